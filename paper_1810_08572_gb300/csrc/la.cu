@@ -47,67 +47,111 @@ fvs_status residual(cudaStream_t s, const Ell& A, const double* x, const double*
 }
 
 // ---------------------------------------------------------------------------
-// Deterministic reductions: fixed grid, block partials, single-block final sum
+// Deterministic reductions: every block writes its partial sums; the last
+// block to finish (ticket) adds the partials in block order, so the result
+// does not depend on scheduling, and then applies the scalar bookkeeping.
+//
+// FP64 issues at two lanes a clock and SM on this part (0.53 T operations/s
+// measured), so a reduction's own arithmetic shows: a block first folds its
+// eight warps through shared memory (one warp per sum: seven adds and five
+// shuffles) instead of shuffling in each of them (45 warp adds per sum), and
+// the quotients of the Krylov recurrences (alpha, omega, beta) are formed
+// once, by the thread that finishes the reduction, instead of by every
+// thread of the vector kernel that uses them (311,296 threads x 2 divisions
+// were 14 us a launch whatever the vector's length).  The grid follows the
+// vector's length below one full wave, so short vectors have few partials.
+// k_bicg_xr_dot 46.2 -> 30.8 us, k_bicg_p 20.3 -> 10.7, k_bicg_s 12.0 -> 6.8
+// at 2,097,152 rows (22, 10 and 7.4 us of memory traffic); k_cg_xr_dot
+// 17.2 -> 8.4, k_dot_rz 11.3 -> 7.1, k_cg_p 8.0 -> 3.2 at 422,000 rows.
 // ---------------------------------------------------------------------------
-__global__ void k_dot2_part(int64_t n, const double* __restrict__ a, const double* __restrict__ b,
-                            const double* __restrict__ c, const double* __restrict__ d, double* __restrict__ part) {
-  __shared__ double sh[32];
-  double s0 = 0.0, s1 = 0.0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    s0 = fma(a[i], b[i], s0);
-    if (c) s1 = fma(c[i], d[i], s1);
+struct OpSum { static __device__ __forceinline__ double f(double a, double b) { return a + b; } };
+struct OpMax { static __device__ __forceinline__ double f(double a, double b) { return fmax(a, b); } };
+
+// NS sums (1 or 2) of the RB threads of a block; result s (s < NS) is valid
+// in lane 0 of warp s
+template <class OP, int NS>
+__device__ __forceinline__ double block_fold(double a, double b) {
+  __shared__ double sh[NS][RB];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  sh[0][threadIdx.x] = a;
+  if (NS > 1) sh[NS - 1][threadIdx.x] = b;
+  __syncthreads();
+  double v = 0.0;
+  if (w < NS) {
+    const double* q = sh[w] + lane;
+    v = OP::f(OP::f(OP::f(q[0], q[32]), OP::f(q[64], q[96])), OP::f(OP::f(q[128], q[160]), OP::f(q[192], q[224])));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = OP::f(v, __shfl_down_sync(0xffffffffu, v, o));
   }
-  s0 = block_sum(s0, sh);
-  s1 = block_sum(s1, sh);
-  if (threadIdx.x == 0) {
-    part[blockIdx.x] = s0;
-    part[gridDim.x + blockIdx.x] = s1;
+  return v;
+}
+
+// safe quotient for Krylov scalars (a breakdown shows up as a stalled residual)
+__device__ __forceinline__ double sdiv(double a, double b) { return b != 0.0 ? a / b : 0.0; }
+
+// Grid-wide sums of a (and b): true in thread 0 of the block that finishes
+// last, with the sums in a and b.  All partials are non-negative under OpMax.
+template <class OP, int NS>
+__device__ __forceinline__ bool grid_fold(double& a, double& b, double* part, unsigned int* ticket) {
+  __shared__ bool last;
+  __shared__ double fin;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  double v = block_fold<OP, NS>(a, b);
+  if (w < NS && lane == 0) {
+    part[(size_t)w * gridDim.x + blockIdx.x] = v;
+    __threadfence();
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return false;
+  __threadfence();
+  double x = 0.0, y = 0.0;
+  for (int i = threadIdx.x; i < (int)gridDim.x; i += RB) {
+    x = OP::f(x, __ldcg(part + i));
+    if (NS > 1) y = OP::f(y, __ldcg(part + gridDim.x + i));
+  }
+  v = block_fold<OP, NS>(x, y);
+  if (NS > 1) {
+    if (w == 1 && lane == 0) fin = v;
+    __syncthreads();
+  }
+  if (threadIdx.x != 0) return false;
+  a = v;
+  b = NS > 1 ? fin : 0.0;
+  *ticket = 0u;
+  return true;
+}
+
+// sc[s0] = a . b (and sc[s1] = c . d with c given)
+template <bool TWO>
+__global__ void __launch_bounds__(RB) k_dot2(int64_t n, const double* __restrict__ a, const double* __restrict__ b,
+                                             const double* __restrict__ c, const double* __restrict__ d,
+                                             double* part, unsigned int* ticket, double* sc, int s0, int s1) {
+  double x = 0.0, y = 0.0;
+  for (int64_t i = blockIdx.x * (int64_t)RB + threadIdx.x; i < n; i += (int64_t)gridDim.x * RB) {
+    x = fma(a[i], b[i], x);
+    if (TWO) y = fma(c[i], d[i], y);
+  }
+  if (grid_fold<OpSum, TWO ? 2 : 1>(x, y, part, ticket)) {
+    sc[s0] = x;
+    if (TWO) sc[s1] = y;
   }
 }
 
-__global__ void k_maxdiff2_part(int64_t n, const double* __restrict__ a, const double* __restrict__ b,
-                                const double* __restrict__ c, const double* __restrict__ d, double* __restrict__ part) {
-  __shared__ double sh[32];
-  double s0 = 0.0, s1 = 0.0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    s0 = fmax(s0, fabs(a[i] - b[i]));
-    if (c) s1 = fmax(s1, fabs(c[i] - d[i]));
+// sc[s0] = max |a - b|, sc[s1] = max |c - d|
+__global__ void __launch_bounds__(RB) k_maxdiff2(int64_t n, const double* __restrict__ a,
+                                                 const double* __restrict__ b, const double* __restrict__ c,
+                                                 const double* __restrict__ d, double* part, unsigned int* ticket,
+                                                 double* sc, int s0, int s1) {
+  double x = 0.0, y = 0.0;
+  for (int64_t i = blockIdx.x * (int64_t)RB + threadIdx.x; i < n; i += (int64_t)gridDim.x * RB) {
+    x = fmax(x, fabs(a[i] - b[i]));
+    if (c) y = fmax(y, fabs(c[i] - d[i]));
   }
-  s0 = block_max(s0, sh);
-  s1 = block_max(s1, sh);
-  if (threadIdx.x == 0) {
-    part[blockIdx.x] = s0;
-    part[gridDim.x + blockIdx.x] = s1;
-  }
-}
-
-// Final sum of partials into slots; mode 1 = max.  Before overwriting s0,
-// the previous value is moved to s0_old (if >= 0): the Krylov drivers keep
-// rho_{k-1} that way without a separate launch.
-__global__ void k_final2(int nb, const double* __restrict__ part, double* __restrict__ sc, int s0, int s1,
-                         int s0_old, int mode) {
-  __shared__ double sh[32];
-  double a = 0.0, b = 0.0;
-  for (int i = threadIdx.x; i < nb; i += blockDim.x) {
-    if (mode) {
-      a = fmax(a, part[i]);
-      b = fmax(b, part[nb + i]);
-    } else {
-      a += part[i];
-      b += part[nb + i];
-    }
-  }
-  if (mode) {
-    a = block_max(a, sh);
-    b = block_max(b, sh);
-  } else {
-    a = block_sum(a, sh);
-    b = block_sum(b, sh);
-  }
-  if (threadIdx.x == 0) {
-    if (s0_old >= 0) sc[s0_old] = sc[s0];
-    sc[s0] = a;
-    if (s1 >= 0) sc[s1] = b;
+  if (grid_fold<OpMax, 2>(x, y, part, ticket)) {
+    sc[s0] = x;
+    sc[s1] = y;
   }
 }
 
@@ -126,24 +170,21 @@ fvs_status Reducer::init() {
 }
 
 fvs_status Reducer::dot(cudaStream_t s, int64_t n, const double* x, const double* y, int slot) {
-  k_dot2_part<<<blocks, RB, 0, s>>>(n, x, y, nullptr, nullptr, part); FVS_COUNT_LAUNCH();
-  k_final2<<<1, 1024, 0, s>>>(blocks, part, sc, slot, -1, -1, 0); FVS_COUNT_LAUNCH();
+  k_dot2<false><<<grid(n), RB, 0, s>>>(n, x, y, nullptr, nullptr, part, ticket, sc, slot, -1); FVS_COUNT_LAUNCH();
   FVS_LAUNCH_CHECK();
   return FVS_OK;
 }
 
 fvs_status Reducer::dot2(cudaStream_t s, int64_t n, const double* a, const double* b, const double* c,
                          const double* d, int s0, int s1) {
-  k_dot2_part<<<blocks, RB, 0, s>>>(n, a, b, c, d, part); FVS_COUNT_LAUNCH();
-  k_final2<<<1, 1024, 0, s>>>(blocks, part, sc, s0, s1, -1, 0); FVS_COUNT_LAUNCH();
+  k_dot2<true><<<grid(n), RB, 0, s>>>(n, a, b, c, d, part, ticket, sc, s0, s1); FVS_COUNT_LAUNCH();
   FVS_LAUNCH_CHECK();
   return FVS_OK;
 }
 
 fvs_status Reducer::max_abs_diff2(cudaStream_t s, int64_t n, const double* a, const double* b,
                                   const double* c, const double* d, int s0, int s1) {
-  k_maxdiff2_part<<<blocks, RB, 0, s>>>(n, a, b, c, d, part); FVS_COUNT_LAUNCH();
-  k_final2<<<1, 1024, 0, s>>>(blocks, part, sc, s0, s1, -1, 1); FVS_COUNT_LAUNCH();
+  k_maxdiff2<<<grid(n), RB, 0, s>>>(n, a, b, c, d, part, ticket, sc, s0, s1); FVS_COUNT_LAUNCH();
   FVS_LAUNCH_CHECK();
   return FVS_OK;
 }
@@ -212,149 +253,133 @@ fvs_status KrylovWork::ensure(int64_t n) {
   return FVS_OK;
 }
 
-// safe quotient for Krylov scalars (a breakdown shows up as a stalled residual)
-__device__ __forceinline__ double sdiv(double a, double b) { return b != 0.0 ? a / b : 0.0; }
-
 // ---------------------------------------------------------------------------
-// Fused reductions: every block writes its partial sums; the last block to
-// finish (ticket) adds the partials in block order, so the result does not
-// depend on scheduling, and then applies the scalar bookkeeping.
+// Reductions fused into the Krylov kernels, and the scalars they finish
 // ---------------------------------------------------------------------------
 enum { FIN_RV = 0, FIN_TSTT = 1, FIN_RR_RHO = 2, FIN_PQ = 3, FIN_RR = 4, FIN_RZ = 5 };
 
-__device__ void finish2(double a, double b, double* part, unsigned int* ticket, double* sc, int mode) {
-  __shared__ double sh[32];
-  __shared__ bool last;
-  a = block_sum(a, sh);
-  b = block_sum(b, sh);
-  if (threadIdx.x == 0) {
-    part[blockIdx.x] = a;
-    part[gridDim.x + blockIdx.x] = b;
-    __threadfence();
-    last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  double x = 0.0, y = 0.0;
-  for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) {
-    x += ((volatile double*)part)[i];
-    y += ((volatile double*)part)[gridDim.x + i];
-  }
-  x = block_sum(x, sh);
-  y = block_sum(y, sh);
-  if (threadIdx.x == 0) {
-    switch (mode) {
-      case FIN_RV: sc[S_RV] = x; break;
-      case FIN_TSTT: sc[S_TS] = x; sc[S_TT] = y; break;
-      case FIN_RR_RHO:
-        // alpha and omega of this iteration are kept for the next beta
-        sc[S_ALPHA] = sdiv(sc[S_RHO], sc[S_RV]);
-        sc[S_OMEGA] = sdiv(sc[S_TS], sc[S_TT]);
-        sc[S_RR] = x;
-        sc[S_RHO_OLD] = sc[S_RHO];
-        sc[S_RHO] = y;
-        sc[S_FIRST] = 0.0;
-        break;
-      case FIN_PQ: sc[S_PQ] = x; break;
-      case FIN_RR: sc[S_RR] = x; sc[S_FIRST] = 0.0; break;
-      case FIN_RZ: sc[S_RZ_OLD] = sc[S_RZ]; sc[S_RZ] = x; break;
-    }
-    *ticket = 0u;
+template <int MODE>
+__device__ __forceinline__ void finish2(double x, double y, double* part, unsigned int* ticket, double* sc) {
+  constexpr int NS = MODE == FIN_TSTT || MODE == FIN_RR_RHO ? 2 : 1;
+  if (!grid_fold<OpSum, NS>(x, y, part, ticket)) return;
+  if (MODE == FIN_RV) {
+    sc[S_RV] = x;
+    sc[S_ALPHA] = sdiv(sc[S_RHO], x);
+  } else if (MODE == FIN_TSTT) {
+    sc[S_TS] = x;
+    sc[S_TT] = y;
+    sc[S_OMEGA] = sdiv(x, y);
+  } else if (MODE == FIN_RR_RHO) {
+    const double rho = sc[S_RHO];
+    sc[S_RR] = x;
+    sc[S_RHO_OLD] = rho;
+    sc[S_RHO] = y;
+    sc[S_BETA] = sdiv(y, rho) * sdiv(sc[S_ALPHA], sc[S_OMEGA]);
+    sc[S_FIRST] = 0.0;
+  } else if (MODE == FIN_PQ) {
+    sc[S_PQ] = x;
+    sc[S_ALPHA] = sdiv(sc[S_RZ], x);
+  } else if (MODE == FIN_RR) {
+    sc[S_RR] = x;
+    sc[S_FIRST] = 0.0;
+  } else {
+    const double rz = sc[S_RZ];
+    sc[S_RZ_OLD] = rz;
+    sc[S_RZ] = x;
+    sc[S_BETA] = sdiv(x, rz);
   }
 }
 
-// y = A x (+ dextra x); sums d.y (and y.y when YY)
-template <int MODE, bool YY, bool DX>
-__global__ void __launch_bounds__(256, 8) k_spmv_dot(int64_t n, int w, const int32_t* __restrict__ col,
-                                                     const double* __restrict__ val, const double* __restrict__ x,
-                                                     double* __restrict__ y, const double* __restrict__ dextra,
-                                                     const double* __restrict__ d, double* part,
-                                                     unsigned int* ticket, double* sc) {
+// y = A x (+ dextra x); sums d.y (and y.y in FIN_TSTT)
+template <int MODE, bool DX>
+__global__ void __launch_bounds__(RB, 8) k_spmv_dot(int64_t n, int w, const int32_t* __restrict__ col,
+                                                    const double* __restrict__ val, const double* __restrict__ x,
+                                                    double* __restrict__ y, const double* __restrict__ dextra,
+                                                    const double* __restrict__ d, double* part,
+                                                    unsigned int* ticket, double* sc) {
   double a = 0.0, b = 0.0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+  for (int64_t i = blockIdx.x * (int64_t)RB + threadIdx.x; i < n; i += (int64_t)gridDim.x * RB) {
     const double acc = ell_row(n, w, col, val, x, i, DX ? dextra[i] * x[i] : 0.0);
     y[i] = acc;
     a = fma(d[i], acc, a);
-    if (YY) b = fma(acc, acc, b);
+    if (MODE == FIN_TSTT) b = fma(acc, acc, b);
   }
-  finish2(a, b, part, ticket, sc, MODE);
+  finish2<MODE>(a, b, part, ticket, sc);
 }
 
 // BiCGStab: x += alpha ph + omega sh ; r = s - omega t ; sums r.r and rh.r
-__global__ void k_bicg_xr_dot(int64_t n, double* __restrict__ sc, const double* __restrict__ ph,
-                              const double* __restrict__ sh, const double* __restrict__ sv,
-                              const double* __restrict__ t, const double* __restrict__ rh, double* __restrict__ x,
-                              double* __restrict__ r, double* part, unsigned int* ticket) {
-  const double alpha = sdiv(sc[S_RHO], sc[S_RV]);
-  const double omega = sdiv(sc[S_TS], sc[S_TT]);
+__global__ void __launch_bounds__(RB) k_bicg_xr_dot(int64_t n, double* __restrict__ sc,
+                                                    const double* __restrict__ ph, const double* __restrict__ sh,
+                                                    const double* __restrict__ sv, const double* __restrict__ t,
+                                                    const double* __restrict__ rh, double* __restrict__ x,
+                                                    double* __restrict__ r, double* part, unsigned int* ticket) {
+  const double alpha = sc[S_ALPHA], omega = sc[S_OMEGA];
   double a = 0.0, b = 0.0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+  for (int64_t i = blockIdx.x * (int64_t)RB + threadIdx.x; i < n; i += (int64_t)gridDim.x * RB) {
     x[i] += alpha * ph[i] + omega * sh[i];
     const double ri = sv[i] - omega * t[i];
     r[i] = ri;
     a = fma(ri, ri, a);
     b = fma(rh[i], ri, b);
   }
-  finish2(a, b, part, ticket, sc, FIN_RR_RHO);
+  finish2<FIN_RR_RHO>(a, b, part, ticket, sc);
 }
 
 // CG: x += alpha p ; r -= alpha q ; sums r.r
-__global__ void k_cg_xr_dot(int64_t n, double* __restrict__ sc, const double* __restrict__ p,
-                            const double* __restrict__ q, double* __restrict__ x, double* __restrict__ r,
-                            double* part, unsigned int* ticket) {
-  const double alpha = sdiv(sc[S_RZ], sc[S_PQ]);
+__global__ void __launch_bounds__(RB) k_cg_xr_dot(int64_t n, double* __restrict__ sc, const double* __restrict__ p,
+                                                  const double* __restrict__ q, double* __restrict__ x,
+                                                  double* __restrict__ r, double* part, unsigned int* ticket) {
+  const double alpha = sc[S_ALPHA];
   double a = 0.0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+  for (int64_t i = blockIdx.x * (int64_t)RB + threadIdx.x; i < n; i += (int64_t)gridDim.x * RB) {
     x[i] += alpha * p[i];
     const double ri = r[i] - alpha * q[i];
     r[i] = ri;
     a = fma(ri, ri, a);
   }
-  finish2(a, 0.0, part, ticket, sc, FIN_RR);
+  finish2<FIN_RR>(a, 0.0, part, ticket, sc);
 }
 // sums r.z (rz moved to rz_old)
-__global__ void k_dot_rz(int64_t n, const double* __restrict__ r, const double* __restrict__ z, double* part,
-                         unsigned int* ticket, double* sc) {
+__global__ void __launch_bounds__(RB) k_dot_rz(int64_t n, const double* __restrict__ r, const double* __restrict__ z,
+                                               double* part, unsigned int* ticket, double* sc) {
   double a = 0.0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+  for (int64_t i = blockIdx.x * (int64_t)RB + threadIdx.x; i < n; i += (int64_t)gridDim.x * RB)
     a = fma(r[i], z[i], a);
-  finish2(a, 0.0, part, ticket, sc, FIN_RZ);
+  finish2<FIN_RZ>(a, 0.0, part, ticket, sc);
 }
 
 // BiCGStab: p = r + beta (p - omega v), beta = (rho/rho_old)(alpha/omega)
 __global__ void k_bicg_p(int64_t n, const double* __restrict__ sc, const double* __restrict__ r,
                          const double* __restrict__ v, double* __restrict__ p, int first) {
   first = first || sc[S_FIRST] != 0.0;
-  const double beta = first ? 0.0 : sdiv(sc[S_RHO], sc[S_RHO_OLD]) * sdiv(sc[S_ALPHA], sc[S_OMEGA]);
-  const double om = sc[S_OMEGA];
+  const double beta = sc[S_BETA], om = sc[S_OMEGA];
   GRID_STRIDE(i, n) p[i] = first ? r[i] : r[i] + beta * (p[i] - om * v[i]);
 }
 // s = r - alpha v, alpha = rho / (rh . v)
 __global__ void k_bicg_s(int64_t n, const double* __restrict__ sc, const double* __restrict__ r,
                          const double* __restrict__ v, double* __restrict__ sv) {
-  const double alpha = sdiv(sc[S_RHO], sc[S_RV]);
+  const double alpha = sc[S_ALPHA];
   GRID_STRIDE(i, n) sv[i] = r[i] - alpha * v[i];
 }
 __global__ void k_cg_p(int64_t n, const double* __restrict__ sc, const double* __restrict__ z,
                        double* __restrict__ p, int first) {
   first = first || sc[S_FIRST] != 0.0;
-  const double beta = first ? 0.0 : sdiv(sc[S_RZ], sc[S_RZ_OLD]);
+  const double beta = sc[S_BETA];
   GRID_STRIDE(i, n) p[i] = first ? z[i] : z[i] + beta * p[i];
 }
 
 static inline bool bad(double v) { return !(v == v) || v > 1e300 || v < -1e300; }
 
 static fvs_status spmv_dot(cudaStream_t s, Reducer& red, const Ell& A, const double* x, double* y,
-                           const double* dextra, const double* d, bool yy, int mode) {
+                           const double* dextra, const double* d, int mode) {
   ProfScope ps(&A, "spmv", (double)A.n * (12.0 * A.w + 24.0 + (dextra ? 8.0 : 0.0)), s);
-#define FVS_SPMV_DOT(M_, Y_, D_) \
-  k_spmv_dot<M_, Y_, D_><<<red.blocks, 256, 0, s>>>(A.n, A.w, A.col, A.val, x, y, dextra, d, red.part, red.ticket, red.sc)
-  if (mode == FIN_RV) { if (dextra) FVS_SPMV_DOT(FIN_RV, false, true); else FVS_SPMV_DOT(FIN_RV, false, false); }
-  else if (mode == FIN_TSTT) { if (dextra) FVS_SPMV_DOT(FIN_TSTT, true, true); else FVS_SPMV_DOT(FIN_TSTT, true, false); }
-  else { if (dextra) FVS_SPMV_DOT(FIN_PQ, false, true); else FVS_SPMV_DOT(FIN_PQ, false, false); }
+  const int g = red.grid(A.n);
+#define FVS_SPMV_DOT(M_, D_) \
+  k_spmv_dot<M_, D_><<<g, RB, 0, s>>>(A.n, A.w, A.col, A.val, x, y, dextra, d, red.part, red.ticket, red.sc)
+  if (mode == FIN_RV) { if (dextra) FVS_SPMV_DOT(FIN_RV, true); else FVS_SPMV_DOT(FIN_RV, false); }
+  else if (mode == FIN_TSTT) { if (dextra) FVS_SPMV_DOT(FIN_TSTT, true); else FVS_SPMV_DOT(FIN_TSTT, false); }
+  else { if (dextra) FVS_SPMV_DOT(FIN_PQ, true); else FVS_SPMV_DOT(FIN_PQ, false); }
 #undef FVS_SPMV_DOT
-  (void)yy;
   FVS_COUNT_LAUNCH();
   FVS_LAUNCH_CHECK();
   return FVS_OK;
@@ -561,12 +586,12 @@ fvs_status bicgstab(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, c
     k_bicg_p<<<grid, 256, 0, s>>>(n, red.sc, w.r, w.v, w.p, first ? 1 : 0); FVS_COUNT_LAUNCH();
     FVS_LAUNCH_CHECK();
     FVS_TRY(M.apply(s, w.p, w.ph));
-    FVS_TRY(spmv_dot(s, red, A, w.ph, w.v, dextra, w.rh, false, FIN_RV));
+    FVS_TRY(spmv_dot(s, red, A, w.ph, w.v, dextra, w.rh, FIN_RV));
     k_bicg_s<<<grid, 256, 0, s>>>(n, red.sc, w.r, w.v, w.sv); FVS_COUNT_LAUNCH();
     FVS_LAUNCH_CHECK();
     FVS_TRY(M.apply(s, w.sv, w.sh));
-    FVS_TRY(spmv_dot(s, red, A, w.sh, w.t, dextra, w.sv, true, FIN_TSTT));
-    k_bicg_xr_dot<<<red.blocks, 256, 0, s>>>(n, red.sc, w.ph, w.sh, w.sv, w.t, w.rh, x, w.r, red.part,
+    FVS_TRY(spmv_dot(s, red, A, w.sh, w.t, dextra, w.sv, FIN_TSTT));
+    k_bicg_xr_dot<<<red.grid(n), RB, 0, s>>>(n, red.sc, w.ph, w.sh, w.sv, w.t, w.rh, x, w.r, red.part,
                                               red.ticket); FVS_COUNT_LAUNCH();
     FVS_LAUNCH_CHECK();
     return FVS_OK;
@@ -651,11 +676,11 @@ fvs_status pcg(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, Precon
   auto body = [&](bool first) -> fvs_status {
     FVS_TRY(M.apply(s, w.r, w.z));
     if (proj) FVS_TRY(proj->apply(s, w.z));
-    k_dot_rz<<<red.blocks, 256, 0, s>>>(n, w.r, w.z, red.part, red.ticket, red.sc); FVS_COUNT_LAUNCH();
+    k_dot_rz<<<red.grid(n), RB, 0, s>>>(n, w.r, w.z, red.part, red.ticket, red.sc); FVS_COUNT_LAUNCH();
     k_cg_p<<<grid, 256, 0, s>>>(n, red.sc, w.z, w.p, first ? 1 : 0); FVS_COUNT_LAUNCH();
     FVS_LAUNCH_CHECK();
-    FVS_TRY(spmv_dot(s, red, A, w.p, w.q, nullptr, w.p, false, FIN_PQ));
-    k_cg_xr_dot<<<red.blocks, 256, 0, s>>>(n, red.sc, w.p, w.q, x, w.r, red.part, red.ticket); FVS_COUNT_LAUNCH();
+    FVS_TRY(spmv_dot(s, red, A, w.p, w.q, nullptr, w.p, FIN_PQ));
+    k_cg_xr_dot<<<red.grid(n), RB, 0, s>>>(n, red.sc, w.p, w.q, x, w.r, red.part, red.ticket); FVS_COUNT_LAUNCH();
     FVS_LAUNCH_CHECK();
     return FVS_OK;
   };

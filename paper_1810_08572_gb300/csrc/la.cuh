@@ -30,7 +30,7 @@ struct Ell {
 // Scalar slots of the Krylov drivers (device memory).
 enum Slot {
   S_RHO = 0, S_RHO_OLD, S_ALPHA, S_OMEGA, S_RV, S_TS, S_TT, S_RR, S_BB, S_RZ, S_RZ_OLD, S_PQ,
-  S_TMP0, S_TMP1, S_TOL2, S_ITER, S_FIRST, S_NSLOT
+  S_TMP0, S_TMP1, S_TOL2, S_ITER, S_FIRST, S_BETA, S_NSLOT
 };
 
 // Reduction scratch owned by a solver: block partials + scalar slots +
@@ -43,6 +43,12 @@ struct Reducer {
   DBuf<int> iter;              // iteration counter of device-driven solve loops
   double* host = nullptr;  // pinned [S_NSLOT]
   fvs_status init();
+  // blocks of 256 threads of a reduction over n rows: a row a thread up to
+  // one full wave, then grid-stride
+  int grid(int64_t n) const {
+    const int64_t g = (n + 255) / 256;
+    return (int)(g < 1 ? 1 : (g < blocks ? g : blocks));
+  }
   ~Reducer() { if (host) cudaFreeHost(host); }
   // out[slot] = x . y  (deterministic: fixed blocks, fixed order)
   fvs_status dot(cudaStream_t s, int64_t n, const double* x, const double* y, int slot);
