@@ -48,6 +48,41 @@ def test_forward_and_gradients_match_fp64_reference(fvs):
     np.testing.assert_allclose(S.get_params(), p * 0.5, rtol=1e-7)
 
 
+@pytest.mark.parametrize("net,rows", [
+    ((3, 128, 4, 4), 1), ((3, 128, 4, 4), 127), ((3, 128, 4, 4), 129), ((3, 128, 4, 4), 3 * 128 * 160 + 5),
+    ((1, 16, 1, 1), 64), ((20, 40, 2, 17), 385), ((128, 128, 1, 128), 130),
+    ((3, 128, 5, 4), 200), ((3, 128, 6, 4), 200),    # two and one tiles a CTA in flight
+    ((3, 128, 8, 4), 300)])                          # weights beyond shared memory: layer by layer
+def test_network_shapes_match_fp64_reference(fvs, net, rows):
+    """Prediction and gradients over the tile edges, padded widths and the
+    network sizes that change how many tiles a CTA holds.  BF16 operands have
+    a relative rounding error of 2^-9; a sum of K products of independently
+    rounded operands keeps that relative error of its root mean square, and
+    each of the L layers adds its own, so the root-mean-square error stays
+    below 2^-8 L of the root-mean-square output (a factor two for the two
+    operands)."""
+    nin, hidden, layers, nout = net
+    sizes = [nin] + [hidden] * layers + [nout]
+    S = fvs.Surrogate(nin, hidden, layers, nout, seed=5)
+    p = S.get_params()
+    params = ref.unflatten(p, sizes)
+    rng = np.random.default_rng(rows)
+    X = rng.normal(size=(rows, nin))
+    T = rng.normal(size=(rows, nout))
+    rms = lambda a: np.sqrt(np.mean(np.square(a)))
+    Y = S.predict(X)
+    Yr, _ = ref.forward(params, X)
+    tol = 2.0 ** -8 * len(sizes)
+    assert rms(Y - Yr) <= tol * rms(Yr)
+    if rows > 1000:
+        X, T = X[:1000], T[:1000]
+    g, loss = S.gradients(X, T)
+    gr = ref.flatten(ref.backward(params, X, T))
+    assert abs(loss - ref.loss(params, X, T)) <= 2 * tol * ref.loss(params, X, T)
+    # back-propagation passes through the layers a second time
+    assert rms(g - gr) <= 2 * tol * rms(gr)
+
+
 def test_adam_steps_match_oracle(fvs):
     """Two full-batch Adam steps on the GPU (FP32 master weights) against the
     FP64 Adam of the oracle fed with the GPU's own gradients at the same
