@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(RB) k_maxdiff2(int64_t n, const double* __rest
   }
   if (grid_fold<OpMax, 2>(x, y, part, ticket)) {
     sc[s0] = x;
-    sc[s1] = y;
+    if (s1 >= 0) sc[s1] = y;
   }
 }
 
