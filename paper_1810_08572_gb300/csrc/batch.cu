@@ -1410,6 +1410,7 @@ struct BMat {
 
 __device__ __forceinline__ FsLaw b_law(FsLaw w, double Tl) {
   w.Tl = Tl;
+  law_derive(w);
   return w;
 }
 
@@ -1791,7 +1792,7 @@ __global__ void kb_energy_base(int64_t Nc, int Sp, int W, const int32_t* cf, con
   }
 }
 // source linearisation at the current iterate (Eq. 20); Jacobi diagonal of the pass
-__global__ void kb_energy_lin(int64_t Nc, int Sp, const double* V, BMat m, const double* Tliq, double dt,
+__global__ void kb_energy_lin(int64_t Nc, int Sp, const double* V, BMat m, const double* Tliq, double idt,
                               const double* Tm, const double* fsm, const double* fsn, const double* base,
                               const double* kevd, double* dextra, double* rhs, double* x, double* jd) {
   BSAMPLE;
@@ -1799,11 +1800,12 @@ __global__ void kb_energy_lin(int64_t Nc, int Sp, const double* V, BMat m, const
   BROW(c, Nc) {
     const int64_t e = c * Sp + s;
     const double t = Tm[e];
-    const double dfs = fs_slope(law, t);
-    const double a = m.rho * m.L * V[c] / dt;
+    const double dfs = fs_slope(law, t, fsm[e]);
+    const double v = V[c] * idt;
+    const double a = m.rho * m.L * v;
     const double Sp_ = a * dfs;
     const double Sc = a * (fsm[e] - fsn[e] - dfs * t);
-    const double dx = m.rho * m.cp * V[c] / dt - Sp_;
+    const double dx = m.rho * m.cp * v - Sp_;
     dextra[e] = dx;
     rhs[e] = base[e] + Sc;
     x[e] = t;
@@ -1822,11 +1824,12 @@ __global__ void kb_energy_update(int64_t Nc, int Sp, BMat m, const double* Tliq,
     const int64_t e = c * Sp + s;
     if (!go) { Tnext[e] = Tm[e]; fsnext[e] = fsm[e]; continue; }
     const double t = Tm[e];
-    const double dfs = fs_slope(law, t);
-    const double H = m.cp * Tlin[e] + m.L * (1.0 - fsm[e] - dfs * (Tlin[e] - t));
-    const double T = T_of_H(law, m.cp, m.L, H);
-    Tnext[e] = T;
-    fsnext[e] = fs_of(law, T);
+    const double f = fsm[e], tl = Tlin[e];
+    const double dfs = fs_slope(law, t, f);
+    const double H = m.cp * tl + m.L * (1.0 - f - dfs * (tl - t));
+    double fs;
+    Tnext[e] = T_of_H(law, H, t, fs);
+    fsnext[e] = fs;
   }
 }
 // first iterate of the latent-heat loop: T^n extrapolated linearly in time
@@ -2221,7 +2224,7 @@ static fvs_status batch_step(Batch& B, double dt, int& failures, int (&its)[4]) 
     a.maxit = B.props.max_krylov_iters;
     int left = 1;
     for (int it = 1; it <= B.props.max_e_iters && left > 0; ++it) {
-      kb_energy_lin<<<gc, blk, 0, st>>>(Nc, Sp, m->V, mt, B.Tliq, dt, B.Tnew, B.fsnew, B.fs, B.ebase, B.kevd, B.edx,
+      kb_energy_lin<<<gc, blk, 0, st>>>(Nc, Sp, m->V, mt, B.Tliq, 1.0 / dt, B.Tnew, B.fsnew, B.fs, B.ebase, B.kevd, B.edx,
                                         B.erhs, B.Tlin, B.jd); FVS_COUNT_LAUNCH();
       int it2 = 0, fail = 0;
       FVS_TRY(bbicgstab(B, op, J, np, B.erhs, B.Tlin, a, it2, fail, &B.ge));

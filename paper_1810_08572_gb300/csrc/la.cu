@@ -3,10 +3,9 @@
 #include <cstdlib>
 
 #include "la.cuh"
+#include "reduce.cuh"
 
 namespace fvs {
-
-static constexpr int RB = 256;  // threads per reduction block
 
 // ---------------------------------------------------------------------------
 // SpMV and residual (ELL, one thread per row, slot-major coalesced loads)
@@ -44,83 +43,6 @@ fvs_status residual(cudaStream_t s, const Ell& A, const double* x, const double*
   k_residual<<<stride_grid(A.n, 256), 256, 0, s>>>(A.n, A.w, A.col, A.val, x, b, r, dextra); FVS_COUNT_LAUNCH();
   FVS_LAUNCH_CHECK();
   return FVS_OK;
-}
-
-// ---------------------------------------------------------------------------
-// Deterministic reductions: every block writes its partial sums; the last
-// block to finish (ticket) adds the partials in block order, so the result
-// does not depend on scheduling, and then applies the scalar bookkeeping.
-//
-// FP64 issues at two lanes a clock and SM on this part (0.53 T operations/s
-// measured), so a reduction's own arithmetic shows: a block first folds its
-// eight warps through shared memory (one warp per sum: seven adds and five
-// shuffles) instead of shuffling in each of them (45 warp adds per sum), and
-// the quotients of the Krylov recurrences (alpha, omega, beta) are formed
-// once, by the thread that finishes the reduction, instead of by every
-// thread of the vector kernel that uses them (311,296 threads x 2 divisions
-// were 14 us a launch whatever the vector's length).  The grid follows the
-// vector's length below one full wave, so short vectors have few partials.
-// k_bicg_xr_dot 46.2 -> 30.8 us, k_bicg_p 20.3 -> 10.7, k_bicg_s 12.0 -> 6.8
-// at 2,097,152 rows (22, 10 and 7.4 us of memory traffic); k_cg_xr_dot
-// 17.2 -> 8.4, k_dot_rz 11.3 -> 7.1, k_cg_p 8.0 -> 3.2 at 422,000 rows.
-// ---------------------------------------------------------------------------
-struct OpSum { static __device__ __forceinline__ double f(double a, double b) { return a + b; } };
-struct OpMax { static __device__ __forceinline__ double f(double a, double b) { return fmax(a, b); } };
-
-// NS sums (1 or 2) of the RB threads of a block; result s (s < NS) is valid
-// in lane 0 of warp s
-template <class OP, int NS>
-__device__ __forceinline__ double block_fold(double a, double b) {
-  __shared__ double sh[NS][RB];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  sh[0][threadIdx.x] = a;
-  if (NS > 1) sh[NS - 1][threadIdx.x] = b;
-  __syncthreads();
-  double v = 0.0;
-  if (w < NS) {
-    const double* q = sh[w] + lane;
-    v = OP::f(OP::f(OP::f(q[0], q[32]), OP::f(q[64], q[96])), OP::f(OP::f(q[128], q[160]), OP::f(q[192], q[224])));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = OP::f(v, __shfl_down_sync(0xffffffffu, v, o));
-  }
-  return v;
-}
-
-// safe quotient for Krylov scalars (a breakdown shows up as a stalled residual)
-__device__ __forceinline__ double sdiv(double a, double b) { return b != 0.0 ? a / b : 0.0; }
-
-// Grid-wide sums of a (and b): true in thread 0 of the block that finishes
-// last, with the sums in a and b.  All partials are non-negative under OpMax.
-template <class OP, int NS>
-__device__ __forceinline__ bool grid_fold(double& a, double& b, double* part, unsigned int* ticket) {
-  __shared__ bool last;
-  __shared__ double fin;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  double v = block_fold<OP, NS>(a, b);
-  if (w < NS && lane == 0) {
-    part[(size_t)w * gridDim.x + blockIdx.x] = v;
-    __threadfence();
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-  __syncthreads();
-  if (!last) return false;
-  __threadfence();
-  double x = 0.0, y = 0.0;
-  for (int i = threadIdx.x; i < (int)gridDim.x; i += RB) {
-    x = OP::f(x, __ldcg(part + i));
-    if (NS > 1) y = OP::f(y, __ldcg(part + gridDim.x + i));
-  }
-  v = block_fold<OP, NS>(x, y);
-  if (NS > 1) {
-    if (w == 1 && lane == 0) fin = v;
-    __syncthreads();
-  }
-  if (threadIdx.x != 0) return false;
-  a = v;
-  b = NS > 1 ? fin : 0.0;
-  *ticket = 0u;
-  return true;
 }
 
 // sc[s0] = a . b (and sc[s1] = c . d with c given)
@@ -253,14 +175,17 @@ fvs_status KrylovWork::ensure(int64_t n) {
   return FVS_OK;
 }
 
+// safe quotient for Krylov scalars (a breakdown shows up as a stalled residual)
+__device__ __forceinline__ double sdiv(double a, double b) { return b != 0.0 ? a / b : 0.0; }
+
 // ---------------------------------------------------------------------------
 // Reductions fused into the Krylov kernels, and the scalars they finish
 // ---------------------------------------------------------------------------
-enum { FIN_RV = 0, FIN_TSTT = 1, FIN_RR_RHO = 2, FIN_PQ = 3, FIN_RR = 4, FIN_RZ = 5 };
+enum { FIN_RV = 0, FIN_TSTT = 1, FIN_RR_RHO = 2, FIN_PQ = 3, FIN_RR = 4, FIN_RZ = 5, FIN_START = 6, FIN_TRUE = 7 };
 
 template <int MODE>
 __device__ __forceinline__ void finish2(double x, double y, double* part, unsigned int* ticket, double* sc) {
-  constexpr int NS = MODE == FIN_TSTT || MODE == FIN_RR_RHO ? 2 : 1;
+  constexpr int NS = MODE == FIN_TSTT || MODE == FIN_RR_RHO || MODE == FIN_START ? 2 : 1;
   if (!grid_fold<OpSum, NS>(x, y, part, ticket)) return;
   if (MODE == FIN_RV) {
     sc[S_RV] = x;
@@ -282,6 +207,11 @@ __device__ __forceinline__ void finish2(double x, double y, double* part, unsign
   } else if (MODE == FIN_RR) {
     sc[S_RR] = x;
     sc[S_FIRST] = 0.0;
+  } else if (MODE == FIN_START) {
+    sc[S_RR] = sc[S_RHO] = x;
+    sc[S_BB] = y;
+  } else if (MODE == FIN_TRUE) {
+    sc[S_RR] = x;
   } else {
     const double rz = sc[S_RZ];
     sc[S_RZ_OLD] = rz;
@@ -305,6 +235,32 @@ __global__ void __launch_bounds__(RB, 8) k_spmv_dot(int64_t n, int w, const int3
     if (MODE == FIN_TSTT) b = fma(acc, acc, b);
   }
   finish2<MODE>(a, b, part, ticket, sc);
+}
+
+// BiCGStab without a projection: start (r = rh = b - A x, sums r.r = rh.r and
+// b.b) and end (r.r of the true residual, r itself not stored) in one launch
+// each instead of a residual, a copy and two dot products (2,097,152 rows of
+// 27 entries: 128 and 124 us, the residual alone 126 us; at 184,320 rows 19
+// and 17 us, where the separate launches took 45 and 31)
+template <int MODE, bool DX>
+__global__ void __launch_bounds__(RB, 8) k_residual_dot(int64_t n, int w, const int32_t* __restrict__ col,
+                                                        const double* __restrict__ val, const double* __restrict__ x,
+                                                        const double* __restrict__ dextra,
+                                                        const double* __restrict__ b, double* __restrict__ r,
+                                                        double* __restrict__ rh, double* part,
+                                                        unsigned int* ticket, double* sc) {
+  double rr = 0.0, bb = 0.0;
+  for (int64_t i = blockIdx.x * (int64_t)RB + threadIdx.x; i < n; i += (int64_t)gridDim.x * RB) {
+    const double acc = ell_row(n, w, col, val, x, i, DX ? dextra[i] * x[i] : 0.0);
+    const double bi = b[i], ri = bi - acc;
+    if (MODE == FIN_START) {
+      r[i] = ri;
+      rh[i] = ri;
+      bb = fma(bi, bi, bb);
+    }
+    rr = fma(ri, ri, rr);
+  }
+  finish2<MODE>(rr, bb, part, ticket, sc);
 }
 
 // BiCGStab: x += alpha ph + omega sh ; r = s - omega t ; sums r.r and rh.r
@@ -380,6 +336,22 @@ static fvs_status spmv_dot(cudaStream_t s, Reducer& red, const Ell& A, const dou
   else if (mode == FIN_TSTT) { if (dextra) FVS_SPMV_DOT(FIN_TSTT, true); else FVS_SPMV_DOT(FIN_TSTT, false); }
   else { if (dextra) FVS_SPMV_DOT(FIN_PQ, true); else FVS_SPMV_DOT(FIN_PQ, false); }
 #undef FVS_SPMV_DOT
+  FVS_COUNT_LAUNCH();
+  FVS_LAUNCH_CHECK();
+  return FVS_OK;
+}
+
+template <int MODE>
+static fvs_status residual_dot(cudaStream_t s, Reducer& red, const Ell& A, const double* x, const double* dextra,
+                               const double* b, double* r, double* rh) {
+  ProfScope ps(&A, "residual", (double)A.n * (12.0 * A.w + (MODE == FIN_START ? 32.0 : 16.0) + (dextra ? 8.0 : 0.0)), s);
+  const int g = red.grid(A.n);
+  if (dextra)
+    k_residual_dot<MODE, true><<<g, RB, 0, s>>>(A.n, A.w, A.col, A.val, x, dextra, b, r, rh, red.part, red.ticket,
+                                                red.sc);
+  else
+    k_residual_dot<MODE, false><<<g, RB, 0, s>>>(A.n, A.w, A.col, A.val, x, dextra, b, r, rh, red.part, red.ticket,
+                                                 red.sc);
   FVS_COUNT_LAUNCH();
   FVS_LAUNCH_CHECK();
   return FVS_OK;
@@ -558,18 +530,18 @@ fvs_status bicgstab(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, c
   }
   FVS_TRY(w.ensure(n));
   const int grid = stride_grid(n, 256);
-  FVS_TRY(residual(s, A, x, b, w.r, dextra));
-  if (proj) FVS_TRY(proj->apply(s, w.r));
-  FVS_TRY(vcopy(s, n, w.r, w.rh));
-  // ||b|| of the (projected) right side; rho_0 = rh . r
-  const double* bb = b;
-  if (proj) {
+  // r = rh = b - A x; ||b|| of the (projected) right side; rho_0 = rh . r
+  if (!proj) {
+    FVS_TRY(residual_dot<FIN_START>(s, red, A, x, dextra, b, w.r, w.rh));
+  } else {
+    FVS_TRY(residual(s, A, x, b, w.r, dextra));
+    FVS_TRY(proj->apply(s, w.r));
+    FVS_TRY(vcopy(s, n, w.r, w.rh));
     FVS_TRY(vcopy(s, n, b, w.q));
     FVS_TRY(proj->apply(s, w.q));
-    bb = w.q;
+    FVS_TRY(red.dot2(s, n, w.q, w.q, w.r, w.r, S_BB, S_RR));
+    FVS_TRY(red.dot(s, n, w.rh, w.r, S_RHO));
   }
-  FVS_TRY(red.dot2(s, n, bb, bb, w.r, w.r, S_BB, S_RR));
-  FVS_TRY(red.dot(s, n, w.rh, w.r, S_RHO));
   FVS_TRY(red.fetch(s));
   double bnorm = fmax(sqrt(red.host[S_BB]), bnorm_floor);
   if (bnorm == 0.0) bnorm = 1.0;
@@ -633,9 +605,13 @@ fvs_status bicgstab(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, c
     }
   }
   // recompute the true residual (the recursive one drifts)
-  FVS_TRY(residual(s, A, x, b, w.r, dextra));
-  if (proj) FVS_TRY(proj->apply(s, w.r));
-  FVS_TRY(red.dot(s, n, w.r, w.r, S_RR));
+  if (!proj) {
+    FVS_TRY(residual_dot<FIN_TRUE>(s, red, A, x, dextra, b, nullptr, nullptr));
+  } else {
+    FVS_TRY(residual(s, A, x, b, w.r, dextra));
+    FVS_TRY(proj->apply(s, w.r));
+    FVS_TRY(red.dot(s, n, w.r, w.r, S_RR));
+  }
   FVS_TRY(red.fetch(s));
   res.relres = sqrt(red.host[S_RR]) / bnorm;
   res.converged = res.relres <= rtol * 10.0 && !bad(res.relres);

@@ -13,6 +13,7 @@
 #include <cmath>
 
 #include "fslaw.cuh"
+#include "reduce.cuh"
 #include "solver.cuh"
 
 extern "C" const char* fvs_last_error(void);
@@ -530,17 +531,18 @@ __global__ void k_energy_base(int64_t Nc, int W, const int32_t* cf, const int8_t
 }
 
 // source linearisation at the current iterate (Eq. 20): S_p, S_c
-__global__ void k_energy_lin(int64_t Nc, const double* V, Mat m, double dt, const double* Tm, const double* fsm,
+__global__ void k_energy_lin(int64_t Nc, const double* V, Mat m, double idt, const double* Tm, const double* fsm,
                              const double* fsn, const double* base, double* dextra, double* rhs, double* x,
                              const double* rcp, const double* rL, const uint8_t* metal, const double* kdiag,
                              double* jinv) {
   GS(c, Nc) {
-    const double t = Tm[c];
-    const double dfs = metal[c] ? fs_slope(m.law, t) : 0.0;
-    const double a = rL[c] * V[c] / dt;
+    const double t = Tm[c], f = fsm[c];
+    const double dfs = metal[c] ? fs_slope(m.law, t, f) : 0.0;
+    const double v = V[c] * idt;
+    const double a = rL[c] * v;
     const double Sp = a * dfs;
-    const double Sc = a * (fsm[c] - fsn[c] - dfs * t);
-    const double dx = rcp[c] * V[c] / dt - Sp;
+    const double Sc = a * (f - fsn[c] - dfs * t);
+    const double dx = rcp[c] * v - Sp;
     dextra[c] = dx;
     jinv[c] = 1.0 / (kdiag[c] + dx);   // Jacobi preconditioner of the pass
     rhs[c] = base[c] + Sc;
@@ -553,21 +555,34 @@ __global__ void k_inverse(int64_t n, const double* a, double* inv) {
 }
 
 // enthalpy-to-temperature inversion of the linearised update:
-// H = cp T_lin + L (1 - fs^m - dfs (T_lin - T^m)), T = H^-1(H), fs = fs(T)
-__global__ void k_energy_update(int64_t Nc, Mat m, const double* Tlin, const double* Tm, const double* fsm,
-                                double* Tnext, double* fsnext, const uint8_t* metal) {
-  GS(c, Nc) {
-    if (!metal[c]) {      // mold: no latent heat
-      Tnext[c] = Tlin[c];
-      fsnext[c] = 0.0;
-      continue;
+// H = cp T_lin + L (1 - fs^m - dfs (T_lin - T^m)), T = H^-1(H), fs = fs(T),
+// and the largest changes max |T - T^m|, max |fs - fs^m| (the stop rule) into
+// sc[s0], sc[s1].  Bound by the FP64 pipe: with the law's quotients formed
+// beforehand 130 us at 2,097,152 cells (139 us, and 19 us for the maxima in
+// launches of their own, before); Scheil law, 184,320 cells: 75 us (423 us
+// before, Newton's method from T_liq and three more powers a cell).
+__global__ void __launch_bounds__(RB) k_energy_update(int64_t Nc, Mat m, const double* __restrict__ Tlin,
+                                                      const double* __restrict__ Tm, const double* __restrict__ fsm,
+                                                      double* __restrict__ Tnext, double* __restrict__ fsnext,
+                                                      const uint8_t* __restrict__ metal, double* part,
+                                                      unsigned int* ticket, double* sc, int s0, int s1) {
+  double dT = 0.0, df = 0.0;
+  for (int64_t c = blockIdx.x * (int64_t)RB + threadIdx.x; c < Nc; c += (int64_t)gridDim.x * RB) {
+    const double tl = Tlin[c], t = Tm[c], f = fsm[c];
+    double T = tl, fs = 0.0;      // mold: no latent heat
+    if (metal[c]) {
+      const double dfs = fs_slope(m.law, t, f);
+      const double H = m.cp * tl + m.L * (1.0 - f - dfs * (tl - t));
+      T = T_of_H(m.law, H, t, fs);
     }
-    const double t = Tm[c];
-    const double dfs = fs_slope(m.law, t);
-    const double H = m.cp * Tlin[c] + m.L * (1.0 - fsm[c] - dfs * (Tlin[c] - t));
-    const double T = T_of_H(m.law, m.cp, m.L, H);
     Tnext[c] = T;
-    fsnext[c] = fs_of(m.law, T);
+    fsnext[c] = fs;
+    dT = fmax(dT, fabs(T - t));
+    df = fmax(df, fabs(fs - f));
+  }
+  if (grid_fold<OpMax, 2>(dT, df, part, ticket)) {
+    sc[s0] = dT;
+    sc[s1] = df;
   }
 }
 
@@ -1378,12 +1393,12 @@ fvs_status solver_step(fvs_solver s, double dt, fvs_step_stats* stats) {
     J.dinv = s->jinv_m;
     // the three components are judged against the largest right side (a
     // component with a near-zero right side would otherwise chase roundoff)
+    const int slot[3] = {S_TMP0, S_TMP1, S_TS};
+    for (int d = 0; d < 3; ++d)
+      FVS_TRY(s->red.dot(st, na, s->mrhs.p + d * na, s->mrhs.p + d * na, slot[d]));
+    FVS_TRY(s->red.fetch(st));
     double bmax = 0.0;
-    for (int d = 0; d < 3; ++d) {
-      FVS_TRY(s->red.dot(st, na, s->mrhs.p + d * na, s->mrhs.p + d * na, S_TMP0 + (d == 2 ? 0 : d)));
-      FVS_TRY(s->red.fetch(st));
-      bmax = std::max(bmax, sqrt(s->red.host[S_TMP0 + (d == 2 ? 0 : d)]));
-    }
+    for (int d = 0; d < 3; ++d) bmax = std::max(bmax, sqrt(s->red.host[slot[d]]));
     for (int d = 0; d < 3; ++d) {
       SolveResult r;
       FVS_TRY(bicgstab(st, s->red, s->kw, s->M, nullptr, J, s->mrhs.p + d * na, s->mx.p + d * na,
@@ -1502,7 +1517,7 @@ fvs_status solver_step(fvs_solver s, double dt, fvs_step_stats* stats) {
       // inexact inner solves: early passes only need to resolve a fraction
       // of the nonlinear change; the last passes reach e_rtol
       const double rtol_m = std::max(s->props.e_rtol, std::min(1e-4, 1e-5 * dT_prev));
-      k_energy_lin<<<stride_grid(Nc, 256), 256, 0, st>>>(Nc, m->V, mt, dt, Tm, fsm, s->fs, s->ebase, s->edx,
+      k_energy_lin<<<stride_grid(Nc, 256), 256, 0, st>>>(Nc, m->V, mt, 1.0 / dt, Tm, fsm, s->fs, s->ebase, s->edx,
                                                           s->erhs, s->Tlin, s->rcp, s->rL, s->metal, s->Ke.diag,
                                                           s->jinv_e);
       FVS_COUNT_LAUNCH();
@@ -1517,10 +1532,10 @@ fvs_status solver_step(fvs_solver s, double dt, fvs_step_stats* stats) {
         set_error("energy pass %d: relative residual %.3e after %d iterations", it, r.relres, r.iters);
       }
       // next iterate, then its change against the current one
-      k_energy_update<<<stride_grid(Nc, 256), 256, 0, st>>>(Nc, mt, s->Tlin, Tm, fsm, s->Tit, s->fsit, s->metal);
+      k_energy_update<<<s->red.grid(Nc), RB, 0, st>>>(Nc, mt, s->Tlin, Tm, fsm, s->Tit, s->fsit, s->metal,
+                                                      s->red.part, s->red.ticket, s->red.sc, S_TMP0, S_TMP1);
       FVS_COUNT_LAUNCH();
       FVS_LAUNCH_CHECK();
-      FVS_TRY(s->red.max_abs_diff2(st, Nc, s->Tit, Tm, s->fsit, fsm, S_TMP0, S_TMP1));
       dswap(s->Tit, Tm);
       dswap(s->fsit, fsm);
       FVS_TRY(s->red.fetch(st));
