@@ -524,88 +524,234 @@ __global__ void k_max_int(int64_t n, const int32_t* a, int* out) {
 
 // ---------------------------------------------------------------------------
 // coarsest level: dense copy, connected parts, pins, Gauss-Jordan inverse.
-// Larger coarsest levels (n > SMEM_COARSEST) are inverted in place in global
-// memory by the whole GPU: one small pivot launch and one elimination launch
-// per column (FP64 arithmetic is scarce on this part, so the O(n^3) work is
-// spread over every SM instead of one block).
+// Larger coarsest levels (n > SMEM_COARSEST) are inverted in global memory by
+// the whole GPU, DB columns a launch: n^3 FP64 multiply-adds at 0.53 T/s are
+// 1.2 ms for 850 rows and the block steps take 3.8 ms (70 us each; 0.7 ms at
+// 330 rows), where a pivot and an elimination launch per column took 11.3 ms
+// (6.6 us each, bound by latency) and parts and folds 3.2 ms.
 // ---------------------------------------------------------------------------
 __global__ void k_dense_fill(int n, int w, const int32_t* col, const double* val, double* M) {
   GS(i, n) {
     for (int k = 0; k < w; ++k) M[(int64_t)i * n + col[(int64_t)k * n + i]] += val[(int64_t)k * n + i];
   }
 }
-// Connected parts of the symmetric pattern of M: the block builds a bit
-// matrix of the pattern and the row sums in shared memory, then one thread
-// runs a breadth-first search over 32-bit words.  Each singular part (zero
-// row sums) gets its first (lowest) row pinned.  'order' lists the rows
-// grouped by part, parts in order of discovery.
+// Connected parts of the pattern (either direction couples), one block: every
+// row starts with its own index as label, takes the smallest label across
+// its nonzero entries, and follows labels to their root between the rounds
+// (a label is never larger than its row, so the walk ends; at most n rounds,
+// a few in practice).  Parts are numbered by their smallest row; a singular
+// part (row sums zero) pins that row: its row of M becomes the identity's.
 static constexpr int DENSE_PARTS_MAX = 1024;
-static size_t dense_parts_smem(int n) {
-  const size_t nw = (size_t)(n + 31) / 32;
-  return 2 * (size_t)n * sizeof(double) + ((size_t)n * nw + nw + (size_t)n) * sizeof(uint32_t);
+__global__ void __launch_bounds__(1024) k_dense_parts(int n, int w, const int32_t* col, const double* val, double* M,
+                                                      int32_t* lab, uint8_t* sing, int* ncomp_out) {
+  __shared__ int lb[DENSE_PARTS_MAX], id[DENSE_PARTS_MAX];
+  __shared__ double rs[DENSE_PARTS_MAX], dg[DENSE_PARTS_MAX];
+  __shared__ uint8_t sg[DENSE_PARTS_MAX];
+  __shared__ int changed;
+  const int i = threadIdx.x;
+  const bool in = i < n;
+  if (in) {
+    double r = 0.0, d = 0.0;
+    for (int k = 0; k < w; ++k) {
+      const double v = val[(int64_t)k * n + i];
+      r += v;
+      if (col[(int64_t)k * n + i] == i) d += v;
+    }
+    rs[i] = r;
+    dg[i] = fabs(d);
+    lb[i] = i;
+  }
+  __syncthreads();
+  for (int round = 0; round < n; ++round) {
+    if (i == 0) changed = 0;
+    __syncthreads();
+    if (in) {
+      int m = lb[i];
+      const int m0 = m;
+      for (int k = 0; k < w; ++k) {
+        if (val[(int64_t)k * n + i] == 0.0) continue;
+        const int j = col[(int64_t)k * n + i];
+        m = min(m, atomicMin(&lb[j], m));
+      }
+      if (m < m0) atomicMin(&lb[i], m);
+    }
+    __syncthreads();
+    if (in) {
+      int r = lb[i];
+      for (int k = 0; k < n && lb[r] != r; ++k) r = lb[r];
+      if (r < lb[i]) atomicMin(&lb[i], r);
+    }
+    __syncthreads();
+    if (in) {
+      // every coupling has to join equal labels before the rounds end
+      for (int k = 0; k < w; ++k)
+        if (val[(int64_t)k * n + i] != 0.0 && lb[col[(int64_t)k * n + i]] != lb[i]) changed = 1;
+    }
+    __syncthreads();
+    const int go = changed;
+    __syncthreads();
+    if (!go) break;
+  }
+  // numbers of the parts: smallest rows in order
+  if (in) {
+    int k = 0;
+    for (int j = 0; j < i; ++j) k += lb[j] == j ? 1 : 0;
+    id[i] = k;   // parts with a smaller first row
+    if (i == n - 1) *ncomp_out = k + (lb[i] == i ? 1 : 0);
+  }
+  __syncthreads();
+  if (in && lb[i] == i) {
+    double r = 0.0, sc = 0.0;
+    for (int j = i; j < n; ++j)
+      if (lb[j] == i) { r += rs[j]; sc += dg[j]; }
+    sg[i] = fabs(r) <= 1e-9 * sc ? 1 : 0;
+    sing[id[i]] = sg[i];
+  }
+  __syncthreads();
+  if (in) lab[i] = id[lb[i]];
+  for (int q = 0; q < n; ++q) {
+    if (lb[q] != q || !sg[q]) continue;
+    if (in) M[(int64_t)q * n + i] = i == q ? 1.0 : 0.0;
+  }
 }
-__global__ void __launch_bounds__(1024) k_dense_parts(int n, double* M, int32_t* lab, uint8_t* sing, int32_t* order,
-                                                      int* ncomp_out) {
-  extern __shared__ double psm[];
-  const int nw = (n + 31) / 32;
-  double* rs = psm;                                   // [n] row sums
-  double* dg = rs + n;                                // [n] |diagonal|
-  uint32_t* adj = (uint32_t*)(dg + n);                // [n][nw]
-  uint32_t* vis = adj + (size_t)n * nw;               // [nw]
-  int* queue = (int*)(vis + nw);                      // [n]
-  for (int e = threadIdx.x; e < n * nw; e += blockDim.x) adj[e] = 0u;
-  for (int e = threadIdx.x; e < nw; e += blockDim.x) vis[e] = 0u;
-  __syncthreads();
-  for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-    const int i = e / n, j = e - i * n;
-    if (M[e] != 0.0) {
-      atomicOr(&adj[i * nw + (j >> 5)], 1u << (j & 31));
-      atomicOr(&adj[j * nw + (i >> 5)], 1u << (i & 31));
+// One block step of the in-place Gauss-Jordan inverse, from A to B: with K the
+// rows and columns k0 .. k0 + bs - 1 and D = A[K][K],
+//   B[K][K] = D^-1,  B[K][j] = D^-1 A[K][j],  B[i][K] = -A[i][K] D^-1,
+//   B[i][j] = A[i][j] - A[i][K] D^-1 A[K][j].
+// A 32 x 64 tile a block; every block inverts D for itself (16 x 16, rows
+// exchanged within D), then forms G = A[i][K] D^-1 and the rank-16 update.
+// Rows of K take G = -D^-1 and columns of K take the identity for A[K][j],
+// both with A[i][j] = 0, so that all four cases are the one update.
+constexpr int DB = 16, DT_R = 32, DT_C = 64;
+__global__ void __launch_bounds__(256) k_gj_block(int n, int k0, const double* __restrict__ A, double* __restrict__ B,
+                                                  int* err) {
+  __shared__ double D[DB][DB + 1], G[DT_R][DB + 1], C[DT_R][DB + 1], Rt[DB][DT_C];
+  __shared__ int prow[DB];
+  const int t = threadIdx.x, bs = min(DB, n - k0);
+  const int i0 = blockIdx.y * DT_R, j0 = blockIdx.x * DT_C;
+  {
+    const int r = t >> 4, c = t & 15;
+    D[r][c] = (r < bs && c < bs) ? A[(int64_t)(k0 + r) * n + k0 + c] : (r == c ? 1.0 : 0.0);
+    for (int q = t; q < DT_R * DB; q += 256) {
+      const int i = i0 + (q >> 4), k = q & 15;
+      C[q >> 4][k] = (i < n && k < bs) ? A[(int64_t)i * n + k0 + k] : 0.0;
+    }
+    for (int q = t; q < DB * DT_C; q += 256) {
+      const int k = q >> 6, j = j0 + (q & 63);
+      const bool inK = j >= k0 && j < k0 + bs;
+      Rt[k][q & 63] = (k < bs && j < n) ? (inK ? (j == k0 + k ? 1.0 : 0.0) : A[(int64_t)(k0 + k) * n + j]) : 0.0;
     }
   }
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    double a = 0.0;
-    for (int j = 0; j < n; ++j) a += M[(int64_t)i * n + j];
-    rs[i] = a;
-    dg[i] = fabs(M[(int64_t)i * n + i]);
-  }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int nc = 0, qt = 0;
-    for (int s0 = 0; s0 < n; ++s0) {
-      if ((vis[s0 >> 5] >> (s0 & 31)) & 1u) continue;
-      const int start = qt;
-      int qh = qt;
-      queue[qt++] = s0;
-      vis[s0 >> 5] |= 1u << (s0 & 31);
-      while (qh < qt) {
-        const int i = queue[qh++];
-        lab[i] = nc;
-        for (int w = 0; w < nw; ++w) {
-          uint32_t c = adj[i * nw + w] & ~vis[w];
-          vis[w] |= c;
-          while (c) {
-            const int b = __ffs(c) - 1;
-            c &= c - 1u;
-            queue[qt++] = w * 32 + b;
-          }
-        }
+  // D <- D^-1: Gauss-Jordan with row exchanges, undone as column exchanges
+  for (int k = 0; k < DB; ++k) {
+    if (t < 32) {
+      double best = t >= k && t < DB ? fabs(D[t][k]) : -1.0;
+      int p = t;
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) {
+        const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+        const int op = __shfl_xor_sync(0xffffffffu, p, o);
+        if (ob > best || (ob == best && op < p)) { best = ob; p = op; }
       }
-      double r = 0.0, sc = 0.0;
-      for (int q = start; q < qt; ++q) {
-        r += rs[queue[q]];
-        sc += dg[queue[q]];
+      if (t == 0) {
+        prow[k] = p;
+        if (!(best > 1e-300)) atomicOr(err, 16);
       }
-      const bool sg = fabs(r) <= 1e-9 * sc;
-      sing[nc] = sg ? 1 : 0;
-      if (sg)   // pin the first row of the part: p = 0 there
-        for (int j = 0; j < n; ++j) M[(int64_t)s0 * n + j] = (j == s0) ? 1.0 : 0.0;
-      ++nc;
     }
-    *ncomp_out = nc;
+    __syncthreads();
+    const int p = prow[k], r = t >> 4, c = t & 15;
+    // the pivot row scaled, every other row eliminated, from the old values
+    const double piv = D[p][k], inv = piv != 0.0 ? 1.0 / piv : 0.0;
+    const double prc = c == k ? 1.0 : D[p][c];
+    const int src = r == p ? k : r;     // the row that lands in r
+    const double f = D[src][k];
+    const double v = r == k ? prc * inv : (c == k ? 0.0 : D[src][c]) - f * (prc * inv);
+    __syncthreads();
+    D[r][c] = v;
+    __syncthreads();
+  }
+  for (int k = DB - 1; k >= 0; --k) {
+    const int p = prow[k];
+    if (p != k && t < DB) { const double v = D[t][k]; D[t][k] = D[t][p]; D[t][p] = v; }
+    __syncthreads();
+  }
+  for (int q = t; q < DT_R * DB; q += 256) {
+    const int r = q >> 4, k = q & 15, i = i0 + r;
+    double g = 0.0;
+    if (i >= k0 && i < k0 + bs) {
+      g = -D[i - k0][k];
+    } else {
+#pragma unroll
+      for (int m = 0; m < DB; ++m) g = fma(C[r][m], D[m][k], g);
+    }
+    G[r][k] = g;
   }
   __syncthreads();
-  for (int q = threadIdx.x; q < n; q += blockDim.x) order[q] = queue[q];
+  // 256 threads: eight rows apart by 4 in r, 64 columns as 2 x 32
+  const int tc = t & 31, tr = t >> 5;
+  double acc[4][2];
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const int i = i0 + tr + 8 * a, j = j0 + tc + 32 * c;
+      const bool out = i >= n || j >= n || (i >= k0 && i < k0 + bs) || (j >= k0 && j < k0 + bs);
+      acc[a][c] = out ? 0.0 : A[(int64_t)i * n + j];
+    }
+#pragma unroll
+  for (int k = 0; k < DB; ++k) {
+    const double r0 = Rt[k][tc], r1 = Rt[k][tc + 32];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      const double g = G[tr + 8 * a][k];
+      acc[a][0] = fma(-g, r0, acc[a][0]);
+      acc[a][1] = fma(-g, r1, acc[a][1]);
+    }
+  }
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const int i = i0 + tr + 8 * a, j = j0 + tc + 32 * c;
+      if (i < n && j < n) B[(int64_t)i * n + j] = acc[a][c];
+    }
+}
+// The block steps exchange rows inside a block only.  That is enough for the
+// diagonally dominant systems of the face couplings; to be sure of any other,
+// the inverse is tried on a vector v of numbers in [-1, 1): y = B v, and
+// |A y - v| has to be small against |A| |y| + |v| in every row, else err
+// and the columns are taken one by one with pivots from the whole column.
+__device__ __forceinline__ double probe_entry(int i) {
+  return (double)((uint32_t)(i + 1) * 2654435761u >> 8) * (2.0 / 16777216.0) - 1.0;
+}
+__global__ void k_dense_probe(int n, const double* __restrict__ Minv, double* __restrict__ y) {
+  const int lane = threadIdx.x & 31, row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (row >= n) return;
+  double a = 0.0;
+  for (int j = lane; j < n; j += 32) a = fma(Minv[(int64_t)row * n + j], probe_entry(j), a);
+  a = warp_sum(a);
+  if (lane == 0) y[row] = a;
+}
+__global__ void k_dense_check(int n, int w, const int32_t* col, const double* val, const int32_t* lab,
+                              const uint8_t* sing, const double* y, int* err) {
+  GS(i, n) {
+    bool pinned = sing[lab[i]] != 0;
+    for (int j = 0; j < (int)i && pinned; ++j) pinned = lab[j] != lab[i];
+    const double v = probe_entry((int)i);
+    double z = -v, sc = fabs(v);
+    if (pinned) {
+      z += y[i];
+      sc += fabs(y[i]);
+    } else {
+      for (int k = 0; k < w; ++k) {
+        const double q = val[(int64_t)k * n + i] * y[col[(int64_t)k * n + i]];
+        z += q;
+        sc += fabs(q);
+      }
+    }
+    if (!(fabs(z) <= 1e-9 * sc)) atomicOr(err, 16);
+  }
 }
 // column k: partial pivot (largest |M[i][k]|, i >= k, lowest index on ties),
 // row swap, scaling of the pivot row, elimination factors
@@ -681,28 +827,57 @@ __global__ void k_gj_unswap(int n, double* M, const int32_t* perm, const int* er
     }
   }
 }
-// M <- P M (LEFT) or M P (!LEFT), P v = v - (mean of v on each singular part)
-template <bool LEFT>
-__global__ void k_dense_fold(int n, double* M, const int32_t* lab, const uint8_t* sing, const int32_t* order,
-                             const int* ncomp, const int* err) {
-  if (*err) return;
-  const int ncs = *ncomp;
-  GS(t, n) {
-    int pos = 0;
-    for (int c = 0; c < ncs; ++c) {
-      int cnt = 0;
-      double sum = 0.0;
-      for (int q = pos; q < n && lab[order[q]] == c; ++q, ++cnt)
-        sum += LEFT ? M[(int64_t)order[q] * n + t] : M[(int64_t)t * n + order[q]];
-      if (sing[c]) {
-        const double m = sum / (double)cnt;
-        for (int q = pos; q < pos + cnt; ++q) {
-          if (LEFT) M[(int64_t)order[q] * n + t] -= m;
-          else M[(int64_t)t * n + order[q]] -= m;
-        }
+// M <- P M, P v = v - (mean of v on each singular part): 32 columns a block,
+// 32 threads a column
+__global__ void __launch_bounds__(1024) k_dense_fold_rows(int n, double* M, const int32_t* lab, const uint8_t* sing,
+                                                          const int* ncomp) {
+  __shared__ double sum[32][33];
+  __shared__ int cnt[32];
+  const int tc = threadIdx.x & 31, tr = threadIdx.x >> 5, j = blockIdx.x * 32 + tc;
+  for (int c = 0; c < *ncomp; ++c) {
+    if (!sing[c]) continue;
+    double a = 0.0;
+    int m = 0;
+    for (int i = tr; i < n; i += 32)
+      if (lab[i] == c) {
+        ++m;
+        if (j < n) a += M[(int64_t)i * n + j];
       }
-      pos += cnt;
+    sum[tr][tc] = a;
+    if (tc == 0) cnt[tr] = m;
+    __syncthreads();
+    a = 0.0;
+    m = 0;
+    for (int q = 0; q < 32; ++q) {
+      a += sum[q][tc];
+      m += cnt[q];
     }
+    a /= (double)m;
+    if (j < n)
+      for (int i = tr; i < n; i += 32)
+        if (lab[i] == c) M[(int64_t)i * n + j] -= a;
+    __syncthreads();
+  }
+}
+// M <- M P: a warp a row
+__global__ void k_dense_fold_cols(int n, double* M, const int32_t* lab, const uint8_t* sing, const int* ncomp) {
+  const int lane = threadIdx.x & 31, row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (row >= n) return;
+  double* Mi = M + (int64_t)row * n;
+  for (int c = 0; c < *ncomp; ++c) {
+    if (!sing[c]) continue;
+    double a = 0.0;
+    int m = 0;
+    for (int j = lane; j < n; j += 32)
+      if (lab[j] == c) { a += Mi[j]; ++m; }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      a += __shfl_xor_sync(0xffffffffu, a, o);
+      m += __shfl_xor_sync(0xffffffffu, m, o);
+    }
+    a /= (double)m;
+    for (int j = lane; j < n; j += 32)
+      if (lab[j] == c) Mi[j] -= a;
   }
 }
 
@@ -1606,62 +1781,44 @@ fvs_status Amg::coarsest_setup(cudaStream_t s) {
       k_coarsest_smem<<<1, 1024, sh, s>>>(nc, A.w, A.col, A.val, Ainv, clab, csing, ncd, err, 1);
       FVS_COUNT_LAUNCH();
     } else {
-      DBuf<double>& fac = gj_fac;
-      DBuf<int32_t>& perm = gj_perm;
-      DBuf<int32_t> order;
-      FVS_TRY(fac.alloc(nc)); FVS_TRY(perm.alloc(nc)); FVS_TRY(order.alloc(nc));
-      FVS_CUDA(cudaMemsetAsync(Ainv.p, 0, (size_t)nc * nc * sizeof(double), s));
-      k_dense_fill<<<stride_grid(nc, 128), 128, 0, s>>>(nc, A.w, A.col, A.val, Ainv); FVS_COUNT_LAUNCH();
-      static bool parts_attr[64] = {false};
-      int dev = 0;
-      cudaGetDevice(&dev);
-      if (dev >= 0 && dev < 64 && !parts_attr[dev]) {
-        FVS_CUDA(cudaFuncSetAttribute(k_dense_parts, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)dense_parts_smem(DENSE_PARTS_MAX)));
-        parts_attr[dev] = true;
+      FVS_TRY(gj_tmp.alloc((size_t)nc * nc + 1)); FVS_TRY(gj_fac.alloc(nc));
+      // the block steps go back and forth between two arrays and end in Ainv
+      const int steps = (nc + DB - 1) / DB;
+      auto fill = [&](double* M) -> fvs_status {
+        FVS_CUDA(cudaMemsetAsync(M, 0, (size_t)nc * nc * sizeof(double), s));
+        k_dense_fill<<<stride_grid(nc, 128), 128, 0, s>>>(nc, A.w, A.col, A.val, M); FVS_COUNT_LAUNCH();
+        k_dense_parts<<<1, 1024, 0, s>>>(nc, A.w, A.col, A.val, M, clab, csing, ncd); FVS_COUNT_LAUNCH();
+        FVS_LAUNCH_CHECK();
+        return FVS_OK;
+      };
+      double* src = (steps & 1) ? gj_tmp.p : Ainv.p;
+      double* dst = (steps & 1) ? Ainv.p : gj_tmp.p;
+      FVS_TRY(fill(src));
+      for (int k0 = 0; k0 < nc; k0 += DB) {
+        k_gj_block<<<dim3((nc + DT_C - 1) / DT_C, (nc + DT_R - 1) / DT_R), 256, 0, s>>>(nc, k0, src, dst, err);
+        FVS_COUNT_LAUNCH();
+        std::swap(src, dst);
       }
-      k_dense_parts<<<1, 1024, dense_parts_smem(nc), s>>>(nc, Ainv, clab, csing, order, ncd); FVS_COUNT_LAUNCH();
-      const int eb = std::min(nc, 4 * sm_count());
-      // 2 nc launches whose cost is mostly launch latency: capture them once
-      // per level size and buffer set, then replay the graph
-      const uint64_t key = ((uint64_t)nc << 40) ^ (uint64_t)(uintptr_t)Ainv.p ^ ((uint64_t)(uintptr_t)fac.p << 1) ^
-                           ((uint64_t)(uintptr_t)perm.p << 2) ^ ((uint64_t)(uintptr_t)err.p << 3) ^ (uint64_t)eb;
-      bool replayed = false;
-      if (graphs_enabled() && s != nullptr) {
-        if (!gj_exec || gj_key != key) {
-          if (gj_exec) cudaGraphExecDestroy(gj_exec);
-          gj_exec = nullptr;
-          gj_key = 0;
-          cudaGraph_t g = nullptr;
-          if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
-            for (int k = 0; k < nc; ++k) {
-              k_gj_pivot<<<1, 256, 0, s>>>(nc, k, Ainv, fac, perm, err);
-              k_gj_elim<<<eb, 128, 0, s>>>(nc, k, Ainv, fac, err);
-            }
-            if (cudaStreamEndCapture(s, &g) == cudaSuccess && g) {
-              if (cudaGraphInstantiate(&gj_exec, g, 0) != cudaSuccess) gj_exec = nullptr;
-              cudaGraphDestroy(g);
-            }
-          }
-          cudaGetLastError();   // a failed capture leaves the eager launches below
-          if (gj_exec) gj_key = key;
-        }
-        if (gj_exec && cudaGraphLaunch(gj_exec, s) == cudaSuccess) {
-          replayed = true;
-          __atomic_add_fetch(&g_launches, 2ULL * (unsigned long long)nc, __ATOMIC_RELAXED);
-        }
-      }
-      if (!replayed) {
+      k_dense_probe<<<(nc + 7) / 8, 256, 0, s>>>(nc, Ainv, gj_fac); FVS_COUNT_LAUNCH();
+      k_dense_check<<<stride_grid(nc, 128), 128, 0, s>>>(nc, A.w, A.col, A.val, clab, csing, gj_fac, err);
+      FVS_COUNT_LAUNCH();
+      FVS_LAUNCH_CHECK();
+      int bad = 0;
+      FVS_TRY(read_int(s, err, &bad));
+      if (bad) {
+        DBuf<int32_t>& perm = gj_perm;
+        FVS_TRY(perm.alloc(nc));
+        FVS_TRY(err.zero(s));
+        FVS_TRY(fill(Ainv));
+        const int eb = std::min(nc, 4 * sm_count());
         for (int k = 0; k < nc; ++k) {
-          k_gj_pivot<<<1, 256, 0, s>>>(nc, k, Ainv, fac, perm, err); FVS_COUNT_LAUNCH();
-          k_gj_elim<<<eb, 128, 0, s>>>(nc, k, Ainv, fac, err); FVS_COUNT_LAUNCH();
+          k_gj_pivot<<<1, 256, 0, s>>>(nc, k, Ainv, gj_fac, perm, err); FVS_COUNT_LAUNCH();
+          k_gj_elim<<<eb, 128, 0, s>>>(nc, k, Ainv, gj_fac, err); FVS_COUNT_LAUNCH();
         }
+        k_gj_unswap<<<stride_grid(nc, 128), 128, 0, s>>>(nc, Ainv, perm, err); FVS_COUNT_LAUNCH();
       }
-      k_gj_unswap<<<stride_grid(nc, 128), 128, 0, s>>>(nc, Ainv, perm, err); FVS_COUNT_LAUNCH();
-      k_dense_fold<true><<<stride_grid(nc, 128), 128, 0, s>>>(nc, Ainv, clab, csing, order, ncd, err);
-      FVS_COUNT_LAUNCH();
-      k_dense_fold<false><<<stride_grid(nc, 128), 128, 0, s>>>(nc, Ainv, clab, csing, order, ncd, err);
-      FVS_COUNT_LAUNCH();
+      k_dense_fold_rows<<<(nc + 31) / 32, 1024, 0, s>>>(nc, Ainv, clab, csing, ncd); FVS_COUNT_LAUNCH();
+      k_dense_fold_cols<<<(nc + 7) / 8, 256, 0, s>>>(nc, Ainv, clab, csing, ncd); FVS_COUNT_LAUNCH();
     }
     FVS_LAUNCH_CHECK();
   }

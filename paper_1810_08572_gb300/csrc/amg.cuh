@@ -84,15 +84,11 @@ struct Amg : Precond {
   fvs_status refresh(cudaStream_t s, const int32_t* act, const uint8_t* ppe);
   fvs_status apply(cudaStream_t s, const double* r, double* z) override;
   uint64_t version = 0;          // bumped by every setup
-  // coarsest inverse above the shared-memory size: one pivot and one
-  // elimination launch per column, replayed as a captured graph (kept while
-  // the level size and buffers stay the same)
-  DBuf<double> gj_fac;
+  // coarsest inverse above the shared-memory size: the block steps' second
+  // array, a vector, and the row exchanges of the column-by-column fallback
+  DBuf<double> gj_tmp, gj_fac;
   DBuf<int32_t> gj_perm;
   DBuf<int> c_err, c_ncd;
-  cudaGraphExec_t gj_exec = nullptr;
-  uint64_t gj_key = 0;
-  ~Amg() { if (gj_exec) cudaGraphExecDestroy(gj_exec); }
   uint64_t signature() const override {
     // Chebyshev weights are launch arguments: new bounds need a new graph
     return version * 2654435761ULL + (opt.fp32 ? 1 : 0) + (masked ? 2 : 0) +

@@ -380,3 +380,18 @@ def test_energy_line_preconditioner_changes_only_the_iterations(fvs, monkeypatch
     for k in ("T", "U", "P", "FS"):
         assert rel(lin[k], jac[k]) <= 1e-10, (k, rel(lin[k], jac[k]))
     assert its_l <= 0.6 * its_j, (its_l, its_j)
+
+
+@pytest.mark.parametrize("jitter,shape", [(0.0, (16, 16, 2)), (0.2, (24, 24, 1)), (0.2, (31, 31, 1)), (0.2, (20, 19, 2))])
+def test_dense_level_of_every_size_matches_the_single_grid_solve(fvs, jitter, shape):
+    """Systems of 161 to 1000 rows are one dense level (block Gauss-Jordan
+    inverse, tiles and last blocks of every remainder, three pockets pinned
+    and projected): two steps equal the single-grid solve's, both solved to
+    1e-13."""
+    m = box_mesh(*shape, cases.CAVITY, jitter=jitter, jitter_seed=13, permute_seed=14)
+    T0 = pockets_field(m, seed=6)
+    u0 = np.random.default_rng(3).normal(scale=2e-3, size=(len(T0), 3))
+    dense, _ = _run(fvs, m, cases.props(**TIGHT), T0, u0, 2)
+    single, _ = _run(fvs, m, cases.props(p_solver=1, **TIGHT), T0, u0, 2)
+    for k in ("T", "U", "P", "FLUX"):
+        assert rel(dense[k], single[k]) <= 1e-10, k
