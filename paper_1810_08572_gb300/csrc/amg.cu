@@ -1079,8 +1079,12 @@ __global__ void k_coarse_solve(int n, const double* __restrict__ Ainv, const T* 
 // ---------------------------------------------------------------------------
 // V-cycle kernels
 // ---------------------------------------------------------------------------
+// Weights of the sweeps lie in device memory (k_sweep_weights), not in the
+// launch arguments, so a refresh that moves the Chebyshev interval neither
+// reads the bounds back nor changes a captured cycle.
 template <typename T>
-__global__ void k_jac0(int64_t n, T omega, const T* dinv, const T* b, T* x) {
+__global__ void k_jac0(int64_t n, const double* __restrict__ wp, const T* dinv, const T* b, T* x) {
+  const T omega = (T)wp[0];
   GS(i, n) x[i] = omega * dinv[i] * b[i];
 }
 // Fine level: (A x)_i over every slot of the row (one thread per row; the
@@ -1093,9 +1097,10 @@ __device__ __forceinline__ T fine_row(int64_t n, int w, const int32_t* __restric
 
 // y = x + omega D^-1 (b - A x)
 template <typename T>
-__global__ void k_jac(int64_t n, int w, const int32_t* __restrict__ col, const T* __restrict__ val, T omega,
-                      const T* __restrict__ dinv, const T* __restrict__ b, const T* __restrict__ x,
-                      T* __restrict__ y) {
+__global__ void k_jac(int64_t n, int w, const int32_t* __restrict__ col, const T* __restrict__ val,
+                      const double* __restrict__ wp, const T* __restrict__ dinv, const T* __restrict__ b,
+                      const T* __restrict__ x, T* __restrict__ y) {
+  const T omega = (T)wp[0];
   GS(i, n) {
     const T acc = fine_row(n, w, col, val, x, i);
     y[i] = x[i] + omega * dinv[i] * (b[i] - acc);
@@ -1169,9 +1174,10 @@ __global__ void k_resid_g(int64_t n, const int32_t* __restrict__ col, const T* _
 }
 // y = x + omega D^-1 (b - A x) on a coarse level
 template <typename T, int G>
-__global__ void k_jac_g(int64_t n, const int32_t* __restrict__ col, const T* __restrict__ val, T omega,
-                        const T* __restrict__ dinv, const T* __restrict__ b, const T* __restrict__ x,
-                        T* __restrict__ y, const int32_t* __restrict__ rlen) {
+__global__ void k_jac_g(int64_t n, const int32_t* __restrict__ col, const T* __restrict__ val,
+                        const double* __restrict__ wp, const T* __restrict__ dinv, const T* __restrict__ b,
+                        const T* __restrict__ x, T* __restrict__ y, const int32_t* __restrict__ rlen) {
+  const T omega = (T)wp[0];
   const int lane = threadIdx.x & 31, q = lane & (G - 1);
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -1188,9 +1194,10 @@ __global__ void k_jac_g(int64_t n, const int32_t* __restrict__ col, const T* __r
 // before x (nullptr: zero).  xp and y may be the same array (each row reads
 // its own xp entry before writing y); x is gathered and must differ from y.
 template <typename T>
-__global__ void k_cheb(int64_t n, int w, const int32_t* __restrict__ col, const T* __restrict__ val, T alpha,
-                       T beta, const T* __restrict__ dinv, const T* __restrict__ b, const T* __restrict__ x,
-                       const T* xp, T* y) {
+__global__ void k_cheb(int64_t n, int w, const int32_t* __restrict__ col, const T* __restrict__ val,
+                       const double* __restrict__ wp, const T* __restrict__ dinv, const T* __restrict__ b,
+                       const T* __restrict__ x, const T* xp, T* y) {
+  const T alpha = (T)wp[0], beta = (T)wp[1];
   GS(i, n) {
     const T acc = fine_row(n, w, col, val, x, i);
     const T xi = x[i];
@@ -1199,9 +1206,10 @@ __global__ void k_cheb(int64_t n, int w, const int32_t* __restrict__ col, const 
   }
 }
 template <typename T, int G>
-__global__ void k_cheb_g(int64_t n, const int32_t* __restrict__ col, const T* __restrict__ val, T alpha, T beta,
-                         const T* __restrict__ dinv, const T* __restrict__ b, const T* __restrict__ x, const T* xp,
-                         T* y, const int32_t* __restrict__ rlen) {
+__global__ void k_cheb_g(int64_t n, const int32_t* __restrict__ col, const T* __restrict__ val,
+                         const double* __restrict__ wp, const T* __restrict__ dinv, const T* __restrict__ b,
+                         const T* __restrict__ x, const T* xp, T* y, const int32_t* __restrict__ rlen) {
+  const T alpha = (T)wp[0], beta = (T)wp[1];
   const int lane = threadIdx.x & 31, q = lane & (G - 1);
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -1235,6 +1243,32 @@ __global__ void k_gershgorin(int64_t n, int w, const double* __restrict__ val, c
   if ((threadIdx.x & 31) == 0) atomicMax(out, (unsigned long long)__double_as_longlong(m));
 }
 
+// Weights of every level's sweeps from its bound b (gb, bit pattern of a
+// double): a row of 2 * steps values, w0 (the first sweep from a given
+// iterate), unused, then alpha_k, beta_k of step k.  Chebyshev on
+// [b / ratio, b], centre th, half-width de: w0 = 1 / th, and step k >= 1 has
+// rho_k = 1 / (2 th / de - rho_{k-1}), rho_0 = de / th, alpha = 2 rho_k / de,
+// beta = rho_k rho_{k-1}.  Without a usable bound (or ratio 0) every step is
+// weighted Jacobi.
+__global__ void k_sweep_weights(int nl, int steps, const unsigned long long* gb, double ratio, double omega,
+                                double* w) {
+  const int l = threadIdx.x;
+  if (l >= nl) return;
+  double* q = w + (size_t)l * 2 * steps;
+  const double b = ratio > 1.0 ? __longlong_as_double((long long)gb[l]) : 0.0;
+  const bool cheb = b > 0.0 && b < 1e300;
+  const double th = 0.5 * (b + b / ratio), de = 0.5 * (b - b / ratio);
+  double rho = cheb ? de / th : 0.0;
+  q[0] = cheb ? 1.0 / th : omega;
+  q[1] = 0.0;
+  for (int k = 1; k < steps; ++k) {
+    const double rn = cheb ? 1.0 / (2.0 * th / de - rho) : 0.0;
+    q[2 * k] = cheb ? 2.0 * rn / de : omega;
+    q[2 * k + 1] = rn * rho;
+    rho = rn;
+  }
+}
+
 // lanes per row of a coarse level from its mean stored row length
 // (FVS_AMG_LANES forces one count)
 static int coarse_lanes(const AmgLevel& L) {
@@ -1265,8 +1299,9 @@ __global__ void k_restrict(int64_t nc, const int32_t* mptr, const int32_t* midx,
 // restriction and the next level's first Jacobi iterate: bc = R r,
 // xc = omega Dc^-1 bc
 template <typename T>
-__global__ void k_restrict_jac0(int64_t nc, const int32_t* mptr, const int32_t* midx, const T* r, T* bc, T omega,
-                                const T* dinvc, T* xc) {
+__global__ void k_restrict_jac0(int64_t nc, const int32_t* mptr, const int32_t* midx, const T* r, T* bc,
+                                const double* __restrict__ wp, const T* dinvc, T* xc) {
+  const T omega = (T)wp[0];
   GS(I, nc) {
     T s = 0;
     for (int32_t m = mptr[I]; m < mptr[I + 1]; ++m) s += r[midx[m]];
@@ -1568,88 +1603,97 @@ fvs_status Amg::setup(cudaStream_t s, const Ell& A) {
     // attempts 0-2: distance-1 independent sets on ever wider strength
     // graphs; attempt 3, only where those would stall the coarsening: the
     // distance-2 set on the first graph
-    const int first = l >= opt.mis2_from ? 3 : 0;
-    for (int attempt = first; attempt < 4; ++attempt) {
-      if (first == 0 && attempt == 3 && (double)nc <= opt.mis2_ratio * (double)n) break;   // keep the distance-1 result
-      mis2 = attempt == 3;
-      const double theta = (attempt == 0 || mis2) ? opt.theta : 0.0;
-      const int absval = attempt == 2 ? 1 : 0;
-      FVS_TRY(st.zero(s));
-      if (l == 0) {
-        k_mark_decoupled<<<stride_grid(n, 256), 256, 0, s>>>(n, cur->w, cur->col, cur->val, st);
+    // (from level mis2_from on the distance-2 set comes first, and the
+    // attempts follow only where it coarsens too little or leaves a row out)
+    bool placed = false;   // aggregates assigned to every row
+    for (int plan = l >= opt.mis2_from ? 0 : 1; plan < 2 && !placed; ++plan) {
+      const int first = plan == 0 ? 3 : 0;
+      for (int attempt = first; attempt < 4; ++attempt) {
+        if (first == 0 && attempt == 3 && (double)nc <= opt.mis2_ratio * (double)n) break;   // keep the distance-1 result
+        mis2 = attempt == 3;
+        const double theta = (attempt == 0 || mis2) ? opt.theta : 0.0;
+        const int absval = attempt == 2 ? 1 : 0;
+        FVS_TRY(st.zero(s));
+        if (l == 0) {
+          k_mark_decoupled<<<stride_grid(n, 256), 256, 0, s>>>(n, cur->w, cur->col, cur->val, st);
+          FVS_COUNT_LAUNCH();
+        }
+        k_strong<<<stride_grid(n, 256), 256, 0, s>>>(n, cur->w, cur->col, cur->val, mo, theta, absval, mask);
         FVS_COUNT_LAUNCH();
-      }
-      k_strong<<<stride_grid(n, 256), 256, 0, s>>>(n, cur->w, cur->col, cur->val, mo, theta, absval, mask);
-      FVS_COUNT_LAUNCH();
-      FVS_LAUNCH_CHECK();
-      tick(1);
-      if (mis2) { FVS_TRY(t1.alloc(n)); FVS_TRY(r1.alloc(n)); }
-      for (int round = 0;; round += 2) {
-        // two independent-set rounds per check (rounds after completion change nothing)
-        FVS_TRY(cnt.zero(s));
-        for (int q = 0; q < 2; ++q) {
-          int* cq = q == 1 ? cnt.p : cnt.p + 1;
-          if (mis2) {
-            k_mis2_max1<<<stride_grid(n, 256), 256, 0, s>>>(n, cur->col, mask, st, t1); FVS_COUNT_LAUNCH();
-            k_mis2_select<<<stride_grid(n, 256), 256, 0, s>>>(n, cur->col, mask, st, t1, st2); FVS_COUNT_LAUNCH();
-            k_mis2_near<<<stride_grid(n, 256), 256, 0, s>>>(n, cur->col, mask, st2, r1); FVS_COUNT_LAUNCH();
-            k_mis2_remove<<<stride_grid(n, 256), 256, 0, s>>>(n, cur->col, mask, st2, r1, st, cq); FVS_COUNT_LAUNCH();
-          } else {
-            k_mis_select<<<stride_grid(n, 256), 256, 0, s>>>(n, cur->w, cur->col, mask, st, st2); FVS_COUNT_LAUNCH();
-            k_mis_remove<<<stride_grid(n, 256), 256, 0, s>>>(n, cur->w, cur->col, mask, st2, st, cq);
-            FVS_COUNT_LAUNCH();
+        FVS_LAUNCH_CHECK();
+        tick(1);
+        if (mis2) { FVS_TRY(t1.alloc(n)); FVS_TRY(r1.alloc(n)); }
+        for (int round = 0;; round += 2) {
+          // two independent-set rounds per check (rounds after completion change nothing)
+          FVS_TRY(cnt.zero(s));
+          for (int q = 0; q < 2; ++q) {
+            int* cq = q == 1 ? cnt.p : cnt.p + 1;
+            if (mis2) {
+              k_mis2_max1<<<stride_grid(n, 256), 256, 0, s>>>(n, cur->col, mask, st, t1); FVS_COUNT_LAUNCH();
+              k_mis2_select<<<stride_grid(n, 256), 256, 0, s>>>(n, cur->col, mask, st, t1, st2); FVS_COUNT_LAUNCH();
+              k_mis2_near<<<stride_grid(n, 256), 256, 0, s>>>(n, cur->col, mask, st2, r1); FVS_COUNT_LAUNCH();
+              k_mis2_remove<<<stride_grid(n, 256), 256, 0, s>>>(n, cur->col, mask, st2, r1, st, cq); FVS_COUNT_LAUNCH();
+            } else {
+              k_mis_select<<<stride_grid(n, 256), 256, 0, s>>>(n, cur->w, cur->col, mask, st, st2); FVS_COUNT_LAUNCH();
+              k_mis_remove<<<stride_grid(n, 256), 256, 0, s>>>(n, cur->w, cur->col, mask, st2, st, cq);
+              FVS_COUNT_LAUNCH();
+            }
+          }
+          FVS_LAUNCH_CHECK();
+          int und = 0;
+          FVS_TRY(read_int(s, cnt, &und));
+          if (und == 0) break;
+          if (round >= 62) {
+            set_error("AMG aggregation did not finish");
+            return FVS_ERR_NOT_CONVERGED;
           }
         }
-        FVS_LAUNCH_CHECK();
-        int und = 0;
-        FVS_TRY(read_int(s, cnt, &und));
-        if (und == 0) break;
-        if (round >= 62) {
-          set_error("AMG aggregation did not finish");
+        FVS_TRY(flag.zero(s));
+        k_is_root<<<stride_grid(n, 256), 256, 0, s>>>(n, st, flag); FVS_COUNT_LAUNCH();
+        FVS_TRY(exclusive_scan(s, sw, n + 1, flag, rid));
+        FVS_CUDA(cudaMemcpyAsync(&nc, rid.p + n, sizeof(int), cudaMemcpyDeviceToHost, s));
+        FVS_CUDA(cudaStreamSynchronize(s));
+        if ((double)nc <= 0.6 * (double)n) break;
+      }
+      if (dbg) {
+        // rows without a strong coupling in the last attempt become singletons
+        FVS_TRY(cnt.zero(s));
+        k_count_isolated<<<stride_grid(n, 256), 256, 0, s>>>(n, mask, cnt); FVS_COUNT_LAUNCH();
+        int iso = 0;
+        FVS_TRY(read_int(s, cnt, &iso));
+        fprintf(stderr, "[fvs amg] level %d: %lld rows (w%d) -> %d aggregates%s, %d rows without strong couplings\n",
+                l, (long long)n, cur->w, nc, mis2 ? " (distance-2 set)" : "", iso);
+      }
+      if (plan == 0 && !(nc > 0 && (double)nc <= 0.6 * (double)n)) continue;
+      if (nc <= 0 || nc >= n || (double)nc > 0.85 * (double)n) break;  // stagnation: L is the coarsest
+      tick(2);
+      FVS_TRY(L->agg.alloc(n));
+      k_assign<<<stride_grid(n, 256), 256, 0, s>>>(n, cur->w, cur->col, cur->val, mask, st, rid, L->agg, err,
+                                                   mis2 ? 1 : 0);
+      FVS_COUNT_LAUNCH();
+      if (mis2) {
+        // nodes two hops from a root: up to three passes of joining an
+        // assigned neighbour's aggregate; any left over is a setup failure
+        DBuf<int32_t> agg2;
+        FVS_TRY(agg2.alloc(n));
+        int left = 0;
+        for (int pass = 0; pass < 3; ++pass) {
+          FVS_TRY(cnt.zero(s));
+          k_assign_near<<<stride_grid(n, 256), 256, 0, s>>>(n, cur->col, cur->val, mask, st, L->agg, agg2, cnt);
+          FVS_COUNT_LAUNCH();
+          FVS_CUDA(cudaMemcpyAsync(L->agg.p, agg2.p, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
+          FVS_TRY(read_int(s, cnt, &left));
+          if (left == 0) break;
+        }
+        if (left && plan == 0) continue;
+        if (left) {
+          set_error("AMG aggregation left %d rows without an aggregate at level %d", left, l);
           return FVS_ERR_NOT_CONVERGED;
         }
       }
-      FVS_TRY(flag.zero(s));
-      k_is_root<<<stride_grid(n, 256), 256, 0, s>>>(n, st, flag); FVS_COUNT_LAUNCH();
-      FVS_TRY(exclusive_scan(s, sw, n + 1, flag, rid));
-      FVS_CUDA(cudaMemcpyAsync(&nc, rid.p + n, sizeof(int), cudaMemcpyDeviceToHost, s));
-      FVS_CUDA(cudaStreamSynchronize(s));
-      if ((double)nc <= 0.6 * (double)n) break;
+      placed = true;
     }
-    if (dbg) {
-      // rows without a strong coupling in the last attempt become singletons
-      FVS_TRY(cnt.zero(s));
-      k_count_isolated<<<stride_grid(n, 256), 256, 0, s>>>(n, mask, cnt); FVS_COUNT_LAUNCH();
-      int iso = 0;
-      FVS_TRY(read_int(s, cnt, &iso));
-      fprintf(stderr, "[fvs amg] level %d: %lld rows (w%d) -> %d aggregates%s, %d rows without strong couplings\n",
-              l, (long long)n, cur->w, nc, mis2 ? " (distance-2 set)" : "", iso);
-    }
-    if (nc <= 0 || nc >= n || (double)nc > 0.85 * (double)n) break;  // stagnation: L is the coarsest
-    tick(2);
-    FVS_TRY(L->agg.alloc(n));
-    k_assign<<<stride_grid(n, 256), 256, 0, s>>>(n, cur->w, cur->col, cur->val, mask, st, rid, L->agg, err,
-                                                 mis2 ? 1 : 0);
-    FVS_COUNT_LAUNCH();
-    if (mis2) {
-      // nodes two hops from a root: up to three passes of joining an
-      // assigned neighbour's aggregate; any left over is a setup failure
-      DBuf<int32_t> agg2;
-      FVS_TRY(agg2.alloc(n));
-      int left = 0;
-      for (int pass = 0; pass < 3; ++pass) {
-        FVS_TRY(cnt.zero(s));
-        k_assign_near<<<stride_grid(n, 256), 256, 0, s>>>(n, cur->col, cur->val, mask, st, L->agg, agg2, cnt);
-        FVS_COUNT_LAUNCH();
-        FVS_CUDA(cudaMemcpyAsync(L->agg.p, agg2.p, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
-        FVS_TRY(read_int(s, cnt, &left));
-        if (left == 0) break;
-      }
-      if (left) {
-        set_error("AMG aggregation left %d rows without an aggregate at level %d", left, l);
-        return FVS_ERR_NOT_CONVERGED;
-      }
-    }
+    if (!placed) break;
     DBuf<int32_t> mc;
     FVS_TRY(mc.alloc(nc + 1));
     FVS_TRY(mc.zero(s));
@@ -1713,40 +1757,56 @@ fvs_status Amg::setup(cudaStream_t s, const Ell& A) {
             "coarsest %.2f fp32 %.2f\n", nc, ncomp, tph[0], tph[1], tph[2], tph[3], tph[4], tph[5], tph[6]);
   }
   FVS_TRY(count_stored(s));
-  if (opt.smoother == 1) FVS_TRY(cheb_bounds(s));
+  FVS_TRY(sweep_weights(s));
   ready = true;
   return FVS_OK;
 }
 
-fvs_status Amg::cheb_bounds(cudaStream_t s) {
+fvs_status Amg::sweep_weights(cudaStream_t s) {
   const int nl = (int)lv.size();
+  const bool cheb = opt.smoother == 1;
   FVS_TRY(gbound.alloc(nl + 1));
-  FVS_CUDA(cudaMemsetAsync(gbound.p, 0, sizeof(unsigned long long) * nl, s));
-  for (int l = 0; l + 1 < nl; ++l) {   // the coarsest level is solved, not smoothed
+  FVS_TRY(weights.alloc((size_t)nl * 2 * sweep_steps()));
+  if (cheb) FVS_CUDA(cudaMemsetAsync(gbound.p, 0, sizeof(unsigned long long) * nl, s));
+  for (int l = 0; cheb && l + 1 < nl; ++l) {   // the coarsest level is solved, not smoothed
     AmgLevel* L = lv[l].get();
     if (L->n == 0) continue;
     k_gershgorin<<<stride_grid(L->n, 256), 256, 0, s>>>(L->n, L->A->w, L->A->val, L->dinv,
                                                        L->rlen.n ? L->rlen.p : nullptr, gbound.p + l);
     FVS_COUNT_LAUNCH();
   }
+  k_sweep_weights<<<1, 32, 0, s>>>(nl, sweep_steps(), gbound, cheb ? opt.cheb_ratio : 0.0, opt.omega, weights);
+  FVS_COUNT_LAUNCH();
   FVS_LAUNCH_CHECK();
-  std::vector<unsigned long long> h(nl, 0ULL);
-  FVS_CUDA(cudaMemcpyAsync(h.data(), gbound.p, sizeof(unsigned long long) * nl, cudaMemcpyDeviceToHost, s));
-  FVS_CUDA(cudaStreamSynchronize(s));
-  for (int l = 0; l < nl; ++l) {
-    double v;
-    memcpy(&v, &h[l], sizeof(v));
-    lv[l]->cheb_b = std::isfinite(v) ? v : 0.0;
-  }
-  ++bound_epoch;
   return FVS_OK;
 }
 
-// the first sweep from a given iterate: weighted Jacobi, or the first step
-// of the Chebyshev recurrence (weight 1 / theta, theta the interval's centre)
-double Amg::first_weight(const AmgLevel& L) const {
-  if (opt.smoother != 1 || !(L.cheb_b > 0.0)) return opt.omega;
-  return 2.0 / (L.cheb_b * (1.0 + 1.0 / opt.cheb_ratio));
+// everything a captured cycle holds: a hierarchy rebuilt or refreshed into the
+// same buffers replays the same graph
+uint64_t Amg::signature() const {
+  uint64_t h = 1469598103934665603ULL;
+  auto mix = [&](uint64_t v) { h ^= v + 0x9e3779b97f4a7c15ULL + (h << 6) + (h >> 2); };
+  auto ptr = [&](const void* p) { mix((uint64_t)(uintptr_t)p); };
+  mix((uint64_t)lv.size() * 64 + (opt.fp32 ? 1 : 0) + (masked ? 2 : 0) + (opt.smoother == 1 ? 4 : 0));
+  mix((uint64_t)opt.npre * 1000 + (uint64_t)opt.npost);
+  mix((uint64_t)(opt.coarse_scale * 1048576.0));
+  mix((uint64_t)nc * 4096 + (uint64_t)ncomp);
+  for (uint8_t g : sing_host) mix(g);
+  for (const void* p : {(const void*)Ainv.p, (const void*)fine_lab.p, (const void*)csing.p, (const void*)csum.p,
+                        (const void*)ccnt.p, (const void*)cpart.p, (const void*)weights.p})
+    ptr(p);
+  for (const auto& up : lv) {
+    const AmgLevel& L = *up;
+    mix((uint64_t)L.n * 128 + (uint64_t)L.A->w);
+    mix((uint64_t)(L.stored * 16.0 / (double)(L.n > 0 ? L.n : 1)));   // lanes a row
+    for (const void* p : {(const void*)L.A->col.p, (const void*)L.A->val.p, (const void*)L.dinv.p,
+                          (const void*)L.dinvf.p, (const void*)L.valf.p, (const void*)L.rlen.p, (const void*)L.agg.p,
+                          (const void*)L.mptr.p, (const void*)L.midx.p, (const void*)L.b.p, (const void*)L.x.p,
+                          (const void*)L.y.p, (const void*)L.r.p, (const void*)L.t.p, (const void*)L.bf.p,
+                          (const void*)L.xf.p, (const void*)L.yf.p, (const void*)L.rf.p, (const void*)L.tf.p})
+      ptr(p);
+  }
+  return h;
 }
 
 fvs_status Amg::coarsest_setup(cudaStream_t s) {
@@ -2012,7 +2072,7 @@ fvs_status Amg::refresh(cudaStream_t s, const int32_t* act, const uint8_t* ppe) 
             tph[0], tph[1], tph[2], tph[3]);
   masked = true;
   FVS_TRY(count_stored(s));
-  if (opt.smoother == 1) FVS_TRY(cheb_bounds(s));
+  FVS_TRY(sweep_weights(s));
   ready = true;
   return FVS_OK;
 }
@@ -2080,43 +2140,36 @@ fvs_status Amg::vcycle_t(cudaStream_t s, int l, const T* b, T* y, bool x0_ready)
   const char* n_res = f32 ? (cl ? "residual_f32_coarse" : "residual_f32") : (cl ? "residual_vc_coarse" : "residual_vc");
   const int G = rl ? coarse_lanes(*L) : 1;   // coarse levels: G lanes per row
   const int gg = stride_grid(n * G, 256);
-  const T w0 = (T)first_weight(*L);
+  const double* wl = weights.p + (size_t)l * 2 * sweep_steps();   // this level's sweep weights
   auto jac = [&](T* xin, T* xout) {
     ProfScope ps(pkey, n_jac, jac_bytes, s);
-    if (!rl) k_jac<T><<<g, 256, 0, s>>>(n, A.w, A.col, val, w0, dinv, b, xin, xout);
-    else if (G == 1) k_jac_g<T, 1><<<gg, 256, 0, s>>>(n, A.col, val, w0, dinv, b, xin, xout, rl);
-    else if (G == 2) k_jac_g<T, 2><<<gg, 256, 0, s>>>(n, A.col, val, w0, dinv, b, xin, xout, rl);
-    else if (G == 4) k_jac_g<T, 4><<<gg, 256, 0, s>>>(n, A.col, val, w0, dinv, b, xin, xout, rl);
-    else k_jac_g<T, 8><<<gg, 256, 0, s>>>(n, A.col, val, w0, dinv, b, xin, xout, rl);
+    if (!rl) k_jac<T><<<g, 256, 0, s>>>(n, A.w, A.col, val, wl, dinv, b, xin, xout);
+    else if (G == 1) k_jac_g<T, 1><<<gg, 256, 0, s>>>(n, A.col, val, wl, dinv, b, xin, xout, rl);
+    else if (G == 2) k_jac_g<T, 2><<<gg, 256, 0, s>>>(n, A.col, val, wl, dinv, b, xin, xout, rl);
+    else if (G == 4) k_jac_g<T, 4><<<gg, 256, 0, s>>>(n, A.col, val, wl, dinv, b, xin, xout, rl);
+    else k_jac_g<T, 8><<<gg, 256, 0, s>>>(n, A.col, val, wl, dinv, b, xin, xout, rl);
     FVS_COUNT_LAUNCH();
   };
-  // Chebyshev smoother: interval [cb / ratio, cb], centre th, half-width de;
-  // step k >= 1 of the recurrence has rho_k = 1 / (2 th / de - rho_{k-1}),
-  // rho_0 = de / th, alpha = 2 rho_k / de, beta = rho_k rho_{k-1}
-  const bool cheb = opt.smoother == 1 && L->cheb_b > 0.0;
-  const double cb = L->cheb_b, th = 0.5 * (cb + cb / opt.cheb_ratio), de = 0.5 * (cb - cb / opt.cheb_ratio);
-  auto cheb_step = [&](T* xin, const T* xprev, T* xout, double& rho) {
-    const double rn = 1.0 / (2.0 * th / de - rho);
-    const T alpha = (T)(2.0 * rn / de), beta = (T)(rn * rho);
-    rho = rn;
+  const bool cheb = opt.smoother == 1;
+  auto cheb_step = [&](T* xin, const T* xprev, T* xout, int k) {   // step k of the recurrence
+    const double* ab = wl + 2 * k;
     ProfScope ps(pkey, n_jac, jac_bytes + vb * (double)n, s);
-    if (!rl) k_cheb<T><<<g, 256, 0, s>>>(n, A.w, A.col, val, alpha, beta, dinv, b, xin, xprev, xout);
-    else if (G == 1) k_cheb_g<T, 1><<<gg, 256, 0, s>>>(n, A.col, val, alpha, beta, dinv, b, xin, xprev, xout, rl);
-    else if (G == 2) k_cheb_g<T, 2><<<gg, 256, 0, s>>>(n, A.col, val, alpha, beta, dinv, b, xin, xprev, xout, rl);
-    else if (G == 4) k_cheb_g<T, 4><<<gg, 256, 0, s>>>(n, A.col, val, alpha, beta, dinv, b, xin, xprev, xout, rl);
-    else k_cheb_g<T, 8><<<gg, 256, 0, s>>>(n, A.col, val, alpha, beta, dinv, b, xin, xprev, xout, rl);
+    if (!rl) k_cheb<T><<<g, 256, 0, s>>>(n, A.w, A.col, val, ab, dinv, b, xin, xprev, xout);
+    else if (G == 1) k_cheb_g<T, 1><<<gg, 256, 0, s>>>(n, A.col, val, ab, dinv, b, xin, xprev, xout, rl);
+    else if (G == 2) k_cheb_g<T, 2><<<gg, 256, 0, s>>>(n, A.col, val, ab, dinv, b, xin, xprev, xout, rl);
+    else if (G == 4) k_cheb_g<T, 4><<<gg, 256, 0, s>>>(n, A.col, val, ab, dinv, b, xin, xprev, xout, rl);
+    else k_cheb_g<T, 8><<<gg, 256, 0, s>>>(n, A.col, val, ab, dinv, b, xin, xprev, xout, rl);
     FVS_COUNT_LAUNCH();
   };
   if (!x0_ready) {
     ProfScope ps(pkey, n_jac0, 3.0 * vb * (double)n, s);
-    k_jac0<T><<<g, 256, 0, s>>>(n, w0, dinv, b, xa); FVS_COUNT_LAUNCH();
+    k_jac0<T><<<g, 256, 0, s>>>(n, wl, dinv, b, xa); FVS_COUNT_LAUNCH();
   }
   {
-    double rho = cheb ? de / th : 0.0;
     const T* xprev = nullptr;   // the pre-smoothing starts from zero
     for (int k = 1; k < opt.npre; ++k) {
       if (cheb) {
-        cheb_step(xa, xprev, xb, rho);
+        cheb_step(xa, xprev, xb, k);
         xprev = xa;
       } else {
         jac(xa, xb);
@@ -2140,7 +2193,7 @@ fvs_status Amg::vcycle_t(cudaStream_t s, int l, const T* b, T* y, bool x0_ready)
     T* cx = f32 ? (T*)C->xf.p : (T*)C->x.p;
     const T* cdinv = f32 ? (const T*)C->dinvf.p : (const T*)C->dinv.p;
     k_restrict_jac0<T><<<stride_grid(C->n, 256), 256, 0, s>>>(C->n, L->mptr, L->midx, r, cbv,
-                                                             (T)first_weight(*C), cdinv, cx);
+                                                             wl + 2 * sweep_steps(), cdinv, cx);
   } else {
     k_restrict<T><<<stride_grid(C->n, 256), 256, 0, s>>>(C->n, L->mptr, L->midx, r, cbv);
   }
@@ -2149,10 +2202,9 @@ fvs_status Amg::vcycle_t(cudaStream_t s, int l, const T* b, T* y, bool x0_ready)
   FVS_TRY(vcycle_t<T>(s, l + 1, cbv, cy, next_sweeps));
   k_prolong<T><<<g, 256, 0, s>>>(n, L->agg, cy, (T)opt.coarse_scale, xa); FVS_COUNT_LAUNCH();
   {
-    double rho = cheb ? de / th : 0.0;
     for (int k = 0; k < opt.npost; ++k) {
       T* out = (k == opt.npost - 1) ? y : xb;
-      if (cheb && k > 0) cheb_step(xa, xb, out, rho);   // xb holds the iterate before xa
+      if (cheb && k > 0) cheb_step(xa, xb, out, k);   // xb holds the iterate before xa
       else jac(xa, out);
       xb = xa;
       xa = out;

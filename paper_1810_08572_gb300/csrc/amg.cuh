@@ -28,7 +28,6 @@ struct AmgLevel {
   DBuf<uint8_t> dirty;  // rows changed since the last setup or refresh
   int64_t n = 0;
   double stored = 0.0;  // operator entries the V-cycle reads (coarse levels: sum of rlen)
-  double cheb_b = 0.0;  // Chebyshev smoother: Gershgorin bound of the spectrum of D^-1 A
 };
 
 struct AmgOptions {
@@ -89,11 +88,7 @@ struct Amg : Precond {
   DBuf<double> gj_tmp, gj_fac;
   DBuf<int32_t> gj_perm;
   DBuf<int> c_err, c_ncd;
-  uint64_t signature() const override {
-    // Chebyshev weights are launch arguments: new bounds need a new graph
-    return version * 2654435761ULL + (opt.fp32 ? 1 : 0) + (masked ? 2 : 0) +
-           (opt.smoother == 1 ? bound_epoch * 4 : 0);
-  }
+  uint64_t signature() const override;
   // subtract the component mean on every singular component (fine level)
   fvs_status project(cudaStream_t s, double* v);
   int levels() const { return (int)lv.size(); }
@@ -105,12 +100,12 @@ struct Amg : Precond {
   fvs_status vcycle_t(cudaStream_t s, int l, const T* b, T* y, bool x0_ready = false);
   fvs_status coarsest_setup(cudaStream_t s);
   fvs_status setup_fp32(cudaStream_t s);
-  // Chebyshev smoother: Gershgorin bounds of every smoothed level (after a
-  // setup or a refresh, when the operator values are final)
-  fvs_status cheb_bounds(cudaStream_t s);
-  double first_weight(const AmgLevel& L) const;   // weight of the first sweep
+  // sweep weights of every smoothed level (after a setup or a refresh, when
+  // the operator values are final)
+  fvs_status sweep_weights(cudaStream_t s);
+  int sweep_steps() const { return opt.npre > opt.npost ? opt.npre : opt.npost; }
   DBuf<unsigned long long> gbound;
-  uint64_t bound_epoch = 0;
+  DBuf<double> weights;
 };
 
 struct AmgProjector : Projector {

@@ -85,7 +85,7 @@ fvs_status Reducer::init() {
   FVS_TRY(sc.zero(st));
   FVS_TRY(ticket.alloc(1));
   FVS_TRY(ticket.zero(st));
-  FVS_TRY(iter.alloc(1));
+  FVS_TRY(iter.alloc(2));
   FVS_TRY(iter.zero(st));
   if (!host) FVS_CUDA(cudaMallocHost(&host, S_NSLOT * sizeof(double)));
   return FVS_OK;
@@ -324,6 +324,8 @@ __global__ void k_cg_p(int64_t n, const double* __restrict__ sc, const double* _
   GRID_STRIDE(i, n) p[i] = first ? z[i] : z[i] + beta * p[i];
 }
 
+constexpr int MAX_RESTARTS = 3;   // from the true residual, once the recursive one has met the tolerance
+
 static inline bool bad(double v) { return !(v == v) || v > 1e300 || v < -1e300; }
 
 static fvs_status spmv_dot(cudaStream_t s, Reducer& red, const Ell& A, const double* x, double* y,
@@ -434,24 +436,26 @@ static fvs_status run_body(cudaStream_t s, IterGraph* g, uint64_t key, bool firs
 // trip per iteration).  Bounded by maxit; a NaN residual or a breakdown of
 // the BiCGStab recurrence also stops the loop (the host then restarts or
 // reports).
-__global__ void k_ctl_bicg(cudaGraphConditionalHandle h, double* sc, int* it, int maxit) {
-  const int n = ++(*it);
+__global__ void k_ctl_bicg(cudaGraphConditionalHandle h, double* sc, int* it) {
+  const int n = ++it[0], maxit = it[1];
   sc[S_ITER] = (double)n;
   const double rr = sc[S_RR];
   const bool go = n < maxit && rr > sc[S_TOL2] && rr == rr && rr < 1e300 && sc[S_TT] != 0.0 &&
                   sc[S_RV] != 0.0 && sc[S_RHO] != 0.0;
   cudaGraphSetConditional(h, go ? 1u : 0u);
 }
-__global__ void k_ctl_cg(cudaGraphConditionalHandle h, double* sc, int* it, int maxit) {
-  const int n = ++(*it);
+__global__ void k_ctl_cg(cudaGraphConditionalHandle h, double* sc, int* it) {
+  const int n = ++it[0], maxit = it[1];
   sc[S_ITER] = (double)n;
   const double rr = sc[S_RR];
   const bool go = n < maxit && rr > sc[S_TOL2] && rr == rr && rr < 1e300;
   cudaGraphSetConditional(h, go ? 1u : 0u);
 }
-__global__ void k_loop_init(double* sc, int* it, double tol2, int fresh) {
+// (the bound lies beside the counter: a loop captured once serves every bound)
+__global__ void k_loop_init(double* sc, int* it, int maxit, double tol2, int fresh) {
   sc[S_FIRST] = fresh ? 1.0 : 0.0;
-  *it = 0;
+  it[0] = 0;
+  it[1] = maxit;
   sc[S_ITER] = 0.0;
   sc[S_TOL2] = tol2;
 }
@@ -488,9 +492,9 @@ static bool run_loop(cudaStream_t s, IterGraph* g, uint64_t key, Reducer& red, d
         const unsigned long long before = __atomic_load_n(&g_launches, __ATOMIC_RELAXED);
         fvs_status r = body(false);
         if (bicg)
-          k_ctl_bicg<<<1, 1, 0, s>>>(h, red.sc.p, red.iter.p, maxit);
+          k_ctl_bicg<<<1, 1, 0, s>>>(h, red.sc.p, red.iter.p);
         else
-          k_ctl_cg<<<1, 1, 0, s>>>(h, red.sc.p, red.iter.p, maxit);
+          k_ctl_cg<<<1, 1, 0, s>>>(h, red.sc.p, red.iter.p);
         g->loop_kernels = __atomic_load_n(&g_launches, __ATOMIC_RELAXED) - before + 1;
         __atomic_sub_fetch(&g_launches, g->loop_kernels - 1, __ATOMIC_RELAXED);
         cudaGraph_t out = nullptr;
@@ -509,7 +513,7 @@ static bool run_loop(cudaStream_t s, IterGraph* g, uint64_t key, Reducer& red, d
     }
     g->loop_key = key;
   }
-  k_loop_init<<<1, 1, 0, s>>>(red.sc.p, red.iter.p, tol2, fresh ? 1 : 0);
+  k_loop_init<<<1, 1, 0, s>>>(red.sc.p, red.iter.p, maxit, tol2, fresh ? 1 : 0);
   FVS_COUNT_LAUNCH();
   const cudaError_t e = cudaGraphLaunch(g->loop, s);
   if (e != cudaSuccess) {
@@ -574,47 +578,62 @@ fvs_status bicgstab(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, c
   bool fresh = true;
   int it = 0;
   const double tol2 = (rtol * bnorm) * (rtol * bnorm);
-  while (it < maxit) {
-    bool looped = false;
-    {
-      fvs_status st = FVS_OK;
-      looped = run_loop(s, graph, key, red, tol2, maxit - it, true, fresh, body, st);
-      FVS_TRY(st);
+  for (int again = 0;; ++again) {
+    while (it < maxit) {
+      bool looped = false;
+      {
+        fvs_status st = FVS_OK;
+        looped = run_loop(s, graph, key, red, tol2, maxit - it, true, fresh, body, st);
+        FVS_TRY(st);
+      }
+      if (!looped) FVS_TRY(run_body(s, graph, key, fresh, body));
+      fresh = false;
+      FVS_TRY(red.fetch(s));
+      const int done = looped ? (int)red.host[S_ITER] : 1;
+      if (looped) __atomic_add_fetch(&g_launches, graph->loop_kernels * (unsigned long long)done, __ATOMIC_RELAXED);
+      it += done;
+      rn = sqrt(red.host[S_RR]);
+      res.iters = it;
+      res.relres = rn / bnorm;
+      if (bad(rn)) return FVS_OK;
+      if (res.relres <= rtol) {
+        res.converged = true;
+        break;
+      }
+      // restart on breakdown of the shadow residual
+      if (red.host[S_TT] == 0.0 || red.host[S_RV] == 0.0 || red.host[S_RHO] == 0.0) {
+        FVS_TRY(residual(s, A, x, b, w.r, dextra));
+        if (proj) FVS_TRY(proj->apply(s, w.r));
+        FVS_TRY(vcopy(s, n, w.r, w.rh));
+        FVS_TRY(red.dot(s, n, w.rh, w.r, S_RHO));
+        fresh = true;
+      }
     }
-    if (!looped) FVS_TRY(run_body(s, graph, key, fresh, body));
-    fresh = false;
-    FVS_TRY(red.fetch(s));
-    const int done = looped ? (int)red.host[S_ITER] : 1;
-    if (looped) __atomic_add_fetch(&g_launches, graph->loop_kernels * (unsigned long long)done, __ATOMIC_RELAXED);
-    it += done;
-    rn = sqrt(red.host[S_RR]);
-    res.iters = it;
-    res.relres = rn / bnorm;
-    if (bad(rn)) return FVS_OK;
-    if (res.relres <= rtol) {
-      res.converged = true;
-      break;
-    }
-    // restart on breakdown of the shadow residual
-    if (red.host[S_TT] == 0.0 || red.host[S_RV] == 0.0 || red.host[S_RHO] == 0.0) {
+    // recompute the true residual (the recursive one drifts)
+    if (!proj) {
+      FVS_TRY(residual_dot<FIN_TRUE>(s, red, A, x, dextra, b, nullptr, nullptr));
+    } else {
       FVS_TRY(residual(s, A, x, b, w.r, dextra));
-      if (proj) FVS_TRY(proj->apply(s, w.r));
+      FVS_TRY(proj->apply(s, w.r));
+      FVS_TRY(red.dot(s, n, w.r, w.r, S_RR));
+    }
+    FVS_TRY(red.fetch(s));
+    res.relres = sqrt(red.host[S_RR]) / bnorm;
+    const bool met = res.converged;   // the recursive residual reached rtol
+    res.converged = res.relres <= rtol * 10.0 && !bad(res.relres);
+    // the recursive residual drifted too far from the true one (tight
+    // tolerances on large systems): start again from the true residual
+    // rather than give the solve up
+    if (res.converged || !met || bad(res.relres) || again == MAX_RESTARTS || it >= maxit) break;
+    res.converged = false;
+    if (!proj) {
+      FVS_TRY(residual_dot<FIN_START>(s, red, A, x, dextra, b, w.r, w.rh));
+    } else {
       FVS_TRY(vcopy(s, n, w.r, w.rh));
       FVS_TRY(red.dot(s, n, w.rh, w.r, S_RHO));
-      fresh = true;
     }
+    fresh = true;
   }
-  // recompute the true residual (the recursive one drifts)
-  if (!proj) {
-    FVS_TRY(residual_dot<FIN_TRUE>(s, red, A, x, dextra, b, nullptr, nullptr));
-  } else {
-    FVS_TRY(residual(s, A, x, b, w.r, dextra));
-    FVS_TRY(proj->apply(s, w.r));
-    FVS_TRY(red.dot(s, n, w.r, w.r, S_RR));
-  }
-  FVS_TRY(red.fetch(s));
-  res.relres = sqrt(red.host[S_RR]) / bnorm;
-  res.converged = res.relres <= rtol * 10.0 && !bad(res.relres);
   return FVS_OK;
 }
 
@@ -662,33 +681,42 @@ fvs_status pcg(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, Precon
   };
   const uint64_t key = graph_key(A, nullptr, M, b, x, w, red) ^ (proj ? 0x70636770ULL : 0x70636700ULL);
   const double tol2 = (rtol * bnorm) * (rtol * bnorm);
-  for (int it = 0; it < maxit;) {
-    bool looped = false;
-    {
-      fvs_status st = FVS_OK;
-      looped = run_loop(s, graph, key, red, tol2, maxit - it, false, it == 0, body, st);
-      FVS_TRY(st);
+  bool fresh = true;
+  int it = 0;
+  for (int again = 0;; ++again) {
+    while (it < maxit) {
+      bool looped = false;
+      {
+        fvs_status st = FVS_OK;
+        looped = run_loop(s, graph, key, red, tol2, maxit - it, false, fresh, body, st);
+        FVS_TRY(st);
+      }
+      if (!looped) FVS_TRY(run_body(s, graph, key, fresh, body));
+      fresh = false;
+      FVS_TRY(red.fetch(s));
+      const int done = looped ? (int)red.host[S_ITER] : 1;
+      if (looped) __atomic_add_fetch(&g_launches, graph->loop_kernels * (unsigned long long)done, __ATOMIC_RELAXED);
+      it += done;
+      const double rn = sqrt(red.host[S_RR]);
+      res.iters = it;
+      res.relres = rn / bnorm;
+      if (bad(rn)) return FVS_OK;
+      if (res.relres <= rtol) {
+        res.converged = true;
+        break;
+      }
     }
-    if (!looped) FVS_TRY(run_body(s, graph, key, it == 0, body));
+    FVS_TRY(residual(s, A, x, b, w.r, nullptr));
+    if (proj) FVS_TRY(proj->apply(s, w.r));
+    FVS_TRY(red.dot(s, n, w.r, w.r, S_RR));
     FVS_TRY(red.fetch(s));
-    const int done = looped ? (int)red.host[S_ITER] : 1;
-    if (looped) __atomic_add_fetch(&g_launches, graph->loop_kernels * (unsigned long long)done, __ATOMIC_RELAXED);
-    it += done;
-    const double rn = sqrt(red.host[S_RR]);
-    res.iters = it;
-    res.relres = rn / bnorm;
-    if (bad(rn)) return FVS_OK;
-    if (res.relres <= rtol) {
-      res.converged = true;
-      break;
-    }
+    res.relres = sqrt(red.host[S_RR]) / bnorm;
+    const bool met = res.converged;
+    res.converged = res.relres <= rtol * 10.0 && !bad(res.relres);
+    if (res.converged || !met || bad(res.relres) || again == MAX_RESTARTS || it >= maxit) break;
+    res.converged = false;
+    fresh = true;    // from the true residual, as in bicgstab
   }
-  FVS_TRY(residual(s, A, x, b, w.r, nullptr));
-  if (proj) FVS_TRY(proj->apply(s, w.r));
-  FVS_TRY(red.dot(s, n, w.r, w.r, S_RR));
-  FVS_TRY(red.fetch(s));
-  res.relres = sqrt(red.host[S_RR]) / bnorm;
-  res.converged = res.relres <= rtol * 10.0 && !bad(res.relres);
   return FVS_OK;
 }
 

@@ -40,7 +40,7 @@ struct Reducer {
   DBuf<double> part;   // [2*blocks]
   DBuf<double> sc;     // [S_NSLOT]
   DBuf<unsigned int> ticket;   // last-block counter of the fused reductions
-  DBuf<int> iter;              // iteration counter of device-driven solve loops
+  DBuf<int> iter;              // device-driven solve loops: iteration counter and its bound
   double* host = nullptr;  // pinned [S_NSLOT]
   fvs_status init();
   // blocks of 256 threads of a reduction over n rows: a row a thread up to

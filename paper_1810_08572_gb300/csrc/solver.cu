@@ -1172,11 +1172,21 @@ static fvs_status assemble_pressure(fvs_solver s) {
     // is one matrix-vector product per V-cycle, cheaper than the several
     // latency-bound launches per level that the small levels below it cost
     s->amg.opt.coarsest = SOLVER_COARSEST;
-    // BiCGStab (non-orthogonal meshes) takes a V(1,2) cycle: the second
-    // post-sweep saves more iterations than it costs (128^3 jittered cavity,
-    // 20 steps: 429 -> 352 iterations, 49.4 -> 48.8 ms a step); CG keeps the
-    // symmetric V(1,1)
-    s->amg.opt.npost = m->orthogonal ? 1 : 2;
+    // Distance-2 aggregates from the fine level on (about five rows each, not
+    // two and a half) with a stronger over-correction: a few more iterations,
+    // but the levels below the fine one hold a third of the entries, and FP64
+    // multiply-adds are what a cycle is bound by.  Chebyshev sweeps, V(1,2)
+    // under BiCGStab (non-orthogonal meshes), the symmetric V(2,2) under CG.
+    // Against distance-1 sets with V(1,2) / V(1,1) Jacobi, time (iterations of
+    // the last step): 128^3 jittered, 3 steps to 1e-12, 229 -> 197 ms (30 ->
+    // 29); 96^3 half frozen, FP32 cycle, 133 -> 112 ms; casting in its mold
+    // 50 -> 42 ms (39 -> 30); AMG-CG on 96 x 96 x 48 11.0 -> 7.0 ms (53 -> 34).
+    s->amg.opt.mis2_from = 0;
+    s->amg.opt.coarse_scale = 2.3;
+    s->amg.opt.smoother = 1;
+    s->amg.opt.cheb_ratio = 6.0;
+    s->amg.opt.npre = m->orthogonal ? 2 : 1;
+    s->amg.opt.npost = 2;
     // the vertex-interpolation couplings are small next to the face
     // couplings; leaving them out of the hierarchy cuts the bytes of every
     // V-cycle sweep (7 instead of 27 entries a fine row, narrower Galerkin

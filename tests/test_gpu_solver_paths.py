@@ -395,3 +395,21 @@ def test_dense_level_of_every_size_matches_the_single_grid_solve(fvs, jitter, sh
     single, _ = _run(fvs, m, cases.props(p_solver=1, **TIGHT), T0, u0, 2)
     for k in ("T", "U", "P", "FLUX"):
         assert rel(dense[k], single[k]) <= 1e-10, k
+
+
+@pytest.mark.parametrize("jitter,precision", [(0.2, 0), (0.2, 1), (0.0, 0), (0.0, 1)])
+def test_aggregation_and_smoother_change_only_the_iterations(fvs, monkeypatch, jitter, precision):
+    """The default hierarchy (distance-2 aggregates, Chebyshev sweeps) and one
+    on distance-1 aggregates with weighted Jacobi precondition the same
+    solves: three steps with three pockets agree to the solve tolerance."""
+    m = box_mesh(32, 32, 8, cases.CAVITY, jitter=jitter, jitter_seed=91, permute_seed=92)
+    T0 = pockets_field(m, seed=5)
+    u0 = np.random.default_rng(12).normal(scale=2e-3, size=(len(T0), 3))
+    props = cases.props(precision=precision, **TIGHT)
+    default, _ = _steps_with_stats(fvs, m, props, T0, u0, 3)
+    for k, v in (("SMOOTHER", "0"), ("MIS2_FROM", "99"), ("SCALE", "1.5"), ("NPRE", "1"), ("NPOST", "1")):
+        monkeypatch.setenv("FVS_AMG_" + k, v)
+    other, _ = _steps_with_stats(fvs, m, props, T0, u0, 3)
+    tol = 1e-10 if precision == 0 else 1e-8
+    for k in ("T", "U", "P", "FLUX"):
+        assert rel(default[k], other[k]) <= tol, k
