@@ -87,3 +87,28 @@ def test_exact_polynomial_and_device_evaluation(fvs):
     Yd = torch.empty((1000, 1), dtype=torch.float64, device="cuda")
     P(torch.tensor(Xt, device="cuda"), Yd)
     np.testing.assert_array_equal(Yd.cpu().numpy(), P(Xt))
+
+
+@pytest.mark.parametrize("fams,degree,nout", [
+    ([0], 0, 1), ([1], 24, 3), ([0, 1], 1, 8), ([1, 0, 1, 0, 1], 3, 5), ([0, 1] * 4, 2, 4)])
+def test_evaluation_over_inputs_degrees_and_outputs(fvs, fams, degree, nout):
+    """One to eight inputs, degree 0 to the largest, every padding of the
+    outputs, at one point, a block's edge and past it, against the oracle's
+    expansion with the same coefficients.  Each of the P terms is a product
+    of d basis values with a relative rounding error of a few ulps a degree:
+    the sum is within 1e-13 (degree + 1) P of its largest term."""
+    d = len(fams)
+    pars = [(1.0 + j, 0.5 + 0.25 * j) if f == 0 else (-1.0 - j, 2.0 + j) for j, f in enumerate(fams)]
+    P = fvs.Pce(fams, pars, degree, nout)
+    truth = ref.PCE(fams, pars, degree)
+    rng = np.random.default_rng(degree)
+    m = 3 * P.num_terms() + 7
+    X = ref.latin_hypercube(fams, pars, m, seed=2)
+    P.fit(X, rng.normal(size=(m, nout)))
+    truth.coef = P.coefficients()
+    for n in (1, 128, 300):
+        Xt = ref.latin_hypercube(fams, pars, n, seed=n)
+        V = truth.vandermonde(Xt)
+        scale = (np.abs(V)[:, :, None] * np.abs(truth.coef)[None]).max(axis=1)
+        tol = 1e-13 * (degree + 1) * P.num_terms() * scale
+        assert np.all(np.abs(P(Xt) - V @ truth.coef) <= tol)
