@@ -1065,15 +1065,15 @@ __global__ void __launch_bounds__(1024) k_coarsest_smem(int n, int w, const int3
 
 // coarsest solve: y = Ainv b with the projections already folded into Ainv;
 // one warp per row, FP64 arithmetic whatever the vector type
-template <typename T>
-__global__ void k_coarse_solve(int n, const double* __restrict__ Ainv, const T* __restrict__ b, T* __restrict__ y) {
+template <typename T, typename Y>
+__global__ void k_coarse_solve(int n, const double* __restrict__ Ainv, const T* __restrict__ b, Y* __restrict__ y) {
   const int lane = threadIdx.x & 31;
   const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (row >= n) return;
   double a = 0.0;
   for (int j = lane; j < n; j += 32) a = fma(Ainv[(int64_t)row * n + j], (double)b[j], a);
   a = warp_sum(a);
-  if (lane == 0) y[row] = (T)a;
+  if (lane == 0) y[row] = (Y)a;
 }
 
 // ---------------------------------------------------------------------------
@@ -1096,14 +1096,14 @@ __device__ __forceinline__ T fine_row(int64_t n, int w, const int32_t* __restric
 }
 
 // y = x + omega D^-1 (b - A x)
-template <typename T>
+template <typename T, typename Y>
 __global__ void k_jac(int64_t n, int w, const int32_t* __restrict__ col, const T* __restrict__ val,
                       const double* __restrict__ wp, const T* __restrict__ dinv, const T* __restrict__ b,
-                      const T* __restrict__ x, T* __restrict__ y) {
+                      const T* __restrict__ x, Y* __restrict__ y) {
   const T omega = (T)wp[0];
   GS(i, n) {
     const T acc = fine_row(n, w, col, val, x, i);
-    y[i] = x[i] + omega * dinv[i] * (b[i] - acc);
+    y[i] = (Y)(x[i] + omega * dinv[i] * (b[i] - acc));
   }
 }
 template <typename T>
@@ -1173,10 +1173,10 @@ __global__ void k_resid_g(int64_t n, const int32_t* __restrict__ col, const T* _
   }
 }
 // y = x + omega D^-1 (b - A x) on a coarse level
-template <typename T, int G>
+template <typename T, typename Y, int G>
 __global__ void k_jac_g(int64_t n, const int32_t* __restrict__ col, const T* __restrict__ val,
                         const double* __restrict__ wp, const T* __restrict__ dinv, const T* __restrict__ b,
-                        const T* __restrict__ x, T* __restrict__ y, const int32_t* __restrict__ rlen) {
+                        const T* __restrict__ x, Y* __restrict__ y, const int32_t* __restrict__ rlen) {
   const T omega = (T)wp[0];
   const int lane = threadIdx.x & 31, q = lane & (G - 1);
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -1186,29 +1186,29 @@ __global__ void k_jac_g(int64_t n, const int32_t* __restrict__ col, const T* __r
     const bool ok = i < n;
     T acc = ok ? coarse_part<T, G>(n, col, val, XVec<T>{x}, rlen[i], i, q) : (T)0;
     acc = lanes_sum<T, G>(acc);
-    if (ok && q == 0) y[i] = x[i] + omega * dinv[i] * (b[i] - acc);
+    if (ok && q == 0) y[i] = (Y)(x[i] + omega * dinv[i] * (b[i] - acc));
   }
 }
 // Chebyshev sweep (three-term recurrence of the Chebyshev polynomials in
 // D^-1 A): y = x + beta (x - xp) + alpha D^-1 (b - A x), xp the iterate
 // before x (nullptr: zero).  xp and y may be the same array (each row reads
 // its own xp entry before writing y); x is gathered and must differ from y.
-template <typename T>
+template <typename T, typename Y>
 __global__ void k_cheb(int64_t n, int w, const int32_t* __restrict__ col, const T* __restrict__ val,
                        const double* __restrict__ wp, const T* __restrict__ dinv, const T* __restrict__ b,
-                       const T* __restrict__ x, const T* xp, T* y) {
+                       const T* __restrict__ x, const T* xp, Y* y) {
   const T alpha = (T)wp[0], beta = (T)wp[1];
   GS(i, n) {
     const T acc = fine_row(n, w, col, val, x, i);
     const T xi = x[i];
     const T d = xp ? xi - xp[i] : xi;
-    y[i] = xi + beta * d + alpha * dinv[i] * (b[i] - acc);
+    y[i] = (Y)(xi + beta * d + alpha * dinv[i] * (b[i] - acc));
   }
 }
-template <typename T, int G>
+template <typename T, typename Y, int G>
 __global__ void k_cheb_g(int64_t n, const int32_t* __restrict__ col, const T* __restrict__ val,
                          const double* __restrict__ wp, const T* __restrict__ dinv, const T* __restrict__ b,
-                         const T* __restrict__ x, const T* xp, T* y, const int32_t* __restrict__ rlen) {
+                         const T* __restrict__ x, const T* xp, Y* y, const int32_t* __restrict__ rlen) {
   const T alpha = (T)wp[0], beta = (T)wp[1];
   const int lane = threadIdx.x & 31, q = lane & (G - 1);
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -1221,7 +1221,7 @@ __global__ void k_cheb_g(int64_t n, const int32_t* __restrict__ col, const T* __
     if (ok && q == 0) {
       const T xi = x[i];
       const T d = xp ? xi - xp[i] : xi;
-      y[i] = xi + beta * d + alpha * dinv[i] * (b[i] - acc);
+      y[i] = (Y)(xi + beta * d + alpha * dinv[i] * (b[i] - acc));
     }
   }
 }
@@ -2077,6 +2077,18 @@ fvs_status Amg::refresh(cudaStream_t s, const int32_t* act, const uint8_t* ppe) 
   return FVS_OK;
 }
 
+int Amg::single_part(MeanPart& m) {
+  int nsing = 0, first = -1;
+  for (int c = 0; c < ncomp; ++c)
+    if (sing_host[c]) { ++nsing; if (first < 0) first = c; }
+  if (lv[0]->n == 0 || nsing == 0) return 0;
+  if (nsing > 1) return 2;
+  m.lab = (masked || ncomp > 1) ? fine_lab.p : nullptr;
+  m.want = ncomp > 1 ? first : -1;
+  m.cnt = m.lab ? ccnt.p + first : nullptr;
+  return 1;
+}
+
 fvs_status Amg::project(cudaStream_t s, double* v) {
   const int64_t n = lv[0]->n;
   if (n == 0 || ncomp == 0) return FVS_OK;
@@ -2104,14 +2116,14 @@ fvs_status Amg::project(cudaStream_t s, double* v) {
   return FVS_OK;
 }
 
-template <typename T>
-fvs_status Amg::vcycle_t(cudaStream_t s, int l, const T* b, T* y, bool x0_ready) {
+template <typename T, typename Y>
+fvs_status Amg::vcycle_t(cudaStream_t s, int l, const T* b, Y* y, bool x0_ready) {
   AmgLevel* L = lv[l].get();
   const Ell& A = *L->A;
   const int64_t n = L->n;
   if (n == 0) return FVS_OK;
   if (l + 1 == (int)lv.size()) {
-    k_coarse_solve<T><<<(nc + 7) / 8, 256, 0, s>>>(nc, Ainv.p, b, y); FVS_COUNT_LAUNCH();
+    k_coarse_solve<T, Y><<<(nc + 7) / 8, 256, 0, s>>>(nc, Ainv.p, b, y); FVS_COUNT_LAUNCH();
     FVS_LAUNCH_CHECK();
     return FVS_OK;
   }
@@ -2141,24 +2153,26 @@ fvs_status Amg::vcycle_t(cudaStream_t s, int l, const T* b, T* y, bool x0_ready)
   const int G = rl ? coarse_lanes(*L) : 1;   // coarse levels: G lanes per row
   const int gg = stride_grid(n * G, 256);
   const double* wl = weights.p + (size_t)l * 2 * sweep_steps();   // this level's sweep weights
-  auto jac = [&](T* xin, T* xout) {
+  auto jac = [&](T* xin, auto* xout) {
+    using O = std::remove_pointer_t<decltype(xout)>;
     ProfScope ps(pkey, n_jac, jac_bytes, s);
-    if (!rl) k_jac<T><<<g, 256, 0, s>>>(n, A.w, A.col, val, wl, dinv, b, xin, xout);
-    else if (G == 1) k_jac_g<T, 1><<<gg, 256, 0, s>>>(n, A.col, val, wl, dinv, b, xin, xout, rl);
-    else if (G == 2) k_jac_g<T, 2><<<gg, 256, 0, s>>>(n, A.col, val, wl, dinv, b, xin, xout, rl);
-    else if (G == 4) k_jac_g<T, 4><<<gg, 256, 0, s>>>(n, A.col, val, wl, dinv, b, xin, xout, rl);
-    else k_jac_g<T, 8><<<gg, 256, 0, s>>>(n, A.col, val, wl, dinv, b, xin, xout, rl);
+    if (!rl) k_jac<T, O><<<g, 256, 0, s>>>(n, A.w, A.col, val, wl, dinv, b, xin, xout);
+    else if (G == 1) k_jac_g<T, O, 1><<<gg, 256, 0, s>>>(n, A.col, val, wl, dinv, b, xin, xout, rl);
+    else if (G == 2) k_jac_g<T, O, 2><<<gg, 256, 0, s>>>(n, A.col, val, wl, dinv, b, xin, xout, rl);
+    else if (G == 4) k_jac_g<T, O, 4><<<gg, 256, 0, s>>>(n, A.col, val, wl, dinv, b, xin, xout, rl);
+    else k_jac_g<T, O, 8><<<gg, 256, 0, s>>>(n, A.col, val, wl, dinv, b, xin, xout, rl);
     FVS_COUNT_LAUNCH();
   };
   const bool cheb = opt.smoother == 1;
-  auto cheb_step = [&](T* xin, const T* xprev, T* xout, int k) {   // step k of the recurrence
+  auto cheb_step = [&](T* xin, const T* xprev, auto* xout, int k) {   // step k of the recurrence
+    using O = std::remove_pointer_t<decltype(xout)>;
     const double* ab = wl + 2 * k;
     ProfScope ps(pkey, n_jac, jac_bytes + vb * (double)n, s);
-    if (!rl) k_cheb<T><<<g, 256, 0, s>>>(n, A.w, A.col, val, ab, dinv, b, xin, xprev, xout);
-    else if (G == 1) k_cheb_g<T, 1><<<gg, 256, 0, s>>>(n, A.col, val, ab, dinv, b, xin, xprev, xout, rl);
-    else if (G == 2) k_cheb_g<T, 2><<<gg, 256, 0, s>>>(n, A.col, val, ab, dinv, b, xin, xprev, xout, rl);
-    else if (G == 4) k_cheb_g<T, 4><<<gg, 256, 0, s>>>(n, A.col, val, ab, dinv, b, xin, xprev, xout, rl);
-    else k_cheb_g<T, 8><<<gg, 256, 0, s>>>(n, A.col, val, ab, dinv, b, xin, xprev, xout, rl);
+    if (!rl) k_cheb<T, O><<<g, 256, 0, s>>>(n, A.w, A.col, val, ab, dinv, b, xin, xprev, xout);
+    else if (G == 1) k_cheb_g<T, O, 1><<<gg, 256, 0, s>>>(n, A.col, val, ab, dinv, b, xin, xprev, xout, rl);
+    else if (G == 2) k_cheb_g<T, O, 2><<<gg, 256, 0, s>>>(n, A.col, val, ab, dinv, b, xin, xprev, xout, rl);
+    else if (G == 4) k_cheb_g<T, O, 4><<<gg, 256, 0, s>>>(n, A.col, val, ab, dinv, b, xin, xprev, xout, rl);
+    else k_cheb_g<T, O, 8><<<gg, 256, 0, s>>>(n, A.col, val, ab, dinv, b, xin, xprev, xout, rl);
     FVS_COUNT_LAUNCH();
   };
   if (!x0_ready) {
@@ -2199,31 +2213,50 @@ fvs_status Amg::vcycle_t(cudaStream_t s, int l, const T* b, T* y, bool x0_ready)
   }
   FVS_COUNT_LAUNCH();
   FVS_LAUNCH_CHECK();
-  FVS_TRY(vcycle_t<T>(s, l + 1, cbv, cy, next_sweeps));
+  FVS_TRY((vcycle_t<T, T>(s, l + 1, cbv, cy, next_sweeps)));
   k_prolong<T><<<g, 256, 0, s>>>(n, L->agg, cy, (T)opt.coarse_scale, xa); FVS_COUNT_LAUNCH();
   {
-    for (int k = 0; k < opt.npost; ++k) {
-      T* out = (k == opt.npost - 1) ? y : xb;
-      if (cheb && k > 0) cheb_step(xa, xb, out, k);   // xb holds the iterate before xa
+    // the last sweep writes y; xb holds the iterate before xa
+    auto sweep = [&](auto* out, int k) {
+      if (cheb && k > 0) cheb_step(xa, xb, out, k);
       else jac(xa, out);
-      xb = xa;
-      xa = out;
+    };
+    for (int k = 0; k + 1 < opt.npost; ++k) {
+      sweep(xb, k);
+      T* t = xa; xa = xb; xb = t;
     }
+    sweep(y, opt.npost - 1);
   }
   FVS_LAUNCH_CHECK();
   return FVS_OK;
 }
 
+// mixed precision: the V-cycle runs in FP32, the Krylov method around it in FP64
 fvs_status Amg::apply(cudaStream_t s, const double* r, double* z) {
-  if (!opt.fp32) return vcycle_t<double>(s, 0, r, z);
-  // mixed precision: the V-cycle runs in FP32, the Krylov method around it in FP64
+  if (!opt.fp32) return vcycle_t<double, double>(s, 0, r, z);
   AmgLevel* L = lv[0].get();
   const int64_t n = L->n;
   k_convert<double, float><<<stride_grid(n, 256), 256, 0, s>>>(n, r, L->bf.p); FVS_COUNT_LAUNCH();
-  FVS_TRY(vcycle_t<float>(s, 0, L->bf.p, L->yf.p));
-  k_convert<float, double><<<stride_grid(n, 256), 256, 0, s>>>(n, L->yf.p, z); FVS_COUNT_LAUNCH();
   FVS_LAUNCH_CHECK();
-  return FVS_OK;
+  return vcycle_t<float, double>(s, 0, L->bf.p, z);
+}
+FirstSweep Amg::first(double*) {
+  FirstSweep f;
+  if (lv.size() < 2 || lv[0]->n == 0) return f;
+  AmgLevel* L = lv[0].get();
+  f.mode = opt.fp32 ? 2 : 1;
+  f.w = weights.p;
+  f.dinv = L->dinv.p;
+  f.x = L->x.p;
+  f.dinvf = L->dinvf.p;
+  f.bf = L->bf.p;
+  f.xf = L->xf.p;
+  return f;
+}
+fvs_status Amg::rest(cudaStream_t s, const double* r, double* z) {
+  if (lv.size() < 2 || lv[0]->n == 0) return apply(s, r, z);
+  if (!opt.fp32) return vcycle_t<double, double>(s, 0, r, z, true);
+  return vcycle_t<float, double>(s, 0, lv[0]->bf.p, z, true);
 }
 
 // FP32 copies of the level operators and vectors (mixed precision)

@@ -82,6 +82,8 @@ struct Amg : Precond {
   // so a new setup is needed.
   fvs_status refresh(cudaStream_t s, const int32_t* act, const uint8_t* ppe);
   fvs_status apply(cudaStream_t s, const double* r, double* z) override;
+  FirstSweep first(double* z) override;
+  fvs_status rest(cudaStream_t s, const double* r, double* z) override;
   uint64_t version = 0;          // bumped by every setup
   // coarsest inverse above the shared-memory size: the block steps' second
   // array, a vector, and the row exchanges of the column-by-column fallback
@@ -91,13 +93,15 @@ struct Amg : Precond {
   uint64_t signature() const override;
   // subtract the component mean on every singular component (fine level)
   fvs_status project(cudaStream_t s, double* v);
+  int single_part(MeanPart& m);   // see Projector::single
   int levels() const { return (int)lv.size(); }
 
  private:
   // x0_ready: the level's first Jacobi iterate from zero is already in its x
-  // (formed by the restriction from the level above)
-  template <typename T>
-  fvs_status vcycle_t(cudaStream_t s, int l, const T* b, T* y, bool x0_ready = false);
+  // (formed by the restriction from the level above, or by the Krylov kernel
+  // that formed b); y may be of another type on the fine level
+  template <typename T, typename Y>
+  fvs_status vcycle_t(cudaStream_t s, int l, const T* b, Y* y, bool x0_ready = false);
   fvs_status coarsest_setup(cudaStream_t s);
   fvs_status setup_fp32(cudaStream_t s);
   // sweep weights of every smoothed level (after a setup or a refresh, when
@@ -111,6 +115,7 @@ struct Amg : Precond {
 struct AmgProjector : Projector {
   Amg* amg = nullptr;
   fvs_status apply(cudaStream_t s, double* v) override { return amg->project(s, v); }
+  int single(MeanPart& m) override { return amg->single_part(m); }
 };
 
 // Pinned dense inverses of Sp coarsest systems at once (one block each):

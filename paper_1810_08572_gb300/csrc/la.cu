@@ -181,12 +181,12 @@ __device__ __forceinline__ double sdiv(double a, double b) { return b != 0.0 ? a
 // ---------------------------------------------------------------------------
 // Reductions fused into the Krylov kernels, and the scalars they finish
 // ---------------------------------------------------------------------------
-enum { FIN_RV = 0, FIN_TSTT = 1, FIN_RR_RHO = 2, FIN_PQ = 3, FIN_RR = 4, FIN_RZ = 5, FIN_START = 6, FIN_TRUE = 7 };
+enum { FIN_RV = 0, FIN_TSTT = 1, FIN_RR_RHO = 2, FIN_PQ = 3, FIN_RR = 4, FIN_RZ = 5, FIN_START = 6, FIN_TRUE = 7, FIN_RZM = 8 };
 
 template <int MODE>
-__device__ __forceinline__ void finish2(double x, double y, double* part, unsigned int* ticket, double* sc) {
-  constexpr int NS = MODE == FIN_TSTT || MODE == FIN_RR_RHO || MODE == FIN_START ? 2 : 1;
-  if (!grid_fold<OpSum, NS>(x, y, part, ticket)) return;
+__device__ __forceinline__ bool finish2(double x, double y, double* part, unsigned int* ticket, double* sc) {
+  constexpr int NS = MODE == FIN_TSTT || MODE == FIN_RR_RHO || MODE == FIN_START || MODE == FIN_RZM ? 2 : 1;
+  if (!grid_fold<OpSum, NS>(x, y, part, ticket)) return false;
   if (MODE == FIN_RV) {
     sc[S_RV] = x;
     sc[S_ALPHA] = sdiv(sc[S_RHO], x);
@@ -217,7 +217,9 @@ __device__ __forceinline__ void finish2(double x, double y, double* part, unsign
     sc[S_RZ_OLD] = rz;
     sc[S_RZ] = x;
     sc[S_BETA] = sdiv(x, rz);
+    if (MODE == FIN_RZM) sc[S_MEAN] = y;
   }
+  return true;
 }
 
 // y = A x (+ dextra x); sums d.y (and y.y in FIN_TSTT)
@@ -235,6 +237,43 @@ __global__ void __launch_bounds__(RB, 8) k_spmv_dot(int64_t n, int w, const int3
     if (MODE == FIN_TSTT) b = fma(acc, acc, b);
   }
   finish2<MODE>(a, b, part, ticket, sc);
+}
+
+template <int PM>
+__device__ __forceinline__ double first_weight(const FirstSweep& f) {
+  return PM != 0 && f.w ? f.w[0] : 1.0;
+}
+template <int PM>
+__device__ __forceinline__ void first_sweep(const FirstSweep& f, double w, int64_t i, double v) {
+  if (PM == 1) f.x[i] = w * f.dinv[i] * v;
+  if (PM == 2) {
+    const float b = (float)v;
+    f.bf[i] = b;
+    f.xf[i] = (float)w * f.dinvf[i] * b;
+  }
+}
+// the first sweep alone (before the first iteration of a CG recurrence)
+template <int PM>
+__global__ void k_first_sweep(int64_t n, FirstSweep f, const double* __restrict__ v) {
+  const double w = first_weight<PM>(f);
+  GRID_STRIDE(i, n) first_sweep<PM>(f, w, i, v[i]);
+}
+
+// Device-driven solve loop: the thread that finishes the last reduction of an
+// iteration decides whether the conditional while-node runs the body again
+// (no host round trip, no launch of its own).  Bounded by it[1]; a NaN
+// residual or a breakdown of the BiCGStab recurrence also stops the loop (the
+// host then restarts or reports).
+struct LoopCtl {
+  cudaGraphConditionalHandle h;
+  int* it = nullptr;    // counter and bound; null: no loop
+};
+__device__ __forceinline__ void loop_next(const LoopCtl& c, double* sc, bool alive) {
+  if (!c.it) return;
+  const int n = ++c.it[0];
+  sc[S_ITER] = (double)n;
+  const double rr = sc[S_RR];
+  cudaGraphSetConditional(c.h, n < c.it[1] && rr > sc[S_TOL2] && rr == rr && rr < 1e300 && alive ? 1u : 0u);
 }
 
 // BiCGStab without a projection: start (r = rh = b - A x, sums r.r = rh.r and
@@ -268,7 +307,8 @@ __global__ void __launch_bounds__(RB) k_bicg_xr_dot(int64_t n, double* __restric
                                                     const double* __restrict__ ph, const double* __restrict__ sh,
                                                     const double* __restrict__ sv, const double* __restrict__ t,
                                                     const double* __restrict__ rh, double* __restrict__ x,
-                                                    double* __restrict__ r, double* part, unsigned int* ticket) {
+                                                    double* __restrict__ r, double* part, unsigned int* ticket,
+                                                    LoopCtl ctl) {
   const double alpha = sc[S_ALPHA], omega = sc[S_OMEGA];
   double a = 0.0, b = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)RB + threadIdx.x; i < n; i += (int64_t)gridDim.x * RB) {
@@ -278,51 +318,94 @@ __global__ void __launch_bounds__(RB) k_bicg_xr_dot(int64_t n, double* __restric
     a = fma(ri, ri, a);
     b = fma(rh[i], ri, b);
   }
-  finish2<FIN_RR_RHO>(a, b, part, ticket, sc);
+  if (finish2<FIN_RR_RHO>(a, b, part, ticket, sc))
+    loop_next(ctl, sc, sc[S_TT] != 0.0 && sc[S_RV] != 0.0 && sc[S_RHO] != 0.0);
 }
 
-// CG: x += alpha p ; r -= alpha q ; sums r.r
+// CG: x += alpha p ; r -= alpha q ; sums r.r, and the preconditioner's first
+// sweep on the new r
+template <int PM>
 __global__ void __launch_bounds__(RB) k_cg_xr_dot(int64_t n, double* __restrict__ sc, const double* __restrict__ p,
                                                   const double* __restrict__ q, double* __restrict__ x,
-                                                  double* __restrict__ r, double* part, unsigned int* ticket) {
-  const double alpha = sc[S_ALPHA];
+                                                  double* __restrict__ r, FirstSweep f, double* part,
+                                                  unsigned int* ticket, LoopCtl ctl) {
+  const double alpha = sc[S_ALPHA], w = first_weight<PM>(f);
   double a = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)RB + threadIdx.x; i < n; i += (int64_t)gridDim.x * RB) {
     x[i] += alpha * p[i];
     const double ri = r[i] - alpha * q[i];
     r[i] = ri;
+    first_sweep<PM>(f, w, i, ri);
     a = fma(ri, ri, a);
   }
-  finish2<FIN_RR>(a, 0.0, part, ticket, sc);
+  if (finish2<FIN_RR>(a, 0.0, part, ticket, sc)) loop_next(ctl, sc, true);
 }
-// sums r.z (rz moved to rz_old)
+// CG: sums r.z (rz moved to rz_old); with a mean to project out of z also the
+// mean of z over its rows (r has zero sum there, so r.z is that of the
+// projected z), which k_cg_p subtracts as it reads z
+__device__ __forceinline__ bool in_mean(const MeanPart& m, int64_t i) {
+  return !m.lab || (m.want < 0 ? m.lab[i] >= 0 : m.lab[i] == m.want);
+}
+template <bool MEAN>
 __global__ void __launch_bounds__(RB) k_dot_rz(int64_t n, const double* __restrict__ r, const double* __restrict__ z,
-                                               double* part, unsigned int* ticket, double* sc) {
-  double a = 0.0;
-  for (int64_t i = blockIdx.x * (int64_t)RB + threadIdx.x; i < n; i += (int64_t)gridDim.x * RB)
-    a = fma(r[i], z[i], a);
-  finish2<FIN_RZ>(a, 0.0, part, ticket, sc);
+                                               MeanPart m, double* part, unsigned int* ticket, double* sc) {
+  double a = 0.0, b = 0.0;
+  for (int64_t i = blockIdx.x * (int64_t)RB + threadIdx.x; i < n; i += (int64_t)gridDim.x * RB) {
+    const double zi = z[i];
+    a = fma(r[i], zi, a);
+    if (MEAN && in_mean(m, i)) b += zi;
+  }
+  if (!MEAN) {
+    finish2<FIN_RZ>(a, 0.0, part, ticket, sc);
+  } else if (finish2<FIN_RZM>(a, b, part, ticket, sc)) {
+    const double c = m.cnt ? *m.cnt : (double)n;
+    sc[S_MEAN] = c > 0.0 ? sc[S_MEAN] / c : 0.0;
+  }
 }
 
-// BiCGStab: p = r + beta (p - omega v), beta = (rho/rho_old)(alpha/omega)
+// BiCGStab: p = r + beta (p - omega v), beta = (rho/rho_old)(alpha/omega),
+// and the preconditioner's first sweep on p
+template <int PM>
 __global__ void k_bicg_p(int64_t n, const double* __restrict__ sc, const double* __restrict__ r,
-                         const double* __restrict__ v, double* __restrict__ p, int first) {
+                         const double* __restrict__ v, double* __restrict__ p, int first, FirstSweep f) {
   first = first || sc[S_FIRST] != 0.0;
-  const double beta = sc[S_BETA], om = sc[S_OMEGA];
-  GRID_STRIDE(i, n) p[i] = first ? r[i] : r[i] + beta * (p[i] - om * v[i]);
+  const double beta = sc[S_BETA], om = sc[S_OMEGA], w = first_weight<PM>(f);
+  GRID_STRIDE(i, n) {
+    const double pi = first ? r[i] : r[i] + beta * (p[i] - om * v[i]);
+    p[i] = pi;
+    first_sweep<PM>(f, w, i, pi);
+  }
 }
-// s = r - alpha v, alpha = rho / (rh . v)
+// s = r - alpha v, alpha = rho / (rh . v), and the first sweep on s
+template <int PM>
 __global__ void k_bicg_s(int64_t n, const double* __restrict__ sc, const double* __restrict__ r,
-                         const double* __restrict__ v, double* __restrict__ sv) {
-  const double alpha = sc[S_ALPHA];
-  GRID_STRIDE(i, n) sv[i] = r[i] - alpha * v[i];
+                         const double* __restrict__ v, double* __restrict__ sv, FirstSweep f) {
+  const double alpha = sc[S_ALPHA], w = first_weight<PM>(f);
+  GRID_STRIDE(i, n) {
+    const double si = r[i] - alpha * v[i];
+    sv[i] = si;
+    first_sweep<PM>(f, w, i, si);
+  }
 }
+template <bool MEAN>
 __global__ void k_cg_p(int64_t n, const double* __restrict__ sc, const double* __restrict__ z,
-                       double* __restrict__ p, int first) {
+                       double* __restrict__ p, int first, MeanPart m) {
   first = first || sc[S_FIRST] != 0.0;
-  const double beta = sc[S_BETA];
-  GRID_STRIDE(i, n) p[i] = first ? z[i] : z[i] + beta * p[i];
+  const double beta = sc[S_BETA], mean = MEAN ? sc[S_MEAN] : 0.0;
+  GRID_STRIDE(i, n) {
+    double zi = z[i];
+    if (MEAN && in_mean(m, i)) zi -= mean;
+    p[i] = first ? zi : zi + beta * p[i];
+  }
 }
+#define FVS_BY_MODE(mode_, CALL)   \
+  do {                             \
+    if ((mode_) == 2) { constexpr int PM = 2; CALL; } \
+    else if ((mode_) == 1) { constexpr int PM = 1; CALL; } \
+    else { constexpr int PM = 0; CALL; } \
+    FVS_COUNT_LAUNCH();            \
+    FVS_LAUNCH_CHECK();            \
+  } while (0)
 
 constexpr int MAX_RESTARTS = 3;   // from the true residual, once the recursive one has met the tolerance
 
@@ -396,17 +479,17 @@ static uint64_t graph_key(const Ell& A, const double* dextra, const Precond& M, 
 
 template <typename F>
 static fvs_status run_body(cudaStream_t s, IterGraph* g, uint64_t key, bool first, F& body) {
-  if (first || !g || g->disabled || !graphs_enabled() || s == nullptr) return body(first);
+  if (first || !g || g->disabled || !graphs_enabled() || s == nullptr) return body(first, LoopCtl());
   if (!g->exec || g->key != key) {
     g->reset();
     cudaGraph_t graph = nullptr;
     if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
       cudaGetLastError();
       g->disabled = true;
-      return body(first);
+      return body(first, LoopCtl());
     }
     const unsigned long long before = __atomic_load_n(&g_launches, __ATOMIC_RELAXED);
-    fvs_status r = body(false);
+    fvs_status r = body(false, LoopCtl());
     g->kernels = __atomic_load_n(&g_launches, __ATOMIC_RELAXED) - before;
     __atomic_sub_fetch(&g_launches, g->kernels, __ATOMIC_RELAXED);   // counted when replayed
     cudaError_t e = cudaStreamEndCapture(s, &graph);
@@ -414,7 +497,7 @@ static fvs_status run_body(cudaStream_t s, IterGraph* g, uint64_t key, bool firs
       if (graph) cudaGraphDestroy(graph);
       cudaGetLastError();
       g->disabled = true;
-      return body(first);
+      return body(first, LoopCtl());
     }
     e = cudaGraphInstantiate(&g->exec, graph, 0);
     cudaGraphDestroy(graph);
@@ -422,7 +505,7 @@ static fvs_status run_body(cudaStream_t s, IterGraph* g, uint64_t key, bool firs
       cudaGetLastError();
       g->exec = nullptr;
       g->disabled = true;
-      return body(first);
+      return body(first, LoopCtl());
     }
     g->key = key;
   }
@@ -431,26 +514,6 @@ static fvs_status run_body(cudaStream_t s, IterGraph* g, uint64_t key, bool firs
   return FVS_OK;
 }
 
-// Loop controllers: the last node of each iteration decides on the device
-// whether the conditional while-node runs the body again (no host round
-// trip per iteration).  Bounded by maxit; a NaN residual or a breakdown of
-// the BiCGStab recurrence also stops the loop (the host then restarts or
-// reports).
-__global__ void k_ctl_bicg(cudaGraphConditionalHandle h, double* sc, int* it) {
-  const int n = ++it[0], maxit = it[1];
-  sc[S_ITER] = (double)n;
-  const double rr = sc[S_RR];
-  const bool go = n < maxit && rr > sc[S_TOL2] && rr == rr && rr < 1e300 && sc[S_TT] != 0.0 &&
-                  sc[S_RV] != 0.0 && sc[S_RHO] != 0.0;
-  cudaGraphSetConditional(h, go ? 1u : 0u);
-}
-__global__ void k_ctl_cg(cudaGraphConditionalHandle h, double* sc, int* it) {
-  const int n = ++it[0], maxit = it[1];
-  sc[S_ITER] = (double)n;
-  const double rr = sc[S_RR];
-  const bool go = n < maxit && rr > sc[S_TOL2] && rr == rr && rr < 1e300;
-  cudaGraphSetConditional(h, go ? 1u : 0u);
-}
 // (the bound lies beside the counter: a loop captured once serves every bound)
 __global__ void k_loop_init(double* sc, int* it, int maxit, double tol2, int fresh) {
   sc[S_FIRST] = fresh ? 1.0 : 0.0;
@@ -464,7 +527,7 @@ __global__ void k_loop_init(double* sc, int* it, int maxit, double tol2, int fre
 // conditional while-node; returns false (nothing launched) when the loop
 // graph cannot be used, so the caller iterates from the host instead.
 template <typename F>
-static bool run_loop(cudaStream_t s, IterGraph* g, uint64_t key, Reducer& red, double tol2, int maxit, bool bicg, bool fresh,
+static bool run_loop(cudaStream_t s, IterGraph* g, uint64_t key, Reducer& red, double tol2, int maxit, bool fresh,
                      F& body, fvs_status& st) {
   st = FVS_OK;
   if (!g || g->loop_disabled || !graphs_enabled() || s == nullptr || maxit <= 0) return false;
@@ -490,13 +553,12 @@ static bool run_loop(cudaStream_t s, IterGraph* g, uint64_t key, Reducer& red, d
            cudaSuccess;
       if (ok) {
         const unsigned long long before = __atomic_load_n(&g_launches, __ATOMIC_RELAXED);
-        fvs_status r = body(false);
-        if (bicg)
-          k_ctl_bicg<<<1, 1, 0, s>>>(h, red.sc.p, red.iter.p);
-        else
-          k_ctl_cg<<<1, 1, 0, s>>>(h, red.sc.p, red.iter.p);
-        g->loop_kernels = __atomic_load_n(&g_launches, __ATOMIC_RELAXED) - before + 1;
-        __atomic_sub_fetch(&g_launches, g->loop_kernels - 1, __ATOMIC_RELAXED);
+        LoopCtl ctl;
+        ctl.h = h;
+        ctl.it = red.iter.p;
+        fvs_status r = body(false, ctl);
+        g->loop_kernels = __atomic_load_n(&g_launches, __ATOMIC_RELAXED) - before;
+        __atomic_sub_fetch(&g_launches, g->loop_kernels, __ATOMIC_RELAXED);
         cudaGraph_t out = nullptr;
         const cudaError_t e = cudaStreamEndCapture(s, &out);
         ok = r == FVS_OK && e == cudaSuccess;
@@ -558,17 +620,16 @@ fvs_status bicgstab(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, c
   }
   // K x has zero sum on every singular part (zero column sums), so the
   // Krylov vectors stay in the range once r is projected
-  auto body = [&](bool first) -> fvs_status {
-    k_bicg_p<<<grid, 256, 0, s>>>(n, red.sc, w.r, w.v, w.p, first ? 1 : 0); FVS_COUNT_LAUNCH();
-    FVS_LAUNCH_CHECK();
-    FVS_TRY(M.apply(s, w.p, w.ph));
+  const FirstSweep fp = M.first(w.ph), fs = M.first(w.sh);
+  auto body = [&](bool first, const LoopCtl& ctl) -> fvs_status {
+    FVS_BY_MODE(fp.mode, (k_bicg_p<PM><<<grid, 256, 0, s>>>(n, red.sc, w.r, w.v, w.p, first ? 1 : 0, fp)));
+    FVS_TRY(M.rest(s, w.p, w.ph));
     FVS_TRY(spmv_dot(s, red, A, w.ph, w.v, dextra, w.rh, FIN_RV));
-    k_bicg_s<<<grid, 256, 0, s>>>(n, red.sc, w.r, w.v, w.sv); FVS_COUNT_LAUNCH();
-    FVS_LAUNCH_CHECK();
-    FVS_TRY(M.apply(s, w.sv, w.sh));
+    FVS_BY_MODE(fs.mode, (k_bicg_s<PM><<<grid, 256, 0, s>>>(n, red.sc, w.r, w.v, w.sv, fs)));
+    FVS_TRY(M.rest(s, w.sv, w.sh));
     FVS_TRY(spmv_dot(s, red, A, w.sh, w.t, dextra, w.sv, FIN_TSTT));
     k_bicg_xr_dot<<<red.grid(n), RB, 0, s>>>(n, red.sc, w.ph, w.sh, w.sv, w.t, w.rh, x, w.r, red.part,
-                                              red.ticket); FVS_COUNT_LAUNCH();
+                                              red.ticket, ctl); FVS_COUNT_LAUNCH();
     FVS_LAUNCH_CHECK();
     return FVS_OK;
   };
@@ -583,7 +644,7 @@ fvs_status bicgstab(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, c
       bool looped = false;
       {
         fvs_status st = FVS_OK;
-        looped = run_loop(s, graph, key, red, tol2, maxit - it, true, fresh, body, st);
+        looped = run_loop(s, graph, key, red, tol2, maxit - it, fresh, body, st);
         FVS_TRY(st);
       }
       if (!looped) FVS_TRY(run_body(s, graph, key, fresh, body));
@@ -668,18 +729,34 @@ fvs_status pcg(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, Precon
     res.converged = true;
     return FVS_OK;
   }
-  auto body = [&](bool first) -> fvs_status {
-    FVS_TRY(M.apply(s, w.r, w.z));
-    if (proj) FVS_TRY(proj->apply(s, w.z));
-    k_dot_rz<<<red.grid(n), RB, 0, s>>>(n, w.r, w.z, red.part, red.ticket, red.sc); FVS_COUNT_LAUNCH();
-    k_cg_p<<<grid, 256, 0, s>>>(n, red.sc, w.z, w.p, first ? 1 : 0); FVS_COUNT_LAUNCH();
+  const FirstSweep f = M.first(w.z);
+  MeanPart mp;
+  const int how = proj ? proj->single(mp) : 0;
+  auto body = [&](bool first, const LoopCtl& ctl) -> fvs_status {
+    // (the first sweep on r is done already)
+    FVS_TRY(M.rest(s, w.r, w.z));
+    if (how == 2) FVS_TRY(proj->apply(s, w.z));
+    if (how == 1) {
+      k_dot_rz<true><<<red.grid(n), RB, 0, s>>>(n, w.r, w.z, mp, red.part, red.ticket, red.sc); FVS_COUNT_LAUNCH();
+      k_cg_p<true><<<grid, 256, 0, s>>>(n, red.sc, w.z, w.p, first ? 1 : 0, mp); FVS_COUNT_LAUNCH();
+    } else {
+      k_dot_rz<false><<<red.grid(n), RB, 0, s>>>(n, w.r, w.z, mp, red.part, red.ticket, red.sc); FVS_COUNT_LAUNCH();
+      k_cg_p<false><<<grid, 256, 0, s>>>(n, red.sc, w.z, w.p, first ? 1 : 0, mp); FVS_COUNT_LAUNCH();
+    }
     FVS_LAUNCH_CHECK();
     FVS_TRY(spmv_dot(s, red, A, w.p, w.q, nullptr, w.p, FIN_PQ));
-    k_cg_xr_dot<<<red.grid(n), RB, 0, s>>>(n, red.sc, w.p, w.q, x, w.r, red.part, red.ticket); FVS_COUNT_LAUNCH();
+    FVS_BY_MODE(f.mode, (k_cg_xr_dot<PM><<<red.grid(n), RB, 0, s>>>(n, red.sc, w.p, w.q, x, w.r, f, red.part,
+                                                                    red.ticket, ctl)));
+    return FVS_OK;
+  };
+  auto prepare = [&]() -> fvs_status {
+    if (f.mode == 1) { k_first_sweep<1><<<grid, 256, 0, s>>>(n, f, w.r); FVS_COUNT_LAUNCH(); }
+    if (f.mode == 2) { k_first_sweep<2><<<grid, 256, 0, s>>>(n, f, w.r); FVS_COUNT_LAUNCH(); }
     FVS_LAUNCH_CHECK();
     return FVS_OK;
   };
-  const uint64_t key = graph_key(A, nullptr, M, b, x, w, red) ^ (proj ? 0x70636770ULL : 0x70636700ULL);
+  FVS_TRY(prepare());
+  const uint64_t key = graph_key(A, nullptr, M, b, x, w, red) ^ (0x70636770ULL + (uint64_t)how);
   const double tol2 = (rtol * bnorm) * (rtol * bnorm);
   bool fresh = true;
   int it = 0;
@@ -688,7 +765,7 @@ fvs_status pcg(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, Precon
       bool looped = false;
       {
         fvs_status st = FVS_OK;
-        looped = run_loop(s, graph, key, red, tol2, maxit - it, false, fresh, body, st);
+        looped = run_loop(s, graph, key, red, tol2, maxit - it, fresh, body, st);
         FVS_TRY(st);
       }
       if (!looped) FVS_TRY(run_body(s, graph, key, fresh, body));
@@ -716,6 +793,7 @@ fvs_status pcg(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, Precon
     if (res.converged || !met || bad(res.relres) || again == MAX_RESTARTS || it >= maxit) break;
     res.converged = false;
     fresh = true;    // from the true residual, as in bicgstab
+    FVS_TRY(prepare());
   }
   return FVS_OK;
 }
