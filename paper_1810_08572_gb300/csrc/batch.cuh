@@ -24,7 +24,7 @@ constexpr int BATCH_NCM = 8;   // liquid pockets per sample handled by the null-
 
 // per-sample scalar slots of the batched Krylov drivers: sc[slot * Sp + s]
 enum BSlot {
-  B_RHO = 0, B_RHO_OLD, B_ALPHA, B_OMEGA, B_RV, B_TS, B_TT, B_RR, B_BB, B_RZ, B_RZ_OLD, B_PQ, B_TOL2,
+  B_RHO = 0, B_RHO_OLD, B_ALPHA, B_OMEGA, B_RV, B_TS, B_TT, B_RR, B_BB, B_RZ, B_RZ_OLD, B_PQ, B_TOL2, B_BETA,
   B_FIRST, B_T0, B_T1, B_T2, B_NSLOT
 };
 
@@ -104,6 +104,7 @@ struct Batch {
 
   // per-sample inputs
   DBuf<double> Tliq, Twall, Tmelt;   // [Sp]
+  DBuf<double> lawd;                 // [3*Sp] constants of each sample's solid-fraction law
   // grain growth (Eq. 24-26): r^2 [Nc*Sp] when D_s > 0
   double grain_kp = 0.0, grain_Ds = 0.0;
   DBuf<double> r2;
@@ -152,11 +153,14 @@ struct Batch {
   DBuf<uint8_t> csing;            // [Sp][nc]
   DBuf<int> cncomp;               // [Sp]
   DBuf<int32_t> cid;              // compact projected part per (s, coarsest part) [Sp*nc]
-  DBuf<double> ccnt, csum;        // [Sp*BATCH_NCM]
+  DBuf<double> ccnt, csum;        // [BATCH_NCM*Sp] 1 / rows of each projected part, its mean
+  DBuf<int> npart;                // [Sp] projected parts of each sample
+  DBuf<int8_t> pid;               // [Nc*Sp] projected part of every fine row (-1: none)
   DBuf<int> ccount;               // [Sp*nc] fine rows per coarsest part
   bool amg_ok = false;
   bool fp32 = false;              // FP32 V-cycle inside the FP64 Krylov method
   AmgOptions aopt;
+  bool two_sweeps = false;        // V(2,2) instead of V(1,1)
 
   // reductions
   int nb = 0;                     // row blocks of the reduction kernels
