@@ -67,7 +67,10 @@ struct Amg : Precond {
   bool masked = false;            // the projection reads the fine labels (rows with label -1 take no part)
   int refreshes = 0;              // refreshes since the setup
 
-  fvs_status setup(cudaStream_t s, const Ell& A);
+  // diagonal_first: seven slots a row, the diagonal in slot 0 and no other
+  // slot of a row holding it (but zeros that point at the row itself)
+  fvs_status setup(cudaStream_t s, const Ell& A, bool diagonal_first = false);
+  bool diag_first = false;
   fvs_status count_stored(cudaStream_t s);   // AmgLevel::stored of every level
   // The operator's values changed on the same rows: rows of cells without
   // pressure (ppe[act[i]] == 0: frozen since the setup) leave their

@@ -64,7 +64,7 @@ static inline void dswap_b(DBuf<T>& a, DBuf<T>& b) {
 // reduction but the plain dot products is fused into the kernel that forms its
 // operands.  At 4,608 rows x 32 samples a dot product takes 6.8 us (12.4 with
 // a walk over 38 partials a lane, one load at a time), r.z with the parts'
-// sums 10.8 (36.9 as three launches), the CG update with r.r 9.2 (19.5 as
+// sums 13.1 (36.9 as three launches), the CG update with r.r 9.0 (19.5 as
 // three).
 struct RSum { static __device__ __forceinline__ double f(double a, double b) { return a + b; } };
 struct RMax { static __device__ __forceinline__ double f(double a, double b) { return fmax(a, b); } };

@@ -10,20 +10,33 @@ namespace fvs {
 // ---------------------------------------------------------------------------
 // SpMV and residual (ELL, one thread per row, slot-major coalesced loads)
 // ---------------------------------------------------------------------------
+// the row kernels by width (7: face-only rows) and by whether the matrix streams
+#define FVS_BY_ROW(A_, CALL)                                                     \
+  do {                                                                           \
+    const bool big_ = (A_).n * (int64_t)(A_).w * 12 > L2_KEEP_BYTES;             \
+    if ((A_).w == 7 && big_) { constexpr int W = 7; constexpr bool CS = true; CALL; }        \
+    else if ((A_).w == 7) { constexpr int W = 7; constexpr bool CS = false; CALL; }          \
+    else if (big_) { constexpr int W = 0; constexpr bool CS = true; CALL; }      \
+    else { constexpr int W = 0; constexpr bool CS = false; CALL; }               \
+    FVS_COUNT_LAUNCH();                                                          \
+  } while (0)
+
+template <int W, bool CS>
 __global__ void k_spmv(int64_t n, int w, const int32_t* __restrict__ col, const double* __restrict__ val,
                        const double* __restrict__ x, double* __restrict__ y,
                        const double* __restrict__ dextra) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const double acc = ell_row(n, w, col, val, x, i, dextra ? dextra[i] * x[i] : 0.0);
+    const double acc = ell_row<W, CS>(n, w, col, val, x, i, dextra ? dextra[i] * x[i] : 0.0);
     y[i] = acc;
   }
 }
 
+template <int W, bool CS>
 __global__ void k_residual(int64_t n, int w, const int32_t* __restrict__ col, const double* __restrict__ val,
                            const double* __restrict__ x, const double* __restrict__ b, double* __restrict__ r,
                            const double* __restrict__ dextra) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const double acc = ell_row(n, w, col, val, x, i, dextra ? dextra[i] * x[i] : 0.0);
+    const double acc = ell_row<W, CS>(n, w, col, val, x, i, dextra ? dextra[i] * x[i] : 0.0);
     r[i] = b[i] - acc;
   }
 }
@@ -31,7 +44,7 @@ __global__ void k_residual(int64_t n, int w, const int32_t* __restrict__ col, co
 fvs_status spmv(cudaStream_t s, const Ell& A, const double* x, double* y, const double* dextra) {
   if (A.n == 0) return FVS_OK;
   ProfScope ps(&A, "spmv", (double)A.n * (12.0 * A.w + 16.0 + (dextra ? 8.0 : 0.0)), s);
-  k_spmv<<<stride_grid(A.n, 256), 256, 0, s>>>(A.n, A.w, A.col, A.val, x, y, dextra); FVS_COUNT_LAUNCH();
+  FVS_BY_ROW(A, (k_spmv<W, CS><<<stride_grid(A.n, 256), 256, 0, s>>>(A.n, A.w, A.col, A.val, x, y, dextra)));
   FVS_LAUNCH_CHECK();
   return FVS_OK;
 }
@@ -40,7 +53,7 @@ fvs_status residual(cudaStream_t s, const Ell& A, const double* x, const double*
                     const double* dextra) {
   if (A.n == 0) return FVS_OK;
   ProfScope ps(&A, "residual", (double)A.n * (12.0 * A.w + 24.0 + (dextra ? 8.0 : 0.0)), s);
-  k_residual<<<stride_grid(A.n, 256), 256, 0, s>>>(A.n, A.w, A.col, A.val, x, b, r, dextra); FVS_COUNT_LAUNCH();
+  FVS_BY_ROW(A, (k_residual<W, CS><<<stride_grid(A.n, 256), 256, 0, s>>>(A.n, A.w, A.col, A.val, x, b, r, dextra)));
   FVS_LAUNCH_CHECK();
   return FVS_OK;
 }
@@ -223,15 +236,15 @@ __device__ __forceinline__ bool finish2(double x, double y, double* part, unsign
 }
 
 // y = A x (+ dextra x); sums d.y (and y.y in FIN_TSTT)
-template <int MODE, bool DX>
-__global__ void __launch_bounds__(RB, 8) k_spmv_dot(int64_t n, int w, const int32_t* __restrict__ col,
+template <int MODE, bool DX, int W, bool CS>
+__global__ void __launch_bounds__(RB, W > 0 ? 6 : 8) k_spmv_dot(int64_t n, int w, const int32_t* __restrict__ col,
                                                     const double* __restrict__ val, const double* __restrict__ x,
                                                     double* __restrict__ y, const double* __restrict__ dextra,
                                                     const double* __restrict__ d, double* part,
                                                     unsigned int* ticket, double* sc) {
   double a = 0.0, b = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)RB + threadIdx.x; i < n; i += (int64_t)gridDim.x * RB) {
-    const double acc = ell_row(n, w, col, val, x, i, DX ? dextra[i] * x[i] : 0.0);
+    const double acc = ell_row<W, CS>(n, w, col, val, x, i, DX ? dextra[i] * x[i] : 0.0);
     y[i] = acc;
     a = fma(d[i], acc, a);
     if (MODE == FIN_TSTT) b = fma(acc, acc, b);
@@ -281,8 +294,8 @@ __device__ __forceinline__ void loop_next(const LoopCtl& c, double* sc, bool ali
 // each instead of a residual, a copy and two dot products (2,097,152 rows of
 // 27 entries: 128 and 124 us, the residual alone 126 us; at 184,320 rows 19
 // and 17 us, where the separate launches took 45 and 31)
-template <int MODE, bool DX>
-__global__ void __launch_bounds__(RB, 8) k_residual_dot(int64_t n, int w, const int32_t* __restrict__ col,
+template <int MODE, bool DX, int W, bool CS>
+__global__ void __launch_bounds__(RB, W > 0 ? 6 : 8) k_residual_dot(int64_t n, int w, const int32_t* __restrict__ col,
                                                         const double* __restrict__ val, const double* __restrict__ x,
                                                         const double* __restrict__ dextra,
                                                         const double* __restrict__ b, double* __restrict__ r,
@@ -290,7 +303,7 @@ __global__ void __launch_bounds__(RB, 8) k_residual_dot(int64_t n, int w, const 
                                                         unsigned int* ticket, double* sc) {
   double rr = 0.0, bb = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)RB + threadIdx.x; i < n; i += (int64_t)gridDim.x * RB) {
-    const double acc = ell_row(n, w, col, val, x, i, DX ? dextra[i] * x[i] : 0.0);
+    const double acc = ell_row<W, CS>(n, w, col, val, x, i, DX ? dextra[i] * x[i] : 0.0);
     const double bi = b[i], ri = bi - acc;
     if (MODE == FIN_START) {
       r[i] = ri;
@@ -312,8 +325,8 @@ __global__ void __launch_bounds__(RB) k_bicg_xr_dot(int64_t n, double* __restric
   const double alpha = sc[S_ALPHA], omega = sc[S_OMEGA];
   double a = 0.0, b = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)RB + threadIdx.x; i < n; i += (int64_t)gridDim.x * RB) {
-    x[i] += alpha * ph[i] + omega * sh[i];
-    const double ri = sv[i] - omega * t[i];
+    x[i] = fma(alpha, ph[i], fma(omega, sh[i], x[i]));
+    const double ri = fma(-omega, t[i], sv[i]);
     r[i] = ri;
     a = fma(ri, ri, a);
     b = fma(rh[i], ri, b);
@@ -411,33 +424,34 @@ constexpr int MAX_RESTARTS = 3;   // from the true residual, once the recursive 
 
 static inline bool bad(double v) { return !(v == v) || v > 1e300 || v < -1e300; }
 
+template <int MODE, bool DX>
+static void launch_spmv_dot(cudaStream_t s, Reducer& red, const Ell& A, const double* x, double* y,
+                            const double* dextra, const double* d) {
+  FVS_BY_ROW(A, (k_spmv_dot<MODE, DX, W, CS><<<red.grid(A.n), RB, 0, s>>>(A.n, A.w, A.col, A.val, x, y, dextra, d,
+                                                                          red.part, red.ticket, red.sc)));
+}
+template <int MODE>
 static fvs_status spmv_dot(cudaStream_t s, Reducer& red, const Ell& A, const double* x, double* y,
-                           const double* dextra, const double* d, int mode) {
+                           const double* dextra, const double* d) {
   ProfScope ps(&A, "spmv", (double)A.n * (12.0 * A.w + 24.0 + (dextra ? 8.0 : 0.0)), s);
-  const int g = red.grid(A.n);
-#define FVS_SPMV_DOT(M_, D_) \
-  k_spmv_dot<M_, D_><<<g, RB, 0, s>>>(A.n, A.w, A.col, A.val, x, y, dextra, d, red.part, red.ticket, red.sc)
-  if (mode == FIN_RV) { if (dextra) FVS_SPMV_DOT(FIN_RV, true); else FVS_SPMV_DOT(FIN_RV, false); }
-  else if (mode == FIN_TSTT) { if (dextra) FVS_SPMV_DOT(FIN_TSTT, true); else FVS_SPMV_DOT(FIN_TSTT, false); }
-  else { if (dextra) FVS_SPMV_DOT(FIN_PQ, true); else FVS_SPMV_DOT(FIN_PQ, false); }
-#undef FVS_SPMV_DOT
-  FVS_COUNT_LAUNCH();
+  if (dextra) launch_spmv_dot<MODE, true>(s, red, A, x, y, dextra, d);
+  else launch_spmv_dot<MODE, false>(s, red, A, x, y, dextra, d);
   FVS_LAUNCH_CHECK();
   return FVS_OK;
 }
 
+template <int MODE, bool DX>
+static void launch_residual_dot(cudaStream_t s, Reducer& red, const Ell& A, const double* x, const double* dextra,
+                                const double* b, double* r, double* rh) {
+  FVS_BY_ROW(A, (k_residual_dot<MODE, DX, W, CS><<<red.grid(A.n), RB, 0, s>>>(A.n, A.w, A.col, A.val, x, dextra, b, r,
+                                                                              rh, red.part, red.ticket, red.sc)));
+}
 template <int MODE>
 static fvs_status residual_dot(cudaStream_t s, Reducer& red, const Ell& A, const double* x, const double* dextra,
                                const double* b, double* r, double* rh) {
   ProfScope ps(&A, "residual", (double)A.n * (12.0 * A.w + (MODE == FIN_START ? 32.0 : 16.0) + (dextra ? 8.0 : 0.0)), s);
-  const int g = red.grid(A.n);
-  if (dextra)
-    k_residual_dot<MODE, true><<<g, RB, 0, s>>>(A.n, A.w, A.col, A.val, x, dextra, b, r, rh, red.part, red.ticket,
-                                                red.sc);
-  else
-    k_residual_dot<MODE, false><<<g, RB, 0, s>>>(A.n, A.w, A.col, A.val, x, dextra, b, r, rh, red.part, red.ticket,
-                                                 red.sc);
-  FVS_COUNT_LAUNCH();
+  if (dextra) launch_residual_dot<MODE, true>(s, red, A, x, dextra, b, r, rh);
+  else launch_residual_dot<MODE, false>(s, red, A, x, dextra, b, r, rh);
   FVS_LAUNCH_CHECK();
   return FVS_OK;
 }
@@ -624,10 +638,10 @@ fvs_status bicgstab(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, c
   auto body = [&](bool first, const LoopCtl& ctl) -> fvs_status {
     FVS_BY_MODE(fp.mode, (k_bicg_p<PM><<<grid, 256, 0, s>>>(n, red.sc, w.r, w.v, w.p, first ? 1 : 0, fp)));
     FVS_TRY(M.rest(s, w.p, w.ph));
-    FVS_TRY(spmv_dot(s, red, A, w.ph, w.v, dextra, w.rh, FIN_RV));
+    FVS_TRY(spmv_dot<FIN_RV>(s, red, A, w.ph, w.v, dextra, w.rh));
     FVS_BY_MODE(fs.mode, (k_bicg_s<PM><<<grid, 256, 0, s>>>(n, red.sc, w.r, w.v, w.sv, fs)));
     FVS_TRY(M.rest(s, w.sv, w.sh));
-    FVS_TRY(spmv_dot(s, red, A, w.sh, w.t, dextra, w.sv, FIN_TSTT));
+    FVS_TRY(spmv_dot<FIN_TSTT>(s, red, A, w.sh, w.t, dextra, w.sv));
     k_bicg_xr_dot<<<red.grid(n), RB, 0, s>>>(n, red.sc, w.ph, w.sh, w.sv, w.t, w.rh, x, w.r, red.part,
                                               red.ticket, ctl); FVS_COUNT_LAUNCH();
     FVS_LAUNCH_CHECK();
@@ -744,7 +758,7 @@ fvs_status pcg(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, Precon
       k_cg_p<false><<<grid, 256, 0, s>>>(n, red.sc, w.z, w.p, first ? 1 : 0, mp); FVS_COUNT_LAUNCH();
     }
     FVS_LAUNCH_CHECK();
-    FVS_TRY(spmv_dot(s, red, A, w.p, w.q, nullptr, w.p, FIN_PQ));
+    FVS_TRY(spmv_dot<FIN_PQ>(s, red, A, w.p, w.q, nullptr, w.p));
     FVS_BY_MODE(f.mode, (k_cg_xr_dot<PM><<<red.grid(n), RB, 0, s>>>(n, red.sc, w.p, w.q, x, w.r, f, red.part,
                                                                     red.ticket, ctl)));
     return FVS_OK;

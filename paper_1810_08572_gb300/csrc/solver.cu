@@ -1192,9 +1192,10 @@ static fvs_status assemble_pressure(fvs_solver s) {
     // V-cycle sweep (7 instead of 27 entries a fine row, narrower Galerkin
     // rows below) while the Krylov method keeps the full K
     const char* pc = getenv("FVS_PC_COMPACT");
-    s->pc_compact = m->W > 7 && !(pc && *pc == '0');
+    // (a face-only row keeps its seven entries, its diagonal moved to slot 0)
+    s->pc_compact = m->W >= 7 && !(pc && *pc == '0');
     if (s->pc_compact) FVS_TRY(fill_compact());
-    fvs_status r = s->amg.setup(st, s->pc_compact ? s->Kp : s->K);
+    fvs_status r = s->amg.setup(st, s->pc_compact ? s->Kp : s->K, s->pc_compact);
     if (r == FVS_OK) {
       s->amg_ok = true;
       s->amg_levels = s->amg.levels();
