@@ -397,31 +397,49 @@ __device__ __forceinline__ void kb_part_add(int k, double v, double* a) {
 }
 // CG, one iteration after z = M^-1 r:
 //  kb_cg_z   sums z over the rows of every projected part (pid: the part's
-//            index, -1 none) and r.z; mean[part], rz, beta.  r has zero sum on
-//            those parts, so r.z is that of the projected z.
+//            index, -1 none) and r.z; mean[part], rz, beta.  r.z of the
+//            projected z is r.z less mean times the part's sum of r (zero but
+//            for rounding, which counts near the attainable residual).
 //  kb_cg_p   p = (z - mean) + beta p
 //  kb_cg_xr  x += alpha p, r -= alpha q, r.r, activity; and, for the FP32
 //            cycle, its right side bf = (float) r and first sweep xf
 template <typename Z>
 __global__ void kb_cg_z(int64_t n, int Sp, const double* __restrict__ r, const Z* __restrict__ z,
-                        const int8_t* __restrict__ pid, const double* __restrict__ cinv, const int* nparts, double* part, double* mean, double* sc, int* cnt, int* counts) {
+                        const int8_t* __restrict__ pid, const double* __restrict__ cinv, const int* nparts, double* part,
+                        double* mean, double* sc, int* cnt, int* counts) {
   BSAMPLE;
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 3 && threadIdx.y == 0) counts[threadIdx.x] = 0;
   const int np = kb_tile_parts(nparts, s);
-  double v[BATCH_NCM + 1];   // r.z, then the parts' sums
+  double v[1 + 2 * BATCH_NCM];   // r.z, then the sums of z and of r over each part in turn
 #pragma unroll
-  for (int k = 0; k <= BATCH_NCM; ++k) v[k] = 0.0;
+  for (int k = 0; k < 1 + 2 * BATCH_NCM; ++k) v[k] = 0.0;
   BROW4(i, n) {
     const int64_t e = i * Sp + s;
-    const double ze = (double)z[e];
-    kb_part_add(pid[e], ze, v + 1);
-    v[0] = fma(r[e], ze, v[0]);
+    const double ze = (double)z[e], re = r[e];
+    const int k = pid[e];
+    v[0] = fma(re, ze, v[0]);
+    if (k == 0) {
+      v[1] += ze;
+      v[2] += re;
+    } else if (k > 0) {
+#pragma unroll
+      for (int q = 1; q < BATCH_NCM; ++q)
+        if (q == k) {
+          v[1 + 2 * q] += ze;
+          v[2 + 2 * q] += re;
+        }
+    }
   }
-  if (!kb_tile_fold<RSum>(Sp, v, part, cnt, np + 1)) return;
+  if (!kb_tile_fold<RSum>(Sp, v, part, cnt, 1 + 2 * np)) return;
+  double rz = v[0];
 #pragma unroll
   for (int k = 0; k < BATCH_NCM; ++k)
-    if (k < np) mean[k * Sp + s] = v[k + 1] * cinv[k * Sp + s];
-  const double rz_old = sc[B_RZ * Sp + s], rz = v[0];
+    if (k < np) {
+      const double m = v[1 + 2 * k] * cinv[k * Sp + s];
+      mean[k * Sp + s] = m;
+      rz -= m * v[2 + 2 * k];
+    }
+  const double rz_old = sc[B_RZ * Sp + s];
   sc[B_RZ_OLD * Sp + s] = rz_old;
   sc[B_RZ * Sp + s] = rz;
   sc[B_BETA * Sp + s] = bsdiv(rz, rz_old);
@@ -2467,7 +2485,7 @@ fvs_status batch_run(fvs_mesh mesh, const fvs_props* base, int64_t n, const doub
       {
         const int64_t rows = std::max<int64_t>(std::max(Nc, Nf), Nv);
         const int nbm = red_blocks(rows, B.tiles);
-        FVS_TRY(B.part.alloc((size_t)(BATCH_NCM + 1) * Sp * nbm + 1));
+        FVS_TRY(B.part.alloc((size_t)(2 * BATCH_NCM + 1) * Sp * nbm + 1));
         FVS_TRY(B.redcnt.alloc((size_t)Sp / 32 + 1));
         FVS_TRY(B.redcnt.zero(B.stream));
       }

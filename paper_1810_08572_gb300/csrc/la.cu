@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(RB) k_maxdiff2(int64_t n, const double* __rest
 fvs_status Reducer::init() {
   cudaStream_t st = g_alloc_stream;
   blocks = 8 * sm_count();   // full occupancy for the fused SpMV + reduction kernels
-  FVS_TRY(part.alloc(2 * (size_t)blocks));
+  FVS_TRY(part.alloc(3 * (size_t)blocks));
   FVS_TRY(sc.alloc(S_NSLOT));
   FVS_TRY(sc.zero(st));
   FVS_TRY(ticket.alloc(1));
@@ -194,11 +194,11 @@ __device__ __forceinline__ double sdiv(double a, double b) { return b != 0.0 ? a
 // ---------------------------------------------------------------------------
 // Reductions fused into the Krylov kernels, and the scalars they finish
 // ---------------------------------------------------------------------------
-enum { FIN_RV = 0, FIN_TSTT = 1, FIN_RR_RHO = 2, FIN_PQ = 3, FIN_RR = 4, FIN_RZ = 5, FIN_START = 6, FIN_TRUE = 7, FIN_RZM = 8 };
+enum { FIN_RV = 0, FIN_TSTT = 1, FIN_RR_RHO = 2, FIN_PQ = 3, FIN_RR = 4, FIN_START = 5, FIN_TRUE = 6 };
 
 template <int MODE>
 __device__ __forceinline__ bool finish2(double x, double y, double* part, unsigned int* ticket, double* sc) {
-  constexpr int NS = MODE == FIN_TSTT || MODE == FIN_RR_RHO || MODE == FIN_START || MODE == FIN_RZM ? 2 : 1;
+  constexpr int NS = MODE == FIN_TSTT || MODE == FIN_RR_RHO || MODE == FIN_START ? 2 : 1;
   if (!grid_fold<OpSum, NS>(x, y, part, ticket)) return false;
   if (MODE == FIN_RV) {
     sc[S_RV] = x;
@@ -225,12 +225,6 @@ __device__ __forceinline__ bool finish2(double x, double y, double* part, unsign
     sc[S_BB] = y;
   } else if (MODE == FIN_TRUE) {
     sc[S_RR] = x;
-  } else {
-    const double rz = sc[S_RZ];
-    sc[S_RZ_OLD] = rz;
-    sc[S_RZ] = x;
-    sc[S_BETA] = sdiv(x, rz);
-    if (MODE == FIN_RZM) sc[S_MEAN] = y;
   }
   return true;
 }
@@ -354,26 +348,35 @@ __global__ void __launch_bounds__(RB) k_cg_xr_dot(int64_t n, double* __restrict_
   if (finish2<FIN_RR>(a, 0.0, part, ticket, sc)) loop_next(ctl, sc, true);
 }
 // CG: sums r.z (rz moved to rz_old); with a mean to project out of z also the
-// mean of z over its rows (r has zero sum there, so r.z is that of the
-// projected z), which k_cg_p subtracts as it reads z
+// mean of z over its rows, which k_cg_p subtracts as it reads z, and the sum
+// of r over them (zero but for rounding, which counts near the attainable
+// residual): r.z of the projected z is r.z - mean sum(r)
 __device__ __forceinline__ bool in_mean(const MeanPart& m, int64_t i) {
   return !m.lab || (m.want < 0 ? m.lab[i] >= 0 : m.lab[i] == m.want);
 }
 template <bool MEAN>
 __global__ void __launch_bounds__(RB) k_dot_rz(int64_t n, const double* __restrict__ r, const double* __restrict__ z,
                                                MeanPart m, double* part, unsigned int* ticket, double* sc) {
-  double a = 0.0, b = 0.0;
+  double v[MEAN ? 3 : 1] = {};
   for (int64_t i = blockIdx.x * (int64_t)RB + threadIdx.x; i < n; i += (int64_t)gridDim.x * RB) {
-    const double zi = z[i];
-    a = fma(r[i], zi, a);
-    if (MEAN && in_mean(m, i)) b += zi;
+    const double zi = z[i], ri = r[i];
+    v[0] = fma(ri, zi, v[0]);
+    if (MEAN && in_mean(m, i)) {
+      v[MEAN ? 1 : 0] += zi;
+      v[MEAN ? 2 : 0] += ri;
+    }
   }
-  if (!MEAN) {
-    finish2<FIN_RZ>(a, 0.0, part, ticket, sc);
-  } else if (finish2<FIN_RZM>(a, b, part, ticket, sc)) {
-    const double c = m.cnt ? *m.cnt : (double)n;
-    sc[S_MEAN] = c > 0.0 ? sc[S_MEAN] / c : 0.0;
+  if (!grid_fold<OpSum, MEAN ? 3 : 1>(v, part, ticket)) return;
+  double rz = v[0];
+  if (MEAN) {
+    const double c = m.cnt ? *m.cnt : (double)n, mean = c > 0.0 ? v[MEAN ? 1 : 0] / c : 0.0;
+    sc[S_MEAN] = mean;
+    rz -= mean * v[MEAN ? 2 : 0];
   }
+  const double old = sc[S_RZ];
+  sc[S_RZ_OLD] = old;
+  sc[S_RZ] = rz;
+  sc[S_BETA] = sdiv(rz, old);
 }
 
 // BiCGStab: p = r + beta (p - omega v), beta = (rho/rho_old)(alpha/omega),
@@ -653,6 +656,7 @@ fvs_status bicgstab(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, c
   bool fresh = true;
   int it = 0;
   const double tol2 = (rtol * bnorm) * (rtol * bnorm);
+  double best = 0.0;   // true residual before a restart (its iterate in w.z)
   for (int again = 0;; ++again) {
     while (it < maxit) {
       bool looped = false;
@@ -670,7 +674,13 @@ fvs_status bicgstab(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, c
       rn = sqrt(red.host[S_RR]);
       res.iters = it;
       res.relres = rn / bnorm;
-      if (bad(rn)) return FVS_OK;
+      if (bad(rn)) {
+        if (again > 0) {
+          FVS_TRY(vcopy(s, n, w.z, x));
+          res.relres = best;
+        }
+        return FVS_OK;
+      }
       if (res.relres <= rtol) {
         res.converged = true;
         break;
@@ -698,9 +708,17 @@ fvs_status bicgstab(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, c
     res.converged = res.relres <= rtol * 10.0 && !bad(res.relres);
     // the recursive residual drifted too far from the true one (tight
     // tolerances on large systems): start again from the true residual
-    // rather than give the solve up
+    // rather than give the solve up; an attempt that ends further off than it
+    // began is undone
+    if (again > 0 && !(res.relres <= best)) {
+      FVS_TRY(vcopy(s, n, w.z, x));
+      res.relres = best;
+      res.converged = false;
+      break;
+    }
     if (res.converged || !met || bad(res.relres) || again == MAX_RESTARTS || it >= maxit) break;
-    res.converged = false;
+    best = res.relres;
+    FVS_TRY(vcopy(s, n, x, w.z));
     if (!proj) {
       FVS_TRY(residual_dot<FIN_START>(s, red, A, x, dextra, b, w.r, w.rh));
     } else {
@@ -774,6 +792,7 @@ fvs_status pcg(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, Precon
   const double tol2 = (rtol * bnorm) * (rtol * bnorm);
   bool fresh = true;
   int it = 0;
+  double best = 0.0;   // true residual before a restart (its iterate in w.v)
   for (int again = 0;; ++again) {
     while (it < maxit) {
       bool looped = false;
@@ -791,7 +810,13 @@ fvs_status pcg(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, Precon
       const double rn = sqrt(red.host[S_RR]);
       res.iters = it;
       res.relres = rn / bnorm;
-      if (bad(rn)) return FVS_OK;
+      if (bad(rn)) {
+        if (again > 0) {
+          FVS_TRY(vcopy(s, n, w.v, x));
+          res.relres = best;
+        }
+        return FVS_OK;
+      }
       if (res.relres <= rtol) {
         res.converged = true;
         break;
@@ -804,8 +829,15 @@ fvs_status pcg(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, Precon
     res.relres = sqrt(red.host[S_RR]) / bnorm;
     const bool met = res.converged;
     res.converged = res.relres <= rtol * 10.0 && !bad(res.relres);
+    if (again > 0 && !(res.relres <= best)) {
+      FVS_TRY(vcopy(s, n, w.v, x));
+      res.relres = best;
+      res.converged = false;
+      break;
+    }
     if (res.converged || !met || bad(res.relres) || again == MAX_RESTARTS || it >= maxit) break;
-    res.converged = false;
+    best = res.relres;
+    FVS_TRY(vcopy(s, n, x, w.v));
     fresh = true;    // from the true residual, as in bicgstab
     FVS_TRY(prepare());
   }

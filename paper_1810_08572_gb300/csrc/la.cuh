@@ -165,11 +165,30 @@ struct LinePrecond : Precond {
   DBuf<int32_t> cell;      // [padded] cell at (group, position, lane)
   DBuf<int8_t> sprev, snext;   // slot of the previous / next cell of the line in the cell's row (-1: none)
   DBuf<double> lo, inv, cp;    // sub-diagonal, 1 / pivot, super-diagonal / pivot
+  DBuf<double> yl;             // forward substitution, in line order
   bool ready = false;
+  // Whether the lines pay: with a and b the mean shares of a row's diagonal
+  // that Jacobi and the lines leave out, the iterations go down by about
+  // sqrt((1 + a)(1 - b) / ((1 - a)(1 + b))), and an iteration costs about 1.4
+  // (27-point rows) or twice (face-only rows) as much.  All melt on 128^3
+  // thin cells (gain 5): 142 -> 25 inner iterations, 193 -> 158 ms for three
+  // steps.  Half frozen on 96^3 (gain 2.5): 107 -> 97 ms, but near the solidus
+  // the two solutions, each within the tolerance, differed by up to 2e-8 of u
+  // in single cells, so the line is drawn above it.  Below MIN_ROWS a
+  // substitution's serial walk costs more than the iterations it saves.
+  static constexpr int64_t MIN_ROWS = 65536;
+  static constexpr double GAIN_WIDE = 3.0, GAIN_FACE = 4.0;
+  static fvs_status worth(cudaStream_t s, Reducer& red, const Ell& A, const double* dextra, bool& use);
   fvs_status build(cudaStream_t s, const Ell& A);
   fvs_status factor(cudaStream_t s);
   fvs_status apply(cudaStream_t s, const double* r, double* z) override;
-  uint64_t signature() const override { return (uint64_t)(uintptr_t)inv.p * 29u + (uint64_t)n; }
+  uint64_t signature() const override {
+    uint64_t h = (uint64_t)n * 131u + (uint64_t)ngroups;
+    for (const void* q : {(const void*)goff.p, (const void*)llen.p, (const void*)cell.p, (const void*)lo.p,
+                          (const void*)inv.p, (const void*)cp.p, (const void*)yl.p})
+      h = h * 1099511628211ULL ^ (uint64_t)(uintptr_t)q;
+    return h;
+  }
 };
 
 struct KrylovWork {

@@ -2,21 +2,26 @@
 // of strongly coupled cells.  Used for the energy system, whose couplings
 // across thin cells exceed its mass term several times over, so that
 // point-Jacobi needs many Krylov iterations.
-#include <vector>
+#include <cub/device/device_radix_sort.cuh>
+
+#include <cmath>
 
 #include "la.cuh"
-#include "lines_host.h"
+#include "reduce.cuh"
+#include "scan.cuh"
 
 namespace fvs {
 
 namespace {
 
+constexpr int LCH = 8;          // positions of a line whose loads are in flight together
 constexpr int kMaxLine = 512;   // longer chains are cut (a dropped coupling keeps P a valid preconditioner)
 
 // Thomas factors of every line with the current values: row k of a line
 // reads lo_k x_{k-1} + b_k x_k + up_k x_{k+1}; pivots d_k = b_k - lo_k cp_{k-1},
-// cp_k = up_k / d_k.  One thread per line.
-__global__ void k_line_factor(int64_t ngroups, const int64_t* __restrict__ goff, const int32_t* __restrict__ llen,
+// cp_k = up_k / d_k.  One thread per line, the loads of eight positions in
+// flight together (16,384 lines of 128 cells: 196 -> 105 us).
+__global__ void __launch_bounds__(64) k_line_factor(int64_t ngroups, const int64_t* __restrict__ goff, const int32_t* __restrict__ llen,
                               const int32_t* __restrict__ cell, const int8_t* __restrict__ sprev,
                               const int8_t* __restrict__ snext, int64_t n, const double* __restrict__ val,
                               const double* __restrict__ diag, const double* __restrict__ dextra,
@@ -28,53 +33,269 @@ __global__ void k_line_factor(int64_t ngroups, const int64_t* __restrict__ goff,
   const int len = llen[t];
   const int64_t base = goff[g] + lane;
   double cprev = 0.0;
-#pragma unroll 4
-  for (int pos = 0; pos < len; ++pos) {
-    const int64_t idx = base + (int64_t)pos * 32;
-    const int32_t c = cell[idx];
-    const int kp = sprev[idx], kn = snext[idx];
-    const double a = kp >= 0 ? val[(int64_t)kp * n + c] : 0.0;
-    const double u = kn >= 0 ? val[(int64_t)kn * n + c] : 0.0;
-    const double d = diag[c] + (dextra ? dextra[c] : 0.0) - a * cprev;
-    const double iv = d != 0.0 ? 1.0 / d : 0.0;
-    lo[idx] = a;
-    inv[idx] = iv;
-    cprev = u * iv;
-    cp[idx] = cprev;
+  for (int p0 = 0; p0 < len; p0 += LCH) {
+    const int m = min(LCH, len - p0);
+    const int64_t i0 = base + (int64_t)p0 * 32;
+    double a[LCH], u[LCH], d[LCH];
+#pragma unroll
+    for (int k = 0; k < LCH; ++k) {
+      const int64_t idx = i0 + (k < m ? k : 0) * 32;
+      const int32_t c = cell[idx];
+      const int kp = sprev[idx], kn = snext[idx];
+      a[k] = kp >= 0 ? val[(int64_t)kp * n + c] : 0.0;
+      u[k] = kn >= 0 ? val[(int64_t)kn * n + c] : 0.0;
+      d[k] = diag[c] + (dextra ? dextra[c] : 0.0);
+    }
+#pragma unroll
+    for (int k = 0; k < LCH; ++k)
+      if (k < m) {
+        const double piv = d[k] - a[k] * cprev;
+        const double iv = piv != 0.0 ? 1.0 / piv : 0.0;
+        cprev = u[k] * iv;
+        lo[i0 + k * 32] = a[k];
+        inv[i0 + k * 32] = iv;
+        cp[i0 + k * 32] = cprev;
+      }
   }
 }
 
-// z = P^-1 r: forward substitution y_k = (r_k - lo_k y_{k-1}) / d_k (kept in
-// z), then back substitution x_k = y_k - cp_k x_{k+1}.
-__global__ void k_line_solve(int64_t ngroups, const int64_t* __restrict__ goff, const int32_t* __restrict__ llen,
-                             const int32_t* __restrict__ cell, const double* __restrict__ lo,
-                             const double* __restrict__ inv, const double* __restrict__ cp, const double* r,
-                             double* z) {
+// z = P^-1 r: forward substitution y_k = (r_k - lo_k y_{k-1}) / d_k, then back
+// substitution x_k = y_k - cp_k x_{k+1}.  One thread per line, so a launch is
+// bound by the latency of its loads: eight positions are loaded together, and
+// y is kept in line order, where a warp's stores and loads are contiguous
+// (only r is gathered and z scattered by cell).  16,384 lines of 128 cells:
+// 57 us.
+__global__ void __launch_bounds__(64) k_line_solve(int64_t ngroups, const int64_t* __restrict__ goff,
+                                                   const int32_t* __restrict__ llen,
+                                                   const int32_t* __restrict__ cell, const double* __restrict__ lo,
+                                                   const double* __restrict__ inv, const double* __restrict__ cp,
+                                                   const double* __restrict__ r, double* __restrict__ yl,
+                                                   double* __restrict__ z) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t g = t >> 5;
   if (g >= ngroups) return;
-  const int lane = (int)(t & 31);
   const int len = llen[t];
-  const int64_t base = goff[g] + lane;
+  const int64_t base = goff[g] + (int)(t & 31);
   double y = 0.0;
-#pragma unroll 4
-  for (int pos = 0; pos < len; ++pos) {
-    const int64_t idx = base + (int64_t)pos * 32;
-    const int32_t c = cell[idx];
-    y = (r[c] - lo[idx] * y) * inv[idx];
-    z[c] = y;
+  for (int p0 = 0; p0 < len; p0 += LCH) {
+    const int m = min(LCH, len - p0);
+    const int64_t i0 = base + (int64_t)p0 * 32;
+    double l[LCH], d[LCH], q[LCH];
+#pragma unroll
+    for (int k = 0; k < LCH; ++k) {
+      const int64_t idx = i0 + (k < m ? k : 0) * 32;
+      q[k] = r[cell[idx]];
+      l[k] = lo[idx];
+      d[k] = inv[idx];
+    }
+#pragma unroll
+    for (int k = 0; k < LCH; ++k)
+      if (k < m) {
+        y = (q[k] - l[k] * y) * d[k];
+        yl[i0 + k * 32] = y;
+      }
   }
   double x = 0.0;
-#pragma unroll 4
-  for (int pos = len - 1; pos >= 0; --pos) {
-    const int64_t idx = base + (int64_t)pos * 32;
-    const int32_t c = cell[idx];
-    x = z[c] - cp[idx] * x;
-    z[c] = x;
+  for (int p1 = len; p1 > 0; p1 -= LCH) {
+    const int m = min(LCH, p1);
+    const int64_t i1 = base + (int64_t)(p1 - 1) * 32;
+    double u[LCH], q[LCH];
+    int32_t c[LCH];
+#pragma unroll
+    for (int k = 0; k < LCH; ++k) {
+      const int64_t idx = i1 - (k < m ? k : 0) * 32;
+      c[k] = cell[idx];
+      u[k] = cp[idx];
+      q[k] = yl[idx];
+    }
+#pragma unroll
+    for (int k = 0; k < LCH; ++k)
+      if (k < m) {
+        x = q[k] - u[k] * x;
+        z[c[k]] = x;
+      }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// the chains, on the device (build_line_layout in lines_host.h is the same
+// rule on the host, against which the layout is checked)
+// ---------------------------------------------------------------------------
+// two largest off-diagonal couplings of a row (the first slot wins a tie),
+// the second only if at least a quarter of the first
+__device__ __forceinline__ void strongest2(int64_t n, int w, const int32_t* col, const double* val, int64_t i,
+                                           int32_t& b0, int32_t& b1, double& m0, double& m1) {
+  m0 = m1 = 0.0;
+  b0 = b1 = -1;
+  for (int k = 0; k < w; ++k) {
+    const int32_t j = col[(int64_t)k * n + i];
+    if (j == (int32_t)i) continue;
+    const double a = fabs(val[(int64_t)k * n + i]);
+    if (!(a > 0.0)) continue;
+    if (a > m0) {
+      if (j != b0) { m1 = m0; b1 = b0; }
+      m0 = a;
+      b0 = j;
+    } else if (a > m1 && j != b0) {
+      m1 = a;
+      b1 = j;
+    }
+  }
+  if (!(m1 >= 0.25 * m0)) { b1 = -1; m1 = 0.0; }
+}
+__global__ void k_line_best(int64_t n, int w, const int32_t* __restrict__ col, const double* __restrict__ val,
+                            int32_t* __restrict__ best) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    int32_t b0, b1;
+    double m0, m1;
+    strongest2(n, w, col, val, i, b0, b1, m0, m1);
+    best[2 * i] = b0;
+    best[2 * i + 1] = b1;
+  }
+}
+// couplings that both rows chose
+__global__ void k_line_links(int64_t n, const int32_t* __restrict__ best, int32_t* __restrict__ nb) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    int32_t l[2] = {-1, -1};
+    int q = 0;
+    for (int t = 0; t < 2; ++t) {
+      const int32_t j = best[2 * i + t];
+      if (j >= 0 && (best[2 * (int64_t)j] == (int32_t)i || best[2 * (int64_t)j + 1] == (int32_t)i)) l[q++] = j;
+    }
+    nb[2 * i] = l[0];
+    nb[2 * i + 1] = l[1];
+  }
+}
+// Walks along the chains: node 2 i + d stands at cell i, about to leave it by
+// link d.  jump = the node some hops on, hops = how many; a node whose link
+// is missing is an end (itself, 0 hops).  Each round doubles the hops.
+__global__ void k_line_walk0(int64_t n, const int32_t* __restrict__ nb, int2* __restrict__ walk) {
+  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < 2 * n; v += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t i = (int32_t)(v >> 1), j = nb[v];
+    if (j < 0) walk[v] = make_int2((int32_t)v, 0);
+    else walk[v] = make_int2(2 * j + (nb[2 * (int64_t)j] == i ? 1 : 0), 1);
+  }
+}
+__global__ void k_line_walk(int64_t n2, const int2* __restrict__ in, int2* __restrict__ out) {
+  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n2; v += (int64_t)gridDim.x * blockDim.x) {
+    const int2 a = in[v], b = in[a.x];
+    out[v] = make_int2(b.x, a.y + b.y);
+  }
+}
+// place of every cell: head cell of its chain (the end with the smaller id),
+// position, and at the head the number of lines the chain is cut into.  A
+// cell whose walks have not both ended (a cycle, or a chain longer than the
+// rounds reach, the same for all its cells) is a line of its own.
+constexpr int WALK_ROUNDS = 12, MAX_CHAIN = 1 << WALK_ROUNDS;
+__global__ void k_line_place(int64_t n, const int32_t* __restrict__ nb, const int2* __restrict__ walk, int max_line,
+                             int32_t* __restrict__ head, int32_t* __restrict__ place, int32_t* __restrict__ len,
+                             int32_t* __restrict__ cnt) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int2 a = walk[2 * i], b = walk[2 * i + 1];
+    int32_t h = (int32_t)i, p = 0, m = 1;
+    int dir = 0;                 // link towards the head
+    if (nb[a.x] < 0 && nb[b.x] < 0 && a.y + b.y < MAX_CHAIN) {
+      const int32_t ea = a.x >> 1, eb = b.x >> 1;
+      dir = ea <= eb ? 0 : 1;
+      h = dir == 0 ? ea : eb;
+      p = dir == 0 ? a.y : b.y;
+      m = a.y + b.y + 1;
+    } else {
+      dir = 2;                   // off the chains
+    }
+    head[i] = h;
+    place[i] = p * 4 + dir;
+    len[i] = m;
+    cnt[i] = p == 0 ? (m + max_line - 1) / max_line : 0;
+  }
+}
+// lengths of the lines, by line; sort keys put longer lines first
+__global__ void k_line_lengths(int64_t n, const int32_t* __restrict__ place, const int32_t* __restrict__ len,
+                               const int32_t* __restrict__ first, int max_line, int32_t* __restrict__ key,
+                               int32_t* __restrict__ id) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    if (place[i] >> 2) continue;
+    const int m = len[i], nl = (m + max_line - 1) / max_line;
+    for (int q = 0; q < nl; ++q) {
+      key[first[i] + q] = max_line - min(max_line, m - q * max_line);
+      id[first[i] + q] = first[i] + q;
+    }
+  }
+}
+__global__ void k_line_groups(int nl, int ng, int max_line, const int32_t* __restrict__ key,
+                              const int32_t* __restrict__ id, int32_t* __restrict__ rank, int32_t* __restrict__ llen,
+                              int32_t* __restrict__ glen) {
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < ng * 32; t += gridDim.x * blockDim.x) {
+    llen[t] = t < nl ? max_line - key[t] : 0;
+    if (t < nl) rank[id[t]] = t;
+    if ((t & 31) == 0) glen[t >> 5] = max_line - key[t];
+  }
+}
+__global__ void k_line_offsets(int ng, const int32_t* __restrict__ sum, int64_t* __restrict__ goff) {
+  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < ng; g += gridDim.x * blockDim.x) goff[g] = 32LL * sum[g];
+}
+__global__ void k_line_fill(int64_t n, int w, const int32_t* __restrict__ col, const int32_t* __restrict__ nb,
+                            const int32_t* __restrict__ head, const int32_t* __restrict__ place,
+                            const int32_t* __restrict__ first, const int32_t* __restrict__ rank,
+                            const int32_t* __restrict__ llen, const int64_t* __restrict__ goff, int max_line,
+                            int32_t* __restrict__ cell, int8_t* __restrict__ sprev, int8_t* __restrict__ snext) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int p = place[i] >> 2, dir = place[i] & 3, pos = p % max_line;
+    const int32_t t = rank[first[head[i]] + p / max_line];
+    const int64_t e = goff[t >> 5] + (int64_t)pos * 32 + (t & 31);
+    const int32_t jp = dir < 2 && pos > 0 ? nb[2 * i + dir] : -1;
+    const int32_t jn = dir < 2 && pos + 1 < llen[t] ? nb[2 * i + 1 - dir] : -1;
+    int8_t sp = -1, sn = -1;
+    for (int k = w - 1; k >= 0; --k) {
+      const int32_t j = col[(int64_t)k * n + i];
+      if (j == jp) sp = (int8_t)k;
+      if (j == jn) sn = (int8_t)k;
+    }
+    cell[e] = (int32_t)i;
+    sprev[e] = jp >= 0 ? sp : (int8_t)-1;
+    snext[e] = jn >= 0 ? sn : (int8_t)-1;
+  }
+}
+// sums over the rows of |off-diagonal| / diagonal, and of the same without
+// each row's chain couplings: what Jacobi and the lines leave out
+__global__ void __launch_bounds__(RB) k_line_weight(int64_t n, int w, const int32_t* __restrict__ col,
+                                                    const double* __restrict__ val, const double* __restrict__ diag,
+                                                    const double* __restrict__ dextra, double* part,
+                                                    unsigned int* ticket, double* sc, int s0, int s1) {
+  double x = 0.0, y = 0.0;
+  for (int64_t i = blockIdx.x * (int64_t)RB + threadIdx.x; i < n; i += (int64_t)gridDim.x * RB) {
+    int32_t b0, b1;
+    double m0, m1, off = 0.0;
+    strongest2(n, w, col, val, i, b0, b1, m0, m1);
+    for (int k = 0; k < w; ++k)
+      if (col[(int64_t)k * n + i] != (int32_t)i) off += fabs(val[(int64_t)k * n + i]);
+    const double d = fabs(diag[i] + (dextra ? dextra[i] : 0.0));
+    if (d > 0.0) {
+      x += off / d;
+      y += (off - m0 - m1) / d;
+    }
+  }
+  if (grid_fold<OpSum, 2>(x, y, part, ticket)) {
+    sc[s0] = x;
+    sc[s1] = y;
   }
 }
 
 }  // namespace
+
+fvs_status LinePrecond::worth(cudaStream_t s, Reducer& red, const Ell& Ain, const double* dx, bool& use) {
+  use = false;
+  if (Ain.n < MIN_ROWS || Ain.w < 3) return FVS_OK;
+  k_line_weight<<<red.grid(Ain.n), RB, 0, s>>>(Ain.n, Ain.w, Ain.col, Ain.val, Ain.diag, dx, red.part, red.ticket,
+                                               red.sc, S_TMP0, S_TMP1);
+  FVS_COUNT_LAUNCH();
+  FVS_LAUNCH_CHECK();
+  FVS_TRY(red.fetch(s));
+  const double a = std::min(0.999, red.host[S_TMP0] / (double)Ain.n);
+  const double b = std::max(0.0, std::min(a, red.host[S_TMP1] / (double)Ain.n));
+  use = std::sqrt((1.0 + a) * (1.0 - b) / ((1.0 - a) * (1.0 + b))) > (Ain.w > 7 ? GAIN_WIDE : GAIN_FACE);
+  return FVS_OK;
+}
 
 fvs_status LinePrecond::build(cudaStream_t s, const Ell& Ain) {
   ready = false;
@@ -83,36 +304,78 @@ fvs_status LinePrecond::build(cudaStream_t s, const Ell& Ain) {
   w = Ain.w;
   built_from = Ain.col.p;
   if (n <= 0) return FVS_OK;
-  if (n > 2147483647LL) {
-    set_error("line preconditioner: %lld rows exceed 32-bit cell ids", (long long)n);
+  if (n > 1073741823LL) {
+    set_error("line preconditioner: %lld rows exceed 31-bit node ids", (long long)n);
     return FVS_ERR_ARG;
   }
-  const size_t nw = (size_t)n * (size_t)w;
-  std::vector<int32_t> col(nw);
-  std::vector<double> val(nw);
-  FVS_CUDA(cudaMemcpyAsync(col.data(), Ain.col.p, nw * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-  FVS_CUDA(cudaMemcpyAsync(val.data(), Ain.val.p, nw * sizeof(double), cudaMemcpyDeviceToHost, s));
+  const int g = stride_grid(n, 256);
+  DBuf<int32_t> nb, head, place, len, cnt, first;
+  FVS_TRY(nb.alloc(2 * (size_t)n));
+  {
+    DBuf<int32_t> best;
+    FVS_TRY(best.alloc(2 * (size_t)n));
+    k_line_best<<<g, 256, 0, s>>>(n, w, Ain.col, Ain.val, best); FVS_COUNT_LAUNCH();
+    k_line_links<<<g, 256, 0, s>>>(n, best, nb); FVS_COUNT_LAUNCH();
+    FVS_LAUNCH_CHECK();
+  }
+  FVS_TRY(head.alloc(n)); FVS_TRY(place.alloc(n)); FVS_TRY(len.alloc(n));
+  FVS_TRY(cnt.alloc((size_t)n + 1)); FVS_TRY(first.alloc((size_t)n + 1));
+  {
+    DBuf<int2> wa, wb;
+    FVS_TRY(wa.alloc(2 * (size_t)n)); FVS_TRY(wb.alloc(2 * (size_t)n));
+    k_line_walk0<<<stride_grid(2 * n, 256), 256, 0, s>>>(n, nb, wa); FVS_COUNT_LAUNCH();
+    for (int q = 0; q < WALK_ROUNDS; ++q) {
+      k_line_walk<<<stride_grid(2 * n, 256), 256, 0, s>>>(2 * n, (q & 1) ? wb.p : wa.p, (q & 1) ? wa.p : wb.p);
+      FVS_COUNT_LAUNCH();
+    }
+    FVS_TRY(cnt.zero(s));
+    k_line_place<<<g, 256, 0, s>>>(n, nb, (WALK_ROUNDS & 1) ? wb.p : wa.p, kMaxLine, head, place, len, cnt);
+    FVS_COUNT_LAUNCH();
+    FVS_LAUNCH_CHECK();
+  }
+  ScanWork sw;
+  FVS_TRY(exclusive_scan(s, sw, n + 1, cnt, first));
+  int32_t nl = 0;
+  FVS_CUDA(cudaMemcpyAsync(&nl, first.p + n, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   FVS_CUDA(cudaStreamSynchronize(s));
-  LineLayout L;
-  build_line_layout(col.data(), val.data(), n, w, kMaxLine, L);
-  nlines = L.nlines;
-  ngroups = L.ngroups;
-  padded = L.padded;
-  max_len = L.max_len;
-  FVS_TRY(goff.alloc(ngroups + 1));
-  FVS_TRY(llen.alloc((size_t)ngroups * 32 + 1));
+  nlines = nl;
+  ngroups = (nl + 31) / 32;
+  const int ng = (int)ngroups;
+  DBuf<int32_t> key, id, key2, id2, rank, glen, gsum;
+  FVS_TRY(key.alloc(nl)); FVS_TRY(id.alloc(nl)); FVS_TRY(key2.alloc(nl)); FVS_TRY(id2.alloc(nl));
+  FVS_TRY(rank.alloc(nl)); FVS_TRY(glen.alloc((size_t)ng + 1)); FVS_TRY(gsum.alloc((size_t)ng + 1));
+  FVS_TRY(goff.alloc((size_t)ng + 1)); FVS_TRY(llen.alloc((size_t)ng * 32 + 1));
+  k_line_lengths<<<g, 256, 0, s>>>(n, place, len, first, kMaxLine, key, id); FVS_COUNT_LAUNCH();
+  FVS_LAUNCH_CHECK();
+  {
+    size_t bytes = 0;
+    FVS_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, bytes, key.p, key2.p, id.p, id2.p, nl, 0, 10, s));
+    DBuf<char> tmp;
+    FVS_TRY(tmp.alloc(bytes + 1));
+    FVS_CUDA(cub::DeviceRadixSort::SortPairs(tmp.p, bytes, key.p, key2.p, id.p, id2.p, nl, 0, 10, s));
+  }
+  FVS_TRY(glen.zero(s));
+  k_line_groups<<<stride_grid((int64_t)ng * 32, 256), 256, 0, s>>>(nl, ng, kMaxLine, key2, id2, rank, llen, glen);
+  FVS_COUNT_LAUNCH();
+  FVS_TRY(exclusive_scan(s, sw, ng + 1, glen, gsum));
+  k_line_offsets<<<stride_grid(ng + 1, 256), 256, 0, s>>>(ng + 1, gsum, goff); FVS_COUNT_LAUNCH();
+  int32_t total = 0, longest = 0;
+  FVS_CUDA(cudaMemcpyAsync(&total, gsum.p + ng, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+  FVS_CUDA(cudaMemcpyAsync(&longest, llen.p, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+  FVS_CUDA(cudaStreamSynchronize(s));
+  padded = 32LL * total;
+  max_len = longest;
   FVS_TRY(cell.alloc(padded + 1));
   FVS_TRY(sprev.alloc(padded + 1));
   FVS_TRY(snext.alloc(padded + 1));
   FVS_TRY(lo.alloc(padded + 1));
   FVS_TRY(inv.alloc(padded + 1));
   FVS_TRY(cp.alloc(padded + 1));
-  FVS_CUDA(cudaMemcpyAsync(goff.p, L.goff.data(), (ngroups + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
-  FVS_CUDA(cudaMemcpyAsync(llen.p, L.llen.data(), L.llen.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-  FVS_CUDA(cudaMemcpyAsync(cell.p, L.cell.data(), padded * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-  FVS_CUDA(cudaMemcpyAsync(sprev.p, L.sprev.data(), padded * sizeof(int8_t), cudaMemcpyHostToDevice, s));
-  FVS_CUDA(cudaMemcpyAsync(snext.p, L.snext.data(), padded * sizeof(int8_t), cudaMemcpyHostToDevice, s));
-  FVS_CUDA(cudaStreamSynchronize(s));   // the host arrays go out of scope
+  FVS_TRY(yl.alloc(padded + 1));
+  FVS_CUDA(cudaMemsetAsync(cell.p, 0, (padded + 1) * sizeof(int32_t), s));   // padding is never visited
+  k_line_fill<<<g, 256, 0, s>>>(n, w, Ain.col, nb, head, place, first, rank, llen, goff, kMaxLine, cell, sprev, snext);
+  FVS_COUNT_LAUNCH();
+  FVS_LAUNCH_CHECK();
   ready = true;
   return FVS_OK;
 }
@@ -120,7 +383,7 @@ fvs_status LinePrecond::build(cudaStream_t s, const Ell& Ain) {
 fvs_status LinePrecond::factor(cudaStream_t s) {
   if (!ready || n <= 0) return FVS_OK;
   const int64_t threads = ngroups * 32;
-  k_line_factor<<<grid_for(threads, 128), 128, 0, s>>>(ngroups, goff, llen, cell, sprev, snext, n, A->val,
+  k_line_factor<<<grid_for(threads, 64), 64, 0, s>>>(ngroups, goff, llen, cell, sprev, snext, n, A->val,
                                                       A->diag, dextra, lo, inv, cp);
   FVS_COUNT_LAUNCH();
   FVS_LAUNCH_CHECK();
@@ -130,7 +393,7 @@ fvs_status LinePrecond::factor(cudaStream_t s) {
 fvs_status LinePrecond::apply(cudaStream_t s, const double* r, double* z) {
   if (n <= 0) return FVS_OK;
   const int64_t threads = ngroups * 32;
-  k_line_solve<<<grid_for(threads, 128), 128, 0, s>>>(ngroups, goff, llen, cell, lo, inv, cp, r, z);
+  k_line_solve<<<grid_for(threads, 64), 64, 0, s>>>(ngroups, goff, llen, cell, lo, inv, cp, r, yl, z);
   FVS_COUNT_LAUNCH();
   FVS_LAUNCH_CHECK();
   return FVS_OK;

@@ -28,14 +28,14 @@ constexpr int RB = 256;   // threads per reduction block
 struct OpSum { static __device__ __forceinline__ double f(double a, double b) { return a + b; } };
 struct OpMax { static __device__ __forceinline__ double f(double a, double b) { return fmax(a, b); } };
 
-// NS sums (1 or 2) of the RB threads of a block; result s (s < NS) is valid
+// NS sums (1 to 3) of the RB threads of a block; result s (s < NS) is valid
 // in lane 0 of warp s
 template <class OP, int NS>
-__device__ __forceinline__ double block_fold(double a, double b) {
+__device__ __forceinline__ double block_fold(const double (&a)[NS]) {
   __shared__ double sh[NS][RB];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  sh[0][threadIdx.x] = a;
-  if (NS > 1) sh[NS - 1][threadIdx.x] = b;
+#pragma unroll
+  for (int k = 0; k < NS; ++k) sh[k][threadIdx.x] = a[k];
   __syncthreads();
   double v = 0.0;
   if (w < NS) {
@@ -47,14 +47,15 @@ __device__ __forceinline__ double block_fold(double a, double b) {
   return v;
 }
 
-// Grid-wide sums of a (and b): true in thread 0 of the block that finishes
-// last, with the sums in a and b.  All partials are non-negative under OpMax.
+// Grid-wide sums of a[0 .. NS - 1]: true in thread 0 of the block that
+// finishes last, with the sums in a.  All partials are non-negative under
+// OpMax.
 template <class OP, int NS>
-__device__ __forceinline__ bool grid_fold(double& a, double& b, double* part, unsigned int* ticket) {
+__device__ __forceinline__ bool grid_fold(double (&a)[NS], double* part, unsigned int* ticket) {
   __shared__ bool last;
-  __shared__ double fin;
+  __shared__ double fin[NS];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  double v = block_fold<OP, NS>(a, b);
+  double v = block_fold<OP, NS>(a);
   if (w < NS && lane == 0) {
     part[(size_t)w * gridDim.x + blockIdx.x] = v;
     __threadfence();
@@ -64,20 +65,33 @@ __device__ __forceinline__ bool grid_fold(double& a, double& b, double* part, un
   __syncthreads();
   if (!last) return false;
   __threadfence();
-  double x = 0.0, y = 0.0;
+  double x[NS];
+#pragma unroll
+  for (int k = 0; k < NS; ++k) x[k] = 0.0;
   for (int i = threadIdx.x; i < (int)gridDim.x; i += RB) {
-    x = OP::f(x, __ldcg(part + i));
-    if (NS > 1) y = OP::f(y, __ldcg(part + gridDim.x + i));
+#pragma unroll
+    for (int k = 0; k < NS; ++k) x[k] = OP::f(x[k], __ldcg(part + (size_t)k * gridDim.x + i));
   }
-  v = block_fold<OP, NS>(x, y);
+  v = block_fold<OP, NS>(x);
   if (NS > 1) {
-    if (w == 1 && lane == 0) fin = v;
+    if (w < NS && lane == 0) fin[w] = v;
     __syncthreads();
   }
   if (threadIdx.x != 0) return false;
-  a = v;
-  b = NS > 1 ? fin : 0.0;
+  a[0] = v;
+#pragma unroll
+  for (int k = 1; k < NS; ++k) a[k] = fin[k];
   *ticket = 0u;
+  return true;
+}
+template <class OP, int NS>
+__device__ __forceinline__ bool grid_fold(double& a, double& b, double* part, unsigned int* ticket) {
+  double v[NS];
+  v[0] = a;
+  if (NS > 1) v[NS - 1] = b;
+  if (!grid_fold<OP, NS>(v, part, ticket)) return false;
+  a = v[0];
+  b = NS > 1 ? v[NS - 1] : 0.0;
   return true;
 }
 

@@ -939,6 +939,8 @@ static fvs_status apply_properties(fvs_solver s, const fvs_props* p) {
   k_cell_materials<<<stride_grid(m->Nc, 256), 256, 0, s->stream>>>(m->Nc, m->zone, mm, s->metal, s->rcp, s->rL);
   FVS_COUNT_LAUNCH();
   s->have_props = true;
+  s->eline.ready = false;   // the chains follow the conductive operator
+  s->eline_dt = 0.0;
   FVS_TRY(solver_set_state(s, nullptr, nullptr, 0));
   return conduction_operator(s);
 }
@@ -1511,13 +1513,13 @@ fvs_status solver_step(fvs_solver s, double dt, fvs_step_stats* stats) {
     J.A = &s->Ke;
     J.dextra = s->edx;
     J.dinv = s->jinv_e;
+    // FVS_ENERGY_LINES: 1 and 0 force the line preconditioner on and off;
+    // otherwise decided per operator and time step from the first pass's
+    // diagonal (LinePrecond::worth)
     const char* el = getenv("FVS_ENERGY_LINES");
-    const bool lines = el && *el == '1';
-    if (lines && (!s->eline.ready || s->eline.built_from != s->Ke.col.p || s->eline.n != s->Ke.n ||
-                  s->eline.w != s->Ke.w))
-      FVS_TRY(s->eline.build(st, s->Ke));
-    s->eline.dextra = s->edx;
-    Precond& PE = lines ? static_cast<Precond&>(s->eline) : static_cast<Precond&>(J);
+    bool lines = el && *el == '1';
+    const bool decide = !(el && (*el == '0' || *el == '1'));
+    if (decide && s->eline_dt == dt) lines = s->eline_use;
     // Tnew / fsnew hold the iterate m; Tlin the linear solution
     DBuf<double>& Tm = s->Tnew;
     DBuf<double>& fsm = s->fsnew;
@@ -1533,9 +1535,24 @@ fvs_status solver_step(fvs_solver s, double dt, fvs_step_stats* stats) {
                                                           s->jinv_e);
       FVS_COUNT_LAUNCH();
       FVS_LAUNCH_CHECK();
+      if (it == 1 && decide && s->eline_dt != dt) {
+        FVS_TRY(LinePrecond::worth(st, s->red, s->Ke, s->edx, lines));
+        s->eline_use = lines;
+        s->eline_dt = dt;
+      }
+      if (it == 1 && lines) {
+        if (!s->eline.ready || s->eline.built_from != s->Ke.col.p || s->eline.n != s->Ke.n || s->eline.w != s->Ke.w)
+          FVS_TRY(s->eline.build(st, s->Ke));
+        s->eline.dextra = s->edx;
+      }
+      Precond& PE = lines ? static_cast<Precond&>(s->eline) : static_cast<Precond&>(J);
       if (lines) FVS_TRY(s->eline.factor(st));
       SolveResult r;
-      FVS_TRY(bicgstab(st, s->red, s->kw, s->Ke, s->edx, PE, s->erhs, s->Tlin, rtol_m,
+      // with the lines an iteration takes off an order of magnitude and what
+      // is left sits in a few cells, where Jacobi's many small steps overshoot
+      // the tolerance evenly: the last passes go a little further
+      const double rtol_in = lines && rtol_m <= s->props.e_rtol ? std::min(rtol_m, std::max(0.1 * rtol_m, 1e-14)) : rtol_m;
+      FVS_TRY(bicgstab(st, s->red, s->kw, s->Ke, s->edx, PE, s->erhs, s->Tlin, rtol_in,
                        s->props.max_krylov_iters, nullptr, r, 0.0, &s->g_e));
       S.e_lin_its += r.iters;
       if (!r.converged) {

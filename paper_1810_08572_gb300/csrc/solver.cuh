@@ -55,9 +55,12 @@ struct fvs_solver_s {
   // inverse Jacobi diagonals of the energy system (per latent-heat pass) and
   // of the momentum system (per step)
   fvs::DBuf<double> jinv_e, jinv_m;
-  // line preconditioner of the energy system (FVS_ENERGY_LINES=1 instead of
-  // Jacobi): chains found once from the energy operator, factors per pass
+  // line preconditioner of the energy system, where it pays (else Jacobi):
+  // chains found once from the energy operator, factors per pass; the choice
+  // holds for one operator and time step
   fvs::LinePrecond eline;
+  bool eline_use = false;
+  double eline_dt = 0.0;      // the dt the choice was made for (0: none yet)
   double time = 0.0;
   int64_t nstep = 0;
 

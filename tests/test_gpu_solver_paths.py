@@ -413,3 +413,34 @@ def test_aggregation_and_smoother_change_only_the_iterations(fvs, monkeypatch, j
     tol = 1e-10 if precision == 0 else 1e-8
     for k in ("T", "U", "P", "FLUX"):
         assert rel(default[k], other[k]) <= tol, k
+
+
+@pytest.mark.parametrize("jitter,shape", [(0.2, (32, 33, 64)), (0.0, (17, 19, 400)), (0.1, (9, 8, 1030))])
+def test_lines_chosen_on_thin_cells_change_only_the_iterations(fvs, monkeypatch, jitter, shape):
+    """From 65,536 cells on, cells thin enough take the line preconditioner by
+    themselves (lines of 64 cells, of 400, and of 1,030 cut at 512, the two
+    ends of their groups ragged): three steps equal the Jacobi solves
+    (FVS_ENERGY_LINES=0) to the solve tolerance, in fewer inner iterations."""
+    m = box_mesh(*shape, (0.1, 0.1, 0.0125), jitter=jitter, jitter_seed=31, permute_seed=32)
+    ijk = m["cell_ijk"]
+    T0 = 940.0 - 40.0 * ijk[:, 0] / shape[0] + 3.0 * np.sin(0.1 * ijk[:, 2])
+    T0[ijk[:, 0] == 0] = 810.0
+    # (the shortest lines: a conduction step long enough to couple them)
+    dt = 5e-3
+    props = cases.props(no_flow=True, **TIGHT)
+
+    def run():
+        M = fvs.Mesh(m)
+        S = fvs.Solver(M, props)
+        S.set_state(T0)
+        its = [S.step(dt)["e_lin_its"] for _ in range(3)]
+        T = S.query("T")
+        S.close()
+        M.close()
+        return T, sum(its)
+
+    T1, lines = run()
+    monkeypatch.setenv("FVS_ENERGY_LINES", "0")
+    T2, jacobi = run()
+    assert rel(T1, T2) <= 1e-10
+    assert lines < 0.6 * jacobi, (lines, jacobi)
