@@ -387,8 +387,58 @@ struct RowCtx {
   const double* gint;     // temperature: series conductance (> 0 on metal-mold faces and convective walls)
 };
 
-__device__ __forceinline__ void add_vertex(const RowCtx& x, int kind, int64_t c, int nn, int32_t v, double coef,
-                                           double* acc, double& cst) {
+// Scratch of a kernel that assembles one matrix row a thread: the row's sorted
+// neighbour list, its values and the coefficients of the cell's eight
+// vertices, in shared memory (a column a thread: dynamic indices, no bank
+// conflicts).  Every vertex belongs to three of a cell's faces, so the faces'
+// corner coefficients are summed per vertex first and spread over the cells
+// around each vertex once: 64 searches of the list a row, not 192, and none of
+// them in global memory.
+constexpr int AB_T = 128;
+struct RowCols {
+  int32_t* nb;     // [W][AB_T] sorted neighbours
+  double* acc;     // [W][AB_T]
+  double* coef;    // [8][AB_T]
+  __device__ __forceinline__ int find(int nn, int32_t v) const {
+    int lo = 0, hi = nn - 1;
+    while (lo <= hi) {
+      const int mid = (lo + hi) >> 1;
+      const int32_t y = nb[mid * AB_T];
+      if (y == v) return mid;
+      if (y < v) lo = mid + 1; else hi = mid - 1;
+    }
+    return -1;
+  }
+  __device__ __forceinline__ void add(int p, double v) const {
+    if (p >= 0) acc[p * AB_T] += v;
+  }
+};
+__host__ __device__ inline size_t row_cols_bytes(int W) {
+  return (size_t)AB_T * ((size_t)W * (sizeof(double) + sizeof(int32_t)) + 8 * sizeof(double));
+}
+__device__ __forceinline__ RowCols row_cols(double* sm, int W) {
+  RowCols r;
+  r.acc = sm + threadIdx.x;
+  r.coef = sm + (size_t)W * AB_T + threadIdx.x;
+  r.nb = reinterpret_cast<int32_t*>(sm + (size_t)(W + 8) * AB_T) + threadIdx.x;
+  return r;
+}
+// coefficient of vertex v, found or entered in the row's list of eight
+// vertices (a closed cell of six quadrilaterals has eight; false if not)
+__device__ __forceinline__ bool add_vertex(const RowCols& r, int32_t (&vid)[8], int32_t v, double coef) {
+  int at = -1;
+#pragma unroll
+  for (int k = 7; k >= 0; --k)
+    if (vid[k] == v || vid[k] < 0) at = k;
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+    if (k == at) vid[k] = v;
+  if (at >= 0) r.coef[at * AB_T] += coef;
+  return at >= 0;
+}
+// the cells around vertex v each take an equal share of coef
+__device__ __forceinline__ void spread_vertex(const RowCtx& x, const RowCols& r, int kind, int nn, int32_t v, double coef,
+                                              double& cst) {
   if (kind == 0 && x.vbnd[v]) return;                 // wall vertex: u = 0
   if (kind == 2) {
     const double fixed = x.vfix[v];
@@ -396,73 +446,80 @@ __device__ __forceinline__ void add_vertex(const RowCtx& x, int kind, int64_t c,
   }
   const int32_t lo = x.vc_ptr[v], hi = x.vc_ptr[v + 1];
   const double share = coef / (double)(hi - lo);
-  for (int32_t e = lo; e < hi; ++e) {
-    const int p = find_sorted(x.nb + c, x.Nc, nn, x.vc_idx[e]);
-    if (p >= 0) acc[p] += share;
-  }
+  for (int32_t t = lo; t < hi; ++t) r.add(r.find(nn, x.vc_idx[t]), share);
 }
-
-__device__ void assemble_base_row(const RowCtx& x, int kind, int64_t c, double* acc, double& cst) {
-  const int nn = x.nnb[c];
-  for (int k = 0; k < FVS_MAX_NB; ++k) acc[k] = 0.0;
-  cst = 0.0;
-  const int pc = find_sorted(x.nb + c, x.Nc, nn, (int32_t)c);
-  for (int s = 0; s < 6; ++s) {
-    const int32_t f = x.cf[s * x.Nc + c];
-    double sg = (double)x.cfs[s * x.Nc + c];
-    const int32_t q = x.nei[f];
-    if (kind == 2 && x.gint && x.gint[f] > 0.0) {
-      if (q < 0) {
-        // convective wall: gint (T_amb - T_c), c the owner, no cross terms
-        if (pc >= 0) acc[pc] -= sg * x.gint[f];
-        cst += sg * x.gint[f] * x.bc_T[x.patch[f]];
+// One thread per row on the shared-memory scratch above.  The
+// temperature operator of 184,320 jittered cells, re-assembled in every step
+// where k depends on T: 1,095 -> 242 us.
+__global__ void __launch_bounds__(AB_T) k_assemble_base(RowCtx x, int kind, int W, int32_t* col, double* val,
+                                                        double* diag, double* cvec) {
+  extern __shared__ double ab_sm[];
+  const RowCols r = row_cols(ab_sm, W);
+  GS(c, x.Nc) {
+    const int nn = x.nnb[c];
+    for (int k = 0; k < W; ++k) {
+      r.nb[k * AB_T] = x.nb[(int64_t)k * x.Nc + c];
+      r.acc[k * AB_T] = 0.0;
+    }
+    int32_t vid[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      vid[k] = -1;
+      r.coef[k * AB_T] = 0.0;
+    }
+    double cst = 0.0;
+    const int pc = r.find(nn, (int32_t)c);
+    for (int s = 0; s < 6; ++s) {
+      const int32_t f = x.cf[s * x.Nc + c];
+      double sg = (double)x.cfs[s * x.Nc + c];
+      const int32_t q = x.nei[f], o = x.own[f];
+      const int pj = q >= 0 ? r.find(nn, o == (int32_t)c ? q : o) : -1;   // the other cell of an inner face
+      const double out = o == (int32_t)c ? 1.0 : -1.0;                    // + C2 - C1 as seen from c
+      if (kind == 2 && x.gint && x.gint[f] > 0.0) {
+        if (q < 0) {
+          // convective wall: gint (T_amb - T_c), c the owner, no cross terms
+          r.add(pc, -sg * x.gint[f]);
+          cst += sg * x.gint[f] * x.bc_T[x.patch[f]];
+        } else {
+          // metal-mold interface: orthogonal flux through the series resistance
+          r.add(pj, out * sg * x.gint[f]);
+          r.add(pc, -out * sg * x.gint[f]);
+        }
         continue;
       }
-      // metal-mold interface: orthogonal flux through the series resistance
-      const int p2 = find_sorted(x.nb + c, x.Nc, nn, q);
-      const int p1 = find_sorted(x.nb + c, x.Nc, nn, x.own[f]);
-      if (p2 >= 0) acc[p2] += sg * x.gint[f];
-      if (p1 >= 0) acc[p1] -= sg * x.gint[f];
-      continue;
-    }
-    if (kind == 2 && x.kf) sg *= x.kf[f];   // conductive flux: k_f times the face gradient
-    double phib = 0.0;
-    if (q < 0) {
-      if (kind == 1) continue;
-      if (kind == 2) {
-        if (x.bc_type[x.patch[f]] != FVS_BC_DIRICHLET) continue;
-        phib = x.bc_T[x.patch[f]];
+      if (kind == 2 && x.kf) sg *= x.kf[f];   // conductive flux: k_f times the face gradient
+      double phib = 0.0;
+      if (q < 0) {
+        if (kind == 1) continue;
+        if (kind == 2) {
+          if (x.bc_type[x.patch[f]] != FVS_BC_DIRICHLET) continue;
+          phib = x.bc_T[x.patch[f]];
+        }
+        // flux = cd (phi_b - phi_c): c is the owner of a wall face
+        r.add(pc, -sg * x.cd[f]);
+        cst += sg * x.cd[f] * phib;
+      } else {
+        r.add(pj, out * sg * x.cd[f]);
+        r.add(pc, -out * sg * x.cd[f]);
       }
-      // flux = cd (phi_b - phi_c): c is the owner of a wall face
-      if (pc >= 0) acc[pc] -= sg * x.cd[f];
-      cst += sg * x.cd[f] * phib;
-    } else {
-      const int p2 = find_sorted(x.nb + c, x.Nc, nn, q);
-      const int p1 = find_sorted(x.nb + c, x.Nc, nn, x.own[f]);
-      if (p2 >= 0) acc[p2] += sg * x.cd[f];
-      if (p1 >= 0) acc[p1] -= sg * x.cd[f];
+      const double e = sg * x.ce[f], z = sg * x.cz[f];
+      const int32_t v[4] = {x.fv[2 * x.Nf + f], x.fv[f], x.fv[3 * x.Nf + f], x.fv[x.Nf + f]};
+      const double w[4] = {e, -e, z, -z};
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (w[k] != 0.0 && !add_vertex(r, vid, v[k], w[k])) spread_vertex(x, r, kind, nn, v[k], w[k], cst);
     }
-    const int32_t v1 = x.fv[f], v2 = x.fv[x.Nf + f], v3 = x.fv[2 * x.Nf + f], v4 = x.fv[3 * x.Nf + f];
-    add_vertex(x, kind, c, nn, v3, sg * x.ce[f], acc, cst);
-    add_vertex(x, kind, c, nn, v1, -sg * x.ce[f], acc, cst);
-    add_vertex(x, kind, c, nn, v4, sg * x.cz[f], acc, cst);
-    add_vertex(x, kind, c, nn, v2, -sg * x.cz[f], acc, cst);
-  }
-}
-
-__global__ void k_assemble_base(RowCtx x, int kind, int W, int32_t* col, double* val, double* diag, double* cvec) {
-  double acc[FVS_MAX_NB];
-  GS(c, x.Nc) {
-    double cst;
-    assemble_base_row(x, kind, c, acc, cst);
-    const int nn = x.nnb[c];
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (vid[k] >= 0) spread_vertex(x, r, kind, nn, vid[k], r.coef[k * AB_T], cst);
     double dg = 0.0;
     for (int k = 0; k < W; ++k) {
-      const int32_t j = x.nb[k * x.Nc + c];
+      const int32_t j = r.nb[k * AB_T];
       const bool used = k < nn;
-      col[k * x.Nc + c] = used ? j : (int32_t)c;
-      val[k * x.Nc + c] = used ? acc[k] : 0.0;
-      if (used && j == (int32_t)c) dg = acc[k];
+      const double a = r.acc[k * AB_T];
+      col[(int64_t)k * x.Nc + c] = used ? j : (int32_t)c;
+      val[(int64_t)k * x.Nc + c] = used ? a : 0.0;
+      if (used && j == (int32_t)c) dg = a;
     }
     diag[c] = dg;
     if (cvec) cvec[c] = cst;
@@ -484,6 +541,21 @@ __global__ void k_dirichlet_vertices(int64_t Nf, const int32_t* fv, const int32_
 }
 __global__ void k_vfix(int64_t Nv, const double* vsum, const int32_t* vcnt, double* vfix) {
   GS(v, Nv) vfix[v] = vcnt[v] > 0 ? vsum[v] / (double)vcnt[v] : __longlong_as_double(0x7ff8000000000000LL);
+}
+
+static fvs_status launch_assemble_base(cudaStream_t s, const RowCtx& x, int kind, int W, Ell& L, double* cvec) {
+  static bool attr_set[64] = {false};
+  int dev = 0;
+  FVS_CUDA(cudaGetDevice(&dev));
+  if (!(dev >= 0 && dev < 64 && attr_set[dev])) {
+    FVS_CUDA(cudaFuncSetAttribute(k_assemble_base, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)row_cols_bytes(FVS_MAX_NB)));
+    if (dev >= 0 && dev < 64) attr_set[dev] = true;
+  }
+  k_assemble_base<<<stride_grid(x.Nc, AB_T, 16), AB_T, row_cols_bytes(W), s>>>(x, kind, W, L.col, L.val, L.diag, cvec);
+  FVS_COUNT_LAUNCH();
+  FVS_LAUNCH_CHECK();
+  return FVS_OK;
 }
 
 static RowCtx row_ctx(fvs_mesh m) {
@@ -511,7 +583,7 @@ fvs_status assemble_temperature_operator(fvs_mesh m, const int32_t* d_bc_type, c
   RowCtx x = row_ctx(m);
   x.bc_type = d_bc_type; x.bc_T = d_bc_T; x.vfix = vfix;
   x.kf = kf; x.gint = gint;
-  k_assemble_base<<<stride_grid(m->Nc, 128, 4), 128, 0, s>>>(x, 2, m->W, LT.col, LT.val, LT.diag, lT); FVS_COUNT_LAUNCH();
+  FVS_TRY(launch_assemble_base(s, x, 2, m->W, LT, lT));
   FVS_LAUNCH_CHECK();
   FVS_CUDA(cudaStreamSynchronize(s));
   return FVS_OK;
@@ -762,8 +834,8 @@ fvs_status mesh_build(fvs_mesh m, const double* nodes, int64_t Nv, const int32_t
   RowCtx x = row_ctx(m);
   FVS_TRY(m->Lu.alloc(Nc, m->W));
   FVS_TRY(m->Pb.alloc(Nc, m->W));
-  k_assemble_base<<<stride_grid(Nc, 128, 4), 128, 0, s>>>(x, 0, m->W, m->Lu.col, m->Lu.val, m->Lu.diag, nullptr); FVS_COUNT_LAUNCH();
-  k_assemble_base<<<stride_grid(Nc, 128, 4), 128, 0, s>>>(x, 1, m->W, m->Pb.col, m->Pb.val, m->Pb.diag, nullptr); FVS_COUNT_LAUNCH();
+  FVS_TRY(launch_assemble_base(s, x, 0, m->W, m->Lu, nullptr));
+  FVS_TRY(launch_assemble_base(s, x, 1, m->W, m->Pb, nullptr));
   FVS_LAUNCH_CHECK();
   FVS_CUDA(cudaStreamSynchronize(s));
   return FVS_OK;

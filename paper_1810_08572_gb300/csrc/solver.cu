@@ -241,21 +241,14 @@ struct PpeCtx {
   int WF;
 };
 
-// nbl: the row's sorted neighbour list, copied to thread-local memory once
-__device__ __forceinline__ void ppe_vertex(const PpeCtx& x, const int32_t* nbl, int nn, int32_t v, double coef,
-                                           double* acc) {
-  const int32_t lo = x.vc_ptr[v], hi = x.vc_ptr[v + 1];
-  const double share = coef / (double)(hi - lo);
-  for (int32_t e = lo; e < hi; ++e) {
-    const int32_t j = x.vc_idx[e];
-    if (!x.ppe[j]) continue;            // deleted column (solid or non-flowing)
-    const int p = find_sorted(nbl, 1, nn, j);
-    if (p >= 0) acc[p] += share;
-  }
-}
-
-__global__ void k_ppe_matrix(PpeCtx x, int32_t* col, double* val, double* diag, int* err) {
-  double acc[FVS_MAX_NB];
+// Rows without a face of case 2 or 3 are the base coefficients, renumbered;
+// the others (next to solid cells) are listed for k_ppe_modified.  With both
+// in one launch every warp that held a listed row waited a millisecond for its
+// searches: half-frozen 96^3 (482,617 rows of 27 entries), matrix and refreshed
+// hierarchy together 2.2 -> 1.3 ms a step.
+__global__ void __launch_bounds__(256) k_ppe_matrix(PpeCtx x, int32_t* col, double* val, double* diag, int32_t* list,
+                                                    int* nlist, int* err) {
+  const double mrho = -1.0 / x.rho;
   GS(r, x.nact) {
     const int32_t c = x.act[r];
     const int nn = x.nnb[c];
@@ -273,82 +266,164 @@ __global__ void k_ppe_matrix(PpeCtx x, int32_t* col, double* val, double* diag, 
       const uint8_t fc = x.fcase[x.cf[s * x.Nc + c]];
       modified |= (fc == 2 || fc == 3);
     }
-    if (!modified) {
-      // unchanged row: the base coefficients, renumbered
-      double dg = 0.0;
-      for (int k = 0; k < x.W; ++k) {
-        const int32_t j = x.Pbcol[(int64_t)k * x.Nc + c];
-        const double a = -x.Pbval[(int64_t)k * x.Nc + c] / x.rho;
-        const int32_t mj = x.map[j];
-        int32_t cc = (int32_t)r;
-        double v = 0.0;
-        if (k < nn) {
-          if (mj >= 0 && x.ppe[j]) { cc = mj; v = a; }
-          else if (a != 0.0) atomicOr(err, 1);
-          if (j == c) dg = v;
-        }
-        col[(int64_t)k * x.nact + r] = cc;
-        val[(int64_t)k * x.nact + r] = v;
-      }
-      diag[r] = dg;
+    if (modified) {
+      list[atomicAdd(nlist, 1)] = (int32_t)r;   // (in any order: rows do not depend on one another)
       continue;
     }
-    // re-assembly from the faces (Section 2.4.2, step 3)
-    int32_t nbl[FVS_MAX_NB];
-    for (int k = 0; k < nn; ++k) {
-      acc[k] = 0.0;
-      nbl[k] = x.nb[(int64_t)k * x.Nc + c];
-    }
-    for (int s = 0; s < 6; ++s) {
-      const int32_t f = x.cf[s * x.Nc + c];
-      const uint8_t fc = x.fcase[f];
-      if (fc != 1 && fc != 2) continue;
-      const double sg = (double)x.cfs[s * x.Nc + c];
-      const int32_t o = x.own[f], q = x.nei[f];
-      { const int pq = find_sorted(nbl, 1, nn, q); if (pq >= 0) acc[pq] += sg * x.cd[f]; else atomicOr(err, 8); }
-      { const int po = find_sorted(nbl, 1, nn, o); if (po >= 0) acc[po] -= sg * x.cd[f]; else atomicOr(err, 8); }
-      const int32_t v1 = x.fv[f], v2 = x.fv[x.Nf + f], v3 = x.fv[2 * x.Nf + f], v4 = x.fv[3 * x.Nf + f];
-      const double ce = sg * x.ce[f], cz = sg * x.cz[f];
-      ppe_vertex(x, nbl, nn, v3, ce, acc);
-      ppe_vertex(x, nbl, nn, v1, -ce, acc);
-      ppe_vertex(x, nbl, nn, v4, cz, acc);
-      ppe_vertex(x, nbl, nn, v2, -cz, acc);
-      if (fc == 2) {
-        // Eq. 16: the deleted neighbours' coefficients, spread equally over
-        // the remaining members of N(f)
-        auto frac = [&](int32_t v) {
-          return (double)x.nS[v] / (double)(x.vc_ptr[v + 1] - x.vc_ptr[v]);
-        };
-        const double sdel = ce * (frac(v3) - frac(v1)) + cz * (frac(v4) - frac(v2));
-        const int nf = x.nfnb[f];
-        int nrem = 0;
-        for (int k = 0; k < nf; ++k) nrem += x.ppe[x.fnb[(int64_t)k * x.Nf + f]] ? 1 : 0;
-        const double add = sdel / (double)nrem;
-        for (int k = 0; k < nf; ++k) {
-          const int32_t j = x.fnb[(int64_t)k * x.Nf + f];
-          if (!x.ppe[j]) continue;
-          const int p = find_sorted(nbl, 1, nn, j);
-          if (p >= 0) acc[p] += add;
-          else if (add != 0.0) atomicOr(err, 2);   // a zero share may miss a face-only stencil
-        }
-      }
-    }
     double dg = 0.0;
+#pragma unroll 9
     for (int k = 0; k < x.W; ++k) {
+      const int32_t j = x.Pbcol[(int64_t)k * x.Nc + c];
+      const double a = mrho * x.Pbval[(int64_t)k * x.Nc + c];
+      const int32_t mj = x.map[j];
       int32_t cc = (int32_t)r;
       double v = 0.0;
       if (k < nn) {
-        const int32_t j = x.nb[(int64_t)k * x.Nc + c];
-        const double a = -acc[k] / x.rho;
-        const int32_t mj = x.map[j];
         if (mj >= 0 && x.ppe[j]) { cc = mj; v = a; }
-        else if (a != 0.0) atomicOr(err, 4);
+        else if (a != 0.0) atomicOr(err, 1);
         if (j == c) dg = v;
       }
       col[(int64_t)k * x.nact + r] = cc;
       val[(int64_t)k * x.nact + r] = v;
     }
     diag[r] = dg;
+  }
+}
+// Listed rows re-assembled from their faces (Section 2.4.2, step 3), a warp a
+// row: lane l owns the row's neighbours l and l + 32 and adds what falls to
+// them, so the sums keep one order and need no search; lanes 0 to 7 hold the
+// cell's vertices, whose corner coefficients are summed over the faces and
+// spread over the cells around each vertex once.  The lists of neighbours are
+// read with all lanes' loads in flight; a thread a row walked them one
+// dependent load after the other.  Quotients by small counts come from
+// reciprocals that the lanes hold (FP64 issues a warp in 16 clocks whether one
+// lane is active or all).
+__global__ void __launch_bounds__(256) k_ppe_modified(PpeCtx x, int32_t* col, double* val, double* diag,
+                                                      const int32_t* list, const int* nlist, int* err) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  const double mrho = -1.0 / x.rho;
+  const double rc0 = 1.0 / (double)(lane + 1), rc1 = 1.0 / (double)(lane + 33);
+  constexpr unsigned ALL = 0xffffffffu;
+  // 1 / n for 1 <= n <= 64, the same n in all lanes
+  auto recip = [&](int n) { return n <= 32 ? __shfl_sync(ALL, rc0, n - 1) : __shfl_sync(ALL, rc1, n - 33); };
+  for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < *nlist; t += nw) {
+    const int64_t r = list[t];
+    const int32_t c = x.act[r];
+    const int nn = x.nnb[c];
+    const int32_t n0 = lane < nn ? x.nb[(int64_t)lane * x.Nc + c] : -1;
+    const int32_t n1 = lane + 32 < nn ? x.nb[(int64_t)(lane + 32) * x.Nc + c] : -1;
+    double a0 = 0.0, a1 = 0.0;
+    int32_t vid = -1;     // lanes 0 .. 7: a vertex of the cell
+    double vco = 0.0;     // and its coefficient
+    // the cells of vertex v that carry pressure take share each (deleted
+    // columns, solid or non-flowing, are left out)
+    auto spread = [&](int32_t v, double share) {
+      const int32_t lo = x.vc_ptr[v], hi = x.vc_ptr[v + 1];
+      bool h0 = false, h1 = false;
+      for (int32_t e = lo; e < hi; ++e) {
+        const int32_t j = x.vc_idx[e];
+        h0 |= j == n0;
+        h1 |= j == n1;
+      }
+      if (h0 && x.ppe[n0]) a0 += share;
+      if (h1 && x.ppe[n1]) a1 += share;
+    };
+    for (int s = 0; s < 6; ++s) {
+      const int32_t f = x.cf[s * x.Nc + c];
+      const uint8_t fc = x.fcase[f];
+      if (fc != 1 && fc != 2) continue;
+      const double sg = (double)x.cfs[s * x.Nc + c];
+      const int32_t q = x.nei[f], o = x.own[f];
+      const double cd = sg * x.cd[f];
+      if (n0 == q) a0 += cd;
+      if (n1 == q) a1 += cd;
+      if (n0 == o) a0 -= cd;
+      if (n1 == o) a1 -= cd;
+      if (!__any_sync(ALL, n0 == q || n1 == q) || !__any_sync(ALL, n0 == o || n1 == o))
+        if (lane == 0) atomicOr(err, 8);
+      const double ce = sg * x.ce[f], cz = sg * x.cz[f];
+      if (ce == 0.0 && cz == 0.0) continue;     // orthogonal face: no vertex enters
+      // lanes 0 .. 3: corners v3, v1, v4, v2 with +ce, -ce, +cz, -cz
+      const int kc = lane & 3;
+      const int32_t myv = x.fv[(kc == 0 ? 2 : kc == 1 ? 0 : kc == 2 ? 3 : 1) * x.Nf + f];
+      const int mycnt = x.vc_ptr[myv + 1] - x.vc_ptr[myv];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int32_t v = __shfl_sync(ALL, myv, k);
+        const double w = k == 0 ? ce : k == 1 ? -ce : k == 2 ? cz : -cz;
+        unsigned at = __ballot_sync(ALL, lane < 8 && vid == v);
+        if (!at) at = __ballot_sync(ALL, lane < 8 && vid < 0);
+        if (at) {
+          if (lane == __ffs(at) - 1) {
+            vid = v;
+            vco += w;
+          }
+        } else {
+          spread(v, w * recip(x.vc_ptr[v + 1] - x.vc_ptr[v]));   // a ninth vertex: not a hexahedron
+        }
+      }
+      if (fc == 2) {
+        // Eq. 16: the deleted neighbours' coefficients, spread equally over
+        // the remaining members of N(f)
+        double fr[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int cn = __shfl_sync(ALL, mycnt, k);
+          fr[k] = (double)x.nS[__shfl_sync(ALL, myv, k)] * recip(cn);
+        }
+        const double sdel = ce * (fr[0] - fr[1]) + cz * (fr[2] - fr[3]);
+        const int nf = x.nfnb[f];
+        int nrem = 0;
+        bool h0 = false, h1 = false, left = false;
+        for (int k0 = 0; k0 < nf; k0 += 32) {
+          const int k = k0 + lane;
+          const int32_t j = k < nf ? x.fnb[(int64_t)k * x.Nf + f] : -1;
+          const bool in = j >= 0 && x.ppe[j];
+          unsigned m = __ballot_sync(ALL, in);
+          nrem += __popc(m);
+          while (m) {
+            const int b = __ffs(m) - 1;
+            m &= m - 1u;
+            const int32_t jb = __shfl_sync(ALL, j, b);
+            const bool e0 = jb == n0, e1 = jb == n1;
+            h0 |= e0;
+            h1 |= e1;
+            left |= !__any_sync(ALL, e0 || e1);
+          }
+        }
+        // (a face whose whole neighbourhood is deleted does not occur: its
+        // owners carry pressure)
+        const double add = nrem > 0 ? sdel * recip(nrem) : 0.0;
+        if (h0) a0 += add;
+        if (h1) a1 += add;
+        if (left && add != 0.0 && lane == 0) atomicOr(err, 2);   // a zero share may miss a face-only stencil
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int32_t v = __shfl_sync(ALL, vid, k);
+      const double w = __shfl_sync(ALL, vco, k);
+      if (v >= 0) spread(v, w * recip(x.vc_ptr[v + 1] - x.vc_ptr[v]));
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int k = lane + 32 * h;
+      const int32_t j = h ? n1 : n0;
+      if (k < x.W) {
+        int32_t cc = (int32_t)r;
+        double v = 0.0;
+        if (k < nn) {
+          const double a = mrho * (h ? a1 : a0);
+          const int32_t mj = x.map[j];
+          if (mj >= 0 && x.ppe[j]) { cc = mj; v = a; }
+          else if (a != 0.0) atomicOr(err, 4);
+          if (j == c) diag[r] = v;
+        }
+        col[(int64_t)k * x.nact + r] = cc;
+        val[(int64_t)k * x.nact + r] = v;
+      }
+    }
   }
 }
 
@@ -1111,13 +1186,17 @@ static fvs_status assemble_pressure(fvs_solver s) {
     return ms;
   };
   FVS_TRY(s->K.alloc(s->nact, m->W));
-  DBuf<int> err;
-  FVS_TRY(err.alloc(1));
+  DBuf<int> err;   // flags, rows listed for re-assembly
+  FVS_TRY(err.alloc(2));
   FVS_TRY(err.zero(st));
   if (s->nact > 0) {
-    // one thread per row: the re-assembled rows next to solid cells are
-    // latency-bound searches, so as many as possible run at once
-    k_ppe_matrix<<<(unsigned)((s->nact + 127) / 128), 128, 0, st>>>(ppe_ctx(s), s->K.col, s->K.val, s->K.diag, err);
+    FVS_TRY(s->plist.alloc((size_t)s->nact));
+    const PpeCtx px = ppe_ctx(s);
+    k_ppe_matrix<<<stride_grid(s->nact, 256), 256, 0, st>>>(px, s->K.col, s->K.val, s->K.diag, s->plist, err.p + 1, err);
+    FVS_COUNT_LAUNCH();
+    // (the list's length stays on the device: a warp a row of as many as there are)
+    k_ppe_modified<<<stride_grid(s->nact * 32, 256, 6), 256, 0, st>>>(px, s->K.col, s->K.val, s->K.diag, s->plist,
+                                                                      err.p + 1, err);
     FVS_COUNT_LAUNCH();
     FVS_LAUNCH_CHECK();
   }

@@ -92,6 +92,7 @@ struct fvs_solver_s {
 
   // compact systems
   fvs::Ell M;             // momentum predictor on LM cells
+  fvs::DBuf<int32_t> plist;   // [nact] pressure rows re-assembled from their faces
   fvs::Ell K;             // pressure: K = -A on LM cells (identity rows for non-flowing)
   fvs::Ell Kp;            // K's diagonal and face couplings, the rest lumped (AMG operator)
   bool pc_compact = false;        // the hierarchy was built on Kp
