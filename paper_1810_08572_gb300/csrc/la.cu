@@ -98,7 +98,7 @@ fvs_status Reducer::init() {
   FVS_TRY(sc.zero(st));
   FVS_TRY(ticket.alloc(1));
   FVS_TRY(ticket.zero(st));
-  FVS_TRY(iter.alloc(2));
+  FVS_TRY(iter.alloc(3));
   FVS_TRY(iter.zero(st));
   if (!host) FVS_CUDA(cudaMallocHost(&host, S_NSLOT * sizeof(double)));
   return FVS_OK;
@@ -224,7 +224,7 @@ __device__ __forceinline__ bool finish2(double x, double y, double* part, unsign
     sc[S_RR] = sc[S_RHO] = x;
     sc[S_BB] = y;
   } else if (MODE == FIN_TRUE) {
-    sc[S_RR] = x;
+    sc[S_TRUE] = x;
   }
   return true;
 }
@@ -294,7 +294,8 @@ __global__ void __launch_bounds__(RB, W > 0 ? 6 : 8) k_residual_dot(int64_t n, i
                                                         const double* __restrict__ dextra,
                                                         const double* __restrict__ b, double* __restrict__ r,
                                                         double* __restrict__ rh, double* part,
-                                                        unsigned int* ticket, double* sc) {
+                                                        unsigned int* ticket, double* sc, const int* go) {
+  if (MODE == FIN_TRUE && go && !*go) return;   // no loop was entered: the start's residual stands
   double rr = 0.0, bb = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)RB + threadIdx.x; i < n; i += (int64_t)gridDim.x * RB) {
     const double acc = ell_row<W, CS>(n, w, col, val, x, i, DX ? dextra[i] * x[i] : 0.0);
@@ -425,8 +426,6 @@ __global__ void k_cg_p(int64_t n, const double* __restrict__ sc, const double* _
 
 constexpr int MAX_RESTARTS = 3;   // from the true residual, once the recursive one has met the tolerance
 
-static inline bool bad(double v) { return !(v == v) || v > 1e300 || v < -1e300; }
-
 template <int MODE, bool DX>
 static void launch_spmv_dot(cudaStream_t s, Reducer& red, const Ell& A, const double* x, double* y,
                             const double* dextra, const double* d) {
@@ -445,16 +444,16 @@ static fvs_status spmv_dot(cudaStream_t s, Reducer& red, const Ell& A, const dou
 
 template <int MODE, bool DX>
 static void launch_residual_dot(cudaStream_t s, Reducer& red, const Ell& A, const double* x, const double* dextra,
-                                const double* b, double* r, double* rh) {
+                                const double* b, double* r, double* rh, const int* go) {
   FVS_BY_ROW(A, (k_residual_dot<MODE, DX, W, CS><<<red.grid(A.n), RB, 0, s>>>(A.n, A.w, A.col, A.val, x, dextra, b, r,
-                                                                              rh, red.part, red.ticket, red.sc)));
+                                                                              rh, red.part, red.ticket, red.sc, go)));
 }
 template <int MODE>
 static fvs_status residual_dot(cudaStream_t s, Reducer& red, const Ell& A, const double* x, const double* dextra,
-                               const double* b, double* r, double* rh) {
+                               const double* b, double* r, double* rh, const int* go = nullptr) {
   ProfScope ps(&A, "residual", (double)A.n * (12.0 * A.w + (MODE == FIN_START ? 32.0 : 16.0) + (dextra ? 8.0 : 0.0)), s);
-  if (dextra) launch_residual_dot<MODE, true>(s, red, A, x, dextra, b, r, rh);
-  else launch_residual_dot<MODE, false>(s, red, A, x, dextra, b, r, rh);
+  if (dextra) launch_residual_dot<MODE, true>(s, red, A, x, dextra, b, r, rh, go);
+  else launch_residual_dot<MODE, false>(s, red, A, x, dextra, b, r, rh, go);
   FVS_LAUNCH_CHECK();
   return FVS_OK;
 }
@@ -531,21 +530,40 @@ static fvs_status run_body(cudaStream_t s, IterGraph* g, uint64_t key, bool firs
   return FVS_OK;
 }
 
-// (the bound lies beside the counter: a loop captured once serves every bound)
-__global__ void k_loop_init(double* sc, int* it, int maxit, double tol2, int fresh) {
+__host__ __device__ __forceinline__ bool bad(double v) { return !(v == v) || v > 1e300 || v < -1e300; }
+
+// what a residual is measured against
+__host__ __device__ __forceinline__ double residual_scale(double bb, double floor) {
+  const double b = fmax(sqrt(bb), floor);
+  return b == 0.0 ? 1.0 : b;
+}
+
+// The loop's bound and tolerance lie in memory, so that a loop captured once
+// serves every solve.  At the start of a solve the loop is entered only if
+// the residual just formed is finite and above the tolerance.
+__global__ void k_loop_init(double* sc, int* it, int maxit, double rtol, double floor, int fresh, int start) {
+  const double bn = residual_scale(sc[S_BB], floor);
   sc[S_FIRST] = fresh ? 1.0 : 0.0;
   it[0] = 0;
   it[1] = maxit;
   sc[S_ITER] = 0.0;
-  sc[S_TOL2] = tol2;
+  sc[S_TOL2] = (rtol * bn) * (rtol * bn);
+  int go = 1;
+  if (start) {
+    const double rn = sqrt(sc[S_RR]);
+    sc[S_START] = sc[S_RR];
+    go = !(bad(rn) || bad(bn) || rn / bn <= rtol);
+  }
+  it[2] = go;
 }
+__global__ void k_loop_gate(cudaGraphConditionalHandle h, const int* it) { cudaGraphSetConditional(h, it[2] ? 1u : 0u); }
 
 // Runs up to maxit iterations of body() as one graph launch with a
 // conditional while-node; returns false (nothing launched) when the loop
 // graph cannot be used, so the caller iterates from the host instead.
 template <typename F>
-static bool run_loop(cudaStream_t s, IterGraph* g, uint64_t key, Reducer& red, double tol2, int maxit, bool fresh,
-                     F& body, fvs_status& st) {
+static bool run_loop(cudaStream_t s, IterGraph* g, uint64_t key, Reducer& red, double rtol, double floor, int maxit,
+                     bool fresh, bool start, F& body, fvs_status& st) {
   st = FVS_OK;
   if (!g || g->loop_disabled || !graphs_enabled() || s == nullptr || maxit <= 0) return false;
   if (!g->loop || g->loop_key != key) {
@@ -556,13 +574,23 @@ static bool run_loop(cudaStream_t s, IterGraph* g, uint64_t key, Reducer& red, d
     bool ok = cudaGraphCreate(&graph, 0) == cudaSuccess;
     ok = ok && cudaGraphConditionalHandleCreate(&h, graph, 1, cudaGraphCondAssignDefault) == cudaSuccess;
     cudaGraphNodeParams p = {};
-    cudaGraphNode_t node;
+    cudaGraphNode_t node, gate;
+    if (ok) {
+      const int* itp = red.iter.p;
+      void* args[] = {&h, &itp};
+      cudaKernelNodeParams kp = {};
+      kp.func = (void*)k_loop_gate;
+      kp.gridDim = dim3(1);
+      kp.blockDim = dim3(1);
+      kp.kernelParams = args;
+      ok = cudaGraphAddKernelNode(&gate, graph, nullptr, 0, &kp) == cudaSuccess;
+    }
     if (ok) {
       p.type = cudaGraphNodeTypeConditional;
       p.conditional.handle = h;
       p.conditional.type = cudaGraphCondTypeWhile;
       p.conditional.size = 1;
-      ok = cudaGraphAddNode(&node, graph, nullptr, nullptr, 0, &p) == cudaSuccess;
+      ok = cudaGraphAddNode(&node, graph, &gate, nullptr, 1, &p) == cudaSuccess;
     }
     if (ok) {
       cudaGraph_t bodyg = p.conditional.phGraph_out[0];
@@ -592,8 +620,9 @@ static bool run_loop(cudaStream_t s, IterGraph* g, uint64_t key, Reducer& red, d
     }
     g->loop_key = key;
   }
-  k_loop_init<<<1, 1, 0, s>>>(red.sc.p, red.iter.p, maxit, tol2, fresh ? 1 : 0);
+  k_loop_init<<<1, 1, 0, s>>>(red.sc.p, red.iter.p, maxit, rtol, floor, fresh ? 1 : 0, start ? 1 : 0);
   FVS_COUNT_LAUNCH();
+  FVS_COUNT_LAUNCH();   // the gate
   const cudaError_t e = cudaGraphLaunch(g->loop, s);
   if (e != cudaSuccess) {
     set_error("cudaGraphLaunch: %s", cudaGetErrorString(e));
@@ -604,7 +633,8 @@ static bool run_loop(cudaStream_t s, IterGraph* g, uint64_t key, Reducer& red, d
 
 fvs_status bicgstab(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, const double* dextra,
                     Precond& M, const double* b, double* x, double rtol, int maxit, Projector* proj,
-                    SolveResult& res, double bnorm_floor, IterGraph* graph) {
+                    SolveResult& res, double bnorm_floor, IterGraph* graph,
+                    const std::function<fvs_status()>* tail) {
   const int64_t n = A.n;
   res = SolveResult();
   if (n == 0) {
@@ -625,16 +655,6 @@ fvs_status bicgstab(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, c
     FVS_TRY(red.dot2(s, n, w.q, w.q, w.r, w.r, S_BB, S_RR));
     FVS_TRY(red.dot(s, n, w.rh, w.r, S_RHO));
   }
-  FVS_TRY(red.fetch(s));
-  double bnorm = fmax(sqrt(red.host[S_BB]), bnorm_floor);
-  if (bnorm == 0.0) bnorm = 1.0;
-  double rn = sqrt(red.host[S_RR]);
-  res.relres = rn / bnorm;
-  if (bad(rn) || bad(bnorm)) return FVS_OK;   // non-finite data: not converged, no iterations
-  if (res.relres <= rtol) {
-    res.converged = true;
-    return FVS_OK;
-  }
   // K x has zero sum on every singular part (zero column sums), so the
   // Krylov vectors stay in the range once r is projected
   const FirstSweep fp = M.first(w.ph), fs = M.first(w.sh);
@@ -651,23 +671,50 @@ fvs_status bicgstab(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, c
     return FVS_OK;
   };
   const uint64_t key = graph_key(A, dextra, M, b, x, w, red) ^ 0x6b696367ULL;
-  // the first iteration of a recurrence runs from the host; the following
-  // ones run as one device-driven loop (or one graph replay per iteration)
-  bool fresh = true;
-  int it = 0;
+  // r.r of the true residual (projected: formed in q, so that r stays)
+  auto true_residual = [&](const int* go) -> fvs_status {
+    if (!proj) return residual_dot<FIN_TRUE>(s, red, A, x, dextra, b, nullptr, nullptr, go);
+    FVS_TRY(residual(s, A, x, b, w.q, dextra));
+    FVS_TRY(proj->apply(s, w.q));
+    return red.dot(s, n, w.q, w.q, S_TRUE);
+  };
+  // what follows the loop on the device; true: its scalars are of this x
+  auto queue_loop = [&](int left, bool fresh, bool start, bool& looped) -> fvs_status {
+    fvs_status st = FVS_OK;
+    looped = run_loop(s, graph, key, red, rtol, bnorm_floor, left, fresh, start, body, st);
+    FVS_TRY(st);
+    if (!looped) return FVS_OK;
+    FVS_TRY(true_residual(red.iter.p + 2));
+    if (tail) FVS_TRY((*tail)());
+    return FVS_OK;
+  };
+  // the iterations run as one device-driven loop, or the first of a
+  // recurrence from the host and one graph replay each after that
+  bool looped = false;
+  FVS_TRY(queue_loop(maxit, true, true, looped));
+  FVS_TRY(red.fetch(s));
+  const double bnorm = residual_scale(red.host[S_BB], bnorm_floor);
+  double rn = sqrt(red.host[looped ? S_START : S_RR]);
+  res.relres = rn / bnorm;
+  res.tail_done = looped && tail;
+  if (bad(rn) || bad(bnorm)) return FVS_OK;   // non-finite data: not converged, no iterations
+  if (res.relres <= rtol) {
+    res.converged = true;
+    return FVS_OK;
+  }
   const double tol2 = (rtol * bnorm) * (rtol * bnorm);
+  bool queued = looped, fresh = true;
+  int it = 0;
   double best = 0.0;   // true residual before a restart (its iterate in w.z)
   for (int again = 0;; ++again) {
     while (it < maxit) {
-      bool looped = false;
-      {
-        fvs_status st = FVS_OK;
-        looped = run_loop(s, graph, key, red, tol2, maxit - it, fresh, body, st);
-        FVS_TRY(st);
+      if (!queued) {
+        FVS_TRY(queue_loop(maxit - it, fresh, false, looped));
+        if (!looped) FVS_TRY(run_body(s, graph, key, fresh, body));
+        FVS_TRY(red.fetch(s));
       }
-      if (!looped) FVS_TRY(run_body(s, graph, key, fresh, body));
-      fresh = false;
-      FVS_TRY(red.fetch(s));
+      queued = fresh = false;
+      res.tail_done = looped && tail;
       const int done = looped ? (int)red.host[S_ITER] : 1;
       if (looped) __atomic_add_fetch(&g_launches, graph->loop_kernels * (unsigned long long)done, __ATOMIC_RELAXED);
       it += done;
@@ -678,10 +725,11 @@ fvs_status bicgstab(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, c
         if (again > 0) {
           FVS_TRY(vcopy(s, n, w.z, x));
           res.relres = best;
+          res.tail_done = false;
         }
         return FVS_OK;
       }
-      if (res.relres <= rtol) {
+      if (res.relres <= rtol || red.host[S_RR] <= tol2) {
         res.converged = true;
         break;
       }
@@ -694,16 +742,12 @@ fvs_status bicgstab(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, c
         fresh = true;
       }
     }
-    // recompute the true residual (the recursive one drifts)
-    if (!proj) {
-      FVS_TRY(residual_dot<FIN_TRUE>(s, red, A, x, dextra, b, nullptr, nullptr));
-    } else {
-      FVS_TRY(residual(s, A, x, b, w.r, dextra));
-      FVS_TRY(proj->apply(s, w.r));
-      FVS_TRY(red.dot(s, n, w.r, w.r, S_RR));
+    // the true residual (the recursive one drifts)
+    if (!looped) {
+      FVS_TRY(true_residual(nullptr));
+      FVS_TRY(red.fetch(s));
     }
-    FVS_TRY(red.fetch(s));
-    res.relres = sqrt(red.host[S_RR]) / bnorm;
+    res.relres = sqrt(red.host[S_TRUE]) / bnorm;
     const bool met = res.converged;   // the recursive residual reached rtol
     res.converged = res.relres <= rtol * 10.0 && !bad(res.relres);
     // the recursive residual drifted too far from the true one (tight
@@ -714,6 +758,7 @@ fvs_status bicgstab(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, c
       FVS_TRY(vcopy(s, n, w.z, x));
       res.relres = best;
       res.converged = false;
+      res.tail_done = false;
       break;
     }
     if (res.converged || !met || bad(res.relres) || again == MAX_RESTARTS || it >= maxit) break;
@@ -722,7 +767,8 @@ fvs_status bicgstab(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, c
     if (!proj) {
       FVS_TRY(residual_dot<FIN_START>(s, red, A, x, dextra, b, w.r, w.rh));
     } else {
-      FVS_TRY(vcopy(s, n, w.r, w.rh));
+      FVS_TRY(vcopy(s, n, w.q, w.r));
+      FVS_TRY(vcopy(s, n, w.q, w.rh));
       FVS_TRY(red.dot(s, n, w.rh, w.r, S_RHO));
     }
     fresh = true;
@@ -752,15 +798,6 @@ fvs_status pcg(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, Precon
     bb = w.q;
   }
   FVS_TRY(red.dot2(s, n, bb, bb, w.r, w.r, S_BB, S_RR));
-  FVS_TRY(red.fetch(s));
-  double bnorm = sqrt(red.host[S_BB]);
-  if (bnorm == 0.0) bnorm = 1.0;
-  res.relres = sqrt(red.host[S_RR]) / bnorm;
-  if (bad(res.relres) || bad(bnorm)) return FVS_OK;   // non-finite data: not converged
-  if (res.relres <= rtol) {
-    res.converged = true;
-    return FVS_OK;
-  }
   const FirstSweep f = M.first(w.z);
   MeanPart mp;
   const int how = proj ? proj->single(mp) : 0;
@@ -789,21 +826,41 @@ fvs_status pcg(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, Precon
   };
   FVS_TRY(prepare());
   const uint64_t key = graph_key(A, nullptr, M, b, x, w, red) ^ (0x70636770ULL + (uint64_t)how);
+  // r.r of the true residual (formed in q, so that r stays)
+  auto true_residual = [&]() -> fvs_status {
+    FVS_TRY(residual(s, A, x, b, w.q, nullptr));
+    if (proj) FVS_TRY(proj->apply(s, w.q));
+    return red.dot(s, n, w.q, w.q, S_TRUE);
+  };
+  auto queue_loop = [&](int left, bool fresh, bool start, bool& looped) -> fvs_status {
+    fvs_status st = FVS_OK;
+    looped = run_loop(s, graph, key, red, rtol, 0.0, left, fresh, start, body, st);
+    FVS_TRY(st);
+    return looped ? true_residual() : FVS_OK;
+  };
+  // as in bicgstab
+  bool looped = false;
+  FVS_TRY(queue_loop(maxit, true, true, looped));
+  FVS_TRY(red.fetch(s));
+  const double bnorm = residual_scale(red.host[S_BB], 0.0);
+  res.relres = sqrt(red.host[looped ? S_START : S_RR]) / bnorm;
+  if (bad(res.relres) || bad(bnorm)) return FVS_OK;   // non-finite data: not converged
+  if (res.relres <= rtol) {
+    res.converged = true;
+    return FVS_OK;
+  }
   const double tol2 = (rtol * bnorm) * (rtol * bnorm);
-  bool fresh = true;
+  bool queued = looped, fresh = true;
   int it = 0;
   double best = 0.0;   // true residual before a restart (its iterate in w.v)
   for (int again = 0;; ++again) {
     while (it < maxit) {
-      bool looped = false;
-      {
-        fvs_status st = FVS_OK;
-        looped = run_loop(s, graph, key, red, tol2, maxit - it, fresh, body, st);
-        FVS_TRY(st);
+      if (!queued) {
+        FVS_TRY(queue_loop(maxit - it, fresh, false, looped));
+        if (!looped) FVS_TRY(run_body(s, graph, key, fresh, body));
+        FVS_TRY(red.fetch(s));
       }
-      if (!looped) FVS_TRY(run_body(s, graph, key, fresh, body));
-      fresh = false;
-      FVS_TRY(red.fetch(s));
+      queued = fresh = false;
       const int done = looped ? (int)red.host[S_ITER] : 1;
       if (looped) __atomic_add_fetch(&g_launches, graph->loop_kernels * (unsigned long long)done, __ATOMIC_RELAXED);
       it += done;
@@ -817,16 +874,16 @@ fvs_status pcg(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, Precon
         }
         return FVS_OK;
       }
-      if (res.relres <= rtol) {
+      if (res.relres <= rtol || red.host[S_RR] <= tol2) {
         res.converged = true;
         break;
       }
     }
-    FVS_TRY(residual(s, A, x, b, w.r, nullptr));
-    if (proj) FVS_TRY(proj->apply(s, w.r));
-    FVS_TRY(red.dot(s, n, w.r, w.r, S_RR));
-    FVS_TRY(red.fetch(s));
-    res.relres = sqrt(red.host[S_RR]) / bnorm;
+    if (!looped) {
+      FVS_TRY(true_residual());
+      FVS_TRY(red.fetch(s));
+    }
+    res.relres = sqrt(red.host[S_TRUE]) / bnorm;
     const bool met = res.converged;
     res.converged = res.relres <= rtol * 10.0 && !bad(res.relres);
     if (again > 0 && !(res.relres <= best)) {
@@ -839,6 +896,7 @@ fvs_status pcg(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, Precon
     best = res.relres;
     FVS_TRY(vcopy(s, n, x, w.v));
     fresh = true;    // from the true residual, as in bicgstab
+    FVS_TRY(vcopy(s, n, w.q, w.r));
     FVS_TRY(prepare());
   }
   return FVS_OK;

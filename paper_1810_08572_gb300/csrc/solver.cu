@@ -1631,21 +1631,28 @@ fvs_status solver_step(fvs_solver s, double dt, fvs_step_stats* stats) {
       // is left sits in a few cells, where Jacobi's many small steps overshoot
       // the tolerance evenly: the last passes go a little further
       const double rtol_in = lines && rtol_m <= s->props.e_rtol ? std::min(rtol_m, std::max(0.1 * rtol_m, 1e-14)) : rtol_m;
+      // next iterate, then its change against the current one: queued behind
+      // the solve, so that one copy brings both their scalars
+      const std::function<fvs_status()> update = [&]() -> fvs_status {
+        k_energy_update<<<s->red.grid(Nc), RB, 0, st>>>(Nc, mt, s->Tlin, Tm, fsm, s->Tit, s->fsit, s->metal,
+                                                        s->red.part, s->red.ticket, s->red.sc, S_TMP0, S_TMP1);
+        FVS_COUNT_LAUNCH();
+        FVS_LAUNCH_CHECK();
+        return FVS_OK;
+      };
       FVS_TRY(bicgstab(st, s->red, s->kw, s->Ke, s->edx, PE, s->erhs, s->Tlin, rtol_in,
-                       s->props.max_krylov_iters, nullptr, r, 0.0, &s->g_e));
+                       s->props.max_krylov_iters, nullptr, r, 0.0, &s->g_e, &update));
       S.e_lin_its += r.iters;
       if (!r.converged) {
         status = FVS_ERR_NOT_CONVERGED;
         set_error("energy pass %d: relative residual %.3e after %d iterations", it, r.relres, r.iters);
       }
-      // next iterate, then its change against the current one
-      k_energy_update<<<s->red.grid(Nc), RB, 0, st>>>(Nc, mt, s->Tlin, Tm, fsm, s->Tit, s->fsit, s->metal,
-                                                      s->red.part, s->red.ticket, s->red.sc, S_TMP0, S_TMP1);
-      FVS_COUNT_LAUNCH();
-      FVS_LAUNCH_CHECK();
+      if (!r.tail_done) {
+        FVS_TRY(update());
+        FVS_TRY(s->red.fetch(st));
+      }
       dswap(s->Tit, Tm);
       dswap(s->fsit, fsm);
-      FVS_TRY(s->red.fetch(st));
       if (s->red.host[S_TMP0] <= s->props.e_tol_T && s->red.host[S_TMP1] <= 1e-12 && rtol_m <= s->props.e_rtol) {
         conv = true;
         break;

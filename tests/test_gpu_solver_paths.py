@@ -444,3 +444,68 @@ def test_lines_chosen_on_thin_cells_change_only_the_iterations(fvs, monkeypatch,
     T2, jacobi = run()
     assert rel(T1, T2) <= 1e-10
     assert lines < 0.6 * jacobi, (lines, jacobi)
+
+
+@pytest.mark.parametrize("jitter,precision", [(0.2, 0), (0.2, 1), (0.0, 0), (0.0, 1)])
+def test_loops_on_the_device_equal_loops_from_the_host(fvs, jitter, precision):
+    """Solves whose iterations are decided on the device (one wait a solve)
+    and solves driven from the host (as while kernels are timed) take the same
+    steps to the solve tolerance; right sides that meet the tolerance before
+    the first iteration (zero; a relative tolerance above one) enter no loop."""
+    import torch
+    m = box_mesh(20, 18, 6, cases.CAVITY, jitter=jitter, jitter_seed=51, permute_seed=52)
+    T0 = pockets_field(m, seed=6)
+    u0 = np.random.default_rng(13).normal(scale=2e-3, size=(len(T0), 3))
+    props = cases.props(precision=precision, **TIGHT)
+    M = fvs.Mesh(m)
+    out, p_its = [], []
+    for host in (False, True):
+        S = fvs.Solver(M, props)
+        S.profile(host)
+        S.set_state(T0, u0)
+        p_its.append([S.step(1e-3)["p_its"] for _ in range(3)])
+        out.append({k: S.query(k) for k in ("T", "FS", "U", "P", "FLUX")})
+        rhs = torch.zeros(M.n_cells, dtype=torch.float64, device="cuda")
+        p = torch.ones_like(rhs)
+        assert S.pressure_solve(rhs, p, 1e-10)[:2] == (fvs.FVS_OK, 0)
+        assert not p.any()
+        rhs += torch.randn(M.n_cells, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+        assert S.pressure_solve(rhs, p, 2.0)[:2] == (fvs.FVS_OK, 0)
+        status, its, rr = S.pressure_solve(rhs, p, 1e-10)
+        assert status == fvs.FVS_OK and its > 0 and rr <= 1e-9
+        S.close()
+    M.close()
+    tol = 1e-10 if precision == 0 else 1e-8
+    for k in out[0]:
+        assert rel(out[0][k], out[1][k]) <= tol, k
+    assert max(abs(a - b) for a, b in zip(*p_its)) <= 1, p_its
+
+
+@pytest.mark.parametrize("shape,jitter,samples", [((8, 8, 2), 0.0, 3), ((12, 11, 4), 0.0, 33), ((8, 8, 2), 0.2, 5)])
+def test_lockstep_batch_loops_on_the_device_equal_loops_from_the_host(fvs, shape, jitter, samples):
+    """The same for the lockstep batch (one tile, two tiles, BiCGStab on a
+    skewed mesh): per-sample outputs and step counts after 12 steps."""
+    import os
+    import subprocess
+    import sys
+    code = ("import numpy as np\n"
+            "from paper_1810_08572_gb300 import fvs\n"
+            "from fvs_inputs import box_mesh, cases\n"
+            f"m = box_mesh(*{shape}, (0.01, 0.01, 0.0025), jitter={jitter}, jitter_seed=3, permute_seed=4)\n"
+            f"x = np.stack([np.linspace(930, 960, {samples}), np.linspace(740, 690, {samples}), "
+            f"np.linspace(3.2, 4.8, {samples})], axis=1)\n"
+            f"q, s = fvs.uq_batch(fvs.Mesh(m), cases.props(**{TIGHT}), x, 2e-3, 12)\n"
+            "print(' '.join(v.hex() for v in q.ravel().tolist()), '|', *s.tolist())\n")
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    got = []
+    for host in (False, True):
+        env = dict(os.environ, FVS_NO_TUNE="1", PYTHONPATH=root)
+        env.pop("FVS_NO_GRAPHS", None)
+        if host:
+            env["FVS_NO_GRAPHS"] = "1"
+        r = subprocess.run([sys.executable, "-c", code], cwd=root, env=env, capture_output=True, text=True, timeout=300)
+        assert r.returncode == 0, r.stderr[-2000:]
+        q, s = r.stdout.strip().splitlines()[-1].split("|")
+        got.append((np.array([float.fromhex(v) for v in q.split()]), s.split()))
+    assert got[0][1] == got[1][1]
+    np.testing.assert_allclose(got[0][0], got[1][0], rtol=1e-8, equal_nan=True)
