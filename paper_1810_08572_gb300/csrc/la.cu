@@ -105,21 +105,21 @@ fvs_status Reducer::init() {
 }
 
 fvs_status Reducer::dot(cudaStream_t s, int64_t n, const double* x, const double* y, int slot) {
-  k_dot2<false><<<grid(n), RB, 0, s>>>(n, x, y, nullptr, nullptr, part, ticket, sc, slot, -1); FVS_COUNT_LAUNCH();
+  k_dot2<false><<<vgrid(n), RB, 0, s>>>(n, x, y, nullptr, nullptr, part, ticket, sc, slot, -1); FVS_COUNT_LAUNCH();
   FVS_LAUNCH_CHECK();
   return FVS_OK;
 }
 
 fvs_status Reducer::dot2(cudaStream_t s, int64_t n, const double* a, const double* b, const double* c,
                          const double* d, int s0, int s1) {
-  k_dot2<true><<<grid(n), RB, 0, s>>>(n, a, b, c, d, part, ticket, sc, s0, s1); FVS_COUNT_LAUNCH();
+  k_dot2<true><<<vgrid(n), RB, 0, s>>>(n, a, b, c, d, part, ticket, sc, s0, s1); FVS_COUNT_LAUNCH();
   FVS_LAUNCH_CHECK();
   return FVS_OK;
 }
 
 fvs_status Reducer::max_abs_diff2(cudaStream_t s, int64_t n, const double* a, const double* b,
                                   const double* c, const double* d, int s0, int s1) {
-  k_maxdiff2<<<grid(n), RB, 0, s>>>(n, a, b, c, d, part, ticket, sc, s0, s1); FVS_COUNT_LAUNCH();
+  k_maxdiff2<<<vgrid(n), RB, 0, s>>>(n, a, b, c, d, part, ticket, sc, s0, s1); FVS_COUNT_LAUNCH();
   FVS_LAUNCH_CHECK();
   return FVS_OK;
 }
@@ -665,7 +665,7 @@ fvs_status bicgstab(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, c
     FVS_BY_MODE(fs.mode, (k_bicg_s<PM><<<grid, 256, 0, s>>>(n, red.sc, w.r, w.v, w.sv, fs)));
     FVS_TRY(M.rest(s, w.sv, w.sh));
     FVS_TRY(spmv_dot<FIN_TSTT>(s, red, A, w.sh, w.t, dextra, w.sv));
-    k_bicg_xr_dot<<<red.grid(n), RB, 0, s>>>(n, red.sc, w.ph, w.sh, w.sv, w.t, w.rh, x, w.r, red.part,
+    k_bicg_xr_dot<<<red.vgrid(n), RB, 0, s>>>(n, red.sc, w.ph, w.sh, w.sv, w.t, w.rh, x, w.r, red.part,
                                               red.ticket, ctl); FVS_COUNT_LAUNCH();
     FVS_LAUNCH_CHECK();
     return FVS_OK;
@@ -806,15 +806,15 @@ fvs_status pcg(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, Precon
     FVS_TRY(M.rest(s, w.r, w.z));
     if (how == 2) FVS_TRY(proj->apply(s, w.z));
     if (how == 1) {
-      k_dot_rz<true><<<red.grid(n), RB, 0, s>>>(n, w.r, w.z, mp, red.part, red.ticket, red.sc); FVS_COUNT_LAUNCH();
+      k_dot_rz<true><<<red.vgrid(n), RB, 0, s>>>(n, w.r, w.z, mp, red.part, red.ticket, red.sc); FVS_COUNT_LAUNCH();
       k_cg_p<true><<<grid, 256, 0, s>>>(n, red.sc, w.z, w.p, first ? 1 : 0, mp); FVS_COUNT_LAUNCH();
     } else {
-      k_dot_rz<false><<<red.grid(n), RB, 0, s>>>(n, w.r, w.z, mp, red.part, red.ticket, red.sc); FVS_COUNT_LAUNCH();
+      k_dot_rz<false><<<red.vgrid(n), RB, 0, s>>>(n, w.r, w.z, mp, red.part, red.ticket, red.sc); FVS_COUNT_LAUNCH();
       k_cg_p<false><<<grid, 256, 0, s>>>(n, red.sc, w.z, w.p, first ? 1 : 0, mp); FVS_COUNT_LAUNCH();
     }
     FVS_LAUNCH_CHECK();
     FVS_TRY(spmv_dot<FIN_PQ>(s, red, A, w.p, w.q, nullptr, w.p));
-    FVS_BY_MODE(f.mode, (k_cg_xr_dot<PM><<<red.grid(n), RB, 0, s>>>(n, red.sc, w.p, w.q, x, w.r, f, red.part,
+    FVS_BY_MODE(f.mode, (k_cg_xr_dot<PM><<<red.vgrid(n), RB, 0, s>>>(n, red.sc, w.p, w.q, x, w.r, f, red.part,
                                                                     red.ticket, ctl)));
     return FVS_OK;
   };

@@ -509,3 +509,37 @@ def test_lockstep_batch_loops_on_the_device_equal_loops_from_the_host(fvs, shape
         got.append((np.array([float.fromhex(v) for v in q.split()]), s.split()))
     assert got[0][1] == got[1][1]
     np.testing.assert_allclose(got[0][0], got[1][0], rtol=1e-8, equal_nan=True)
+
+
+@pytest.mark.parametrize("shape", [(64, 64, 38), (64, 64, 39), (128, 76, 64), (128, 76, 65)])
+def test_pressure_solve_where_the_reduction_grids_change(fvs, shape):
+    """155,648 rows are one row for each thread of half a wave, 622,592 two
+    rows for each thread of a full one: the solutions at and past both meet
+    the seven-point equations formed here from the grid, independently of the
+    solver's own sums (tolerance: ten times the residual asked for, which is
+    what a solve may end with)."""
+    import torch
+    h = np.array([1e-3, 1.25e-3, 8e-4])
+    m = box_mesh(*shape, tuple(h * shape), permute_seed=61)
+    M = fvs.Mesh(m)
+    S = fvs.Solver(M, cases.props(**TIGHT))
+    S.set_state(np.full(M.n_cells, 960.0))
+    S.step(1e-4)
+    rhs = np.random.default_rng(14).normal(size=M.n_cells)
+    rhs -= rhs.mean()
+    p = torch.zeros(M.n_cells, dtype=torch.float64, device="cuda")
+    status, its, rr = S.pressure_solve(torch.from_numpy(rhs).cuda(), p, 1e-10)
+    assert status == fvs.FVS_OK and its > 0
+    ijk = tuple(np.asarray(m["cell_ijk"]).T)
+    g = np.zeros(shape)
+    b = np.zeros(shape)
+    g[ijk], b[ijk] = p.cpu().numpy(), rhs
+    q = np.zeros(shape)
+    for a in range(3):
+        d = np.diff(g, axis=a) * (h.prod() / h[a] ** 2)
+        pad = [(1, 1) if k == a else (0, 0) for k in range(3)]
+        q += np.diff(np.pad(d, pad), axis=a)
+    scale = (q * b).sum() / (q * q).sum()      # the solver's sign and units
+    assert np.linalg.norm(b - scale * q) <= 1e-9 * np.linalg.norm(b)
+    S.close()
+    M.close()
