@@ -33,13 +33,13 @@ METRIC = "active cell-steps/s at 1e-8 pressure residual (mixed vs FP64) + UQ sam
 
 # CUDA kernel behind each timed class of the solver's kernel timing (the
 # coarse AMG levels run their own sweep kernels; k_jac0 serves every level)
-CUDA_NAME = {"residual_vc": "k_resid<double>", "residual_vc_coarse": "k_resid_g<double>",
-             "jacobi": "k_jac<double>", "jacobi_coarse": "k_jac_g<double>",
+CUDA_NAME = {"residual_vc": "k_fine<double>", "residual_vc_coarse": "k_resid_g<double>",
+             "jacobi": "k_fine<double>", "jacobi_coarse": "k_cheb_g<double>",
              "jacobi0": "k_jac0<double>", "jacobi0_coarse": "k_jac0<double>",
-             "residual_f32": "k_resid<float>", "residual_f32_coarse": "k_resid_g<float>",
-             "jacobi_f32": "k_jac<float>", "jacobi_f32_coarse": "k_jac_g<float>",
+             "residual_f32": "k_fine<float>", "residual_f32_coarse": "k_resid_g<float>",
+             "jacobi_f32": "k_fine<float>", "jacobi_f32_coarse": "k_cheb_g<float>",
              "jacobi0_f32": "k_jac0<float>", "jacobi0_f32_coarse": "k_jac0<float>",
-             "spmv": "k_spmv_dot", "residual": "k_residual"}
+             "spmv": "k_spmv_dot", "residual": "k_residual_dot"}
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum of one ncu
 # capture, cold cache) per algorithmic byte of the same launches on the 96^3
 # cavity, applied to the bench launch (summary under profiles/): k_spmv_dot,
