@@ -1577,7 +1577,6 @@ fvs_status Amg::setup(cudaStream_t s, const Ell& A, bool diagonal_first) {
   ready = false;
   masked = false;
   refreshes = 0;
-  ++version;
   lv.clear();
   opt.theta = env_num("FVS_AMG_THETA", opt.theta);
   opt.omega = env_num("FVS_AMG_OMEGA", opt.omega);
@@ -1976,7 +1975,6 @@ fvs_status Amg::refresh(cudaStream_t s, const int32_t* act, const uint8_t* ppe) 
     return FVS_ERR_STATE;
   }
   ready = false;
-  ++version;
   const bool dbg = getenv("FVS_DEBUG") != nullptr;
   double tph[4] = {0, 0, 0, 0};
   auto t_last = std::chrono::steady_clock::now();

@@ -87,7 +87,7 @@ struct Amg : Precond {
   fvs_status apply(cudaStream_t s, const double* r, double* z) override;
   FirstSweep first(double* z) override;
   fvs_status rest(cudaStream_t s, const double* r, double* z) override;
-  uint64_t version = 0;          // bumped by every setup
+
   // coarsest inverse above the shared-memory size: the block steps' second
   // array, a vector, and the row exchanges of the column-by-column fallback
   DBuf<double> gj_tmp, gj_fac;

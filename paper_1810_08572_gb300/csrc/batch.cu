@@ -827,10 +827,6 @@ __global__ void kb_scale_copy(int64_t n, double a, const double* x, double* y) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     y[i] = a * x[i];
 }
-__global__ void kb_copy_i32(int64_t n, const int32_t* a, int32_t* b) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    b[i] = a[i];
-}
 // the fine operator of every sample written out as per-sample ELL values
 // (used when the fine level itself is the coarsest)
 __global__ void kb_materialize0(int64_t n, int w, int Sp, const double* base, const int32_t* ovr, const int32_t* col,

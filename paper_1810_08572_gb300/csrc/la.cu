@@ -22,16 +22,6 @@ namespace fvs {
   } while (0)
 
 template <int W, bool CS>
-__global__ void k_spmv(int64_t n, int w, const int32_t* __restrict__ col, const double* __restrict__ val,
-                       const double* __restrict__ x, double* __restrict__ y,
-                       const double* __restrict__ dextra) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const double acc = ell_row<W, CS>(n, w, col, val, x, i, dextra ? dextra[i] * x[i] : 0.0);
-    y[i] = acc;
-  }
-}
-
-template <int W, bool CS>
 __global__ void k_residual(int64_t n, int w, const int32_t* __restrict__ col, const double* __restrict__ val,
                            const double* __restrict__ x, const double* __restrict__ b, double* __restrict__ r,
                            const double* __restrict__ dextra) {
@@ -39,14 +29,6 @@ __global__ void k_residual(int64_t n, int w, const int32_t* __restrict__ col, co
     const double acc = ell_row<W, CS>(n, w, col, val, x, i, dextra ? dextra[i] * x[i] : 0.0);
     r[i] = b[i] - acc;
   }
-}
-
-fvs_status spmv(cudaStream_t s, const Ell& A, const double* x, double* y, const double* dextra) {
-  if (A.n == 0) return FVS_OK;
-  ProfScope ps(&A, "spmv", (double)A.n * (12.0 * A.w + 16.0 + (dextra ? 8.0 : 0.0)), s);
-  FVS_BY_ROW(A, (k_spmv<W, CS><<<stride_grid(A.n, 256), 256, 0, s>>>(A.n, A.w, A.col, A.val, x, y, dextra)));
-  FVS_LAUNCH_CHECK();
-  return FVS_OK;
 }
 
 fvs_status residual(cudaStream_t s, const Ell& A, const double* x, const double* b, double* r,

@@ -71,8 +71,6 @@ struct Reducer {
   fvs_status fetch(cudaStream_t s);   // copies sc -> host and waits
 };
 
-// y = A x (+ dextra .* x if dextra)
-fvs_status spmv(cudaStream_t s, const Ell& A, const double* x, double* y, const double* dextra = nullptr);
 // r = b - A x (- dextra .* x)
 fvs_status residual(cudaStream_t s, const Ell& A, const double* x, const double* b, double* r,
                     const double* dextra = nullptr);
