@@ -2197,6 +2197,12 @@ fvs_status Amg::vcycle_t(cudaStream_t s, int l, const T* b, Y* y, bool x0_ready)
   // the fine level of the face-coupling operator has its own kernel, which
   // leaves a matrix that fits in the L2 cache
   const bool fine7 = l == 0 && diag_first;
+  // FP64: a block for every 256 rows, no stride: at 44 to 48 registers five
+  // blocks fit an SM, so a stride grid of eight an SM ends in a wave 3/5 full
+  // (128^3, three steps 155.8 -> 154.1 ms; AMG-CG on 442,368 rows 6.67 ->
+  // 6.60).  FP32 sweeps, half as long, are better off with fewer blocks (a
+  // casting of 422,000 cells 36.7 ms, 37.0 without the stride).
+  const int gf = sizeof(T) == 8 ? (int)std::min<int64_t>((n + 255) / 256, INT32_MAX) : g;
   auto fine = [&](auto launch) {
     if (n * (int64_t)(6 * (4 + sizeof(T))) > L2_KEEP_BYTES) launch(std::true_type());
     else launch(std::false_type());
@@ -2205,7 +2211,7 @@ fvs_status Amg::vcycle_t(cudaStream_t s, int l, const T* b, Y* y, bool x0_ready)
     using O = std::remove_pointer_t<decltype(xout)>;
     ProfScope ps(pkey, n_jac, jac_bytes, s);
     if (fine7) fine([&](auto cs) {
-      k_fine<T, O, FINE_JACOBI, decltype(cs)::value><<<g, 256, 0, s>>>(n, A.col, val, wl, dinv, b, xin, nullptr, xout);
+      k_fine<T, O, FINE_JACOBI, decltype(cs)::value><<<gf, 256, 0, s>>>(n, A.col, val, wl, dinv, b, xin, nullptr, xout);
     });
     else if (!rl) k_jac<T, O><<<g, 256, 0, s>>>(n, A.w, A.col, val, wl, dinv, b, xin, xout);
     else if (G == 1) k_jac_g<T, O, 1><<<gg, 256, 0, s>>>(n, A.col, val, wl, dinv, b, xin, xout, rl);
@@ -2220,7 +2226,7 @@ fvs_status Amg::vcycle_t(cudaStream_t s, int l, const T* b, Y* y, bool x0_ready)
     const double* ab = wl + 2 * k;
     ProfScope ps(pkey, n_jac, jac_bytes + vb * (double)n, s);
     if (fine7) fine([&](auto cs) {
-      k_fine<T, O, FINE_CHEB, decltype(cs)::value><<<g, 256, 0, s>>>(n, A.col, val, ab, dinv, b, xin, xprev, xout);
+      k_fine<T, O, FINE_CHEB, decltype(cs)::value><<<gf, 256, 0, s>>>(n, A.col, val, ab, dinv, b, xin, xprev, xout);
     });
     else if (!rl) k_cheb<T, O><<<g, 256, 0, s>>>(n, A.w, A.col, val, ab, dinv, b, xin, xprev, xout);
     else if (G == 1) k_cheb_g<T, O, 1><<<gg, 256, 0, s>>>(n, A.col, val, ab, dinv, b, xin, xprev, xout, rl);
@@ -2248,7 +2254,7 @@ fvs_status Amg::vcycle_t(cudaStream_t s, int l, const T* b, Y* y, bool x0_ready)
   {
     ProfScope ps(pkey, n_res, res_bytes, s);
     if (fine7) fine([&](auto cs) {
-      k_fine<T, T, FINE_RESID, decltype(cs)::value><<<g, 256, 0, s>>>(n, A.col, val, wl, dinv, b, xa, nullptr, r);
+      k_fine<T, T, FINE_RESID, decltype(cs)::value><<<gf, 256, 0, s>>>(n, A.col, val, wl, dinv, b, xa, nullptr, r);
     });
     else if (!rl) k_resid<T><<<g, 256, 0, s>>>(n, A.w, A.col, val, xa, b, r);
     else if (G == 1) k_resid_g<T, 1><<<gg, 256, 0, s>>>(n, A.col, val, xa, b, r, rl);

@@ -411,8 +411,8 @@ constexpr int MAX_RESTARTS = 3;   // from the true residual, once the recursive 
 template <int MODE, bool DX>
 static void launch_spmv_dot(cudaStream_t s, Reducer& red, const Ell& A, const double* x, double* y,
                             const double* dextra, const double* d) {
-  FVS_BY_ROW(A, (k_spmv_dot<MODE, DX, W, CS><<<red.grid(A.n), RB, 0, s>>>(A.n, A.w, A.col, A.val, x, y, dextra, d,
-                                                                          red.part, red.ticket, red.sc)));
+  FVS_BY_ROW(A, (k_spmv_dot<MODE, DX, W, CS><<<red.rgrid(red.grid(A.n), W > 0 ? 6 : 8), RB, 0, s>>>(
+      A.n, A.w, A.col, A.val, x, y, dextra, d, red.part, red.ticket, red.sc)));
 }
 template <int MODE>
 static fvs_status spmv_dot(cudaStream_t s, Reducer& red, const Ell& A, const double* x, double* y,
@@ -427,8 +427,8 @@ static fvs_status spmv_dot(cudaStream_t s, Reducer& red, const Ell& A, const dou
 template <int MODE, bool DX>
 static void launch_residual_dot(cudaStream_t s, Reducer& red, const Ell& A, const double* x, const double* dextra,
                                 const double* b, double* r, double* rh, const int* go) {
-  FVS_BY_ROW(A, (k_residual_dot<MODE, DX, W, CS><<<red.grid(A.n), RB, 0, s>>>(A.n, A.w, A.col, A.val, x, dextra, b, r,
-                                                                              rh, red.part, red.ticket, red.sc, go)));
+  FVS_BY_ROW(A, (k_residual_dot<MODE, DX, W, CS><<<red.rgrid(red.grid(A.n), W > 0 ? 6 : 8), RB, 0, s>>>(
+      A.n, A.w, A.col, A.val, x, dextra, b, r, rh, red.part, red.ticket, red.sc, go)));
 }
 template <int MODE>
 static fvs_status residual_dot(cudaStream_t s, Reducer& red, const Ell& A, const double* x, const double* dextra,
@@ -647,7 +647,7 @@ fvs_status bicgstab(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, c
     FVS_BY_MODE(fs.mode, (k_bicg_s<PM><<<grid, 256, 0, s>>>(n, red.sc, w.r, w.v, w.sv, fs)));
     FVS_TRY(M.rest(s, w.sv, w.sh));
     FVS_TRY(spmv_dot<FIN_TSTT>(s, red, A, w.sh, w.t, dextra, w.sv));
-    k_bicg_xr_dot<<<red.vgrid(n), RB, 0, s>>>(n, red.sc, w.ph, w.sh, w.sv, w.t, w.rh, x, w.r, red.part,
+    k_bicg_xr_dot<<<red.rgrid(red.vgrid(n), 5), RB, 0, s>>>(n, red.sc, w.ph, w.sh, w.sv, w.t, w.rh, x, w.r, red.part,
                                               red.ticket, ctl); FVS_COUNT_LAUNCH();
     FVS_LAUNCH_CHECK();
     return FVS_OK;
