@@ -616,7 +616,7 @@ static bool run_loop(cudaStream_t s, IterGraph* g, uint64_t key, Reducer& red, d
 fvs_status bicgstab(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, const double* dextra,
                     Precond& M, const double* b, double* x, double rtol, int maxit, Projector* proj,
                     SolveResult& res, double bnorm_floor, IterGraph* graph,
-                    const std::function<fvs_status()>* tail) {
+                    const std::function<fvs_status()>* tail, double asked) {
   const int64_t n = A.n;
   res = SolveResult();
   if (n == 0) {
@@ -685,6 +685,7 @@ fvs_status bicgstab(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, c
     return FVS_OK;
   }
   const double tol2 = (rtol * bnorm) * (rtol * bnorm);
+  const double accept = 10.0 * (asked > rtol ? asked : rtol);
   bool queued = looped, fresh = true;
   int it = 0;
   double best = 0.0;   // true residual before a restart (its iterate in w.z)
@@ -731,7 +732,7 @@ fvs_status bicgstab(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, c
     }
     res.relres = sqrt(red.host[S_TRUE]) / bnorm;
     const bool met = res.converged;   // the recursive residual reached rtol
-    res.converged = res.relres <= rtol * 10.0 && !bad(res.relres);
+    res.converged = res.relres <= accept && !bad(res.relres);
     // the recursive residual drifted too far from the true one (tight
     // tolerances on large systems): start again from the true residual
     // rather than give the solve up; an attempt that ends further off than it

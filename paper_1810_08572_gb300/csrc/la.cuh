@@ -243,10 +243,13 @@ struct Projector {
 // run holds).  Before, a solve waited three times and the energy pass a
 // fourth: a step on 4,096 cells 1.77 -> 1.67 ms, on 184,320 conducting cells
 // 2.50 -> 2.44; the kernels in the loop are the same.
+//
+// rtol is what the iteration works towards; the true residual is judged, and
+// a restart decided, by ten times the larger of rtol and asked.
 fvs_status bicgstab(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, const double* dextra,
                     Precond& M, const double* b, double* x, double rtol, int maxit,
                     Projector* proj, SolveResult& res, double bnorm_floor = 0.0, IterGraph* graph = nullptr,
-                    const std::function<fvs_status()>* tail = nullptr);
+                    const std::function<fvs_status()>* tail = nullptr, double asked = 0.0);
 fvs_status pcg(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, Precond& M,
                const double* b, double* x, double rtol, int maxit, Projector* proj, SolveResult& res,
                IterGraph* graph = nullptr);

@@ -1629,7 +1629,9 @@ fvs_status solver_step(fvs_solver s, double dt, fvs_step_stats* stats) {
       SolveResult r;
       // with the lines an iteration takes off an order of magnitude and what
       // is left sits in a few cells, where Jacobi's many small steps overshoot
-      // the tolerance evenly: the last passes go a little further
+      // the tolerance evenly: the last passes go a little further.  They are
+      // judged by rtol_m all the same: on cells so thin that rounding stops the
+      // residual between the two, the pass is as good as Jacobi's
       const double rtol_in = lines && rtol_m <= s->props.e_rtol ? std::min(rtol_m, std::max(0.1 * rtol_m, 1e-14)) : rtol_m;
       // next iterate, then its change against the current one: queued behind
       // the solve, so that one copy brings both their scalars
@@ -1641,7 +1643,7 @@ fvs_status solver_step(fvs_solver s, double dt, fvs_step_stats* stats) {
         return FVS_OK;
       };
       FVS_TRY(bicgstab(st, s->red, s->kw, s->Ke, s->edx, PE, s->erhs, s->Tlin, rtol_in,
-                       s->props.max_krylov_iters, nullptr, r, 0.0, &s->g_e, &update));
+                       s->props.max_krylov_iters, nullptr, r, 0.0, &s->g_e, &update, rtol_m));
       S.e_lin_its += r.iters;
       if (!r.converged) {
         status = FVS_ERR_NOT_CONVERGED;

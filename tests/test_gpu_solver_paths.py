@@ -543,3 +543,26 @@ def test_pressure_solve_where_the_reduction_grids_change(fvs, shape):
     assert np.linalg.norm(b - scale * q) <= 1e-9 * np.linalg.norm(b)
     S.close()
     M.close()
+
+
+@pytest.mark.parametrize("lines", [None, "0"])
+def test_thin_cells_are_judged_by_the_tolerance_asked_for(fvs, monkeypatch, lines):
+    """Conduction some thousand times the mass term: rounding stops the true
+    residual of the energy solves near 1.5e-13.  With e_rtol 1e-13 (a solve
+    may end with ten times that) the steps converge, with the line
+    preconditioner, which works towards a tenth of the tolerance, as with
+    Jacobi."""
+    if lines is not None:
+        monkeypatch.setenv("FVS_ENERGY_LINES", lines)
+    shape = (32, 32, 64)
+    m = box_mesh(*shape, (0.1, 0.1, 0.0025), permute_seed=32)
+    ijk = m["cell_ijk"]
+    walls = [(cases.BC_DIRICHLET, 930.0), (cases.BC_DIRICHLET, 990.0)] + [(cases.BC_ADIABATIC, 0.0)] * 4
+    M = fvs.Mesh(m)
+    S = fvs.Solver(M, cases.props(no_flow=True, walls=walls, e_rtol=1e-13, e_tol_T=1e-10, max_krylov_iters=4000))
+    S.set_state(960.0 + 8.0 * np.sin(3.0 * ijk[:, 0] / shape[0]) + 3.0 * np.sin(0.1 * ijk[:, 2]))
+    for _ in range(2):
+        st = S.step(0.05, allow_not_converged=True)
+        assert st["status"] == 0, fvs.fvs_last_error()
+    S.close()
+    M.close()
