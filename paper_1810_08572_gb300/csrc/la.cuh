@@ -181,7 +181,14 @@ struct LinePrecond : Precond {
   DBuf<double> lo, inv, cp;    // sub-diagonal, 1 / pivot, super-diagonal / pivot
   DBuf<double> yl;             // forward substitution, in line order
   bool ready = false;
-  // Whether the lines pay: with a and b the mean shares of a row's diagonal
+  // per row of the operator: sum of its off-diagonal magnitudes, and of those
+  // that the lines leave out
+  DBuf<double> off, rest;
+  bool weighed = false;
+  // Whether the lines pay at the given inverse diagonal, which holds the state
+  // (latent heat makes the rows of mushy cells several times as dominant): asked
+  // in every step, so that a step depends on its state and not on the ones
+  // before it.  With a and b the mean shares of a row's diagonal
   // that Jacobi and the lines leave out, the iterations go down by about
   // sqrt((1 + a)(1 - b) / ((1 - a)(1 + b))), and an iteration costs about 1.4
   // (27-point rows) or twice (face-only rows) as much.  All melt on 128^3
@@ -192,7 +199,7 @@ struct LinePrecond : Precond {
   // substitution's serial walk costs more than the iterations it saves.
   static constexpr int64_t MIN_ROWS = 65536;
   static constexpr double GAIN_WIDE = 3.0, GAIN_FACE = 4.0;
-  static fvs_status worth(cudaStream_t s, Reducer& red, const Ell& A, const double* dextra, bool& use);
+  fvs_status worth(cudaStream_t s, Reducer& red, const Ell& A, const double* dinv, bool& use);
   fvs_status build(cudaStream_t s, const Ell& A);
   fvs_status factor(cudaStream_t s);
   fvs_status apply(cudaStream_t s, const double* r, double* z) override;

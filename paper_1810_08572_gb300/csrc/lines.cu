@@ -122,33 +122,53 @@ __global__ void __launch_bounds__(64) k_line_solve(int64_t ngroups, const int64_
 // rule on the host, against which the layout is checked)
 // ---------------------------------------------------------------------------
 // two largest off-diagonal couplings of a row (the first slot wins a tie),
-// the second only if at least a quarter of the first
-__device__ __forceinline__ void strongest2(int64_t n, int w, const int32_t* col, const double* val, int64_t i,
-                                           int32_t& b0, int32_t& b1, double& m0, double& m1) {
-  m0 = m1 = 0.0;
+// the second only if at least a quarter of the first, and the sum of all;
+// the loads of nine slots in flight together.  Magnitudes are compared as bit
+// patterns, which order as they do (FP64 compares issue at two lanes a clock);
+// a NaN counts as no coupling.
+__device__ __forceinline__ void strongest2(int64_t n, int w, const int32_t* __restrict__ col,
+                                           const double* __restrict__ val, int64_t i, int32_t& b0, int32_t& b1,
+                                           double& m0, double& m1, double& off) {
+  constexpr int B = 9;
+  constexpr long long INF = 0x7ff0000000000000LL;
+  long long q0 = 0, q1 = 0;
+  off = 0.0;
   b0 = b1 = -1;
-  for (int k = 0; k < w; ++k) {
-    const int32_t j = col[(int64_t)k * n + i];
-    if (j == (int32_t)i) continue;
-    const double a = fabs(val[(int64_t)k * n + i]);
-    if (!(a > 0.0)) continue;
-    if (a > m0) {
-      if (j != b0) { m1 = m0; b1 = b0; }
-      m0 = a;
-      b0 = j;
-    } else if (a > m1 && j != b0) {
-      m1 = a;
-      b1 = j;
+  for (int k0 = 0; k0 < w; k0 += B) {
+    int32_t c[B];
+    double v[B];
+#pragma unroll
+    for (int k = 0; k < B; ++k) {
+      const bool in = k0 + k < w;
+      c[k] = in ? col[(int64_t)(k0 + k) * n + i] : (int32_t)i;
+      v[k] = in ? val[(int64_t)(k0 + k) * n + i] : 0.0;
+    }
+#pragma unroll
+    for (int k = 0; k < B; ++k) {
+      const int32_t j = c[k];
+      const double a = j != (int32_t)i ? fabs(v[k]) : 0.0;
+      off += a;
+      const long long q = __double_as_longlong(a) > INF ? 0 : __double_as_longlong(a);
+      if (q > q0) {
+        if (j != b0) { q1 = q0; b1 = b0; }
+        q0 = q;
+        b0 = j;
+      } else if (q > q1 && j != b0) {
+        q1 = q;
+        b1 = j;
+      }
     }
   }
+  m0 = __longlong_as_double(q0);
+  m1 = __longlong_as_double(q1);
   if (!(m1 >= 0.25 * m0)) { b1 = -1; m1 = 0.0; }
 }
 __global__ void k_line_best(int64_t n, int w, const int32_t* __restrict__ col, const double* __restrict__ val,
                             int32_t* __restrict__ best) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     int32_t b0, b1;
-    double m0, m1;
-    strongest2(n, w, col, val, i, b0, b1, m0, m1);
+    double m0, m1, o;
+    strongest2(n, w, col, val, i, b0, b1, m0, m1, o);
     best[2 * i] = b0;
     best[2 * i + 1] = b1;
   }
@@ -256,23 +276,28 @@ __global__ void k_line_fill(int64_t n, int w, const int32_t* __restrict__ col, c
     snext[e] = jn >= 0 ? sn : (int8_t)-1;
   }
 }
-// sums over the rows of |off-diagonal| / diagonal, and of the same without
-// each row's chain couplings: what Jacobi and the lines leave out
-__global__ void __launch_bounds__(RB) k_line_weight(int64_t n, int w, const int32_t* __restrict__ col,
-                                                    const double* __restrict__ val, const double* __restrict__ diag,
-                                                    const double* __restrict__ dextra, double* part,
-                                                    unsigned int* ticket, double* sc, int s0, int s1) {
+// sums of a row's off-diagonal magnitudes, and of the same without its chain
+// couplings: what Jacobi and the lines leave out
+__global__ void k_line_sums(int64_t n, int w, const int32_t* __restrict__ col, const double* __restrict__ val,
+                            double* __restrict__ off, double* __restrict__ rest) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    int32_t b0, b1;
+    double m0, m1, o;
+    strongest2(n, w, col, val, i, b0, b1, m0, m1, o);
+    off[i] = o;
+    rest[i] = o - m0 - m1;
+  }
+}
+// both times the rows' inverse diagonals, summed (rows without a diagonal left out)
+__global__ void __launch_bounds__(RB) k_line_weight(int64_t n, const double* __restrict__ off,
+                                                    const double* __restrict__ rest, const double* __restrict__ dinv,
+                                                    double* part, unsigned int* ticket, double* sc, int s0, int s1) {
   double x = 0.0, y = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)RB + threadIdx.x; i < n; i += (int64_t)gridDim.x * RB) {
-    int32_t b0, b1;
-    double m0, m1, off = 0.0;
-    strongest2(n, w, col, val, i, b0, b1, m0, m1);
-    for (int k = 0; k < w; ++k)
-      if (col[(int64_t)k * n + i] != (int32_t)i) off += fabs(val[(int64_t)k * n + i]);
-    const double d = fabs(diag[i] + (dextra ? dextra[i] : 0.0));
-    if (d > 0.0) {
-      x += off / d;
-      y += (off - m0 - m1) / d;
+    const double d = fabs(dinv[i]);
+    if (d < 1e300) {
+      x = fma(off[i], d, x);
+      y = fma(rest[i], d, y);
     }
   }
   if (grid_fold<OpSum, 2>(x, y, part, ticket)) {
@@ -283,11 +308,17 @@ __global__ void __launch_bounds__(RB) k_line_weight(int64_t n, int w, const int3
 
 }  // namespace
 
-fvs_status LinePrecond::worth(cudaStream_t s, Reducer& red, const Ell& Ain, const double* dx, bool& use) {
+fvs_status LinePrecond::worth(cudaStream_t s, Reducer& red, const Ell& Ain, const double* dinv, bool& use) {
   use = false;
   if (Ain.n < MIN_ROWS || Ain.w < 3) return FVS_OK;
-  k_line_weight<<<red.grid(Ain.n), RB, 0, s>>>(Ain.n, Ain.w, Ain.col, Ain.val, Ain.diag, dx, red.part, red.ticket,
-                                               red.sc, S_TMP0, S_TMP1);
+  if (!weighed) {
+    FVS_TRY(off.alloc(Ain.n));
+    FVS_TRY(rest.alloc(Ain.n));
+    k_line_sums<<<stride_grid(Ain.n, 256), 256, 0, s>>>(Ain.n, Ain.w, Ain.col, Ain.val, off, rest);
+    FVS_COUNT_LAUNCH();
+    weighed = true;
+  }
+  k_line_weight<<<red.vgrid(Ain.n), RB, 0, s>>>(Ain.n, off, rest, dinv, red.part, red.ticket, red.sc, S_TMP0, S_TMP1);
   FVS_COUNT_LAUNCH();
   FVS_LAUNCH_CHECK();
   FVS_TRY(red.fetch(s));

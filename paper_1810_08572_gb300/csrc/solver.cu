@@ -1015,7 +1015,6 @@ static fvs_status apply_properties(fvs_solver s, const fvs_props* p) {
   FVS_COUNT_LAUNCH();
   s->have_props = true;
   s->eline.ready = false;   // the chains follow the conductive operator
-  s->eline_dt = 0.0;
   FVS_TRY(solver_set_state(s, nullptr, nullptr, 0));
   return conduction_operator(s);
 }
@@ -1044,6 +1043,7 @@ static fvs_status conduction_operator(fvs_solver s) {
   k_scale_ell<<<stride_grid(m->Nc, 256), 256, 0, s->stream>>>(m->Nc, m->W, -0.5, s->LT.val, s->LT.diag,
                                                              s->Ke.val, s->Ke.diag); FVS_COUNT_LAUNCH();
   FVS_LAUNCH_CHECK();
+  s->eline.weighed = false;
   return FVS_OK;
 }
 
@@ -1087,6 +1087,7 @@ fvs_status solver_set_state(fvs_solver s, const double* T, const double* u, int 
   s->numbered = false;
   s->force_full = false;
   s->amg_ok = false;
+  if (s->n_k > 0) s->eline.ready = false;   // chains of the earlier state's conductivities
   return FVS_OK;
 }
 
@@ -1593,12 +1594,10 @@ fvs_status solver_step(fvs_solver s, double dt, fvs_step_stats* stats) {
     J.dextra = s->edx;
     J.dinv = s->jinv_e;
     // FVS_ENERGY_LINES: 1 and 0 force the line preconditioner on and off;
-    // otherwise decided per operator and time step from the first pass's
-    // diagonal (LinePrecond::worth)
+    // otherwise decided from the first pass's diagonal (LinePrecond::worth)
     const char* el = getenv("FVS_ENERGY_LINES");
     bool lines = el && *el == '1';
     const bool decide = !(el && (*el == '0' || *el == '1'));
-    if (decide && s->eline_dt == dt) lines = s->eline_use;
     // Tnew / fsnew hold the iterate m; Tlin the linear solution
     DBuf<double>& Tm = s->Tnew;
     DBuf<double>& fsm = s->fsnew;
@@ -1614,11 +1613,7 @@ fvs_status solver_step(fvs_solver s, double dt, fvs_step_stats* stats) {
                                                           s->jinv_e);
       FVS_COUNT_LAUNCH();
       FVS_LAUNCH_CHECK();
-      if (it == 1 && decide && s->eline_dt != dt) {
-        FVS_TRY(LinePrecond::worth(st, s->red, s->Ke, s->edx, lines));
-        s->eline_use = lines;
-        s->eline_dt = dt;
-      }
+      if (it == 1 && decide) FVS_TRY(s->eline.worth(st, s->red, s->Ke, s->jinv_e, lines));
       if (it == 1 && lines) {
         if (!s->eline.ready || s->eline.built_from != s->Ke.col.p || s->eline.n != s->Ke.n || s->eline.w != s->Ke.w)
           FVS_TRY(s->eline.build(st, s->Ke));

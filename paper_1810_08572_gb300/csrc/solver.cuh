@@ -56,11 +56,10 @@ struct fvs_solver_s {
   // of the momentum system (per step)
   fvs::DBuf<double> jinv_e, jinv_m;
   // line preconditioner of the energy system, where it pays (else Jacobi):
-  // chains found once from the energy operator, factors per pass; the choice
-  // holds for one operator and time step
+  // chosen in every step, chains found once from the energy operator (with
+  // k(T) from that of the first step after a state was set that takes them),
+  // factors per pass
   fvs::LinePrecond eline;
-  bool eline_use = false;
-  double eline_dt = 0.0;      // the dt the choice was made for (0: none yet)
   double time = 0.0;
   int64_t nstep = 0;
 

@@ -566,3 +566,41 @@ def test_thin_cells_are_judged_by_the_tolerance_asked_for(fvs, monkeypatch, line
         assert st["status"] == 0, fvs.fvs_last_error()
     S.close()
     M.close()
+
+
+@pytest.mark.parametrize("jitter,k_table", [(0.2, None), (0.0, None), (0.2, [(600.0, 190.0), (833.0, 160.0), (913.0, 110.0)])])
+def test_a_solver_set_to_another_state_steps_as_a_fresh_one(fvs, monkeypatch, jitter, k_table):
+    """All melt these thin cells take the line preconditioner, all mushy
+    (latent heat on the diagonal) Jacobi.  A solver that has stepped one state
+    and is set to the other gives the bits, and takes the iterations, of a
+    solver made for it, in both directions and back."""
+    m = box_mesh(32, 33, 64, (0.1, 0.1, 0.0125), jitter=jitter, jitter_seed=31, permute_seed=32)
+    ijk = m["cell_ijk"]
+    waves = 3.0 * np.sin(0.1 * ijk[:, 2]) + 5.0 * np.cos(0.2 * ijk[:, 0])
+    states = {"melt": 950.0 + waves, "mushy": 870.0 + waves}
+    props = cases.props(no_flow=True, k_table=k_table, e_rtol=1e-13, e_tol_T=1e-10, max_krylov_iters=2000)
+    M = fvs.Mesh(m)
+
+    def steps(S, state):
+        S.set_state(states[state])
+        its = [S.step(5e-3)["e_lin_its"] for _ in range(2)]
+        return its, S.query("T"), S.query("FS")
+
+    def fresh(state):
+        S = fvs.Solver(M, props)
+        out = steps(S, state)
+        S.close()
+        return out
+
+    want = {k: fresh(k) for k in states}
+    S = fvs.Solver(M, props)
+    for state in ("melt", "mushy", "melt"):
+        its, T, FS = steps(S, state)
+        assert its == want[state][0], state
+        assert np.array_equal(T, want[state][1]) and np.array_equal(FS, want[state][2]), state
+    S.close()
+    # the two states lie on either side of the rule
+    monkeypatch.setenv("FVS_ENERGY_LINES", "0")
+    assert sum(want["melt"][0]) < 0.6 * sum(fresh("melt")[0])
+    assert want["mushy"][0] == fresh("mushy")[0]
+    M.close()
