@@ -497,6 +497,20 @@ fvs_status fvs_query_fields_noalloc(fvs_solver solver, fvs_field field, double* 
  * bandwidth. */
 fvs_status fvs_measure_fp64_fma(int64_t iters, double* gflops);
 
+/* The lines of the energy solve's line preconditioner for any operator, found
+ * on the GPU as a step finds them (not part of the method: for checking the
+ * layout).  col, val: host arrays, n rows of w slots (1..127), slot k of row
+ * i at k*n + i, unused slots the row itself with value 0.  sizes [4] receives
+ * the number of lines, of groups of 32 lines, of entries, and the longest
+ * line.  The arrays, if all are given and cap_groups and cap_padded suffice, receive
+ * goff [groups + 1] first entry of each group, llen [groups*32] length of each
+ * line, and per entry goff[g] + 32*position + lane (position < llen) cell, the
+ * row there, and sprev / snext, the slots of its neighbours along the line
+ * (-1: none). */
+fvs_status fvs_line_layout(const int32_t* col, const double* val, int64_t n, int32_t w, int64_t* sizes,
+                           int64_t cap_groups, int64_t cap_padded, int64_t* goff, int32_t* llen, int32_t* cell,
+                           int8_t* sprev, int8_t* snext);
+
 /* Current simulated time and step count. */
 fvs_status fvs_get_time(fvs_solver solver, double* time, int64_t* steps);
 

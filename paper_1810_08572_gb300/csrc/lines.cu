@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(64) k_line_solve(int64_t ngroups, const int64_
 
 // ---------------------------------------------------------------------------
 // the chains, on the device (build_line_layout in lines_host.h is the same
-// rule on the host, against which the layout is checked)
+// rule on the host; a test holds the two layouts against one another)
 // ---------------------------------------------------------------------------
 // two largest off-diagonal couplings of a row (the first slot wins a tie),
 // the second only if at least a quarter of the first, and the sum of all;
@@ -202,29 +202,55 @@ __global__ void k_line_walk(int64_t n2, const int2* __restrict__ in, int2* __res
     out[v] = make_int2(b.x, a.y + b.y);
   }
 }
+// The same walks with the smallest cell on the way (x: node, y: hops, z: cell).
+// After 2^rounds >= n hops a walk that has not ended has gone round a cycle,
+// and z is the cycle's smallest cell.
+__global__ void k_line_ring0(int64_t n, const int32_t* __restrict__ nb, int4* __restrict__ walk) {
+  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < 2 * n; v += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t i = (int32_t)(v >> 1), j = nb[v];
+    if (j < 0) walk[v] = make_int4((int32_t)v, 0, i, 0);
+    else walk[v] = make_int4(2 * j + (nb[2 * (int64_t)j] == i ? 1 : 0), 1, min(i, j), 0);
+  }
+}
+__global__ void k_line_ring(int64_t n2, const int4* __restrict__ in, int4* __restrict__ out) {
+  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n2; v += (int64_t)gridDim.x * blockDim.x) {
+    const int4 a = in[v], b = in[a.x];
+    out[v] = make_int4(b.x, a.y + b.y, min(a.z, b.z), 0);
+  }
+}
+// a cycle is cut at its smallest cell, whose second link goes (hops doubled in
+// every round where the walk has not ended; an ended one has fewer)
+__global__ void k_line_cut(int64_t n, const int4* __restrict__ walk, int hops, int32_t* __restrict__ nb) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int4 a = walk[2 * i];
+    if (a.y != hops || a.z != (int32_t)i) continue;
+    const int64_t q = nb[2 * i + 1];
+    nb[2 * i + 1] = -1;
+    nb[2 * q + (nb[2 * q] == (int32_t)i ? 0 : 1)] = -1;
+  }
+}
 // place of every cell: head cell of its chain (the end with the smaller id),
-// position, and at the head the number of lines the chain is cut into.  A
-// cell whose walks have not both ended (a cycle, or a chain longer than the
-// rounds reach, the same for all its cells) is a line of its own.
-constexpr int WALK_ROUNDS = 12, MAX_CHAIN = 1 << WALK_ROUNDS;
+// position, and at the head the number of lines the chain is cut into.  A cell
+// whose walks have not both ended flags open.
+constexpr int WALK_ROUNDS = 12;   // chains of up to 4,096 links
 __global__ void k_line_place(int64_t n, const int32_t* __restrict__ nb, const int2* __restrict__ walk, int max_line,
                              int32_t* __restrict__ head, int32_t* __restrict__ place, int32_t* __restrict__ len,
-                             int32_t* __restrict__ cnt) {
+                             int32_t* __restrict__ cnt, int32_t* __restrict__ open) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const int2 a = walk[2 * i], b = walk[2 * i + 1];
     int32_t h = (int32_t)i, p = 0, m = 1;
     int dir = 0;                 // link towards the head
-    if (nb[a.x] < 0 && nb[b.x] < 0 && a.y + b.y < MAX_CHAIN) {
+    if (nb[a.x] < 0 && nb[b.x] < 0) {
       const int32_t ea = a.x >> 1, eb = b.x >> 1;
       dir = ea <= eb ? 0 : 1;
       h = dir == 0 ? ea : eb;
       p = dir == 0 ? a.y : b.y;
       m = a.y + b.y + 1;
     } else {
-      dir = 2;                   // off the chains
+      *open = 1;
     }
     head[i] = h;
-    place[i] = p * 4 + dir;
+    place[i] = p * 2 + dir;
     len[i] = m;
     cnt[i] = p == 0 ? (m + max_line - 1) / max_line : 0;
   }
@@ -234,7 +260,7 @@ __global__ void k_line_lengths(int64_t n, const int32_t* __restrict__ place, con
                                const int32_t* __restrict__ first, int max_line, int32_t* __restrict__ key,
                                int32_t* __restrict__ id) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    if (place[i] >> 2) continue;
+    if (place[i] >> 1) continue;
     const int m = len[i], nl = (m + max_line - 1) / max_line;
     for (int q = 0; q < nl; ++q) {
       key[first[i] + q] = max_line - min(max_line, m - q * max_line);
@@ -260,11 +286,11 @@ __global__ void k_line_fill(int64_t n, int w, const int32_t* __restrict__ col, c
                             const int32_t* __restrict__ llen, const int64_t* __restrict__ goff, int max_line,
                             int32_t* __restrict__ cell, int8_t* __restrict__ sprev, int8_t* __restrict__ snext) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int p = place[i] >> 2, dir = place[i] & 3, pos = p % max_line;
+    const int p = place[i] >> 1, dir = place[i] & 1, pos = p % max_line;
     const int32_t t = rank[first[head[i]] + p / max_line];
     const int64_t e = goff[t >> 5] + (int64_t)pos * 32 + (t & 31);
-    const int32_t jp = dir < 2 && pos > 0 ? nb[2 * i + dir] : -1;
-    const int32_t jn = dir < 2 && pos + 1 < llen[t] ? nb[2 * i + 1 - dir] : -1;
+    const int32_t jp = pos > 0 ? nb[2 * i + dir] : -1;
+    const int32_t jn = pos + 1 < llen[t] ? nb[2 * i + 1 - dir] : -1;
     int8_t sp = -1, sn = -1;
     for (int k = w - 1; k >= 0; --k) {
       const int32_t j = col[(int64_t)k * n + i];
@@ -351,24 +377,48 @@ fvs_status LinePrecond::build(cudaStream_t s, const Ell& Ain) {
   }
   FVS_TRY(head.alloc(n)); FVS_TRY(place.alloc(n)); FVS_TRY(len.alloc(n));
   FVS_TRY(cnt.alloc((size_t)n + 1)); FVS_TRY(first.alloc((size_t)n + 1));
-  {
+  ScanWork sw;
+  int32_t nl = 0, open = 0;
+  const int g2 = stride_grid(2 * n, 256);
+  // places of all cells, the number of lines, and whether a walk was too short
+  auto walk = [&](int rounds) -> fvs_status {
     DBuf<int2> wa, wb;
-    FVS_TRY(wa.alloc(2 * (size_t)n)); FVS_TRY(wb.alloc(2 * (size_t)n));
-    k_line_walk0<<<stride_grid(2 * n, 256), 256, 0, s>>>(n, nb, wa); FVS_COUNT_LAUNCH();
-    for (int q = 0; q < WALK_ROUNDS; ++q) {
-      k_line_walk<<<stride_grid(2 * n, 256), 256, 0, s>>>(2 * n, (q & 1) ? wb.p : wa.p, (q & 1) ? wa.p : wb.p);
+    DBuf<int32_t> op;
+    FVS_TRY(wa.alloc(2 * (size_t)n)); FVS_TRY(wb.alloc(2 * (size_t)n)); FVS_TRY(op.alloc(1));
+    k_line_walk0<<<g2, 256, 0, s>>>(n, nb, wa); FVS_COUNT_LAUNCH();
+    for (int q = 0; q < rounds; ++q) {
+      k_line_walk<<<g2, 256, 0, s>>>(2 * n, (q & 1) ? wb.p : wa.p, (q & 1) ? wa.p : wb.p);
       FVS_COUNT_LAUNCH();
     }
-    FVS_TRY(cnt.zero(s));
-    k_line_place<<<g, 256, 0, s>>>(n, nb, (WALK_ROUNDS & 1) ? wb.p : wa.p, kMaxLine, head, place, len, cnt);
+    FVS_TRY(cnt.zero(s)); FVS_TRY(op.zero(s));
+    k_line_place<<<g, 256, 0, s>>>(n, nb, (rounds & 1) ? wb.p : wa.p, kMaxLine, head, place, len, cnt, op);
     FVS_COUNT_LAUNCH();
     FVS_LAUNCH_CHECK();
+    FVS_TRY(exclusive_scan(s, sw, n + 1, cnt, first));
+    FVS_CUDA(cudaMemcpyAsync(&nl, first.p + n, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    FVS_CUDA(cudaMemcpyAsync(&open, op.p, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    FVS_CUDA(cudaStreamSynchronize(s));
+    return FVS_OK;
+  };
+  FVS_TRY(walk(WALK_ROUNDS));
+  if (open) {
+    // cycles, or chains of more links than the rounds reach: cut the cycles,
+    // then walk chains of any length
+    int rounds = 0;
+    while ((1LL << rounds) < n) ++rounds;   // (2^30 hops at most: n is bounded above)
+    {
+      DBuf<int4> wa, wb;
+      FVS_TRY(wa.alloc(2 * (size_t)n)); FVS_TRY(wb.alloc(2 * (size_t)n));
+      k_line_ring0<<<g2, 256, 0, s>>>(n, nb, wa); FVS_COUNT_LAUNCH();
+      for (int q = 0; q < rounds; ++q) {
+        k_line_ring<<<g2, 256, 0, s>>>(2 * n, (q & 1) ? wb.p : wa.p, (q & 1) ? wa.p : wb.p);
+        FVS_COUNT_LAUNCH();
+      }
+      k_line_cut<<<g, 256, 0, s>>>(n, (rounds & 1) ? wb.p : wa.p, 1 << rounds, nb); FVS_COUNT_LAUNCH();
+      FVS_LAUNCH_CHECK();
+    }
+    FVS_TRY(walk(rounds));
   }
-  ScanWork sw;
-  FVS_TRY(exclusive_scan(s, sw, n + 1, cnt, first));
-  int32_t nl = 0;
-  FVS_CUDA(cudaMemcpyAsync(&nl, first.p + n, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-  FVS_CUDA(cudaStreamSynchronize(s));
   nlines = nl;
   ngroups = (nl + 31) / 32;
   const int ng = (int)ngroups;
@@ -431,3 +481,47 @@ fvs_status LinePrecond::apply(cudaStream_t s, const double* r, double* z) {
 }
 
 }  // namespace fvs
+
+using namespace fvs;
+
+extern "C" __attribute__((visibility("default"))) fvs_status fvs_line_layout(
+    const int32_t* col, const double* val, int64_t n, int32_t w, int64_t* sizes, int64_t cap_groups,
+    int64_t cap_padded, int64_t* goff, int32_t* llen, int32_t* cell, int8_t* sprev, int8_t* snext) {
+  if (!col || !val || !sizes || n < 1 || w < 1 || w > 127 || n > INT32_MAX / 2 / w) {
+    set_error("fvs_line_layout: bad argument");
+    return FVS_ERR_ARG;
+  }
+  for (int64_t e = 0; e < n * w; ++e)
+    if (col[e] < 0 || col[e] >= n) {
+      set_error("fvs_line_layout: column %d outside the rows", (int)col[e]);
+      return FVS_ERR_ARG;
+    }
+  cudaStream_t st = nullptr;
+  FVS_CUDA(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
+  auto run = [&]() -> fvs_status {
+    AllocStream as(st);
+    Ell A;
+    LinePrecond P;
+    FVS_TRY(A.alloc(n, w));
+    FVS_CUDA(cudaMemcpyAsync(A.col.p, col, (size_t)n * w * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+    FVS_CUDA(cudaMemcpyAsync(A.val.p, val, (size_t)n * w * sizeof(double), cudaMemcpyHostToDevice, st));
+    FVS_TRY(P.build(st, A));
+    sizes[0] = P.nlines;
+    sizes[1] = P.ngroups;
+    sizes[2] = P.padded;
+    sizes[3] = P.max_len;
+    if (goff && llen && cell && sprev && snext && cap_groups >= P.ngroups && cap_padded >= P.padded) {
+      FVS_CUDA(cudaMemcpyAsync(goff, P.goff.p, (P.ngroups + 1) * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+      FVS_CUDA(cudaMemcpyAsync(llen, P.llen.p, P.ngroups * 32 * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+      FVS_CUDA(cudaMemcpyAsync(cell, P.cell.p, P.padded * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+      FVS_CUDA(cudaMemcpyAsync(sprev, P.sprev.p, P.padded, cudaMemcpyDeviceToHost, st));
+      FVS_CUDA(cudaMemcpyAsync(snext, P.snext.p, P.padded, cudaMemcpyDeviceToHost, st));
+    }
+    FVS_CUDA(cudaStreamSynchronize(st));
+    return FVS_OK;
+  };
+  const fvs_status r = run();
+  cudaStreamSynchronize(st);
+  cudaStreamDestroy(st);
+  return r;
+}
