@@ -1373,9 +1373,13 @@ FVS_API fvs_status fvs_surrogate_predict(fvs_surrogate s, const double* X, doubl
     FVS_TRY(upload_xt(s, X, nullptr, n));
     Xd = s->Xd.p;
   }
+  // tiles write their outputs while others still read their inputs: outputs that
+  // overlap the inputs go through an array of their own
+  const bool overlap = on_device && (const char*)Y < (const char*)(X + n * s->nin) &&
+                       (const char*)X < (const char*)(Y + n * s->nout);
   DBuf<double> out;
   double* Yd = Y;
-  if (!on_device) {
+  if (!on_device || overlap) {
     FVS_TRY(out.alloc((size_t)n * s->nout));
     Yd = out.p;
   }
@@ -1399,6 +1403,8 @@ FVS_API fvs_status fvs_surrogate_predict(fvs_surrogate s, const double* X, doubl
   }
   FVS_LAUNCH_CHECK();
   if (!on_device) FVS_CUDA(cudaMemcpyAsync(Y, Yd, n * s->nout * sizeof(double), cudaMemcpyDeviceToHost, s->stream));
+  else if (overlap)
+    FVS_CUDA(cudaMemcpyAsync(Y, Yd, n * s->nout * sizeof(double), cudaMemcpyDeviceToDevice, s->stream));
   FVS_CUDA(cudaStreamSynchronize(s->stream));
   return tc_check(s);
 }

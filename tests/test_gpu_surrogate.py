@@ -149,3 +149,23 @@ def test_surrogate_gain_over_plain_solves(fvs):
     S.predict(Xmc)
     sur_rate = len(Xmc) / (time.perf_counter() - t0)
     assert sur_rate > 1000 * plain_rate, (sur_rate, plain_rate)
+
+
+@pytest.mark.parametrize("widths,shift", [((3, 128, 4, 4), 0), ((3, 128, 4, 4), 1), ((4, 64, 2, 4), 0), ((4, 64, 2, 4), 5)])
+def test_outputs_may_overlap_the_inputs(fvs, widths, shift):
+    """Device inputs and outputs in one array, at its start, at its end, in
+    place and some values apart: the outputs are those of separate arrays."""
+    import torch
+    nin, hidden, layers, nout = widths
+    S = fvs.Surrogate(nin, hidden, layers, nout, seed=4)
+    n = 300001
+    X = torch.randn(n, nin, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(5))
+    want = torch.zeros(n, nout, dtype=torch.float64, device="cuda")
+    S.predict(X, out=want)
+    buf = torch.zeros(n * max(nin, nout) + shift, dtype=torch.float64, device="cuda")
+    at = len(buf) - n * nin if shift else 0
+    xin = buf[at:at + n * nin].view(n, nin)
+    xin.copy_(X)
+    out = buf[:n * nout].view(n, nout)
+    S.predict(xin, out=out)
+    assert torch.equal(out, want)
