@@ -511,6 +511,18 @@ fvs_status fvs_line_layout(const int32_t* col, const double* val, int64_t n, int
                            int64_t cap_groups, int64_t cap_padded, int64_t* goff, int32_t* llen, int32_t* cell,
                            int8_t* sprev, int8_t* snext);
 
+/* The dense inverse that the pressure hierarchy forms of its coarsest level, of
+ * any matrix (not part of the method: for checking it).  col, val: host
+ * arrays as for fvs_line_layout, n in 1..1000, w in 1..1000, every column at
+ * most once a row but for unused slots.  inverse [n*n] host: the inverse with the
+ * first row of every singular part (a connected part whose row sums vanish)
+ * replaced by the identity's, and the mean over each such part projected
+ * out on both sides.  by_columns: 1 if the block steps, which exchange rows
+ * inside a block of 16 only, were refused and the columns taken one by one.
+ * FVS_ERR_NOT_CONVERGED: no inverse (a zero pivot). */
+fvs_status fvs_dense_inverse(const int32_t* col, const double* val, int64_t n, int32_t w, double* inverse,
+                             int32_t* by_columns);
+
 /* Current simulated time and step count. */
 fvs_status fvs_get_time(fvs_solver solver, double* time, int64_t* steps);
 

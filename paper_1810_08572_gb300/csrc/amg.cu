@@ -2366,3 +2366,44 @@ fvs_status amg_coarsest_batched(cudaStream_t s, int n, int w, const int32_t* col
 }
 
 }  // namespace fvs
+
+using namespace fvs;
+
+extern "C" __attribute__((visibility("default"))) fvs_status fvs_dense_inverse(const int32_t* col, const double* val,
+                                                                                int64_t n, int32_t w, double* inverse,
+                                                                                int32_t* by_columns) {
+  if (!col || !val || !inverse || !by_columns || n < 1 || n > 1000 || w < 1 || w > 1000) {
+    set_error("fvs_dense_inverse: bad argument");
+    return FVS_ERR_ARG;
+  }
+  for (int64_t e = 0; e < n * w; ++e)
+    if (col[e] < 0 || col[e] >= n) {
+      set_error("fvs_dense_inverse: column %d outside the rows", (int)col[e]);
+      return FVS_ERR_ARG;
+    }
+  std::vector<double> diag((size_t)n, 0.0);
+  for (int64_t e = 0; e < n * w; ++e)
+    if (col[e] == (int32_t)(e % n)) diag[e % n] += val[e];
+  cudaStream_t st = nullptr;
+  FVS_CUDA(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
+  auto run = [&]() -> fvs_status {
+    AllocStream as(st);
+    Ell A;
+    Amg M;
+    FVS_TRY(A.alloc(n, w));
+    FVS_CUDA(cudaMemcpyAsync(A.col.p, col, (size_t)n * w * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+    FVS_CUDA(cudaMemcpyAsync(A.val.p, val, (size_t)n * w * sizeof(double), cudaMemcpyHostToDevice, st));
+    FVS_CUDA(cudaMemcpyAsync(A.diag.p, diag.data(), (size_t)n * sizeof(double), cudaMemcpyHostToDevice, st));
+    M.opt.coarsest = 1000;   // one level, the coarsest
+    M.opt.max_levels = 1;
+    FVS_TRY(M.setup(st, A));
+    FVS_CUDA(cudaMemcpyAsync(inverse, M.Ainv.p, (size_t)n * n * sizeof(double), cudaMemcpyDeviceToHost, st));
+    FVS_CUDA(cudaStreamSynchronize(st));
+    *by_columns = M.gj_perm.p ? 1 : 0;
+    return FVS_OK;
+  };
+  const fvs_status r = run();
+  cudaStreamSynchronize(st);
+  cudaStreamDestroy(st);
+  return r;
+}

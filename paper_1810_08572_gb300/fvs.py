@@ -131,6 +131,7 @@ _SIGS = {
                       _P, _P], C.c_int),
     "fvs_profile_read": ([_P, C.POINTER(fvs_kernel_time), C.c_int32, C.POINTER(C.c_int32)], C.c_int),
     "fvs_line_layout": ([_P, _P, C.c_int64, C.c_int32, _P, C.c_int64, C.c_int64, _P, _P, _P, _P, _P], C.c_int),
+    "fvs_dense_inverse": ([_P, _P, C.c_int64, C.c_int32, _P, C.POINTER(C.c_int32)], C.c_int),
     "fvs_measure_fp64_fma": ([C.c_int64, C.POINTER(C.c_double)], C.c_int),
     "fvs_pce_create": ([C.c_int32, _P, _P, _P, C.c_int32, C.c_int32, _P, C.POINTER(_P)], C.c_int),
     "fvs_pce_destroy": ([_P], C.c_int),
