@@ -2180,12 +2180,15 @@ fvs_status Amg::vcycle_t(cudaStream_t s, int l, const T* b, Y* y, bool x0_ready)
   const double vb = (double)sizeof(T);
   // kernel timing: every level is credited to the hierarchy's fine operator,
   // coarse levels under their own class names; algorithmic bytes from the
-  // entries a sweep reads (value + column per entry) and its vectors
+  // entries a sweep reads (value + column per entry; k_fine six a row, the
+  // diagonal, of which the residual reads the value, counts as a vector) and
+  // its vectors
   const void* pkey = lv[0]->A;
   const bool cl = l > 0;
-  const double ent = L->stored > 0.0 ? L->stored : (double)n * A.w;
+  const bool fine7 = l == 0 && diag_first;
+  const double ent = fine7 ? 6.0 * (double)n : (L->stored > 0.0 ? L->stored : (double)n * A.w);
   const double jac_bytes = (4.0 + vb) * ent + 4.0 * vb * (double)n;
-  const double res_bytes = (4.0 + vb) * ent + 3.0 * vb * (double)n;
+  const double res_bytes = (4.0 + vb) * ent + (fine7 ? 4.0 : 3.0) * vb * (double)n;
   const int32_t* rl = L->rlen.n ? L->rlen.p : nullptr;   // coarse levels: stored row lengths
   const int g = stride_grid(n, 256);
   const char* n_jac0 = f32 ? (cl ? "jacobi0_f32_coarse" : "jacobi0_f32") : (cl ? "jacobi0_coarse" : "jacobi0");
@@ -2196,7 +2199,6 @@ fvs_status Amg::vcycle_t(cudaStream_t s, int l, const T* b, Y* y, bool x0_ready)
   const double* wl = weights.p + (size_t)l * 2 * sweep_steps();   // this level's sweep weights
   // the fine level of the face-coupling operator has its own kernel, which
   // leaves a matrix that fits in the L2 cache
-  const bool fine7 = l == 0 && diag_first;
   // FP64: a block for every 256 rows, no stride: at 44 to 48 registers five
   // blocks fit an SM, so a stride grid of eight an SM ends in a wave 3/5 full
   // (128^3, three steps 155.8 -> 154.1 ms; AMG-CG on 442,368 rows 6.67 ->
@@ -2224,7 +2226,7 @@ fvs_status Amg::vcycle_t(cudaStream_t s, int l, const T* b, Y* y, bool x0_ready)
   auto cheb_step = [&](T* xin, const T* xprev, auto* xout, int k) {   // step k of the recurrence
     using O = std::remove_pointer_t<decltype(xout)>;
     const double* ab = wl + 2 * k;
-    ProfScope ps(pkey, n_jac, jac_bytes + vb * (double)n, s);
+    ProfScope ps(pkey, n_jac, jac_bytes + (xprev ? vb * (double)n : 0.0), s);
     if (fine7) fine([&](auto cs) {
       k_fine<T, O, FINE_CHEB, decltype(cs)::value><<<gf, 256, 0, s>>>(n, A.col, val, ab, dinv, b, xin, xprev, xout);
     });

@@ -604,3 +604,31 @@ def test_a_solver_set_to_another_state_steps_as_a_fresh_one(fvs, monkeypatch, ji
     assert sum(want["melt"][0]) < 0.6 * sum(fresh("melt")[0])
     assert want["mushy"][0] == fresh("mushy")[0]
     M.close()
+
+
+@pytest.mark.parametrize("jitter,precision", [(0.2, 0), (0.2, 1), (0.0, 0)])
+def test_bytes_credited_to_the_fine_level(fvs, jitter, precision):
+    """The timed fine-level sweeps are credited with what a row reads and
+    writes: six values and columns, and b, x, the (inverse) diagonal and the
+    result, the Chebyshev sweep from a previous iterate also that one.  A V(1,2)
+    cycle has one sweep of each kind after the coarse correction, a V(2,2) cycle a
+    Chebyshev sweep from zero before it as well."""
+    m = box_mesh(20, 18, 6, cases.CAVITY, jitter=jitter, jitter_seed=51, permute_seed=52)
+    M = fvs.Mesh(m)
+    S = fvs.Solver(M, cases.props(precision=precision, **TIGHT))
+    S.profile(True)
+    S.set_state(np.full(M.n_cells, 950.0), np.random.default_rng(13).normal(scale=2e-3, size=(M.n_cells, 3)))
+    st = S.step(1e-3)
+    assert st["amg_levels"] > 1
+    f32 = "_f32" if precision else ""
+    v = 4 if precision else 8
+    got = {r["name"]: r for r in S.profile_read()}
+    res, jac = got[("residual_f32" if precision else "residual_vc") + "@pressure"], got["jacobi" + f32 + "@pressure"]
+    cheb = 5 if jitter else 4.5          # mean over the Chebyshev sweeps of a cycle
+    n_cheb = 1 if jitter else 2
+    assert res["bytes"] == res["launches"] * M.n_cells * (6 * (4 + v) + 4 * v)
+    assert jac["launches"] == res["launches"] * (1 + n_cheb)
+    per_cycle = 6 * (4 + v) * (1 + n_cheb) + 4 * v + n_cheb * cheb * v
+    assert jac["bytes"] == res["launches"] * M.n_cells * per_cycle
+    S.close()
+    M.close()
