@@ -354,7 +354,6 @@ __global__ void kb_bicg_xr(int64_t n, int Sp, double* sc, uint8_t* act, const do
   if (!go) return;
   const double rr = v[0], rho_old = sc[B_RHO * Sp + s], rho = v[1];
   sc[B_RR * Sp + s] = rr;
-  sc[B_RHO_OLD * Sp + s] = rho_old;
   sc[B_RHO * Sp + s] = rho;
   sc[B_BETA * Sp + s] = bsdiv(rho, rho_old) * bsdiv(alpha, omega);
   sc[B_FIRST * Sp + s] = 0.0;
@@ -441,7 +440,6 @@ __global__ void kb_cg_z(int64_t n, int Sp, const double* __restrict__ r, const Z
       rz -= m * v[2 + 2 * k];
     }
   const double rz_old = sc[B_RZ * Sp + s];
-  sc[B_RZ_OLD * Sp + s] = rz_old;
   sc[B_RZ * Sp + s] = rz;
   sc[B_BETA * Sp + s] = bsdiv(rz, rz_old);
 }

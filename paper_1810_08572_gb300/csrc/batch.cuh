@@ -24,7 +24,7 @@ constexpr int BATCH_NCM = 8;   // liquid pockets per sample handled by the null-
 
 // per-sample scalar slots of the batched Krylov drivers: sc[slot * Sp + s]
 enum BSlot {
-  B_RHO = 0, B_RHO_OLD, B_ALPHA, B_OMEGA, B_RV, B_TS, B_TT, B_RR, B_BB, B_RZ, B_RZ_OLD, B_PQ, B_TOL2, B_BETA,
+  B_RHO = 0, B_ALPHA, B_OMEGA, B_RV, B_TS, B_TT, B_RR, B_BB, B_RZ, B_PQ, B_TOL2, B_BETA,
   B_FIRST, B_T0, B_T1, B_T2, B_NSLOT
 };
 

@@ -192,7 +192,6 @@ __device__ __forceinline__ bool finish2(double x, double y, double* part, unsign
   } else if (MODE == FIN_RR_RHO) {
     const double rho = sc[S_RHO];
     sc[S_RR] = x;
-    sc[S_RHO_OLD] = rho;
     sc[S_RHO] = y;
     sc[S_BETA] = sdiv(y, rho) * sdiv(sc[S_ALPHA], sc[S_OMEGA]);
     sc[S_FIRST] = 0.0;
@@ -330,7 +329,7 @@ __global__ void __launch_bounds__(RB) k_cg_xr_dot(int64_t n, double* __restrict_
   }
   if (finish2<FIN_RR>(a, 0.0, part, ticket, sc)) loop_next(ctl, sc, true);
 }
-// CG: sums r.z (rz moved to rz_old); with a mean to project out of z also the
+// CG: sums r.z and forms beta with the one before; with a mean to project out of z also the
 // mean of z over its rows, which k_cg_p subtracts as it reads z, and the sum
 // of r over them (zero but for rounding, which counts near the attainable
 // residual): r.z of the projected z is r.z - mean sum(r)
@@ -357,7 +356,6 @@ __global__ void __launch_bounds__(RB) k_dot_rz(int64_t n, const double* __restri
     rz -= mean * v[MEAN ? 2 : 0];
   }
   const double old = sc[S_RZ];
-  sc[S_RZ_OLD] = old;
   sc[S_RZ] = rz;
   sc[S_BETA] = sdiv(rz, old);
 }

@@ -31,7 +31,7 @@ struct Ell {
 
 // Scalar slots of the Krylov drivers (device memory).
 enum Slot {
-  S_RHO = 0, S_RHO_OLD, S_ALPHA, S_OMEGA, S_RV, S_TS, S_TT, S_RR, S_BB, S_RZ, S_RZ_OLD, S_PQ,
+  S_RHO = 0, S_ALPHA, S_OMEGA, S_RV, S_TS, S_TT, S_RR, S_BB, S_RZ, S_PQ,
   S_TMP0, S_TMP1, S_TOL2, S_ITER, S_FIRST, S_BETA, S_MEAN, S_START, S_TRUE, S_NSLOT
 };
 
