@@ -201,6 +201,7 @@ struct LinePrecond : Precond {
   static constexpr double GAIN_WIDE = 3.0, GAIN_FACE = 4.0;
   fvs_status worth(cudaStream_t s, Reducer& red, const Ell& A, const double* dinv, bool& use);
   fvs_status build(cudaStream_t s, const Ell& A);
+  void drop();     // gives all its memory back
   fvs_status factor(cudaStream_t s);
   fvs_status apply(cudaStream_t s, const double* r, double* z) override;
   uint64_t signature() const override {

@@ -461,6 +461,16 @@ fvs_status LinePrecond::build(cudaStream_t s, const Ell& Ain) {
   return FVS_OK;
 }
 
+void LinePrecond::drop() {
+  ready = weighed = false;
+  goff.release();
+  llen.release();
+  cell.release();
+  sprev.release();
+  snext.release();
+  for (DBuf<double>* b : {&lo, &inv, &cp, &yl, &off, &rest}) b->release();
+}
+
 fvs_status LinePrecond::factor(cudaStream_t s) {
   if (!ready || n <= 0) return FVS_OK;
   const int64_t threads = ngroups * 32;

@@ -1613,10 +1613,20 @@ fvs_status solver_step(fvs_solver s, double dt, fvs_step_stats* stats) {
                                                           s->jinv_e);
       FVS_COUNT_LAUNCH();
       FVS_LAUNCH_CHECK();
-      if (it == 1 && decide) FVS_TRY(s->eline.worth(st, s->red, s->Ke, s->jinv_e, lines));
-      if (it == 1 && lines) {
-        if (!s->eline.ready || s->eline.built_from != s->Ke.col.p || s->eline.n != s->Ke.n || s->eline.w != s->Ke.w)
-          FVS_TRY(s->eline.build(st, s->Ke));
+      if (it == 1) {
+        fvs_status r = decide ? s->eline.worth(st, s->red, s->Ke, s->jinv_e, lines) : FVS_OK;
+        if (r == FVS_OK && lines && (!s->eline.ready || s->eline.built_from != s->Ke.col.p ||
+                                     s->eline.n != s->Ke.n || s->eline.w != s->Ke.w))
+          r = s->eline.build(st, s->Ke);
+        if (r == FVS_ERR_NOMEM && decide) {
+          // the lines need some 150 bytes a cell while their chains are found:
+          // without them the step still runs
+          cudaGetLastError();
+          s->eline.drop();
+          lines = false;
+          r = FVS_OK;
+        }
+        FVS_TRY(r);
         s->eline.dextra = s->edx;
       }
       Precond& PE = lines ? static_cast<Precond&>(s->eline) : static_cast<Precond&>(J);

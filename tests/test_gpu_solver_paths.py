@@ -632,3 +632,64 @@ def test_bytes_credited_to_the_fine_level(fvs, jitter, precision):
     assert jac["bytes"] == res["launches"] * M.n_cells * per_cycle
     S.close()
     M.close()
+
+
+def test_a_step_without_memory_for_lines_takes_jacobi(fvs):
+    """With the device memory taken but for a few MB, a state that would take the
+    line preconditioner steps all the same (with Jacobi's iterations), and takes
+    it once there is memory again."""
+    import ctypes
+    import torch
+    props = cases.props(no_flow=True, **TIGHT)
+
+    def state(m, base):
+        ijk = m["cell_ijk"]
+        return base + 3.0 * np.sin(0.1 * ijk[:, 2]) + 5.0 * np.cos(0.2 * ijk[:, 0])
+
+    # every kernel loaded before the memory is taken
+    m = box_mesh(32, 32, 64, (0.1, 0.1, 0.0125), permute_seed=32)
+    M = fvs.Mesh(m)
+    S = fvs.Solver(M, props)
+    S.set_state(state(m, 950.0))
+    S.step(5e-3)
+    S.close()
+    M.close()
+    m = box_mesh(64, 64, 256, (0.2, 0.2, 0.05), permute_seed=32)
+    M = fvs.Mesh(m)
+    S = fvs.Solver(M, props)
+    # (device arrays: setting the state needs no memory of its own)
+    mushy, melt = (torch.from_numpy(state(m, T)).cuda() for T in (870.0, 950.0))
+    S.set_state(mushy)
+    S.step(5e-3)
+    torch.cuda.synchronize()
+    # all of the device memory, also what the library's pool keeps, but 24 MB
+    cu = ctypes.CDLL("libcuda.so.1")
+    taken = []
+
+    def take(size):
+        p = ctypes.c_uint64()
+        ok = cu.cuMemAllocAsync(ctypes.byref(p), ctypes.c_size_t(size), None) == 0
+        if ok:
+            taken.append(p)
+        return ok
+
+    assert take(24 << 20)
+    try:
+        size = 1 << 38
+        while size >= 1 << 21:
+            if not take(size):
+                size >>= 1
+        cu.cuMemFreeAsync(taken.pop(0), None)
+        torch.cuda.synchronize()
+        S.set_state(melt)
+        tight = S.step(5e-3)
+    finally:
+        for p in taken:
+            cu.cuMemFreeAsync(p, None)
+        torch.cuda.synchronize()
+    S.set_state(melt)
+    roomy = S.step(5e-3)
+    assert tight["status"] == 0 and roomy["status"] == 0
+    assert roomy["e_lin_its"] < 0.6 * tight["e_lin_its"]
+    S.close()
+    M.close()
