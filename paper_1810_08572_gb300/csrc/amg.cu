@@ -886,19 +886,31 @@ __global__ void k_dense_fold_cols(int n, double* M, const int32_t* lab, const ui
 // faster than the global-memory version above.
 static constexpr int SMEM_COARSEST = 160;
 
+__host__ __device__ static inline size_t coarsest_smem_bytes(int n) {
+  return (size_t)n * n * sizeof(double) + 2 * (size_t)n * sizeof(double) + 3 * (size_t)n * sizeof(int);
+}
+// drop: a part of the pattern may hold several null vectors (two liquid regions
+// that touch along an edge are coupled by cross terms that cancel), of which
+// the pin removes one.  A column whose best pivot is rounding next to its
+// diagonal entry is then left out, row and column zero in the inverse,
+// where its quotients (1e15 times the others) would be the preconditioner;
+// without drop such a column is taken as it is, and a zero one refused.
+constexpr double PIVOT_NOISE = 1e-12;
 __global__ void __launch_bounds__(1024) k_coarsest_smem(int n, int w, const int32_t* col, const double* val,
                                                         double* Ainv, int32_t* lab, uint8_t* sing,
-                                                        int* ncomp_out, int* err, int vs) {
+                                                        int* ncomp_out, int* err, int vs, int drop) {
   // one block per sample s = blockIdx.x; values and outputs of sample s sit
   // at stride vs (vs = 1, one block: a single system)
   const int smp = blockIdx.x;
   extern __shared__ double smem[];
   double* M = smem;                          // [n*n] in-place inverse
   double* fac = M + n * n;                   // [n]
-  int* perm = (int*)(fac + n);               // [n] row swaps
+  double* big = fac + n;                     // [n] diagonal (drop)
+  int* perm = (int*)(big + n);               // [n] row swaps
   int* lb = perm + n;                        // [n] labels
   int* order = lb + n;                       // [n] rows grouped by part
   __shared__ int piv, ncs;
+  __shared__ bool leave;
   __shared__ double pval;
   __shared__ uint8_t sg[SMEM_COARSEST];
   for (int e = threadIdx.x; e < n * n; e += blockDim.x) M[e] = 0.0;
@@ -945,15 +957,16 @@ __global__ void __launch_bounds__(1024) k_coarsest_smem(int n, int w, const int3
     for (int i = 0; i < n; ++i) lb[i] = perm[lb[i]];
     for (int c = 0; c < nc; ++c) {
       double rs = 0.0, sc = 0.0;
-      int first = -1;
+      int first = -1, rows = 0;
       for (int i = 0; i < n; ++i) {
         if (lb[i] != c) continue;
         if (first < 0) first = i;
+        ++rows;
         rs += fac[i];
         sc += fabs(M[i * n + i]);
       }
       const bool sgl = fabs(rs) <= 1e-9 * sc;
-      sg[c] = sgl ? 1 : 0;
+      sg[c] = sgl ? (rows > 1 ? 1 : 2) : 0;
       if (sgl) {
         for (int j = 0; j < n; ++j) M[first * n + j] = 0.0;
         M[first * n + first] = 1.0;
@@ -967,6 +980,10 @@ __global__ void __launch_bounds__(1024) k_coarsest_smem(int n, int w, const int3
     ncomp_out[smp] = nc;
   }
   __syncthreads();
+  if (drop) {
+    for (int j = threadIdx.x; j < n; j += blockDim.x) big[j] = fabs(M[j * n + j]);
+    __syncthreads();
+  }
   // in-place Gauss-Jordan with partial (row) pivoting; the pivot search is
   // one warp's, the update a 32 x 32 tiling of the matrix
   for (int k = 0; k < n; ++k) {
@@ -987,9 +1004,19 @@ __global__ void __launch_bounds__(1024) k_coarsest_smem(int n, int w, const int3
         piv = p;
         perm[k] = p;
         pval = best;
+        leave = drop && best >= 0.0 && best <= PIVOT_NOISE * big[k];
       }
     }
     __syncthreads();
+    if (leave) {
+      for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        M[k * n + j] = 0.0;
+        M[j * n + k] = 0.0;
+      }
+      if (threadIdx.x == 0) perm[k] = k;
+      __syncthreads();
+      continue;
+    }
     if (!(pval > 1e-300)) {
       if (threadIdx.x == 0) atomicOr(err, 8);
       return;
@@ -1868,19 +1895,18 @@ fvs_status Amg::coarsest_setup(cudaStream_t s) {
   FVS_TRY(err.zero(s));
   if (nc > 0) {
     if (nc <= SMEM_COARSEST) {
-      const size_t sh = (size_t)nc * nc * sizeof(double) + (size_t)nc * sizeof(double) + 3 * (size_t)nc * sizeof(int);
+      const size_t sh = coarsest_smem_bytes(nc);
       // the attribute is per function, shared by every thread: set it once to
       // the largest size any launch uses (concurrent solvers launch smaller ones)
       static bool attr_set[64] = {false};
       int dev = 0;
       cudaGetDevice(&dev);
       if (dev >= 0 && dev < 64 && !attr_set[dev]) {
-        const size_t shmax = (size_t)SMEM_COARSEST * SMEM_COARSEST * sizeof(double) +
-                             (size_t)SMEM_COARSEST * sizeof(double) + 3 * (size_t)SMEM_COARSEST * sizeof(int);
+        const size_t shmax = coarsest_smem_bytes(SMEM_COARSEST);
         FVS_CUDA(cudaFuncSetAttribute(k_coarsest_smem, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shmax));
         attr_set[dev] = true;
       }
-      k_coarsest_smem<<<1, 1024, sh, s>>>(nc, A.w, A.col, A.val, Ainv, clab, csing, ncd, err, 1);
+      k_coarsest_smem<<<1, 1024, sh, s>>>(nc, A.w, A.col, A.val, Ainv, clab, csing, ncd, err, 1, 0);
       FVS_COUNT_LAUNCH();
     } else {
       FVS_TRY(gj_tmp.alloc((size_t)nc * nc + 1)); FVS_TRY(gj_fac.alloc(nc));
@@ -2355,13 +2381,12 @@ fvs_status amg_coarsest_batched(cudaStream_t s, int n, int w, const int32_t* col
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev >= 0 && dev < 64 && !attr_set[dev]) {
-    const size_t shmax = (size_t)SMEM_COARSEST * SMEM_COARSEST * sizeof(double) +
-                         (size_t)SMEM_COARSEST * sizeof(double) + 3 * (size_t)SMEM_COARSEST * sizeof(int);
+    const size_t shmax = coarsest_smem_bytes(SMEM_COARSEST);
     FVS_CUDA(cudaFuncSetAttribute(k_coarsest_smem, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shmax));
     attr_set[dev] = true;
   }
-  const size_t sh = (size_t)n * n * sizeof(double) + (size_t)n * sizeof(double) + 3 * (size_t)n * sizeof(int);
-  k_coarsest_smem<<<Sp, 1024, sh, s>>>(n, w, col, val, Ainv, lab, sing, ncomp, err, Sp);
+  const size_t sh = coarsest_smem_bytes(n);
+  k_coarsest_smem<<<Sp, 1024, sh, s>>>(n, w, col, val, Ainv, lab, sing, ncomp, err, Sp, 1);
   FVS_COUNT_LAUNCH();
   FVS_LAUNCH_CHECK();
   return FVS_OK;

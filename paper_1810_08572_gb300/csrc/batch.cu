@@ -591,30 +591,42 @@ __global__ void kb_to_double(int64_t n, const float* a, double* b) {
 
 // ---------------------------------------------------------------------------
 // per-sample Galerkin values on the shared aggregation: coarse entry q gets
-// the sum of the listed fine entries (rows of cells without pressure left out)
+// the sum of the listed fine entries (rows of cells without pressure left out).
+// A sum that is rounding next to its entries is zero: the diagonal of an
+// aggregate that holds a whole liquid pocket of a sample (the aggregates are
+// those of the all-liquid operator) would else be inverted as 1e15 times the
+// others, and its part counted as regular.
 // ---------------------------------------------------------------------------
+constexpr double GAL_NOISE = 1e-12;
+__device__ __forceinline__ double gal_sum(double a, double m) { return fabs(a) <= GAL_NOISE * m ? 0.0 : a; }
 __global__ void kb_galerkin0(int64_t nq, int64_t n, int w, int Sp, const int32_t* gptr, const int32_t* gidx,
                              const double* base, const int32_t* ovr, const double* mval, double* cval) {
   BSAMPLE;
   BROW(q, nq) {
-    double a = 0.0;
+    double a = 0.0, m = 0.0;
     for (int32_t t = gptr[q]; t < gptr[q + 1]; ++t) {
       const int32_t e = gidx[t];
       const int32_t k = (int32_t)(e / n), i = (int32_t)(e - (int64_t)k * n);
       const int32_t o = ovr[(int64_t)i * Sp + s];
       if (o == -2) continue;
-      a += o < 0 ? base[e] : mval[(int64_t)o * w + k];
+      const double v = o < 0 ? base[e] : mval[(int64_t)o * w + k];
+      a += v;
+      m += fabs(v);
     }
-    cval[q * Sp + s] = a;
+    cval[q * Sp + s] = gal_sum(a, m);
   }
 }
 __global__ void kb_galerkin(int64_t nq, int Sp, const int32_t* gptr, const int32_t* gidx, const double* val,
                             double* cval) {
   BSAMPLE;
   BROW(q, nq) {
-    double a = 0.0;
-    for (int32_t t = gptr[q]; t < gptr[q + 1]; ++t) a += val[(int64_t)gidx[t] * Sp + s];
-    cval[q * Sp + s] = a;
+    double a = 0.0, m = 0.0;
+    for (int32_t t = gptr[q]; t < gptr[q + 1]; ++t) {
+      const double v = val[(int64_t)gidx[t] * Sp + s];
+      a += v;
+      m += fabs(v);
+    }
+    cval[q * Sp + s] = gal_sum(a, m);
   }
 }
 __global__ void kb_coarse_dinv(int64_t n, int Sp, const int32_t* dslot, const double* val, double* dinv) {
@@ -646,26 +658,26 @@ __global__ void kb_part_count(int64_t n, int Sp, int nc, const int32_t* lab, int
   }
 }
 // compact ids of the singular parts that hold fine rows (at most BATCH_NCM per
-// sample), their number and 1 / rows of each, [k][Sp]
+// sample), their number and 1 / rows of each, [k][Sp]; parts of one coarse row
+// (pockets inside one aggregate, a few cells) as far as there is room
 __global__ void kb_part_ids(int Sp, int nc, const int* count, const uint8_t* sing, const int* ncomp, int32_t* cid,
                             double* cinv, int* nparts, int* err) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= Sp) return;
   int k = 0;
   for (int c = 0; c < BATCH_NCM; ++c) cinv[c * Sp + s] = 0.0;
-  for (int c = 0; c < nc; ++c) {
-    int32_t id = -1;
-    if (c < ncomp[s] && sing[(int64_t)c * Sp + s] && count[(int64_t)s * nc + c] > 0) {
+  for (int c = 0; c < nc; ++c) cid[(int64_t)s * nc + c] = -1;
+  for (int kind = 1; kind <= 2; ++kind)
+    for (int c = 0; c < nc && c < ncomp[s]; ++c) {
+      if (sing[(int64_t)c * Sp + s] != kind || count[(int64_t)s * nc + c] == 0) continue;
       if (k < BATCH_NCM) {
-        id = k;
+        cid[(int64_t)s * nc + c] = k;
         cinv[k * Sp + s] = 1.0 / (double)count[(int64_t)s * nc + c];
         ++k;
-      } else {
+      } else if (kind == 1) {
         atomicOr(err, 16);
       }
     }
-    cid[(int64_t)s * nc + c] = id;
-  }
   nparts[s] = k;
 }
 // projected part of every (row, sample): index into the sample's parts, -1 none
