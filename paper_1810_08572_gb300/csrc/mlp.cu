@@ -481,7 +481,7 @@ __device__ __forceinline__ bool fu_bar_or(int g, bool bad) {
 }
 __global__ void __launch_bounds__(256 * FU_GROUPS, 1)
 k_mlp_predict_tc(int64_t n, FusedNet net, const bf16* __restrict__ wb, const float* __restrict__ w32,
-                 const double* __restrict__ X, double* __restrict__ Y, const float* __restrict__ mu_in,
+                 const double* __restrict__ X, const bf16* __restrict__ Hin, double* __restrict__ Y, const float* __restrict__ mu_in,
                  const float* __restrict__ sd_in, const float* __restrict__ mu_out,
                  const float* __restrict__ sd_out, int* err) {
   extern __shared__ __align__(1024) unsigned char tc_dyn[];
@@ -513,8 +513,11 @@ k_mlp_predict_tc(int64_t n, FusedNet net, const bf16* __restrict__ wb, const flo
        tile += (int64_t)gridDim.x * groups) {
     for (int t = tid; t < 128 * nch0; t += 256) {
       const int ch = t % nch0, r = t / nch0;
-      *reinterpret_cast<uint4*>(act + fu_off(r, ch * 8, net.kd[0])) =
-          fu_input8(X, tile * 128 + r, n, net.nin, ch * 8, mu_in, sd_in);
+      const int64_t mr = tile * 128 + r;
+      uint4 h = make_uint4(0, 0, 0, 0);
+      if (!Hin) h = fu_input8(X, mr, n, net.nin, ch * 8, mu_in, sd_in);
+      else if (mr < n) h = *reinterpret_cast<const uint4*>(Hin + mr * net.kd[0] + ch * 8);
+      *reinterpret_cast<uint4*>(act + fu_off(r, ch * 8, net.kd[0])) = h;
     }
     const int64_t m = tile * 128 + row;
     for (int l = 0; l < net.L; ++l) {
@@ -933,6 +936,7 @@ struct fvs_surrogate_s {
   std::vector<DBuf<float>*> Z;  // pre-activations per layer output
   std::vector<DBuf<bf16>*> D;   // loss gradients per layer output
   DBuf<float> Y;
+  DBuf<bf16> Xn;                // normalised inputs of a prediction with many of them
   DBuf<double> part, lossv, Xd, Td;
   DBuf<int> tc_err;          // set by a tensor-core GEMM whose bounded wait ran out
   ~fvs_surrogate_s() {
@@ -1388,8 +1392,21 @@ FVS_API fvs_status fvs_surrogate_predict(fvs_surrogate s, const double* X, doubl
     FVS_TRY(fused_smem_attr());
     const int groups = fused_fits(net, 3) ? 3 : (fused_fits(net, 2) ? 2 : 1);
     const int grid = (int)std::min<int64_t>((n + 127) / 128, sm_count());
+    // More than 32 inputs are normalised beforehand, by the whole GPU: a tile's
+    // FP64 divisions (128 a column) on its own SM alone, two lanes a clock, are
+    // otherwise most of the call where there are few tiles.  128 inputs, 1000
+    // rows: 117 us in the tiles, 71 beforehand; 20,000 rows 196 and 149, 200,000
+    // (tiles enough for three groups an SM) 888 and 908.  40 inputs: 66 and 48,
+    // 96 and 82, 365 and 364 us.
+    const bool pre = s->nin > 32;
+    if (pre) {
+      FVS_TRY(s->Xn.alloc((size_t)n * s->kd[0]));
+      k_mlp_in<<<stride_grid(n * s->kd[0], 256), 256, 0, s->stream>>>(n, s->nin, s->kd[0], Xd, s->mu_in.p, s->sd_in.p,
+                                                                      s->Xn.p);
+      FVS_COUNT_LAUNCH();
+    }
     k_mlp_predict_tc<<<grid, 256 * groups, net.wbytes + groups * FU_ACT, s->stream>>>(
-        n, net, s->wb.p, s->w32.p, Xd, Yd, s->mu_in.p, s->sd_in.p, s->mu_out.p, s->sd_out.p, s->tc_err.p);
+        n, net, s->wb.p, s->w32.p, Xd, pre ? s->Xn.p : nullptr, Yd, s->mu_in.p, s->sd_in.p, s->mu_out.p, s->sd_out.p, s->tc_err.p);
     FVS_COUNT_LAUNCH();
   } else {
     FVS_TRY(sg_work(s, n + 16, false));

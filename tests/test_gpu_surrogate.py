@@ -169,3 +169,45 @@ def test_outputs_may_overlap_the_inputs(fvs, widths, shift):
     out = buf[:n * nout].view(n, nout)
     S.predict(xin, out=out)
     assert torch.equal(out, want)
+
+
+@pytest.mark.parametrize("n_in", [32, 33, 128])
+@pytest.mark.parametrize("n", [1, 128, 129, 3001])
+def test_prediction_of_many_inputs_matches_fp64_reference(fvs, n_in, n):
+    """Up to 32 inputs are normalised in the network's tiles, more beforehand
+    (full and ragged tiles): both within BF16 rounding of the FP64 forward pass
+    (the bound of the three-input network), host and device arrays alike."""
+    import torch
+    sizes = [n_in, 64, 64, 5]
+    S = fvs.Surrogate(n_in, 64, 2, 5, seed=6)
+    rng = np.random.default_rng(n_in + n)
+    mu, sd = rng.normal(size=n_in).astype(np.float32), rng.uniform(0.5, 2.0, n_in).astype(np.float32)
+    S.set_scaling(mu, sd, np.zeros(5), np.ones(5))
+    X = mu + sd * rng.normal(size=(n, n_in))
+    Yr, _ = ref.forward(ref.unflatten(S.get_params(), sizes), (X - mu) / sd)
+    Y = S.predict(X)
+    assert np.abs(Y - Yr).max() <= 3e-2 * np.abs(Yr).max()
+    Yd = torch.zeros(n, 5, dtype=torch.float64, device="cuda")
+    S.predict(torch.from_numpy(X).cuda(), out=Yd)
+    assert np.array_equal(Yd.cpu().numpy(), Y)
+
+
+def test_prediction_of_many_inputs_uses_the_whole_gpu(fvs):
+    """1000 rows of 128 inputs are eight tiles; their normalisation must not
+    run on eight SMs.  Against a network of three inputs and the same hidden
+    layers, the call takes about 1.4 times as long (2.7 times on eight SMs)."""
+    import torch
+
+    def best(n_in):
+        S = fvs.Surrogate(n_in, 16, 1, 1, seed=6)
+        X = torch.randn(1000, n_in, dtype=torch.float64, device="cuda")
+        Y = torch.zeros(1000, 1, dtype=torch.float64, device="cuda")
+        ts = []
+        for _ in range(50):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            S.predict(X, out=Y)
+            ts.append(time.perf_counter() - t0)
+        return min(ts[10:])
+
+    assert best(128) <= 2.2 * best(3)
