@@ -332,6 +332,8 @@ struct fvs_pce_s {
   int no_pad = 1;              // outputs padded to 1, 2, 4 or 8
   DBuf<PcePrefix> pref;
   DBuf<double> ecoef;          // [P*no_pad]
+  std::vector<PcePrefix> hpref;   // host sides of the two, read by copies in flight
+  std::vector<double> hcoef;
   bool fitted = false;
 };
 
@@ -489,7 +491,7 @@ FVS_API fvs_status fvs_pce_nodes(fvs_pce s, int32_t level, int32_t sparse, doubl
 
 namespace fvs {
 // prefixes, recurrence and coefficients of the evaluation from the fitted
-// coefficients c [P x nout]
+// coefficients c [P x nout] (queued; the caller waits for the stream)
 static fvs_status pce_prepare_eval(fvs_pce s, const std::vector<double>& c) {
   const int d = s->D.d, p = s->D.p, P = s->D.P, no = s->D.nout;
   PceEval& E = s->ev;
@@ -519,8 +521,10 @@ static fvs_status pce_prepare_eval(fvs_pce s, const std::vector<double>& c) {
                                         al + (size_t)(y + 1) * d);
   });
   s->no_pad = no <= 1 ? 1 : (no <= 2 ? 2 : (no <= 4 ? 4 : 8));
-  std::vector<double> e((size_t)P * s->no_pad, 0.0);
-  std::vector<PcePrefix> pre;
+  std::vector<double>& e = s->hcoef;
+  std::vector<PcePrefix>& pre = s->hpref;
+  e.assign((size_t)P * s->no_pad, 0.0);
+  pre.clear();
   for (int k = 0; k < P; ++k) {
     const int8_t* a = al + (size_t)at[k] * d;
     double f = 1.0;
@@ -539,7 +543,6 @@ static fvs_status pce_prepare_eval(fvs_pce s, const std::vector<double>& c) {
   FVS_TRY(s->ecoef.alloc(e.size()));
   FVS_CUDA(cudaMemcpyAsync(s->pref.p, pre.data(), pre.size() * sizeof(PcePrefix), cudaMemcpyHostToDevice, s->stream));
   FVS_CUDA(cudaMemcpyAsync(s->ecoef.p, e.data(), e.size() * sizeof(double), cudaMemcpyHostToDevice, s->stream));
-  FVS_CUDA(cudaStreamSynchronize(s->stream));   // the host arrays must outlive the copies
   return FVS_OK;
 }
 template <int NO>
@@ -590,16 +593,15 @@ FVS_API fvs_status fvs_pce_fit(fvs_pce s, const double* X, const double* Y, int6
   }
   FVS_LAUNCH_CHECK();
   int h = 0;
+  std::vector<double> hc((size_t)P * no);
   FVS_CUDA(cudaMemcpyAsync(&h, err.p, sizeof(int), cudaMemcpyDeviceToHost, st));
+  FVS_CUDA(cudaMemcpyAsync(hc.data(), R.p, hc.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
   FVS_CUDA(cudaStreamSynchronize(st));
   if (h) {
     set_error("fvs_pce_fit: the collocation points do not determine the %d coefficients", P);
     return FVS_ERR_ARG;
   }
   FVS_CUDA(cudaMemcpyAsync(s->coef.p, R.p, (size_t)P * no * sizeof(double), cudaMemcpyDeviceToDevice, st));
-  std::vector<double> hc((size_t)P * no);
-  FVS_CUDA(cudaMemcpyAsync(hc.data(), R.p, hc.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
-  FVS_CUDA(cudaStreamSynchronize(st));
   FVS_TRY(pce_prepare_eval(s, hc));
   s->fitted = true;
   if (rms_resid) {
