@@ -188,7 +188,10 @@ struct LinePrecond : Precond {
   // Whether the lines pay at the given inverse diagonal, which holds the state
   // (latent heat makes the rows of mushy cells several times as dominant): asked
   // in every step, so that a step depends on its state and not on the ones
-  // before it.  With a and b the mean shares of a row's diagonal
+  // before it (35 us), unless no state could take them at that step size: may()
+  // asks for the largest gain, without latent heat, from scale times an operator
+  // that does not depend on the state, and is asked once per operator and step
+  // size.  With a and b the mean shares of a row's diagonal
   // that Jacobi and the lines leave out, the iterations go down by about
   // sqrt((1 + a)(1 - b) / ((1 - a)(1 + b))), and an iteration costs about 1.4
   // (27-point rows) or twice (face-only rows) as much.  All melt on 128^3
@@ -199,6 +202,8 @@ struct LinePrecond : Precond {
   // substitution's serial walk costs more than the iterations it saves.
   static constexpr int64_t MIN_ROWS = 65536;
   static constexpr double GAIN_WIDE = 3.0, GAIN_FACE = 4.0;
+  static fvs_status may(cudaStream_t s, Reducer& red, const Ell& A, double scale, const double* rcp, const double* V,
+                        double idt, bool& use);
   fvs_status worth(cudaStream_t s, Reducer& red, const Ell& A, const double* dinv, bool& use);
   fvs_status build(cudaStream_t s, const Ell& A);
   void drop();     // gives all its memory back

@@ -314,6 +314,30 @@ __global__ void k_line_sums(int64_t n, int w, const int32_t* __restrict__ col, c
     rest[i] = o - m0 - m1;
   }
 }
+// the same over the rows' diagonals of the energy system without latent heat,
+// summed (an operator of w slots, times scale)
+__global__ void __launch_bounds__(RB) k_line_bound(int64_t n, int w, const int32_t* __restrict__ col,
+                                                   const double* __restrict__ val, const double* __restrict__ diag,
+                                                   double scale, const double* __restrict__ rcp,
+                                                   const double* __restrict__ V, double idt, double* part,
+                                                   unsigned int* ticket, double* sc, int s0, int s1) {
+  double x = 0.0, y = 0.0;
+  for (int64_t i = blockIdx.x * (int64_t)RB + threadIdx.x; i < n; i += (int64_t)gridDim.x * RB) {
+    int32_t b0, b1;
+    double m0, m1, o;
+    strongest2(n, w, col, val, i, b0, b1, m0, m1, o);
+    const double d = scale * fabs(diag[i]) + rcp[i] * V[i] * idt;
+    if (d > 0.0) {
+      const double q = scale / d;
+      x = fma(o, q, x);
+      y = fma(o - m0 - m1, q, y);
+    }
+  }
+  if (grid_fold<OpSum, 2>(x, y, part, ticket)) {
+    sc[s0] = x;
+    sc[s1] = y;
+  }
+}
 // both times the rows' inverse diagonals, summed (rows without a diagonal left out)
 __global__ void __launch_bounds__(RB) k_line_weight(int64_t n, const double* __restrict__ off,
                                                     const double* __restrict__ rest, const double* __restrict__ dinv,
@@ -334,6 +358,27 @@ __global__ void __launch_bounds__(RB) k_line_weight(int64_t n, const double* __r
 
 }  // namespace
 
+// from the sums in S_TMP0 and S_TMP1
+static fvs_status line_gain(cudaStream_t s, Reducer& red, int64_t n, int w, bool& use) {
+  FVS_TRY(red.fetch(s));
+  const double a = std::min(0.999, red.host[S_TMP0] / (double)n);
+  const double b = std::max(0.0, std::min(a, red.host[S_TMP1] / (double)n));
+  use = std::sqrt((1.0 + a) * (1.0 - b) / ((1.0 - a) * (1.0 + b))) >
+        (w > 7 ? LinePrecond::GAIN_WIDE : LinePrecond::GAIN_FACE);
+  return FVS_OK;
+}
+
+fvs_status LinePrecond::may(cudaStream_t s, Reducer& red, const Ell& Ain, double scale, const double* rcp,
+                            const double* V, double idt, bool& use) {
+  use = false;
+  if (Ain.n < MIN_ROWS || Ain.w < 3) return FVS_OK;
+  k_line_bound<<<red.grid(Ain.n), RB, 0, s>>>(Ain.n, Ain.w, Ain.col, Ain.val, Ain.diag, scale, rcp, V, idt, red.part,
+                                              red.ticket, red.sc, S_TMP0, S_TMP1);
+  FVS_COUNT_LAUNCH();
+  FVS_LAUNCH_CHECK();
+  return line_gain(s, red, Ain.n, Ain.w, use);
+}
+
 fvs_status LinePrecond::worth(cudaStream_t s, Reducer& red, const Ell& Ain, const double* dinv, bool& use) {
   use = false;
   if (Ain.n < MIN_ROWS || Ain.w < 3) return FVS_OK;
@@ -347,11 +392,7 @@ fvs_status LinePrecond::worth(cudaStream_t s, Reducer& red, const Ell& Ain, cons
   k_line_weight<<<red.vgrid(Ain.n), RB, 0, s>>>(Ain.n, off, rest, dinv, red.part, red.ticket, red.sc, S_TMP0, S_TMP1);
   FVS_COUNT_LAUNCH();
   FVS_LAUNCH_CHECK();
-  FVS_TRY(red.fetch(s));
-  const double a = std::min(0.999, red.host[S_TMP0] / (double)Ain.n);
-  const double b = std::max(0.0, std::min(a, red.host[S_TMP1] / (double)Ain.n));
-  use = std::sqrt((1.0 + a) * (1.0 - b) / ((1.0 - a) * (1.0 + b))) > (Ain.w > 7 ? GAIN_WIDE : GAIN_FACE);
-  return FVS_OK;
+  return line_gain(s, red, Ain.n, Ain.w, use);
 }
 
 fvs_status LinePrecond::build(cudaStream_t s, const Ell& Ain) {

@@ -479,6 +479,8 @@ __device__ __forceinline__ bool fu_bar_or(int g, bool bad) {
       : "memory");
   return any != 0;
 }
+// PRE: the inputs are there already, normalised (Hin, rows of kd[0])
+template <bool PRE>
 __global__ void __launch_bounds__(256 * FU_GROUPS, 1)
 k_mlp_predict_tc(int64_t n, FusedNet net, const bf16* __restrict__ wb, const float* __restrict__ w32,
                  const double* __restrict__ X, const bf16* __restrict__ Hin, double* __restrict__ Y, const float* __restrict__ mu_in,
@@ -513,11 +515,15 @@ k_mlp_predict_tc(int64_t n, FusedNet net, const bf16* __restrict__ wb, const flo
        tile += (int64_t)gridDim.x * groups) {
     for (int t = tid; t < 128 * nch0; t += 256) {
       const int ch = t % nch0, r = t / nch0;
-      const int64_t mr = tile * 128 + r;
-      uint4 h = make_uint4(0, 0, 0, 0);
-      if (!Hin) h = fu_input8(X, mr, n, net.nin, ch * 8, mu_in, sd_in);
-      else if (mr < n) h = *reinterpret_cast<const uint4*>(Hin + mr * net.kd[0] + ch * 8);
-      *reinterpret_cast<uint4*>(act + fu_off(r, ch * 8, net.kd[0])) = h;
+      if (PRE) {
+        const int64_t mr = tile * 128 + r;
+        uint4 h = make_uint4(0, 0, 0, 0);
+        if (mr < n) h = *reinterpret_cast<const uint4*>(Hin + mr * net.kd[0] + ch * 8);
+        *reinterpret_cast<uint4*>(act + fu_off(r, ch * 8, net.kd[0])) = h;
+      } else {
+        *reinterpret_cast<uint4*>(act + fu_off(r, ch * 8, net.kd[0])) =
+            fu_input8(X, tile * 128 + r, n, net.nin, ch * 8, mu_in, sd_in);
+      }
     }
     const int64_t m = tile * 128 + row;
     for (int l = 0; l < net.L; ++l) {
@@ -998,7 +1004,8 @@ static fvs_status fused_smem_attr() {
   int dev = 0;
   FVS_CUDA(cudaGetDevice(&dev));
   if (dev >= 0 && dev < 64 && attr_set[dev]) return FVS_OK;
-  FVS_CUDA(cudaFuncSetAttribute(k_mlp_predict_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, FU_SMEM));
+  FVS_CUDA(cudaFuncSetAttribute(k_mlp_predict_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, FU_SMEM));
+  FVS_CUDA(cudaFuncSetAttribute(k_mlp_predict_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, FU_SMEM));
   FVS_CUDA(cudaFuncSetAttribute(k_mlp_train_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, FU_SMEM));
   FVS_CUDA(cudaFuncSetAttribute(k_mlp_wgrad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, WG_STAGES * WG_STAGE));
   if (dev >= 0 && dev < 64) attr_set[dev] = true;
@@ -1405,7 +1412,8 @@ FVS_API fvs_status fvs_surrogate_predict(fvs_surrogate s, const double* X, doubl
                                                                       s->Xn.p);
       FVS_COUNT_LAUNCH();
     }
-    k_mlp_predict_tc<<<grid, 256 * groups, net.wbytes + groups * FU_ACT, s->stream>>>(
+    auto predict = pre ? k_mlp_predict_tc<true> : k_mlp_predict_tc<false>;
+    predict<<<grid, 256 * groups, net.wbytes + groups * FU_ACT, s->stream>>>(
         n, net, s->wb.p, s->w32.p, Xd, pre ? s->Xn.p : nullptr, Yd, s->mu_in.p, s->sd_in.p, s->mu_out.p, s->sd_out.p, s->tc_err.p);
     FVS_COUNT_LAUNCH();
   } else {

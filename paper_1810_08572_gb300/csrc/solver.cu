@@ -1015,6 +1015,7 @@ static fvs_status apply_properties(fvs_solver s, const fvs_props* p) {
   FVS_COUNT_LAUNCH();
   s->have_props = true;
   s->eline.ready = false;   // the chains follow the conductive operator
+  s->eline_dt = 0.0;
   FVS_TRY(solver_set_state(s, nullptr, nullptr, 0));
   return conduction_operator(s);
 }
@@ -1087,7 +1088,6 @@ fvs_status solver_set_state(fvs_solver s, const double* T, const double* u, int 
   s->numbered = false;
   s->force_full = false;
   s->amg_ok = false;
-  if (s->n_k > 0) s->eline.ready = false;   // chains of the earlier state's conductivities
   return FVS_OK;
 }
 
@@ -1614,10 +1614,21 @@ fvs_status solver_step(fvs_solver s, double dt, fvs_step_stats* stats) {
       FVS_COUNT_LAUNCH();
       FVS_LAUNCH_CHECK();
       if (it == 1) {
-        fvs_status r = decide ? s->eline.worth(st, s->red, s->Ke, s->jinv_e, lines) : FVS_OK;
-        if (r == FVS_OK && lines && (!s->eline.ready || s->eline.built_from != s->Ke.col.p ||
-                                     s->eline.n != s->Ke.n || s->eline.w != s->Ke.w))
-          r = s->eline.build(st, s->Ke);
+        // an operator that does not depend on the state, of the same pattern: with
+        // k(T) the mesh's Laplacian, at the largest conductivity
+        const Ell& chains = s->n_k > 0 ? m->Lu : s->Ke;
+        if (decide && s->eline_dt != dt) {
+          double kmax = s->has_mold ? s->mold_k : 0.0;
+          for (int i = 0; i < s->n_k; ++i) kmax = std::max(kmax, s->k_val[i]);
+          FVS_TRY(LinePrecond::may(st, s->red, chains, s->n_k > 0 ? 0.5 * kmax : 1.0, s->rcp, m->V, 1.0 / dt,
+                                   s->eline_may));
+          s->eline_dt = dt;
+        }
+        fvs_status r = decide && s->eline_may ? s->eline.worth(st, s->red, s->Ke, s->jinv_e, lines) : FVS_OK;
+        if (r == FVS_OK && lines && (!s->eline.ready || s->eline.built_from != chains.col.p ||
+                                     s->eline.n != chains.n || s->eline.w != chains.w))
+          r = s->eline.build(st, chains);
+        s->eline.A = &s->Ke;
         if (r == FVS_ERR_NOMEM && decide) {
           // the lines need some 150 bytes a cell while their chains are found:
           // without them the step still runs

@@ -56,10 +56,11 @@ struct fvs_solver_s {
   // of the momentum system (per step)
   fvs::DBuf<double> jinv_e, jinv_m;
   // line preconditioner of the energy system, where it pays (else Jacobi):
-  // chosen in every step, chains found once from the energy operator (with
-  // k(T) from that of the first step after a state was set that takes them),
-  // factors per pass
+  // chosen in every step, chains found once (from the energy operator, with k(T)
+  // from the mesh's Laplacian), factors per pass
   fvs::LinePrecond eline;
+  double eline_dt = 0.0;      // step size for which eline_may holds (0: none yet)
+  bool eline_may = false;     // whether any state takes the lines at it
   double time = 0.0;
   int64_t nstep = 0;
 
