@@ -397,8 +397,12 @@ __device__ __forceinline__ void gal_emit(int lane, const int32_t* key, const dou
     const unsigned bal = __ballot_sync(0xffffffffu, head);
     if (FILL && head) {
       const int r = base + __popc(bal & ((1u << lane) - 1));
-      double sum = 0.0;
-      for (int q = e; q < P && key[q] == key[e]; ++q) sum += v[q];
+      double sum = 0.0, mag = 0.0;
+      for (int q = e; q < P && key[q] == key[e]; ++q) {
+        sum += v[q];
+        mag += fabs(v[q]);
+      }
+      if (fabs(sum) <= GAL_NOISE * mag) sum = 0.0;
       if (r < wc) {
         ccol[(int64_t)r * nc + I] = key[e];
         cval[(int64_t)r * nc + I] = sum;

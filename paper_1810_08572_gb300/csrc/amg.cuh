@@ -14,6 +14,12 @@
 
 namespace fvs {
 
+// A Galerkin sum that is rounding next to its entries (below GAL_NOISE of the
+// sum of their magnitudes) is zero: the diagonal of an aggregate that holds a
+// whole liquid pocket would else be inverted as 1e15 times the others, and the
+// pocket, a part of the null space, be counted regular.
+constexpr double GAL_NOISE = 1e-12;
+
 struct AmgLevel {
   Ell own;              // coarse operator (levels >= 1)
   const Ell* A = nullptr;

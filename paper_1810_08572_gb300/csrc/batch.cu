@@ -592,12 +592,9 @@ __global__ void kb_to_double(int64_t n, const float* a, double* b) {
 // ---------------------------------------------------------------------------
 // per-sample Galerkin values on the shared aggregation: coarse entry q gets
 // the sum of the listed fine entries (rows of cells without pressure left out).
-// A sum that is rounding next to its entries is zero: the diagonal of an
-// aggregate that holds a whole liquid pocket of a sample (the aggregates are
-// those of the all-liquid operator) would else be inverted as 1e15 times the
-// others, and its part counted as regular.
+// (GAL_NOISE: the aggregates are those of the all-liquid operator, and a
+// sample's last pockets lie inside single ones)
 // ---------------------------------------------------------------------------
-constexpr double GAL_NOISE = 1e-12;
 __device__ __forceinline__ double gal_sum(double a, double m) { return fabs(a) <= GAL_NOISE * m ? 0.0 : a; }
 __global__ void kb_galerkin0(int64_t nq, int64_t n, int w, int Sp, const int32_t* gptr, const int32_t* gidx,
                              const double* base, const int32_t* ovr, const double* mval, double* cval) {

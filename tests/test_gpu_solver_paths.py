@@ -693,3 +693,38 @@ def test_a_step_without_memory_for_lines_takes_jacobi(fvs):
     assert roomy["e_lin_its"] < 0.6 * tight["e_lin_its"]
     S.close()
     M.close()
+
+
+@pytest.mark.parametrize("seed", [264, 5, 6, 7])
+def test_pockets_inside_an_aggregate_count_as_singular_parts(fvs, seed):
+    """Orthogonal cells, mixed precision, melt freezing in a few long steps:
+    small pockets come to lie inside single aggregates.  Every pressure solve
+    converges on the hierarchy, and the parts it finds are those of the flow
+    (cells joined by faces between melt) that hold pressure."""
+    from scipy.sparse import coo_matrix
+    from scipy.sparse.csgraph import connected_components
+    shape = (18, 7, 17)
+    m = box_mesh(*shape, (0.004383343777328541, 0.010227802147099929, 0.0248389480715284), permute_seed=265)
+    n = len(m["cell_ijk"])
+    T0 = 930.0 + 20.0 * np.random.default_rng(seed).random(n)
+    u0 = np.random.default_rng(seed).normal(scale=2e-3, size=(n, 3))
+    fc = np.asarray(m["face_cells"])
+    inner = fc[:, 1] >= 0
+    M = fvs.Mesh(m)
+    S = fvs.Solver(M, cases.props(precision=1, p_rtol=1e-12, mom_rtol=1e-12, e_rtol=1e-13, e_tol_T=1e-10,
+                                  max_krylov_iters=2000))
+    S.set_state(T0, u0)
+    several = 0
+    for _ in range(10):
+        melt = S.query("T") > cases.AL_ALLOY["T_sol"]
+        st = S.step(0.025160986010573472, allow_not_converged=True)
+        assert st["status"] == 0 and st["fallback"] == 0
+        e = fc[inner][melt[fc[inner, 0]] & melt[fc[inner, 1]]]
+        if st["amg_levels"] > 0 and st["p_rebuilt"] == 1 and len(e):
+            _, lab = connected_components(coo_matrix((np.ones(len(e)), (e[:, 0], e[:, 1])), shape=(n, n)), directed=False)
+            parts = len(np.unique(lab[e[:, 0]]))
+            assert st["n_components"] == parts
+            several = max(several, parts)
+    assert several > 2
+    S.close()
+    M.close()
