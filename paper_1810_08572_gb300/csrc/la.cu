@@ -748,8 +748,12 @@ fvs_status bicgstab(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, c
     if (!proj) {
       FVS_TRY(residual_dot<FIN_START>(s, red, A, x, dextra, b, w.r, w.rh));
     } else {
-      FVS_TRY(vcopy(s, n, w.q, w.r));
-      FVS_TRY(vcopy(s, n, w.q, w.rh));
+      // the null vectors' share of x, which a long recurrence can let grow until
+      // its rounding in A x is the residual, is taken out first
+      FVS_TRY(proj->apply(s, x));
+      FVS_TRY(residual(s, A, x, b, w.r, dextra));
+      FVS_TRY(proj->apply(s, w.r));
+      FVS_TRY(vcopy(s, n, w.r, w.rh));
       FVS_TRY(red.dot(s, n, w.rh, w.r, S_RHO));
     }
     fresh = true;
@@ -877,6 +881,11 @@ fvs_status pcg(cudaStream_t s, Reducer& red, KrylovWork& w, const Ell& A, Precon
     best = res.relres;
     FVS_TRY(vcopy(s, n, x, w.v));
     fresh = true;    // from the true residual, as in bicgstab
+    if (proj) {
+      FVS_TRY(proj->apply(s, x));
+      FVS_TRY(residual(s, A, x, b, w.q, nullptr));
+      FVS_TRY(proj->apply(s, w.q));
+    }
     FVS_TRY(vcopy(s, n, w.q, w.r));
     FVS_TRY(prepare());
   }

@@ -1431,6 +1431,7 @@ static fvs_status solve_pressure(fvs_solver s, double rtol, SolveResult& res, in
   JacobiPrecond J;
   J.A = &s->K;
   FVS_TRY(s->pparts.setup(st, s->K, s->act, s->ppe, s->sw));
+  if (fallback) FVS_TRY(s->pparts.apply(st, s->px));   // what the failed solve left of the null vectors
   FVS_TRY(bicgstab(st, s->red, s->kw, s->K, nullptr, J, s->prhs, s->px, rtol, fallback ? maxit * 4 : maxit,
                    &s->pparts, res));
   FVS_TRY(s->pparts.apply(st, s->px));

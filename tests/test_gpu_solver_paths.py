@@ -728,3 +728,20 @@ def test_pockets_inside_an_aggregate_count_as_singular_parts(fvs, seed):
     assert several > 2
     S.close()
     M.close()
+
+
+def test_restart_takes_the_null_vectors_out_of_the_iterate(fvs):
+    """A jittered box, all melt but a thin frozen layer, whose first pressure
+    solve meets a near-breakdown of BiCGStab: the iterate's constant grows until
+    its rounding is the residual.  The solve converges on the hierarchy after a
+    restart (1e-12 asked for)."""
+    from perf import cases as workloads
+    c = dict(kind="step", nx=23, ny=56, nz=50, jitter=0.2, precision=0, steps=5, front=0.912, physics="flow")
+    s = workloads.prepare(c, 477)
+    S = s["solver"]
+    S.set_state(s["T"])
+    for _ in range(3):
+        st = S.step(1e-3, allow_not_converged=True)
+        assert st["status"] == 0 and st["fallback"] == 0, (st, fvs.fvs_last_error())
+    S.close()
+    s["mesh"].close()
