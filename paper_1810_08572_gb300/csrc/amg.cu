@@ -1610,6 +1610,7 @@ fvs_status Amg::setup(cudaStream_t s, const Ell& A, bool diagonal_first) {
   refreshes = 0;
   lv.clear();
   opt.theta = env_num("FVS_AMG_THETA", opt.theta);
+  opt.theta_fine = env_num("FVS_AMG_THETA", opt.theta_fine);
   opt.omega = env_num("FVS_AMG_OMEGA", opt.omega);
   opt.coarse_scale = env_num("FVS_AMG_SCALE", opt.coarse_scale);
   opt.npre = (int)env_num("FVS_AMG_NPRE", opt.npre);
@@ -1683,7 +1684,7 @@ fvs_status Amg::setup(cudaStream_t s, const Ell& A, bool diagonal_first) {
       for (int attempt = first; attempt < 4; ++attempt) {
         if (first == 0 && attempt == 3 && (double)nc <= opt.mis2_ratio * (double)n) break;   // keep the distance-1 result
         mis2 = attempt == 3;
-        const double theta = (attempt == 0 || mis2) ? opt.theta : 0.0;
+        const double theta = (attempt == 0 || mis2) ? (l == 0 ? opt.theta_fine : opt.theta) : 0.0;
         const int absval = attempt == 2 ? 1 : 0;
         FVS_TRY(st.zero(s));
         if (l == 0) {

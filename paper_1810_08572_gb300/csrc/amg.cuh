@@ -37,7 +37,8 @@ struct AmgLevel {
 };
 
 struct AmgOptions {
-  double theta = 0.08;     // strength threshold
+  double theta = 0.08;       // strength threshold
+  double theta_fine = 0.08;  // the same on the fine level
   double omega = 0.85;     // Jacobi damping
   double coarse_scale = 1.5;  // over-correction of the piecewise-constant coarse correction
   int max_levels = 20;

@@ -1265,6 +1265,16 @@ static fvs_status assemble_pressure(fvs_solver s) {
     // 50 -> 42 ms (39 -> 30); AMG-CG on 96 x 96 x 48 11.0 -> 7.0 ms (53 -> 34).
     s->amg.opt.mis2_from = 0;
     s->amg.opt.coarse_scale = 2.3;
+    // On the fine level of an orthogonal mesh a coupling counts from a quarter of
+    // the row's strongest on: from 0.08 on, sets of five cells spread over a
+    // direction a tenth as strong, and AMG-CG was slower than on distance-1 sets
+    // of that threshold (28 x 94 x 37 cells, couplings 1 : 0.10 : 0.01, 153
+    // iterations and 13.6 ms against 90 and 10.8; now 75 and 6.9.  111 x 22 x 32,
+    // 1 : 0.19 : 0.01, 128 and 11.2 against 78 and 9.2; now 83 and 7.5).  0.2 to 0.4
+    // are the same; on the coarse levels 0.25 is worse (64^3 56 -> 85
+    // iterations).  On skewed meshes, never slower than those sets, 0.25 takes
+    // 7 % off 128^3 but adds 4 % on 83 x 61 x 19: left at 0.08.
+    s->amg.opt.theta_fine = m->orthogonal ? 0.25 : 0.08;
     s->amg.opt.smoother = 1;
     s->amg.opt.cheb_ratio = 6.0;
     s->amg.opt.npre = m->orthogonal ? 2 : 1;
