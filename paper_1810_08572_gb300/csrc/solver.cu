@@ -1172,6 +1172,41 @@ static PpeCtx ppe_ctx(fvs_solver s) {
   return x;
 }
 
+// mean over the rows of the all-liquid pressure operator of the smallest
+// coupling's share of the largest (a property of the mesh)
+__global__ void __launch_bounds__(RB) k_coupling_spread(int64_t n, int w, const int32_t* __restrict__ col,
+                                                        const double* __restrict__ val, double* part,
+                                                        unsigned int* ticket, double* sc, int s0, int s1) {
+  double x = 0.0, y = 0.0;
+  for (int64_t i = blockIdx.x * (int64_t)RB + threadIdx.x; i < n; i += (int64_t)gridDim.x * RB) {
+    double hi = 0.0, lo = 1e300;
+    for (int k = 0; k < w; ++k) {
+      const double a = fabs(val[(int64_t)k * n + i]);
+      if (col[(int64_t)k * n + i] == (int32_t)i || a == 0.0) continue;
+      hi = fmax(hi, a);
+      lo = fmin(lo, a);
+    }
+    if (hi > 0.0) {
+      x += lo / hi;
+      y += 1.0;
+    }
+  }
+  if (grid_fold<OpSum, 2>(x, y, part, ticket)) {
+    sc[s0] = x;
+    sc[s1] = y;
+  }
+}
+static fvs_status coupling_spread(fvs_solver s) {
+  fvs_mesh m = s->mesh;
+  k_coupling_spread<<<s->red.grid(m->Nc), RB, 0, s->stream>>>(m->Nc, m->W, m->Pb.col, m->Pb.val, s->red.part,
+                                                             s->red.ticket, s->red.sc, S_TMP0, S_TMP1);
+  FVS_COUNT_LAUNCH();
+  FVS_LAUNCH_CHECK();
+  FVS_TRY(s->red.fetch(s->stream));
+  s->spread = s->red.host[S_TMP1] > 0.0 ? s->red.host[S_TMP0] / s->red.host[S_TMP1] : 1.0;
+  return FVS_OK;
+}
+
 static fvs_status assemble_pressure(fvs_solver s) {
   fvs_mesh m = s->mesh;
   cudaStream_t st = s->stream;
@@ -1265,16 +1300,18 @@ static fvs_status assemble_pressure(fvs_solver s) {
     // 50 -> 42 ms (39 -> 30); AMG-CG on 96 x 96 x 48 11.0 -> 7.0 ms (53 -> 34).
     s->amg.opt.mis2_from = 0;
     s->amg.opt.coarse_scale = 2.3;
-    // On the fine level of an orthogonal mesh a coupling counts from a quarter of
-    // the row's strongest on: from 0.08 on, sets of five cells spread over a
-    // direction a tenth as strong, and AMG-CG was slower than on distance-1 sets
-    // of that threshold (28 x 94 x 37 cells, couplings 1 : 0.10 : 0.01, 153
-    // iterations and 13.6 ms against 90 and 10.8; now 75 and 6.9.  111 x 22 x 32,
-    // 1 : 0.19 : 0.01, 128 and 11.2 against 78 and 9.2; now 83 and 7.5).  0.2 to 0.4
-    // are the same; on the coarse levels 0.25 is worse (64^3 56 -> 85
-    // iterations).  On skewed meshes, never slower than those sets, 0.25 takes
-    // 7 % off 128^3 but adds 4 % on 83 x 61 x 19: left at 0.08.
-    s->amg.opt.theta_fine = m->orthogonal ? 0.25 : 0.08;
+    // On the fine level of an orthogonal mesh with a direction whose couplings are
+    // below a tenth of the strongest, a coupling counts from a quarter of the
+    // row's strongest on: from 0.08 on, sets of five cells spread over the middle
+    // direction, and AMG-CG was slower than on distance-1 sets of that threshold
+    // (28 x 94 x 37 cells, couplings 1 : 0.10 : 0.01, 153 iterations and 13.6 ms
+    // against 90 and 10.8; now 75 and 6.9.  111 x 22 x 32, 1 : 0.19 : 0.01, 128 and
+    // 11.2 against 78 and 9.2; now 83 and 7.5).  0.2 to 0.4 are the same; on the
+    // coarse levels 0.25 is worse (64^3 56 -> 85 iterations), and so it is where
+    // all three directions count (23 x 30 x 6, 1 : 0.39 : 0.23, 1.1 -> 1.4 ms).  Skewed
+    // meshes, never slower than on distance-1 sets, keep 0.08.
+    if (m->orthogonal && s->spread < 0.0) FVS_TRY(coupling_spread(s));
+    s->amg.opt.theta_fine = m->orthogonal && s->spread < 0.1 ? 0.25 : 0.08;
     s->amg.opt.smoother = 1;
     s->amg.opt.cheb_ratio = 6.0;
     s->amg.opt.npre = m->orthogonal ? 2 : 1;

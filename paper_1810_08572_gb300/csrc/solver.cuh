@@ -96,6 +96,7 @@ struct fvs_solver_s {
   fvs::Ell K;             // pressure: K = -A on LM cells (identity rows for non-flowing)
   fvs::Ell Kp;            // K's diagonal and face couplings, the rest lumped (AMG operator)
   bool pc_compact = false;        // the hierarchy was built on Kp
+  double spread = -1.0;           // coupling_spread of the mesh (< 0: not formed yet)
   fvs::DBuf<double> mrhs, mx;     // [3*nact]
   fvs::DBuf<double> prhs, px;     // [nact]
   fvs::DBuf<double> pv, fSv;      // vertex pressure sums / solid fractions [Nv]

@@ -747,7 +747,8 @@ def test_restart_takes_the_null_vectors_out_of_the_iterate(fvs):
     s["mesh"].close()
 
 
-@pytest.mark.parametrize("shape", [(28, 94, 37), (111, 22, 32), (25, 71, 31), (96, 96, 48), (40, 40, 40)])
+@pytest.mark.parametrize("shape", [(28, 94, 37), (111, 22, 32), (25, 71, 31), (96, 96, 48), (40, 40, 40), (23, 30, 6),
+                                   (47, 88, 5)])
 def test_aggregates_follow_the_strong_direction(fvs, monkeypatch, shape):
     """AMG-CG on boxes whose couplings in the second direction are a tenth to a
     fifth of the strongest (and on thin and mildly thin cells): at most 1.25
