@@ -1396,7 +1396,7 @@ __global__ void k_part_sub(int64_t n, const int32_t* lab, const double* sum, con
 
 fvs_status PartProjector::setup(cudaStream_t s, const Ell& K, const int32_t* act, const uint8_t* ppe,
                                 ScanWork& sw) {
-  const int64_t n = K.n;
+  n = K.n;
   ncomp = 0;
   if (n == 0) return FVS_OK;
   FVS_TRY(par.alloc(n + 1)); FVS_TRY(root_flag.alloc(n + 1)); FVS_TRY(root_id.alloc(n + 1));
@@ -1432,7 +1432,6 @@ fvs_status PartProjector::setup(cudaStream_t s, const Ell& K, const int32_t* act
 }
 
 fvs_status PartProjector::apply(cudaStream_t s, double* v) {
-  const int64_t n = lab.n ? (int64_t)lab.n - 1 : 0;
   if (ncomp == 0 || n == 0) return FVS_OK;
   FVS_TRY(sum.zero(s));
   k_part_sum<<<stride_grid(n, 256), 256, 0, s>>>(n, lab, v, sum); FVS_COUNT_LAUNCH();

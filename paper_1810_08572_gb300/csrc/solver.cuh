@@ -23,6 +23,7 @@ struct PartProjector : Projector {
   DBuf<double> sum, cnt;
   DBuf<int> changed;
   int ncomp = 0;
+  int64_t n = 0;    // rows of the system last set up (lab may hold more, of a larger one before)
   // labels of the rows i with ppe[act[i]] (the others are identity rows and
   // stay out of every part)
   fvs_status setup(cudaStream_t s, const Ell& K, const int32_t* act, const uint8_t* ppe, ScanWork& sw);

@@ -775,3 +775,31 @@ def test_aggregates_follow_the_strong_direction(fvs, monkeypatch, shape):
     for k, v in (("SMOOTHER", "0"), ("MIS2_FROM", "99"), ("SCALE", "1.5"), ("NPRE", "1"), ("NPOST", "1"), ("THETA", "0.08")):
         monkeypatch.setenv("FVS_AMG_" + k, v)
     assert two <= 1.25 * its()
+
+
+@pytest.mark.parametrize("jitter", [0.0, 0.2])
+def test_single_grid_solve_of_a_shrinking_system(fvs, jitter):
+    """Melt freezing from one wall in steps of a few layers: the system is
+    renumbered smaller several times, and the single-grid solve's parts are
+    those of the present rows (not of rows that an earlier, larger numbering
+    had).  Every step converges, to the fields of the hierarchy's solve."""
+    shape = (24, 10, 4)
+    m = box_mesh(*shape, (0.024, 0.010, 0.004), jitter=jitter, jitter_seed=5, permute_seed=6)
+    T0 = 860.0 + 3.0 * m["cell_ijk"][:, 0] + np.random.default_rng(2).random(len(m["cell_ijk"]))
+    walls = [(cases.BC_DIRICHLET, 600.0)] + [(cases.BC_ADIABATIC, 0.0)] * 5
+    out = []
+    for p_solver in (1, 0):
+        M = fvs.Mesh(m)
+        S = fvs.Solver(M, cases.props(walls=walls, p_solver=p_solver, **TIGHT))
+        S.set_state(T0, np.random.default_rng(3).normal(scale=2e-3, size=(len(T0), 3)))
+        active = []
+        for _ in range(12):
+            st = S.step(0.03, allow_not_converged=True)
+            assert st["status"] == 0, (p_solver, active, fvs.fvs_last_error())
+            active.append(st["n_active"])
+        assert active[0] > active[-1] > 0 and len(set(active)) >= 4
+        out.append({k: S.query(k) for k in ("T", "U", "P")})
+        S.close()
+        M.close()
+    for k in out[0]:
+        assert rel(out[0][k], out[1][k]) <= 1e-8, k
