@@ -1,6 +1,7 @@
 // Aggregation AMG: setup (strength, parallel MIS aggregation, Galerkin
 // coarse operators, pinned dense coarsest inverse, component labels) and the
-// V-cycle (damped Jacobi, piecewise-constant restriction / prolongation).
+// V-cycle (Chebyshev or weighted-Jacobi sweeps, piecewise-constant restriction /
+// prolongation).
 #include <algorithm>
 #include <chrono>
 #include <climits>
@@ -168,9 +169,9 @@ __global__ void k_assign(int64_t n, int w, const int32_t* col, const double* val
 }
 
 // ---------------------------------------------------------------------------
-// Distance-2 independent set (used where the distance-1 set coarsens a level
-// by less than the accepted ratio: chains and star-like couplings of small
-// coarse levels).  A node becomes a root when its key is the largest among
+// Distance-2 independent set (from level mis2_from on; before it where the
+// distance-1 set coarsens a level by less than the accepted ratio: chains and
+// star-like couplings of small coarse levels).  A node becomes a root when its key is the largest among
 // the undecided nodes within two strong hops; nodes within two hops of a root
 // drop out.  Keys: hash of the index, then the index (0 = not undecided).
 // ---------------------------------------------------------------------------
@@ -1353,8 +1354,10 @@ static int coarse_lanes(const AmgLevel& L) {
   // large levels are bandwidth-bound: two lanes keep whole sectors per slot
   // and most lanes busy; small levels are latency-bound: more lanes per row
   // shorten each lane's chain of dependent gathers (128^3 cavity, cold
-  // launches: 905k-row level 37/43 us with two lanes against 47/69 us with
-  // four; 6k-row level 12 us with two against 8 us with four)
+  // launches, residual/Chebyshev: 566,929-row level 36/43 us with one lane,
+  // 27/41 with two; 6,503-row level with 1, 2, 4, 8 lanes 14.9/19.6,
+  // 11.6/11.3, 8.1/7.8, 6.4/6.0 us.  One count forced on every level, three
+  // steps: 160, 155, 165, 191 ms against 154 by this rule)
   const double mean = L.n > 0 ? L.stored / (double)L.n : 0.0;
   if (mean < 6.0) return 1;
   return L.n >= 65536 ? 2 : (L.n >= 8192 ? 4 : 8);

@@ -1164,8 +1164,8 @@ static fvs_status level_applyf(Batch& B, int l, const float* x, const float* b, 
   return bapplyf(B, OpCoarseT<float>{L.n, L.w, L.col, L.valf.p, L.rlen}, x, b, y, mode, dinv, omega, &L.shape);
 }
 
-// one V-cycle on level l: y = M^-1 b (damped Jacobi, piecewise-constant
-// transfers with over-correction, pinned dense coarsest inverse); V = double,
+// one V-cycle on level l: y = M^-1 b (weighted Jacobi, V(2,2) under CG and
+// V(1,1) under BiCGStab; piecewise-constant transfers with over-correction, pinned dense coarsest inverse); V = double,
 // or float for the mixed-precision path (FP32 copies of every level)
 template <typename V>
 static fvs_status bvcycle_t(Batch& B, int l, const V* b, V* y, bool x0_ready = false) {

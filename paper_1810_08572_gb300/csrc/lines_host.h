@@ -1,6 +1,7 @@
-// Host part of the line preconditioner (la.cuh, lines.cu): the chains of
-// strongly coupled cells and their storage layout.  Plain C++ (no CUDA), so
-// that the layout can be checked without a GPU.
+// The rule of the line preconditioner's chains (la.cuh) in plain C++: which
+// strongly coupled cells form a line, and the lines' storage layout.  The
+// library finds the lines on the device (lines.cu); this form states what
+// they have to be, for the tests that compare the two.
 #pragma once
 
 #include <algorithm>
