@@ -1308,8 +1308,10 @@ static fvs_status assemble_pressure(fvs_solver s) {
     // against 90 and 10.8; now 75 and 6.9.  111 x 22 x 32, 1 : 0.19 : 0.01, 128 and
     // 11.2 against 78 and 9.2; now 83 and 7.5).  0.2 to 0.4 are the same; on the
     // coarse levels 0.25 is worse (64^3 56 -> 85 iterations), and so it is where
-    // all three directions count (23 x 30 x 6, 1 : 0.39 : 0.23, 1.1 -> 1.4 ms).  Skewed
-    // meshes, never slower than on distance-1 sets, keep 0.08.
+    // all three directions count (23 x 30 x 6, 1 : 0.39 : 0.23, 1.1 -> 1.4 ms).  Of 150
+    // drawn cases a dozen went up to 1.5 times as fast, one slower (52 x 95 x 21,
+    // FP32 cycle, 3.3 -> 3.8 ms; 5.0 on distance-1 sets).  Skewed meshes, never
+    // slower than on distance-1 sets, keep 0.08.
     if (m->orthogonal && s->spread < 0.0) FVS_TRY(coupling_spread(s));
     s->amg.opt.theta_fine = m->orthogonal && s->spread < 0.1 ? 0.25 : 0.08;
     s->amg.opt.smoother = 1;
