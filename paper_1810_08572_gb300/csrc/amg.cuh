@@ -6,6 +6,7 @@
 // per singular connected part -- the disjoint liquid pockets of Section 2.5).
 #pragma once
 
+#include <algorithm>
 #include <memory>
 #include <vector>
 
@@ -104,6 +105,9 @@ struct Amg : Precond {
   // subtract the component mean on every singular component (fine level)
   fvs_status project(cudaStream_t s, double* v);
   int single_part(MeanPart& m);   // see Projector::single
+  int singular_parts() const {
+    return (int)std::count_if(sing_host.begin(), sing_host.end(), [](uint8_t c) { return c != 0; });
+  }
   int levels() const { return (int)lv.size(); }
 
  private:

@@ -1442,10 +1442,54 @@ fvs_status PartProjector::apply(cudaStream_t s, double* v) {
   return FVS_OK;
 }
 
+// the hierarchy with its parts' means taken out of what it returns
+struct ProjectedAmg : Precond {
+  Amg* amg = nullptr;
+  fvs_status apply(cudaStream_t s, const double* r, double* z) override {
+    FVS_TRY(amg->apply(s, r, z));
+    return amg->project(s, z);
+  }
+  uint64_t signature() const override { return amg->signature() ^ 0x70726f6aULL; }
+};
+
+// Zero mean of the solution on each part of the hierarchy.  Its parts are
+// connected across faces.  On a skewed mesh two of them that touch along an
+// edge or at a vertex are coupled by the vertex values in one direction: K has
+// a null vector for each of them, but it is not the constant on the part, and
+// taking the means out of a solution leaves a residual (up to 1e-2 where 1e-12
+// was asked for).  The solution with zero means is then found by solving on
+// from the projected one, with the means taken out of every search direction;
+// if that does not get there, the solution stays as the first solve left it.
+static fvs_status project_pressure(fvs_solver s, double rtol, SolveResult& res) {
+  cudaStream_t st = s->stream;
+  if (s->mesh->orthogonal || s->amg.singular_parts() < 2) return s->amg.project(st, s->px);
+  const int64_t n = s->K.n;
+  DBuf<double> solved;
+  FVS_TRY(solved.alloc(n));
+  FVS_TRY(vcopy(st, n, s->px, solved));
+  FVS_TRY(s->amg.project(st, s->px));
+  FVS_TRY(residual(st, s->K, s->px, s->prhs, s->kw.q, nullptr));
+  FVS_TRY(s->amg.project(st, s->kw.q));
+  FVS_TRY(vcopy(st, n, s->prhs, s->kw.r));
+  FVS_TRY(s->amg.project(st, s->kw.r));
+  FVS_TRY(s->red.dot2(st, n, s->kw.r, s->kw.r, s->kw.q, s->kw.q, S_BB, S_RR));
+  FVS_TRY(s->red.fetch(st));
+  if (sqrt(s->red.host[S_RR]) <= 10.0 * rtol * sqrt(s->red.host[S_BB])) return FVS_OK;
+  ProjectedAmg M;
+  M.amg = &s->amg;
+  SolveResult r;
+  FVS_TRY(bicgstab(st, s->red, s->kw, s->K, nullptr, M, s->prhs, s->px, rtol, s->props.max_krylov_iters, &s->aproj, r));
+  s->p_more_its = r.iters;
+  if (!r.converged) return vcopy(st, n, solved, s->px);
+  res.relres = r.relres;
+  return FVS_OK;
+}
+
 // solve K x = rhs (compact) with the configured method; fills stats
 static fvs_status solve_pressure(fvs_solver s, double rtol, SolveResult& res, int& fallback) {
   cudaStream_t st = s->stream;
   fallback = 0;
+  s->p_more_its = 0;
   const int maxit = s->props.max_krylov_iters;
   // on a refreshed hierarchy a slow solve means it has gone stale (e.g. a
   // liquid pocket split by freezing cells): stop early and let the caller
@@ -1458,7 +1502,7 @@ static fvs_status solve_pressure(fvs_solver s, double rtol, SolveResult& res, in
     else
       FVS_TRY(bicgstab(st, s->red, s->kw, s->K, nullptr, s->amg, s->prhs, s->px, rtol, cap, &s->aproj, res, 0.0,
                        &s->g_p));
-    if (res.converged) FVS_TRY(s->amg.project(st, s->px));
+    if (res.converged) FVS_TRY(project_pressure(s, rtol, res));
     return FVS_OK;
   }
   if (s->amg_ok) {
@@ -1468,7 +1512,7 @@ static fvs_status solve_pressure(fvs_solver s, double rtol, SolveResult& res, in
       FVS_TRY(bicgstab(st, s->red, s->kw, s->K, nullptr, s->amg, s->prhs, s->px, rtol, maxit, &s->aproj, res, 0.0,
                        &s->g_p));
     if (res.converged) {
-      FVS_TRY(s->amg.project(st, s->px));
+      FVS_TRY(project_pressure(s, rtol, res));
       return FVS_OK;
     }
   }
@@ -1607,7 +1651,7 @@ fvs_status solver_step(fvs_solver s, double dt, fvs_step_stats* stats) {
     }
     // periodic renumbering and rebuild after a run of refreshes
     if (S.p_rebuilt == 2 && ++s->steps_since_setup >= 25) s->force_full = true;
-    S.p_its = r.iters;
+    S.p_its = r.iters + s->p_more_its;
     S.p_relres = r.relres;
     S.fallback = fb;
     if (!r.converged) {
@@ -1795,7 +1839,7 @@ fvs_status solver_pressure_solve(fvs_solver s, const double* rhs, double* p_out,
   k_p_out<<<stride_grid(m->Nc, 256), 256, 0, st>>>(m->Nc, s->map, s->ppe, m->cell_in, s->px, p_out); FVS_COUNT_LAUNCH();
   FVS_LAUNCH_CHECK();
   FVS_CUDA(cudaStreamSynchronize(st));
-  if (iters) *iters = r.iters;
+  if (iters) *iters = r.iters + s->p_more_its;
   if (relres) *relres = r.relres;
   return r.converged ? FVS_OK : FVS_ERR_NOT_CONVERGED;
 }

@@ -43,6 +43,7 @@ struct fvs_solver_s {
   bool amg_full = false;      // the hierarchy was built (not refreshed) this step
   int steps_since_setup = 0;
   int p_its_ref = 0;          // pressure iterations right after the last full setup
+  int p_more_its = 0;         // iterations that project_pressure took on top
   int64_t nlm = 0;            // liquid + mushy cells
   fvs_props props{};
   std::vector<fvs_patch_bc> bc;
